@@ -374,12 +374,12 @@ fr_status fr_profile_read(fr_ctx* ctx, const char* region, double* ms, uint64_t*
  * replay, so the timed regions run as they do unprofiled. Stays set until changed. */
 fr_status fr_profile_only(fr_ctx* ctx, const char* prefix);
 /* NTT autotuner (run by fr_setup on device contexts unless the environment sets
- * FR_NTT_TUNE=0): for N >= 2^15 it times each shape of a forward + inverse transform on this
+ * FR_NTT_TUNE=0): for N >= 2^14 it times each shape of a forward + inverse transform on this
  * GPU for one batch size per bucket (<= 4, <= 16, <= 64, > 64 limb-polynomials; best of 3
  * runs after a warm-up) and keeps the fastest. Shapes 0..3: radix-8 two-pass kernels (8
  * residues per thread), bit 0 = 8 columns per column-pass CTA (else 4), bit 1 = 256-thread
  * row-pass CTAs (else 128); shape 4 (N = 2^16 only): one launch per transform, a cluster of 8
- * CTAs per polynomial exchanging through distributed shared memory; shape 5 (N = 2^16 only):
+ * CTAs per polynomial exchanging through distributed shared memory; shape 5 (N >= 2^14):
  * radix-16 two-pass kernels (16 residues per thread, one exchange per pass). shapes[4]
  * receives the chosen shape per bucket, us[24] (may be NULL) the measured microseconds,
  * bucket-major, 6 per bucket (-1: shape not available). */
@@ -406,9 +406,9 @@ fr_status fr_inject_alloc_failure(fr_ctx* ctx, int64_t after);
  * outputs, FR_ERR_LEVEL for a level outside the chain. */
 fr_status fr_ntt_time(fr_ctx* ctx, uint32_t npolys, uint32_t level, uint32_t reps, double* us_fwd, double* us_inv);
 
-/* Arithmetic ceiling of the NTT on `device`: forward butterflies (Harvey lazy
- * reduction, Shoup twiddle product, 64-bit residues) per second with every operand in
- * registers, measured by a short microbenchmark. Used as the ALU roofline peak. */
+/* Arithmetic ceiling of the NTT on `device`: forward butterflies of 64-bit residues (the
+ * library's cheapest twiddle product, primes of at most 51 bits) per second with every operand
+ * in registers, measured by a short microbenchmark. Used as the ALU roofline peak. */
 fr_status fr_butterfly_peak(int device, double* butterflies_per_s);
 /* FP64 operations per second on `device`: eight independent fused multiply-add chains per
  * thread with register operands, 8 CTAs of 256 threads per SM (an FMA counts as two). The

@@ -7,6 +7,7 @@
 // reduction by R^2 mod q). All primes are below 2^61, which the lazy
 // accumulation bounds below rely on.
 #pragma once
+#include <cuda_runtime.h>
 #include <cstdint>
 
 typedef uint64_t u64;
@@ -16,10 +17,73 @@ struct DevPrime {
     u64 q;       // modulus
     u64 qinv;    // q^-1 mod 2^64 (Montgomery)
     u64 r2;      // 2^128 mod q
-    u64 ninv;    // N^-1 mod q
-    u64 ninv_s;  // Shoup quotient of ninv
     u64 one_s;   // floor(2^64 / q): Shoup quotient of 1 (x mod q for any 64-bit x)
+    // constants of the NTT's products by twiddles (see TwClass)
+    u64 c2;      // classes 0, 1: 2^(S + 32) mod q, below 2^32
+    u64 off;     // classes 0, 1: the smallest multiple of q not below the bound of a product
+    u64 big;     // class 1: the largest multiple of q up to 2^63
+    u32 bsh;     // classes 0, 1: bits(q) - 32
+    u32 c;       // classes 0, 1: 2^bits(q) - q
+    u32 cls;     // twiddle class
+    u32 pad;
+    uint4 tw_ninv;   // N^-1 as a twiddle of the class
+    uint4 tw_wninv;  // N^-1 times the inverse transform's last twiddle, likewise
 };
+
+// Products x w by the twiddles of the NTT. A twiddle is 16 bytes, in the format of its prime's
+// class:
+//
+// Classes 0 and 1 store w and v = w 2^32 mod q, each split at bit S: (w mod 2^S, w >> S, v mod
+// 2^S, v >> S). With x = xh 2^32 + xl the sum xl w + xh v = a0 + a1 2^S is congruent to x w, and
+// a1's high word counts the 2^(S+32) in it, which are worth c2 = 2^(S+32) mod q each:
+//   r = a0 + (a1 mod 2^32) 2^S + (a1 >> 32) c2.
+// That is six 32 x 32 + 64 -> 64 multiply-adds and nothing else, where the 64-bit Shoup product
+// (quotient x ws >> 64, then x w - quotient q) takes five, four 32-bit products and the carries
+// between them. On GB300 a wide product costs 4.2 issue cycles a warp, a 32-bit product or a shift
+// 2, an add 1; butterflies with operands in registers measured 29 cycles a warp against 39 (44
+// with a conditional subtraction of Harvey's ranges). r is not reduced below 2q: it lies in
+// [0, bound),
+//   bound = (a1max >> 32) c2 + 2^(S+32) + 2^(S+33),
+// and twiddle_class() accepts a prime only when the sums of a transform stay below 2^64:
+//   class 0 (S = 20, primes of at most 51 bits close below a power of two): 16 products and a
+//     residue fit in 64 bits, so a forward transform needs no conditional subtraction at all;
+//   class 1 (S = 29, up to 60 bits): a product and a value below 2^63 fit.
+// Class 2 (any prime below 2^61): (w, floor(w 2^64 / q)), the Shoup product.
+constexpr int kTwS0 = 20, kTwS1 = 29;
+
+__device__ __forceinline__ u64 mul_wide(u32 a, u32 b) {
+    u64 r;
+    asm("mul.wide.u32 %0, %1, %2;" : "=l"(r) : "r"(a), "r"(b));
+    return r;
+}
+__device__ __forceinline__ u64 mad_wide(u32 a, u32 b, u64 c) {
+    u64 r;
+    asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+    return r;
+}
+
+// x w, lazily reduced (any 64-bit x); qm: class 2 the modulus, else DevPrime::c2
+template <int CLS>
+__device__ __forceinline__ u64 mul_tw(u64 x, const uint4& w, u64 qm) {
+    if constexpr (CLS == 2) {
+        const u64 W = (u64)w.y << 32 | w.x, WS = (u64)w.w << 32 | w.z;
+        return x * W - __umul64hi(x, WS) * qm;  // in [0, 2q)
+    } else {
+        constexpr int S = CLS == 0 ? kTwS0 : kTwS1;
+        const u32 xl = (u32)x, xh = (u32)(x >> 32);
+        const u64 a1 = mad_wide(xh, w.w, mul_wide(xl, w.y));
+        const u64 a0 = mad_wide(xh, w.z, mul_wide(xl, w.x));
+        return mad_wide((u32)a1, 1u << S, mad_wide((u32)(a1 >> 32), (u32)qm, a0));
+    }
+}
+
+// any value of a transform to below 2q (classes 0, 1: to below 2^bits(q) plus a little, at most
+// 2q): the bits from bits(q) up times c = 2^bits(q) - q
+__device__ __forceinline__ u64 fold_top(u64 v, u32 bsh, u32 c) {
+    const u32 vh = (u32)(v >> 32);
+    const u32 h = vh >> bsh;
+    return mad_wide(h, c, (u64)(vh - (h << bsh)) << 32 | (u32)v);
+}
 
 __device__ __forceinline__ u64 add_mod(u64 a, u64 b, u64 q) {
     u64 s = a + b;
@@ -27,7 +91,8 @@ __device__ __forceinline__ u64 add_mod(u64 a, u64 b, u64 q) {
 }
 __device__ __forceinline__ u64 sub_mod(u64 a, u64 b, u64 q) { return a >= b ? a - b : a + q - b; }
 
-// x * w mod q for a constant w with Shoup quotient ws; any 64-bit x.
+// x * w mod q for a constant w with Shoup quotient ws; any 64-bit x. Lazily: in [0, 2q).
+__device__ __forceinline__ u64 mul_shoup_lazy(u64 x, u64 w, u64 ws, u64 q) { return x * w - __umul64hi(x, ws) * q; }
 __device__ __forceinline__ u64 mul_shoup(u64 x, u64 w, u64 ws, u64 q) {
     u64 hi = __umul64hi(x, ws);
     u64 r = x * w - hi * q;

@@ -91,7 +91,6 @@ struct fr_ctx {
     bool own_stream = false;
     RingDev rd{};
     DevPrime* d_primes = nullptr;
-    u64 *d_tw = nullptr, *d_itw = nullptr;  // (twiddle, Shoup quotient) pairs [primes][N][2]
     unsigned* d_rot = nullptr;
     double *d_zr = nullptr, *d_zi = nullptr;
     uint32_t ell = 0, n1 = 0, schedule = 0, cheb_n = 0;
@@ -1258,37 +1257,113 @@ u64 inv_mod_2_64(u64 q) {
 // 30-bit halves of a residue below 2^60: low half in bits 0..29, high half in bits 32..61
 u64 split30_host(u64 x) { return (x & 0x3fffffffull) | ((x >> 30) << 32); }
 
+// Twiddle class of prime q and its constants in d (see mul_tw): the first class whose sums
+// provably stay in 64 bits.
+void twiddle_class(u64 q, DevPrime& d) {
+    int b = 64;
+    while (!(q >> (b - 1))) --b;
+    const u128 two64 = (u128)1 << 64;
+    for (u32 cls = 0; cls < 2; ++cls) {
+        const int S = cls == 0 ? kTwS0 : kTwS1;
+        const u64 e = (u64)1 << (S + 32), m = e / q * q, wh = (q - 1) >> S;
+        if (b <= 33 || m == 0 || wh >> 31 || (e - m) >> 32) continue;
+        const u64 a1 = 0xffffffffull * (2 * wh);  // wh < 2^31: no overflow
+        // the product's bound: (a1 >> 32) c2 + (a1 mod 2^32) 2^S + a0
+        const u128 bound = (u128)(a1 >> 32) * (e - m) + (u128)e + (u128)2 * e;
+        const u64 c = ((u64)1 << b) - q, top = ((u64)1 << b) - 1;
+        auto folded = [&](u128 v) { return (u128)top + (v >> b) * c; };  // largest result of fold_top
+        if (bound >> 63 || c >> 32) continue;
+        d.off = (u64)((bound + q - 1) / q) * q;
+        if (cls == 0) {
+            // forward: a canonical residue and 16 stages of at most off each; inverse: operands
+            // below off when a phase starts, sums of 4 stages, folded to below the bound at its end
+            const u128 fwd = (u128)q + (u128)16 * d.off, inv = (u128)16 * d.off;
+            if (fwd >= two64 || folded(fwd) >= (u128)2 * q || folded(inv) >= bound || (fwd >> b) >> 32) continue;
+        } else {
+            // forward: below big after the conditional subtraction, plus off; inverse: both
+            // operands below big
+            d.big = ((u64)1 << 63) / q * q;
+            if (bound >= d.big || (u128)d.big + d.off >= two64 || folded(two64 - 1) >= (u128)2 * q) continue;
+        }
+        d.cls = cls;
+        d.c2 = e - m;
+        d.bsh = (u32)(b - 32);
+        d.c = (u32)c;
+        return;
+    }
+    d.cls = 2;
+    d.off = d.big = 0;
+}
+// Twiddles of one prime in the format of its class.
+struct Twiddler {
+    const DevPrime& d;
+    u64 r32, r32_s;  // 2^32 mod q and its Shoup quotient
+    explicit Twiddler(const DevPrime& dp) : d(dp), r32(((u64)1 << 32) % dp.q), r32_s(frh::shoup_quot(r32, dp.q)) {}
+    uint4 operator()(u64 w) const {
+        if (d.cls == 2) {
+            const u64 ws = frh::shoup_quot(w, d.q);
+            return make_uint4((u32)w, (u32)(w >> 32), (u32)ws, (u32)(ws >> 32));
+        }
+        const int S = d.cls == 0 ? kTwS0 : kTwS1;
+        const u64 v = frh::mul_shoup(w, r32, r32_s, d.q), mask = ((u64)1 << S) - 1;
+        return make_uint4((u32)(w & mask), (u32)(w >> S), (u32)(v & mask), (u32)(v >> S));
+    }
+};
+// One row's twiddles (from a prime's natural-order table) in the order of row_tw_index.
+void row_twiddles(const uint4* nat, int N, int logC, int rho, uint4* out) {
+    const int C = 1 << logC;
+    for (int lb = 0; lb < 4; ++lb)
+        for (int u = 0; u < (8 >> lb); ++u) {
+            out[row_tw_index(logC, true, lb, u, 0)] = nat[((N + rho * C) >> (logC - 3 + lb)) + u];
+            if (lb <= logC - 5)
+                for (int tau = 0; tau < C / 16; ++tau)
+                    out[row_tw_index(logC, false, lb, u, tau)] = nat[((N + rho * C + tau * 16) >> (lb + 1)) + u];
+        }
+}
+
 void build_tables(fr_ctx* c) {
     const frh::Ring& R = c->R;
     const int N = R.N, T = R.total();
     // primes
     std::vector<DevPrime> dp(T);
+    bool fast = true;
     for (int i = 0; i < T; ++i) {
         const u64 q = R.primes[i];
-        u64 inv = 1;  // Newton iteration for q^-1 mod 2^64
-        for (int k = 0; k < 7; ++k) inv *= 2 - q * inv;
-        dp[i].q = q;
-        dp[i].qinv = inv;
+        DevPrime& d = dp[i];
+        std::memset(&d, 0, sizeof(d));
+        d.q = q;
+        d.qinv = inv_mod_2_64(q);
         const u64 r1 = (u64)(((u128)1 << 64) % q);
-        dp[i].r2 = frh::mulm(r1, r1, q);
-        dp[i].ninv = R.tabs[i].ninv;
-        dp[i].ninv_s = frh::shoup_quot(R.tabs[i].ninv, q);
-        dp[i].one_s = frh::shoup_quot(1, q);
+        d.r2 = frh::mulm(r1, r1, q);
+        d.one_s = frh::shoup_quot(1, q);
+        twiddle_class(q, d);
+        fast = fast && d.cls != 2;
+        const u64 ninv = R.tabs[i].ninv;
+        d.tw_ninv = Twiddler(d)(ninv);
+        d.tw_wninv = Twiddler(d)(frh::mulm(ninv, R.tabs[i].itw[1], q));
     }
     c->d_primes = upload_persistent(c, dp.data(), T);
-    // twiddles as (w, Shoup quotient) pairs, one 16-byte load per twiddle: [T][N][2]
-    std::vector<u64> tw((size_t)2 * T * N), itw((size_t)2 * T * N);
-    for (int i = 0; i < T; ++i)
-        for (int k = 0; k < N; ++k) {
-            const size_t o = 2 * ((size_t)i * N + k);
-            tw[o] = R.tabs[i].tw[k];
-            tw[o + 1] = R.tabs[i].tws[k];
-            itw[o] = R.tabs[i].itw[k];
-            itw[o + 1] = R.tabs[i].itws[k];
+    // twiddles, 16 bytes each, in the format of their prime's class: [T][N], and for the radix-16
+    // row pass (N >= 2^14) in its order
+    const bool rows = R.logN >= 14;
+    const int logC = R.logN - R.logN / 2, C = 1 << logC;
+    auto upload_tw = [&](bool inv, uint4** nat, uint4** row) {
+        std::vector<uint4> t((size_t)T * N), r(rows ? (size_t)T * N : 0);
+        for (int i = 0; i < T; ++i) {
+            const auto& w = inv ? R.tabs[i].itw : R.tabs[i].tw;
+            uint4* ti = t.data() + (size_t)i * N;
+            const Twiddler tw(dp[i]);
+            for (int k = 0; k < N; ++k) ti[k] = tw(w[k]);
+            for (int rho = 0; rows && rho < N / C; ++rho)
+                row_twiddles(ti, N, logC, rho, r.data() + (size_t)i * N + (size_t)rho * C);
         }
-    c->d_tw = upload_persistent(c, tw.data(), tw.size());
-    c->d_itw = upload_persistent(c, itw.data(), itw.size());
-    c->rd = RingDev{R.logN, N, T, c->d_primes, (const ulonglong2*)c->d_tw, (const ulonglong2*)c->d_itw};
+        *nat = upload_persistent(c, t.data(), t.size());
+        *row = rows ? upload_persistent(c, r.data(), r.size()) : nullptr;
+    };
+    uint4 *tw, *itw, *rtw, *irtw;
+    upload_tw(false, &tw, &rtw);
+    upload_tw(true, &itw, &irtw);
+    c->rd = RingDev{R.logN, N, T, c->d_primes, tw, itw, rtw, irtw, fast};
     c->d_rot = upload_persistent(c, R.rot_group.data(), R.rot_group.size());
     c->d_zr = upload_persistent(c, R.zr.data(), R.zr.size());
     c->d_zi = upload_persistent(c, R.zi.data(), R.zi.size());

@@ -101,14 +101,26 @@ __host__ __device__ inline int ntt_bucket(int npolys) {
     return npolys <= 4 ? 0 : npolys <= 16 ? 1 : npolys <= 64 ? 2 : 3;
 }
 
+// Order of a row's twiddles for the radix-16 row pass of 2^LOG points (TPR = 2^LOG / 16 threads):
+// 2^LOG entries a row. The 15 of the phase on the high bits are the row's own, (8 >> lb) - 1 + u
+// for register bit lb; the low phase's follow as [(8 >> lb) - 1 + u][thread], so that the lanes of
+// a warp read consecutive entries. In the natural order the threads' 8, 4, 2 entries of a stage
+// lie 128, 64, 32 bytes apart, one cache line each. LOG = 7 runs three low stages (lb <= 2).
+__host__ __device__ constexpr int row_tw_index(int LOG, bool high, int lb, int u, int tau) {
+    return high ? (8 >> lb) - 1 + u : 16 + ((8 >> lb) - 1 + u - (LOG == 7 ? 1 : 0)) * ((1 << LOG) / 16) + tau;
+}
+
 // Ring tables resident on the device for one parameter set.
 struct RingDev {
     int logN;
     int N;
     int nprimes;
     const DevPrime* primes;  // [nprimes]
-    const ulonglong2* tw;    // [nprimes][N] (psi^brev(k), its Shoup quotient)
-    const ulonglong2* itw;   // [nprimes][N] (psi^-brev(k), its Shoup quotient)
+    const uint4* tw;         // [nprimes][N] psi^brev(k) in the prime's twiddle format
+    const uint4* itw;        // [nprimes][N] psi^-brev(k), likewise
+    const uint4* rtw;        // [nprimes][N] the same twiddles in the order of the radix-16 row pass
+    const uint4* irtw;       // (row_tw_index; N >= 2^14, null otherwise)
+    bool fast;               // no prime of twiddle class 2
     unsigned char ntt_shape[FR_NTT_BUCKETS];  // tile shape per batch-size bucket (see launch_ntt)
 };
 

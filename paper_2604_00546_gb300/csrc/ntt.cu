@@ -8,13 +8,19 @@
 // polynomial (N = R C): the first log R stages only couple elements of one
 // column (stride C), the remaining log C stages only couple elements of one
 // row (contiguous). Each pass loads its tile once and writes it once. Inside a
-// pass every thread keeps 8 elements in registers and runs up to 3 radix-2
-// stages on them; the elements are re-distributed through shared memory
-// between these 3-stage phases, so a 256-point sub-transform costs 2
-// exchanges instead of 8. Index arithmetic is shifts and masks only.
+// pass every thread keeps 2^RB elements in registers (RB = 3 or 4) and runs up
+// to RB radix-2 stages on them; the elements are re-distributed through shared
+// memory between these phases, so a 256-point sub-transform costs 2 exchanges
+// with 8 elements a thread and 1 with 16. Index arithmetic is shifts and masks only.
 //
-// Residues stay lazily reduced (Harvey): forward butterflies keep values in
-// [0, 4q), inverse butterflies in [0, 2q); the last pass returns [0, q).
+// The passes are bound by the issue of integer multiplications, so the butterfly's product
+// is the cheapest one its prime allows (TwClass in dev_arith.cuh) and residues stay lazily
+// reduced between stages:
+//   class 0  forward: sums only grow, 16 stages stay below 2^64; inverse: the sums of a phase
+//            (at most 4 stages) grow sixteenfold and are folded at its end;
+//   class 1  one conditional subtraction of `big` (about 2^63) per butterfly;
+//   class 2  Harvey's ranges: forward [0, 4q), inverse [0, 2q).
+// The last pass returns canonical residues.
 // Twiddle of the butterfly pairing x and x + 2^b, in either direction:
 // tw[(M + J) >> (b + 1)] where J is the global index of x and M = R for the
 // column pass, N for the row pass.
@@ -47,201 +53,69 @@ __device__ __forceinline__ const u64* poly_in(const PolyBatch& b, int p, int N, 
     return b.src ? b.src + (long long)(p / b.inner) * b.src_outer + (long long)(p % b.inner) * N : x;
 }
 
-__device__ __forceinline__ u64 shoup_lazy(u64 x, u64 w, u64 ws, u64 q) {
-    return x * w - __umul64hi(x, ws) * q;  // in [0, 2q)
-}
-
-// element index of register e of thread tau in a phase whose 3 bits start at LO
-template <int LO>
+// element index of register e of thread tau in a phase whose RB bits start at LO
+template <int RB, int LO>
 __device__ __forceinline__ int phase_x(int tau, int e) {
-    return ((tau >> LO) << (LO + 3)) | (e << LO) | (tau & ((1 << LO) - 1));
+    return ((tau >> LO) << (LO + RB)) | (e << LO) | (tau & ((1 << LO) - 1));
 }
 
-template <int LOG, bool INV, int PH>
+// Phases of a 2^LOG-point pass with RB bits of the element index in registers: phase PH holds
+// bits [LO, LO + RB) and runs the stages on bits [BFROM, BTO). Forward phases take bits in
+// descending order, inverse ones ascending; with RB = 4 (two phases) the inverse ones mirror the
+// forward ones, so both directions share the order of the row pass's twiddles.
+template <int RB, int LOG, bool INV, int PH>
 struct PhaseInfo {
-    // forward phases take bits in descending order, inverse ones ascending;
-    // a phase covers the 3 bits [LO, LO + 3) and runs the stages on bits [BFROM, BTO)
-    static constexpr int LO = INV ? (3 * PH < LOG - 3 ? 3 * PH : LOG - 3) : (LOG - 3 * (PH + 1) > 0 ? LOG - 3 * (PH + 1) : 0);
-    static constexpr int BFROM = INV ? 3 * PH : LO;
-    static constexpr int BTO = INV ? (3 * PH + 3 < LOG ? 3 * PH + 3 : LOG) : LOG - 3 * PH;
+    static constexpr int P = (LOG + RB - 1) / RB;
+    static constexpr int DOWN = LOG - RB * (PH + 1) > 0 ? LOG - RB * (PH + 1) : 0;
+    static constexpr int UP = RB == 4 ? (PH == 0 ? 0 : LOG - 4) : (RB * PH < LOG - RB ? RB * PH : LOG - RB);
+    static constexpr int LO = INV ? UP : DOWN;
+    static constexpr int BFROM = !INV ? LO : RB == 4 ? LO : RB * PH;
+    static constexpr int BTO = !INV ? LOG - RB * PH
+                               : RB == 4 ? (PH == 0 ? LOG - 4 : LOG)
+                                         : (RB * PH + RB < LOG ? RB * PH + RB : LOG);
+    static_assert(RB != 4 || P == 2, "radix-16 passes have two phases");
 };
-
-// Twiddles of a pass: (w, Shoup quotient) pairs, one 16-byte load each. GLOBAL: the table
-// itself (read-only path), else a copy staged in shared memory.
-template <bool GLOBAL>
-struct Ctx {
-    int Jbase, M;    // global index of the tile's element 0; M = R (column pass) or N (row pass)
-    const ulonglong2* tw;
-    u64 q;
-    bool grow;       // forward only: q < 2^57, values may grow by 2q per stage (16 stages < 33q < 2^62)
-    __device__ __forceinline__ ulonglong2 ld(int i) const {
-        if constexpr (GLOBAL) return __ldg(tw + i);
-        else return tw[i];
-    }
-};
-
-// One radix-2 stage on bit B of the registers of a phase with base bit LO. The butterfly of
-// registers e and e + 2^lb (lb = B - LO) takes twiddle (M + J + x) >> (B + 1), x its element
-// index: M + J and the thread's bits of x above LO + 3 are multiples of 2^(B+1), and x's bits
-// below B + 1 are e's bits up to lb and the thread's bits below LO, so the twiddle is
-// base + (e >> (lb + 1)): the stage needs 4 >> lb distinct twiddles, loaded before its
-// butterflies run.
-template <bool INV, int LO, int B, class C>
-__device__ __forceinline__ void stage(u64 (&v)[8], int tau, const C& c) {
-    constexpr int lb = B - LO;
-    constexpr int NT = 4 >> lb;
-    const u64 q2 = 2 * c.q;
-    const int base = (c.M + c.Jbase + ((tau >> LO) << (LO + 3))) >> (B + 1);
-    ulonglong2 w[NT];
-#pragma unroll
-    for (int u = 0; u < NT; ++u) w[u] = c.ld(base + u);
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-        if (e & (1 << lb)) continue;
-        const int e1 = e | (1 << lb);
-        const ulonglong2 t = w[e >> (lb + 1)];
-        if (!INV) {
-            u64 X = v[e];
-            if (!c.grow) X = X >= q2 ? X - q2 : X;
-            const u64 T = shoup_lazy(v[e1], t.x, t.y, c.q);
-            v[e] = X + T;
-            v[e1] = X - T + q2;
-        } else {
-            const u64 X = v[e], Y = v[e1];
-            u64 S = X + Y;
-            S = S >= q2 ? S - q2 : S;
-            v[e] = S;
-            v[e1] = shoup_lazy(X - Y + q2, t.x, t.y, c.q);
-        }
-    }
-}
-
-template <bool INV, int LO, int BFROM, int BTO, int K, class C>
-__device__ __forceinline__ void stages(u64 (&v)[8], int tau, const C& c) {
-    // forward: bits BTO-1 down to BFROM; inverse: BFROM up to BTO-1
-    if constexpr (K < BTO - BFROM) {
-        constexpr int B = INV ? BFROM + K : BTO - 1 - K;
-        stage<INV, LO, B>(v, tau, c);
-        stages<INV, LO, BFROM, BTO, K + 1>(v, tau, c);
-    }
-}
-
-template <int LOG, bool INV, int PH, class Ex, class C>
-__device__ __forceinline__ void phases(u64 (&v)[8], int tau, const C& c, Ex& ex) {
-    constexpr int P = (LOG + 2) / 3;
-    if constexpr (PH < P) {
-        using I = PhaseInfo<LOG, INV, PH>;
-        if constexpr (PH > 0) {
-            using Prev = PhaseInfo<LOG, INV, PH - 1>;
-            ex.template exchange<Prev::LO, I::LO>(v, tau);
-        }
-        stages<INV, I::LO, I::BFROM, I::BTO, 0>(v, tau, c);
-        phases<LOG, INV, PH + 1>(v, tau, c, ex);
-    }
-}
-
-template <int LOG, bool INV>
+template <int RB, int LOG, bool INV>
 struct LastLo {
-    static constexpr int v = PhaseInfo<LOG, INV, (LOG + 2) / 3 - 1>::LO;
+    static constexpr int v = PhaseInfo<RB, LOG, INV, PhaseInfo<RB, LOG, INV, 0>::P - 1>::LO;
 };
-
-__device__ __forceinline__ u64 reduce4(u64 x, u64 q) {
-    x = x >= 2 * q ? x - 2 * q : x;
-    return x >= q ? x - q : x;
-}
-
-// exchange through shared memory, column layout s[x'][KTC]. With 4 columns x' = x ^ x3 ^
-// (x4 << 1), with 8 columns x' = x ^ x3: the rows a half-warp touches then fall on distinct
-// bank groups in every phase layout.
-template <int KTC>
-__device__ __forceinline__ int col_row(int x) {
-    return KTC == 4 ? x ^ ((x >> 3) & 1) ^ (((x >> 4) & 1) << 1) : x ^ ((x >> 3) & 1);
-}
-
-template <int KTC>
-struct ColEx {
-    u64* s;
-    int col;
-    template <int LA, int LB>
-    __device__ __forceinline__ void exchange(u64 (&v)[8], int tau) {
-#pragma unroll
-        for (int e = 0; e < 8; ++e) s[col_row<KTC>(phase_x<LA>(tau, e)) * KTC + col] = v[e];
-        __syncthreads();
-#pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] = s[col_row<KTC>(phase_x<LB>(tau, e)) * KTC + col];
-        __syncthreads();
-    }
-};
-
-// Shared-memory word of element x of a row: the low 4 bits are XORed with bits 4..6
-// (x4 -> bit 0, x5 -> bit 2, x6 -> bits 1 and 3). For 256-point rows this keeps every
-// half-warp access of the forward (bits from 5, 2, 0) and inverse (0, 3, 5) phase layouts
-// on 16 distinct 8-byte bank pairs.
-__device__ __forceinline__ int row_swz(int x) {
-    return x ^ ((x >> 4) & 1) ^ (((x >> 5) & 1) << 2) ^ (((x >> 6) & 1) * 10);
-}
-
-// exchange through shared memory, one row
-struct RowEx {
-    u64* s;
-    template <int LA, int LB>
-    __device__ __forceinline__ void exchange(u64 (&v)[8], int tau) {
-#pragma unroll
-        for (int e = 0; e < 8; ++e) s[row_swz(phase_x<LA>(tau, e))] = v[e];
-        __syncthreads();
-#pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] = s[row_swz(phase_x<LB>(tau, e))];
-        __syncthreads();
-    }
-};
-
-// column pass: one CTA = KTC columns x S rows; thread (tau, col) with col = threadIdx % KTC
-template <int LOG, bool INV, int KTC>
-__global__ void __launch_bounds__(KTC * (1 << LOG) / 8, 5) k_ntt_col(const __grid_constant__ RingDev R, const __grid_constant__ PolyBatch b) {
-    pdl_wait();
-    pdl_trigger();
-    constexpr int S = 1 << LOG;
-    extern __shared__ u64 sm[];
-    ulonglong2* sw = reinterpret_cast<ulonglong2*>(sm + S * KTC);  // twiddles [0, S)
-    const int N = R.N;
-    const int C = N >> LOG;
-    const int p = blockIdx.y;
-    int pi;
-    u64* x = poly_at(b, p, N, &pi);
-    const u64 q = R.primes[pi].q;
-    const ulonglong2* tw = (INV ? R.itw : R.tw) + (size_t)pi * N;
-    for (int i = threadIdx.x; i < S; i += blockDim.x) sw[i] = __ldg(tw + i);
-    const int col = threadIdx.x & (KTC - 1);
-    const int tau = threadIdx.x / KTC;
-    const int gcol = blockIdx.x * KTC + col;
-    constexpr int L0 = PhaseInfo<LOG, INV, 0>::LO;
-    constexpr int LL = LastLo<LOG, INV>::v;
-    const u64* xin = INV ? x : poly_in(b, p, N, x);  // the column pass is the forward transform's first
-    u64 v[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) v[e] = xin[(long long)phase_x<L0>(tau, e) * C + gcol];
-    __syncthreads();
-    Ctx<false> c{0, S, sw, q, q < (1ull << 57)};
-    ColEx<KTC> ex{sm, col};
-    phases<LOG, INV, 0>(v, tau, c, ex);
-    if (INV) {
-        const DevPrime P = R.primes[pi];
-#pragma unroll
-        for (int e = 0; e < 8; ++e)
-            x[(long long)phase_x<LL>(tau, e) * C + gcol] = mul_shoup(v[e], P.ninv, P.ninv_s, q);
-    } else {
-#pragma unroll
-        for (int e = 0; e < 8; ++e) x[(long long)phase_x<LL>(tau, e) * C + gcol] = v[e];
-    }
-}
 
 // Epilogues of the forward row pass (the last pass of a forward transform): instead of
-// storing the transformed value v (canonical) of poly p at index k in place, the fused
-// epilogue finishes the operation the transform belonged to.
+// storing the transformed values of poly p in place, the fused epilogue finishes the operation
+// the transform belonged to, on W = 1 or 2 consecutive indices from k (16-byte accesses for 2).
+// Values arrive below 2q; every epilogue ends them in a product by a constant, and Shoup's product
+// is exact for any 64-bit operand, so differences are lifted by 2q instead of reduced.
 struct EpiStore {};
 
 // Montgomery form of the transformed value, stored in place (template diagonals).
 struct EpiToMont {};
+
+template <class E>
+constexpr bool in_place = std::is_same<E, EpiStore>::value || std::is_same<E, EpiToMont>::value;
+
+template <int W>
+__device__ __forceinline__ void ld_vec(u64 (&r)[W], const u64* p) {
+    if constexpr (W == 2) {
+        const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(p);
+        r[0] = t.x;
+        r[1] = t.y;
+    } else {
+        r[0] = *p;
+    }
+}
+template <int W>
+__device__ __forceinline__ void st_vec(u64* p, const u64 (&r)[W]) {
+    if constexpr (W == 2) *reinterpret_cast<ulonglong2*>(p) = make_ulonglong2(r[0], r[1]);
+    else *p = r[0];
+}
+// r += a term below q, mod q
+template <int W>
+__device__ __forceinline__ void add_vec(u64 (&r)[W], const u64* p, u64 q) {
+    u64 a[W];
+    ld_vec(a, p);
+#pragma unroll
+    for (int w = 0; w < W; ++w) r[w] = add_mod(r[w], a[w], q);
+}
 
 // ModDown combine: poly p = (job, component t, limb i) of the P -> Q conversions; out =
 // (acc_Q - v) P^-1 (+ sigma_g(c0) for rotations, + the ct addend for relinearisation; a
@@ -251,19 +125,26 @@ struct EpiModDown {
     int npos, level, logN;
     const u64* pinv;
     const u64* pinv_s;
-    __device__ __forceinline__ void put(int p, int k, u64 v, u64 q) const {
+    template <int W>
+    __device__ __forceinline__ void put(int p, int k, const u64 (&v)[W], u64 q) const {
         const int L1 = level + 1, N = 1 << logN;
         const int j = p / (2 * L1), r = p % (2 * L1), t = r / L1, i = r % L1;
         const MDJob& J = jobs.j[j];
-        const u64 a = J.acc[((long long)t * npos + i) * N + k];
-        u64 w = mul_shoup(sub_mod(a, v, q), pinv[i], pinv_s[i], q);
+        u64 o[W];
+        ld_vec(o, J.acc + ((long long)t * npos + i) * N + k);
+#pragma unroll
+        for (int w = 0; w < W; ++w) o[w] = mul_shoup(o[w] + 2 * q - v[w], pinv[i], pinv_s[i], q);
         if (J.mode == 1 || J.mode == 3) {
-            if (t == 0) w = add_mod(w, J.add[(long long)i * N + galois_src_index((u32)k, J.galois, logN)], q);
-            if (J.mode == 3) w = add_mod(w, J.add2[((long long)t * J.add_cap + i) * N + k], q);
+            if (t == 0) {
+#pragma unroll
+                for (int w = 0; w < W; ++w)
+                    o[w] = add_mod(o[w], J.add[(long long)i * N + galois_src_index((u32)(k + w), J.galois, logN)], q);
+            }
+            if (J.mode == 3) add_vec(o, J.add2 + ((long long)t * J.add_cap + i) * N + k, q);
         } else if (J.mode == 2) {
-            w = add_mod(w, J.add[((long long)t * J.add_cap + i) * N + k], q);
+            add_vec(o, J.add + ((long long)t * J.add_cap + i) * N + k, q);
         }
-        J.out[((long long)t * J.out_cap + i) * N + k] = w;
+        st_vec(J.out + ((long long)t * J.out_cap + i) * N + k, o);
     }
 };
 
@@ -280,17 +161,23 @@ struct EpiRescale {
     int add_cap;
     long long add_bs;
     const u64* cres;    // mode 2: [l] constants
-    __device__ __forceinline__ void put(int p, int k, u64 v, u64 q) const {
+    template <int W>
+    __device__ __forceinline__ void put(int p, int k, const u64 (&v)[W], u64 q) const {
         const int bt = p / l, i = p % l;
-        const u64 a = x[((long long)bt * x_cap + i) * N + k];
-        u64 r = mul_shoup(sub_mod(a, v, q), tab->qlinv[i], tab->qlinv_s[i], q);
+        u64 r[W];
+        ld_vec(r, x + ((long long)bt * x_cap + i) * N + k);
+#pragma unroll
+        for (int w = 0; w < W; ++w) r[w] = mul_shoup(r[w] + 2 * q - v[w], tab->qlinv[i], tab->qlinv_s[i], q);
         if (mode == 1) {
-            r = add_mod(r, add[(long long)(bt >> 1) * add_bs + ((long long)(bt & 1) * add_cap + i) * N + k], q);
+            add_vec(r, add + (long long)(bt >> 1) * add_bs + ((long long)(bt & 1) * add_cap + i) * N + k, q);
         } else if (mode == 2) {
-            r = add_mod(r, r, q);
-            if ((bt & 1) == 0) r = sub_mod(r, cres[i], q);
+#pragma unroll
+            for (int w = 0; w < W; ++w) {
+                r[w] = add_mod(r[w], r[w], q);
+                if ((bt & 1) == 0) r[w] = sub_mod(r[w], cres[i], q);
+            }
         }
-        out[((long long)bt * out_cap + i) * N + k] = r;
+        st_vec(out + ((long long)bt * out_cap + i) * N + k, r);
     }
 };
 
@@ -311,11 +198,18 @@ struct EpiLeafRescale {
     int out_cap;
     const RescaleTab* tab;
     int l, N;
-    __device__ __forceinline__ void put(int p, int k, u64 v, u64 q) const {
+    template <int W>
+    __device__ __forceinline__ void put(int p, int k, const u64 (&v)[W], u64 q) const {
         const int bjt = p / l, i = p % l, t = bjt & 1, bj = bjt >> 1, j = bj % nl, b = bj / nl;
-        u64 a = mul_shoup(x[(long long)b * x_bs + ((long long)t * x_cap + i) * N + k], cb[j * L1 + i], cb_s[j * L1 + i], q);
-        if (t == 0) a = add_mod(a, ca[j * L1 + i], q);
-        out[((long long)bjt * out_cap + i) * N + k] = mul_shoup(sub_mod(a, v, q), tab->qlinv[i], tab->qlinv_s[i], q);
+        const u64 lift = 2 * q + (t == 0 ? ca[j * L1 + i] : 0);
+        u64 r[W];
+        ld_vec(r, x + (long long)b * x_bs + ((long long)t * x_cap + i) * N + k);
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+            const u64 a = mul_shoup_lazy(r[w], cb[j * L1 + i], cb_s[j * L1 + i], q);  // the sum is below 5q
+            r[w] = mul_shoup(a + lift - v[w], tab->qlinv[i], tab->qlinv_s[i], q);
+        }
+        st_vec(out + ((long long)bjt * out_cap + i) * N + k, r);
     }
 };
 
@@ -324,8 +218,9 @@ struct EpiLeafRescale {
 // y = conv P^-1 + lift, where conv is the ModDown's P -> Q conversion and lift the centered last
 // limb of the ModDown's output. out = (acc_i P^-1 + d_i - v) q_l^-1 with acc the job's key-switch
 // inner product [2][npos][N] and d its tensor product [3][l+1][N] (d0, d1 the addend; null: no
-// addend, a plain ModDown then rescale); then the modes of EpiRescale. Each step is exact modular arithmetic and the NTT is linear, so this equals
-// ModDown, the addition of (d0, d1) and the rescale one after the other, bit for bit.
+// addend, a plain ModDown then rescale); then the modes of EpiRescale. Each step is exact modular
+// arithmetic and the NTT is linear, so this equals ModDown, the addition of (d0, d1) and the
+// rescale one after the other, bit for bit.
 struct EpiRelinRescale {
     const u64* acc;
     const u64* d;
@@ -339,79 +234,306 @@ struct EpiRelinRescale {
     int add_cap;
     long long add_bs;
     const u64* cres;   // mode 2: [l] constants
-    __device__ __forceinline__ void put(int p, int k, u64 v, u64 q) const {
+    template <int W>
+    __device__ __forceinline__ void put(int p, int k, const u64 (&v)[W], u64 q) const {
         const int jt = p / l, i = p % l, j = jt >> 1, t = jt & 1;
-        const u64 a = acc[((long long)jt * npos + i) * N + k];
-        const u64 dd = d ? d[(((long long)j * 3 + t) * (l + 1) + i) * N + k] : 0;
-        const u64 m = add_mod(mul_shoup(a, pinv[i], pinv_s[i], q), dd, q);
-        u64 r = mul_shoup(sub_mod(m, v, q), tab->qlinv[i], tab->qlinv_s[i], q);
-        if (mode == 1) {
-            r = add_mod(r, add[(long long)j * add_bs + ((long long)t * add_cap + i) * N + k], q);
-        } else if (mode == 2) {
-            r = add_mod(r, r, q);
-            if (t == 0) r = sub_mod(r, cres[i], q);
+        u64 r[W], dd[W];
+        ld_vec(r, acc + ((long long)jt * npos + i) * N + k);
+        if (d) ld_vec(dd, d + (((long long)j * 3 + t) * (l + 1) + i) * N + k);
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+            u64 m = mul_shoup_lazy(r[w], pinv[i], pinv_s[i], q) + 2 * q - v[w];  // below 4q
+            if (d) m += dd[w];
+            r[w] = mul_shoup(m, tab->qlinv[i], tab->qlinv_s[i], q);
         }
-        out[(long long)j * out_bs + ((long long)t * out_cap + i) * N + k] = r;
+        if (mode == 1) {
+            add_vec(r, add + (long long)j * add_bs + ((long long)t * add_cap + i) * N + k, q);
+        } else if (mode == 2) {
+#pragma unroll
+            for (int w = 0; w < W; ++w) {
+                r[w] = add_mod(r[w], r[w], q);
+                if (t == 0) r[w] = sub_mod(r[w], cres[i], q);
+            }
+        }
+        st_vec(out + (long long)j * out_bs + ((long long)t * out_cap + i) * N + k, r);
     }
 };
 
+// Constants of a pass and where its twiddles lie. SRC 0: staged in shared memory, natural
+// order; 1: the table itself, natural order; 2: a row's twiddles in the order of row_tw_index.
+template <int CLS, int SRC, int LOG>
+struct Ctx {
+    int Jbase, M;    // global index of the tile's element 0; M = R (column pass) or N (row pass)
+    const uint4* tw;
+    u64 q, qm, off, big;
+    u32 bsh, c;
+    __device__ __forceinline__ Ctx(int jb, int m, const uint4* t, const DevPrime& P)
+        : Jbase(jb), M(m), tw(t), q(P.q), qm(CLS == 2 ? P.q : P.c2), off(P.off), big(P.big), bsh(P.bsh), c(P.c) {}
+    template <int RB, int LO, int B>
+    __device__ __forceinline__ void load(uint4* w, int tau) const {
+        constexpr int lb = B - LO, NT = (1 << (RB - 1)) >> lb;
+        const int base = (M + Jbase + ((tau >> LO) << (LO + RB))) >> (B + 1);
+#pragma unroll
+        for (int u = 0; u < NT; ++u) {
+            if constexpr (SRC == 0) w[u] = tw[base + u];
+            else if constexpr (SRC == 1) w[u] = __ldg(tw + base + u);
+            else w[u] = __ldg(tw + row_tw_index(LOG, LO != 0, lb, u, tau));
+        }
+    }
+    // a value of the transform to below 2q, and to its canonical residue
+    __device__ __forceinline__ u64 fold(u64 v) const {
+        if constexpr (CLS == 2) return min(v, v - 2 * q);
+        else return fold_top(v, bsh, c);
+    }
+    __device__ __forceinline__ u64 canon(u64 v) const {
+        v = fold(v);
+        return min(v, v - q);
+    }
+    // what a pass that ends in epilogue E keeps of v: the epilogues take values below 2q
+    template <class E>
+    __device__ __forceinline__ u64 finish(u64 v, const DevPrime& P) const {
+        if constexpr (std::is_same<E, EpiStore>::value) return canon(v);
+        else if constexpr (std::is_same<E, EpiToMont>::value) return to_mont(v, P);
+        else return fold(v);
+    }
+};
+
+// One radix-2 stage on bit B of the registers of a phase with base bit LO. The butterfly of
+// registers e and e + 2^lb (lb = B - LO) takes twiddle (M + J + x) >> (B + 1), x its element
+// index: M + J and the thread's bits of x above LO + RB are multiples of 2^(B+1), and x's bits
+// below B + 1 are e's bits up to lb and the thread's bits below LO, so the twiddle is
+// base + (e >> (lb + 1)): the stage needs 2^(RB-1) >> lb distinct twiddles, loaded before its
+// butterflies run. T: stages of this phase run before this one (inverse, class 0: operands are
+// below off 2^T).
+template <bool INV, int CLS, int RB, int LO, int B, int T, class C>
+__device__ __forceinline__ void stage(u64 (&v)[1 << RB], int tau, const C& c) {
+    constexpr int lb = B - LO;
+    uint4 w[(1 << (RB - 1)) >> lb];
+    c.template load<RB, LO, B>(w, tau);
+#pragma unroll
+    for (int e = 0; e < (1 << RB); ++e) {
+        if (e & (1 << lb)) continue;
+        const int e1 = e | (1 << lb);
+        const uint4& t = w[e >> (lb + 1)];
+        if constexpr (!INV) {
+            u64 X = v[e];
+            if constexpr (CLS == 1) X = min(X, X - c.big);  // X - big wraps when X is below
+            if constexpr (CLS == 2) X = min(X, X - 2 * c.q);
+            const u64 Tw = mul_tw<CLS>(v[e1], t, c.qm);
+            v[e] = X + Tw;
+            v[e1] = X + (CLS == 2 ? 2 * c.q : c.off) - Tw;
+        } else {
+            const u64 X = v[e], Y = v[e1];
+            const u64 lift = CLS == 0 ? c.off << T : CLS == 1 ? c.big : 2 * c.q;
+            u64 S = X + Y;
+            if constexpr (CLS != 0) S = min(S, S - lift);
+            v[e] = S;
+            v[e1] = mul_tw<CLS>(X - Y + lift, t, c.qm);
+        }
+    }
+}
+
+template <bool INV, int CLS, int RB, int LO, int BFROM, int BTO, int K, class C>
+__device__ __forceinline__ void stages(u64 (&v)[1 << RB], int tau, const C& c) {
+    // forward: bits BTO-1 down to BFROM; inverse: BFROM up to BTO-1
+    if constexpr (K < BTO - BFROM) {
+        constexpr int B = INV ? BFROM + K : BTO - 1 - K;
+        stage<INV, CLS, RB, LO, B, K>(v, tau, c);
+        stages<INV, CLS, RB, LO, BFROM, BTO, K + 1>(v, tau, c);
+    }
+}
+
+// The phases of a pass, PH .. P - 1, exchanging through ex between them. An inverse column pass
+// ends with its last stage (twiddle 1 of the table) and the product by N^-1 in one: the sums are
+// multiplied by N^-1, the differences by N^-1 times the twiddle (FIN).
+template <int CLS, int RB, int LOG, bool INV, bool FIN, int PH, class Ex, class C>
+__device__ __forceinline__ void phases(u64 (&v)[1 << RB], int tau, const C& c, Ex& ex, const DevPrime& P) {
+    using I = PhaseInfo<RB, LOG, INV, PH>;
+    constexpr bool last = PH == I::P - 1;
+    if constexpr (PH > 0) {
+        using Prev = PhaseInfo<RB, LOG, INV, PH - 1>;
+        ex.template exchange<RB, Prev::LO, I::LO>(v, tau);
+    }
+    constexpr int BTO = I::BTO - (FIN && last ? 1 : 0);
+    stages<INV, CLS, RB, I::LO, I::BFROM, BTO, 0>(v, tau, c);
+    if constexpr (FIN && last) {
+        constexpr int lb = LOG - 1 - I::LO, T = BTO - I::BFROM;
+        const uint4 wn = P.tw_ninv, ww = P.tw_wninv;
+        const u64 lift = CLS == 0 ? c.off << T : CLS == 1 ? c.big : 2 * c.q;
+#pragma unroll
+        for (int e = 0; e < (1 << RB); ++e) {
+            if (e & (1 << lb)) continue;
+            const int e1 = e | (1 << lb);
+            const u64 X = v[e], Y = v[e1];
+            v[e] = mul_tw<CLS>(X + Y, wn, c.qm);
+            v[e1] = mul_tw<CLS>(X - Y + lift, ww, c.qm);
+        }
+    } else if constexpr (INV && CLS == 0) {
+        constexpr int lb = BTO - 1 - I::LO;  // the sums of the phase's last stage
+#pragma unroll
+        for (int e = 0; e < (1 << RB); ++e)
+            if (!(e & (1 << lb))) v[e] = fold_top(v[e], c.bsh, c.c);
+    }
+    if constexpr (!last) phases<CLS, RB, LOG, INV, FIN, PH + 1>(v, tau, c, ex, P);
+}
+
+// exchange through shared memory, column layout s[x'][KTC]. With 4 columns x' = x ^ x3 ^
+// (x4 << 1), with 8 columns x' = x ^ x3 (x4 when 16 elements are in registers): the rows a
+// half-warp touches then fall on distinct bank groups in every phase layout. Wider tiles need no
+// swizzle: a half-warp is one row.
+template <int RB, int KTC>
+__device__ __forceinline__ int col_row(int x) {
+    if constexpr (KTC >= 16) return x;
+    else if constexpr (RB == 4) return x ^ ((x >> 4) & 1);
+    else return KTC == 4 ? x ^ ((x >> 3) & 1) ^ (((x >> 4) & 1) << 1) : x ^ ((x >> 3) & 1);
+}
+
+template <int KTC>
+struct ColEx {
+    u64* s;
+    int col;
+    template <int RB, int LA, int LB>
+    __device__ __forceinline__ void exchange(u64 (&v)[1 << RB], int tau) {
+#pragma unroll
+        for (int e = 0; e < (1 << RB); ++e) s[col_row<RB, KTC>(phase_x<RB, LA>(tau, e)) * KTC + col] = v[e];
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < (1 << RB); ++e) v[e] = s[col_row<RB, KTC>(phase_x<RB, LB>(tau, e)) * KTC + col];
+        if constexpr (RB == 3) __syncthreads();  // another exchange follows
+    }
+};
+
+// Shared-memory word of element x of a row: the low 4 bits are XORed with bits 4..6
+// (x4 -> bit 0, x5 -> bit 2, x6 -> bits 1 and 3). For 256-point rows this keeps every
+// half-warp access of the forward (bits from 5, 2, 0) and inverse (0, 3, 5) phase layouts
+// on 16 distinct 8-byte bank pairs.
+__device__ __forceinline__ int row_swz(int x) {
+    return x ^ ((x >> 4) & 1) ^ (((x >> 5) & 1) << 2) ^ (((x >> 6) & 1) * 10);
+}
+
+// exchange through shared memory, one row of 8 elements a thread
+struct RowEx {
+    u64* s;
+    template <int RB, int LA, int LB>
+    __device__ __forceinline__ void exchange(u64 (&v)[1 << RB], int tau) {
+#pragma unroll
+        for (int e = 0; e < (1 << RB); ++e) s[row_swz(phase_x<RB, LA>(tau, e))] = v[e];
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < (1 << RB); ++e) v[e] = s[row_swz(phase_x<RB, LB>(tau, e))];
+        __syncthreads();
+    }
+};
+
+// exchange through shared memory, one row of 16 elements a thread. A row's 2^LOG / 16 threads
+// are 8 or 16 lanes of one warp, so the exchange needs no block barrier. Word x of a row lies at
+// x ^ ((x >> 4) & 15): a half-warp then touches 16 distinct 8-byte bank pairs both when it
+// stores elements e << LO | tau and when it loads tau << 4 | e; with 128-point rows (two rows a
+// half-warp) odd rows flip bit 3 as well.
+template <int LOG>
+struct RowEx16 {
+    u64* s;
+    int odd;
+    __device__ __forceinline__ int at(int x) const { return x ^ ((x >> 4) & 15) ^ (LOG == 7 ? odd << 3 : 0); }
+    template <int RB, int LA, int LB>
+    __device__ __forceinline__ void exchange(u64 (&v)[1 << RB], int tau) {
+#pragma unroll
+        for (int e = 0; e < (1 << RB); ++e) s[at(phase_x<RB, LA>(tau, e))] = v[e];
+        __syncwarp();
+#pragma unroll
+        for (int e = 0; e < (1 << RB); ++e) v[e] = s[at(phase_x<RB, LB>(tau, e))];
+        __syncwarp();
+    }
+};
+
+// column pass: one CTA = KTC columns x S rows; thread (tau, col) with col = threadIdx % KTC
+template <int RB, int LOG, bool INV, int KTC, int CLS>
+__device__ __forceinline__ void ntt_col_body(const PolyBatch& b, u64* x, const uint4* tw, const DevPrime& P, int p,
+                                             int N, u64* sm) {
+    constexpr int S = 1 << LOG;
+    uint4* sw = reinterpret_cast<uint4*>(sm + S * KTC);  // twiddles [0, S)
+    const int C = N >> LOG;
+    for (int i = threadIdx.x; i < S; i += blockDim.x) sw[i] = __ldg(tw + i);
+    const int col = threadIdx.x & (KTC - 1);
+    const int tau = threadIdx.x / KTC;
+    const int gcol = blockIdx.x * KTC + col;
+    constexpr int L0 = PhaseInfo<RB, LOG, INV, 0>::LO;
+    constexpr int LL = LastLo<RB, LOG, INV>::v;
+    const u64* xin = INV ? x : poly_in(b, p, N, x);  // the column pass is the forward transform's first
+    u64 v[1 << RB];
+#pragma unroll
+    for (int e = 0; e < (1 << RB); ++e) v[e] = xin[(long long)phase_x<RB, L0>(tau, e) * C + gcol];
+    __syncthreads();
+    const Ctx<CLS, 0, LOG> c(0, S, sw, P);
+    ColEx<KTC> ex{sm, col};
+    phases<CLS, RB, LOG, INV, INV, 0>(v, tau, c, ex, P);
+#pragma unroll
+    for (int e = 0; e < (1 << RB); ++e) x[(long long)phase_x<RB, LL>(tau, e) * C + gcol] = INV ? c.canon(v[e]) : v[e];
+}
+
+template <int LOG, bool INV, int KTC>
+__global__ void __launch_bounds__(KTC * (1 << LOG) / 8, 5) k_ntt_col(const __grid_constant__ RingDev R, const __grid_constant__ PolyBatch b) {
+    pdl_wait();
+    pdl_trigger();
+    extern __shared__ __align__(16) u64 sm[];
+    const int p = blockIdx.y;
+    int pi;
+    u64* x = poly_at(b, p, R.N, &pi);
+    const uint4* tw = (INV ? R.itw : R.tw) + (size_t)pi * R.N;
+    const DevPrime P = R.primes[pi];
+    if (P.cls == 0) ntt_col_body<3, LOG, INV, KTC, 0>(b, x, tw, P, p, R.N, sm);
+    else if (P.cls == 1) ntt_col_body<3, LOG, INV, KTC, 1>(b, x, tw, P, p, R.N, sm);
+    else ntt_col_body<3, LOG, INV, KTC, 2>(b, x, tw, P, p, R.N, sm);
+}
+
 // row pass: one CTA = RPC rows of S contiguous elements (RT threads), S/8 threads per row
+template <int LOG, int RPC, bool INV, int CLS, class E>
+__device__ __forceinline__ void ntt_row_body(const PolyBatch& b, u64* x, const uint4* tw, const DevPrime& P, int p,
+                                             int N, u64* sm, const E& epi) {
+    constexpr int S = 1 << LOG;
+    constexpr int TPR = S / 8;  // threads per row
+    const int rloc = threadIdx.x / TPR;
+    const int tau = threadIdx.x % TPR;
+    const int Jbase = (blockIdx.x * RPC + rloc) * S;
+    u64* xr = x + Jbase;
+    const u64* xin = (INV ? poly_in(b, p, N, x) : x) + Jbase;  // the row pass is the inverse's first
+    constexpr int L0 = PhaseInfo<3, LOG, INV, 0>::LO;
+    constexpr int LL = LastLo<3, LOG, INV>::v;
+    u64 v[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[e] = xin[phase_x<3, L0>(tau, e)];
+    const Ctx<CLS, 1, LOG> c(Jbase, N, tw, P);
+    RowEx ex{sm + rloc * S};
+    phases<CLS, 3, LOG, INV, false, 0>(v, tau, c, ex, P);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        const int k = phase_x<3, LL>(tau, e);
+        if constexpr (INV) {
+            xr[k] = v[e];
+        } else {
+            const u64 o[1] = {c.template finish<E>(v[e], P)};
+            if constexpr (in_place<E>) xr[k] = o[0];
+            else epi.put(p, Jbase + k, o, P.q);
+        }
+    }
+}
+
 template <int LOG, int LOGR, bool INV, class E, int RT>
 __global__ void __launch_bounds__(RT, RT == 128 ? 9 : 4) k_ntt_row(const __grid_constant__ RingDev R, const __grid_constant__ PolyBatch b,
                                                                    const __grid_constant__ E epi) {
     pdl_wait();
     pdl_trigger();
-    constexpr int S = 1 << LOG;
-    constexpr int TPR = S / 8;           // threads per row
+    constexpr int TPR = (1 << LOG) / 8;
     constexpr int RPC = (RT / TPR < (1 << LOGR)) ? RT / TPR : (1 << LOGR);  // rows per CTA
-    constexpr int SP = S;                // row stride in shared memory (swizzled, no padding)
-    extern __shared__ u64 sm[];
-    const int N = R.N;
+    extern __shared__ __align__(16) u64 sm[];
     const int p = blockIdx.y;
     int pi;
-    u64* x = poly_at(b, p, N, &pi);
-    const u64 q = R.primes[pi].q;
-    const ulonglong2* tw = (INV ? R.itw : R.tw) + (size_t)pi * N;
-    const int rloc = threadIdx.x / TPR;
-    const int tau = threadIdx.x % TPR;
-    const int rho = blockIdx.x * RPC + rloc;
-    const int Jbase = rho * S;
-    u64* xr = x + Jbase;
-    const u64* xin = (INV ? poly_in(b, p, N, x) : x) + Jbase;  // the row pass is the inverse's first
-    constexpr int L0 = PhaseInfo<LOG, INV, 0>::LO;
-    constexpr int LL = LastLo<LOG, INV>::v;
-    u64 v[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) v[e] = xin[phase_x<L0>(tau, e)];
-    const bool grow = q < (1ull << 57);
-    Ctx<true> c{Jbase, N, tw, q, grow};
-    RowEx ex{sm + rloc * SP};
-    phases<LOG, INV, 0>(v, tau, c, ex);
-    if constexpr (std::is_same<E, EpiToMont>::value) {
-        static_assert(!INV, "epilogues follow forward transforms");
-        const DevPrime P = R.primes[pi];
-#pragma unroll
-        for (int e = 0; e < 8; ++e)
-            xr[phase_x<LL>(tau, e)] = to_mont(grow ? mul_shoup(v[e], 1, P.one_s, q) : reduce4(v[e], q), P);
-    } else if constexpr (!std::is_same<E, EpiStore>::value) {
-        static_assert(!INV, "epilogues follow forward transforms");
-        const u64 one_s = R.primes[pi].one_s;
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const u64 fv = grow ? mul_shoup(v[e], 1, one_s, q) : reduce4(v[e], q);
-            epi.put(p, Jbase + phase_x<LL>(tau, e), fv, q);
-        }
-    } else if (INV) {
-#pragma unroll
-        for (int e = 0; e < 8; ++e) xr[phase_x<LL>(tau, e)] = v[e];
-    } else if (grow) {
-        const u64 one_s = R.primes[pi].one_s;
-#pragma unroll
-        for (int e = 0; e < 8; ++e) xr[phase_x<LL>(tau, e)] = mul_shoup(v[e], 1, one_s, q);
-    } else {
-#pragma unroll
-        for (int e = 0; e < 8; ++e) xr[phase_x<LL>(tau, e)] = reduce4(v[e], q);
-    }
+    u64* x = poly_at(b, p, R.N, &pi);
+    const uint4* tw = (INV ? R.itw : R.tw) + (size_t)pi * R.N;
+    const DevPrime P = R.primes[pi];
+    if (P.cls == 0) ntt_row_body<LOG, RPC, INV, 0>(b, x, tw, P, p, R.N, sm, epi);
+    else if (P.cls == 1) ntt_row_body<LOG, RPC, INV, 1>(b, x, tw, P, p, R.N, sm, epi);
+    else ntt_row_body<LOG, RPC, INV, 2>(b, x, tw, P, p, R.N, sm, epi);
 }
 
 // Single-launch NTT of N = 2^16 (256 x 256) for small batches. A cluster of 8 CTAs of 1024
@@ -425,288 +547,208 @@ __global__ void __launch_bounds__(RT, RT == 128 ? 9 : 4) k_ntt_row(const __grid_
 constexpr int kClusterCtas = 8;
 constexpr size_t kClusterSmem = (size_t)(2 * 8192 + 2 * 256) * sizeof(u64);
 
-template <bool INV, class E>
-__global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(1024, 1)
-    k_ntt_cluster(const __grid_constant__ RingDev R, const __grid_constant__ PolyBatch b,
-                  const __grid_constant__ E epi) {
-    pdl_wait();
-    pdl_trigger();
+template <bool INV, int CLS, class E>
+__device__ __forceinline__ void ntt_cluster_body(const RingDev& R, u64* x, const uint4* tw, const DevPrime& P, int p,
+                                                 u64* sm, const E& epi) {
     namespace cg = cooperative_groups;
     constexpr int LOG = 8, S = 256;
-    extern __shared__ u64 sm[];
     u64* A = sm;              // 32 rows x 256 (row layout) / 256 rows x 32 columns (column layout)
     u64* Bb = sm + 8192;
-    ulonglong2* sw = reinterpret_cast<ulonglong2*>(sm + 16384);  // column-pass twiddles [0, 256)
+    uint4* sw = reinterpret_cast<uint4*>(sm + 16384);  // column-pass twiddles [0, 256)
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank();
     const int N = R.N;
-    const int p = blockIdx.y;
-    int pi;
-    u64* x = poly_at(b, p, N, &pi);
-    const u64 q = R.primes[pi].q;
-    const ulonglong2* tw = (INV ? R.itw : R.tw) + (size_t)pi * N;
     for (int i = threadIdx.x; i < S; i += blockDim.x) sw[i] = __ldg(tw + i);
-    const bool grow = q < (1ull << 57);
     // column-pass coordinates: column 32 rank + col, rows phase_x(tauc, e)
     const int col = threadIdx.x & 31, tauc = threadIdx.x >> 5;
     const int gcol = rank * 32 + col;
     // row-pass coordinates: row 32 rank + rloc, elements phase_x(taur, e)
     const int rloc = threadIdx.x >> 5, taur = threadIdx.x & 31;
     const int rho = rank * 32 + rloc;
+    const Ctx<CLS, 0, LOG> c(0, S, sw, P);
+    const Ctx<CLS, 1, LOG> cr(rho * S, N, tw, P);
     u64 v[8];
+    constexpr int L0 = PhaseInfo<3, LOG, INV, 0>::LO, LL = LastLo<3, LOG, INV>::v;
+    u64* xr = x + (long long)rho * S;
     if constexpr (!INV) {
-        constexpr int L0 = PhaseInfo<LOG, false, 0>::LO, LL = LastLo<LOG, false>::v;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] = x[(long long)phase_x<L0>(tauc, e) * S + gcol];
+        for (int e = 0; e < 8; ++e) v[e] = x[(long long)phase_x<3, L0>(tauc, e) * S + gcol];
         __syncthreads();
-        Ctx<false> c{0, S, sw, q, grow};
         ColEx<32> exc{A, col};
-        phases<LOG, false, 0>(v, tauc, c, exc);
+        phases<CLS, 3, LOG, false, false, 0>(v, tauc, c, exc, P);
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
-            const int row = phase_x<LL>(tauc, e);
+            const int row = phase_x<3, LL>(tauc, e);
             u64* dst = cl.map_shared_rank(Bb, row >> 5);
             dst[(row & 31) * S + gcol] = v[e];
         }
         cl.sync();
         u64* br = Bb + rloc * S;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] = br[phase_x<L0>(taur, e)];
-        Ctx<true> cr{rho * S, N, tw, q, grow};
+        for (int e = 0; e < 8; ++e) v[e] = br[phase_x<3, L0>(taur, e)];
         RowEx exr{A + rloc * S};
-        phases<LOG, false, 0>(v, taur, cr, exr);
-        const u64 one_s = R.primes[pi].one_s;
-        u64* xr = x + (long long)rho * S;
+        phases<CLS, 3, LOG, false, false, 0>(v, taur, cr, exr, P);
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
-            const u64 fv = grow ? mul_shoup(v[e], 1, one_s, q) : reduce4(v[e], q);
-            if constexpr (std::is_same<E, EpiStore>::value) xr[phase_x<LL>(taur, e)] = fv;
-            else if constexpr (std::is_same<E, EpiToMont>::value) xr[phase_x<LL>(taur, e)] = to_mont(fv, R.primes[pi]);
-            else epi.put(p, rho * S + phase_x<LL>(taur, e), fv, q);
+            const int k = phase_x<3, LL>(taur, e);
+            const u64 o[1] = {cr.template finish<E>(v[e], P)};
+            if constexpr (in_place<E>) xr[k] = o[0];
+            else epi.put(p, rho * S + k, o, P.q);
         }
     } else {
-        constexpr int L0 = PhaseInfo<LOG, true, 0>::LO, LL = LastLo<LOG, true>::v;
-        const u64* xr = x + (long long)rho * S;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] = xr[phase_x<L0>(taur, e)];
-        Ctx<true> cr{rho * S, N, tw, q, false};
+        for (int e = 0; e < 8; ++e) v[e] = xr[phase_x<3, L0>(taur, e)];
         RowEx exr{Bb + rloc * S};
-        phases<LOG, true, 0>(v, taur, cr, exr);
+        phases<CLS, 3, LOG, true, false, 0>(v, taur, cr, exr, P);
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
-            const int k = phase_x<LL>(taur, e);
+            const int k = phase_x<3, LL>(taur, e);
             u64* dst = cl.map_shared_rank(A, k >> 5);
             dst[rho * 32 + (k & 31)] = v[e];
         }
         cl.sync();
 #pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] = A[phase_x<L0>(tauc, e) * 32 + col];
-        Ctx<false> c{0, S, sw, q, false};
+        for (int e = 0; e < 8; ++e) v[e] = A[phase_x<3, L0>(tauc, e) * 32 + col];
         ColEx<32> exc{Bb, col};
-        phases<LOG, true, 0>(v, tauc, c, exc);
-        const DevPrime P = R.primes[pi];
+        phases<CLS, 3, LOG, true, true, 0>(v, tauc, c, exc, P);
 #pragma unroll
-        for (int e = 0; e < 8; ++e)
-            x[(long long)phase_x<LL>(tauc, e) * S + gcol] = mul_shoup(v[e], P.ninv, P.ninv_s, q);
+        for (int e = 0; e < 8; ++e) x[(long long)phase_x<3, LL>(tauc, e) * S + gcol] = c.canon(v[e]);
     }
 }
 
-// ---------------------------------------------------------------------------
-// Radix-16 passes for N = 2^16 (tile shape 5): every thread keeps 16 residues and runs 4
-// stages per shared-memory exchange, so each 256-point pass is two 4-stage phases with one
-// exchange (radix 8: three phases, two exchanges) and a stage on register bit lb loads
-// 8 >> lb twiddles for its 8 butterflies. Forward phases take register bits 4..7 then 0..3,
-// inverse ones 0..3 then 4..7. Residues whose 16 elements are contiguous in memory move as
-// 16-byte vectors.
-// ---------------------------------------------------------------------------
-template <int LO>
-__device__ __forceinline__ int px16(int tau, int e) {
-    return ((tau >> LO) << (LO + 4)) | (e << LO) | (tau & ((1 << LO) - 1));
+template <bool INV, class E>
+__global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(1024, 1)
+    k_ntt_cluster(const __grid_constant__ RingDev R, const __grid_constant__ PolyBatch b,
+                  const __grid_constant__ E epi) {
+    pdl_wait();
+    pdl_trigger();
+    extern __shared__ __align__(16) u64 sm[];
+    const int p = blockIdx.y;
+    int pi;
+    u64* x = poly_at(b, p, R.N, &pi);
+    const uint4* tw = (INV ? R.itw : R.tw) + (size_t)pi * R.N;
+    const DevPrime P = R.primes[pi];  // class 0 or 1: the launcher checks
+    if (P.cls == 0) ntt_cluster_body<INV, 0>(R, x, tw, P, p, sm, epi);
+    else ntt_cluster_body<INV, 1>(R, x, tw, P, p, sm, epi);
 }
 
-template <bool INV, int LO, int B, class C>
-__device__ __forceinline__ void stage16(u64 (&v)[16], int tau, const C& c) {
-    constexpr int lb = B - LO;
-    constexpr int NT = 8 >> lb;
-    const u64 q2 = 2 * c.q;
-    const int base = (c.M + c.Jbase + ((tau >> LO) << (LO + 4))) >> (B + 1);
-    ulonglong2 w[NT];
+// ---------------------------------------------------------------------------
+// Radix-16 passes (tile shape 5, N = 2^14 .. 2^16, rings without class-2 primes): every thread
+// keeps 16 residues and runs 4 stages (3 in the low phase of a 128-point pass) per shared-memory
+// exchange, so a pass has one exchange (radix 8: two) and a stage on register bit lb loads
+// 8 >> lb twiddles for its 8 butterflies.
+// ---------------------------------------------------------------------------
+constexpr int kCol16 = 8;  // columns of a column-pass CTA: 64-byte row segments
+
+template <int LOG, bool INV>
+__global__ void __launch_bounds__(kCol16 * (1 << LOG) / 16, (INV ? 6 : 5) * (256 >> LOG))
+    k_ntt_col16(const __grid_constant__ RingDev R, const __grid_constant__ PolyBatch b) {
+    pdl_wait();
+    pdl_trigger();
+    extern __shared__ __align__(16) u64 sm[];
+    const int p = blockIdx.y;
+    int pi;
+    u64* x = poly_at(b, p, R.N, &pi);
+    const uint4* tw = (INV ? R.itw : R.tw) + (size_t)pi * R.N;
+    const DevPrime P = R.primes[pi];
+    if (P.cls == 0) ntt_col_body<4, LOG, INV, kCol16, 0>(b, x, tw, P, p, R.N, sm);
+    else ntt_col_body<4, LOG, INV, kCol16, 1>(b, x, tw, P, p, R.N, sm);
+}
+
+__device__ __forceinline__ void ld_async16(void* dst, const void* src) {
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+}
+
+// Row pass: 128 threads, each warp on its own 512 contiguous elements (2 rows of 256 points or 4
+// of 128), so no block barrier. The phase on the low bits has a thread's 16 elements contiguous
+// (128 bytes): they pass through shared memory in 16-byte chunks, chunk h of a thread at h ^
+// (thread & 7), so that the global side moves 512 contiguous bytes per instruction and epilogues
+// see consecutive elements in consecutive lanes. Reading and writing them thread by thread
+// touches 32 cache lines per instruction, which bounded the pass (the epilogues above all).
+template <int LOG, bool INV, int CLS, class E>
+__device__ __forceinline__ void ntt_row16_body(const PolyBatch& b, u64* x, const uint4* tw, const DevPrime& P, int p,
+                                               int N, u64* sm, const E& epi) {
+    constexpr int S = 1 << LOG, TPR = S / 16;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int tau = lane % TPR;
+    const int Wbase = (blockIdx.x * 4 + warp) * 512;  // the warp's first element
+    const int rho = Wbase / S + lane / TPR;
+    u64* ws = sm + warp * 512;
+    ulonglong2* wc = reinterpret_cast<ulonglong2*>(ws);
+    const Ctx<CLS, 2, LOG> c(rho * S, N, tw + (size_t)rho * S, P);
+    RowEx16<LOG> ex{ws + (lane / TPR) * S, rho & 1};
+    u64 v[16];
+    if constexpr (INV) {
+        const u64* xin = poly_in(b, p, N, x) + Wbase;
 #pragma unroll
-    for (int u = 0; u < NT; ++u) w[u] = c.ld(base + u);
+        for (int j = 0; j < 8; ++j) {
+            const int ch = j * 32 + lane;
+            ld_async16(wc + (ch ^ ((ch >> 3) & 7)), xin + 2 * ch);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncwarp();
 #pragma unroll
-    for (int e = 0; e < 16; ++e) {
-        if (e & (1 << lb)) continue;
-        const int e1 = e | (1 << lb);
-        const ulonglong2 t = w[e >> (lb + 1)];
-        if (!INV) {
-            u64 X = v[e];
-            if (!c.grow) X = X >= q2 ? X - q2 : X;
-            const u64 T = shoup_lazy(v[e1], t.x, t.y, c.q);
-            v[e] = X + T;
-            v[e1] = X - T + q2;
-        } else {
-            const u64 X = v[e], Y = v[e1];
-            u64 S = X + Y;
-            S = S >= q2 ? S - q2 : S;
-            v[e] = S;
-            v[e1] = shoup_lazy(X - Y + q2, t.x, t.y, c.q);
+        for (int h = 0; h < 8; ++h) {
+            const ulonglong2 t = wc[lane * 8 + (h ^ (lane & 7))];
+            v[2 * h] = t.x;
+            v[2 * h + 1] = t.y;
+        }
+        __syncwarp();
+        phases<CLS, 4, LOG, true, false, 0>(v, tau, c, ex, P);
+        u64* xr = x + (long long)rho * S;
+#pragma unroll
+        for (int e = 0; e < 16; ++e) xr[phase_x<4, LOG - 4>(tau, e)] = v[e];
+    } else {
+        const u64* xr = x + (long long)rho * S;
+#pragma unroll
+        for (int e = 0; e < 16; ++e) v[e] = xr[phase_x<4, LOG - 4>(tau, e)];
+        phases<CLS, 4, LOG, false, false, 0>(v, tau, c, ex, P);
+#pragma unroll
+        for (int h = 0; h < 8; ++h)
+            wc[lane * 8 + (h ^ (lane & 7))] =
+                make_ulonglong2(c.template finish<E>(v[2 * h], P), c.template finish<E>(v[2 * h + 1], P));
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int ch = j * 32 + lane;
+            u64 o[2];
+            ld_vec(o, ws + 2 * (ch ^ ((ch >> 3) & 7)));
+            if constexpr (in_place<E>) st_vec(x + Wbase + 2 * ch, o);
+            else epi.put(p, Wbase + 2 * ch, o, P.q);
         }
     }
 }
 
-// the four stages of a phase whose register bits start at LO: forward bits LO+3 .. LO,
-// inverse LO .. LO+3
-template <bool INV, int LO, class C>
-__device__ __forceinline__ void phase16(u64 (&v)[16], int tau, const C& c) {
-    if constexpr (!INV) {
-        stage16<false, LO, LO + 3>(v, tau, c);
-        stage16<false, LO, LO + 2>(v, tau, c);
-        stage16<false, LO, LO + 1>(v, tau, c);
-        stage16<false, LO, LO>(v, tau, c);
-    } else {
-        stage16<true, LO, LO>(v, tau, c);
-        stage16<true, LO, LO + 1>(v, tau, c);
-        stage16<true, LO, LO + 2>(v, tau, c);
-        stage16<true, LO, LO + 3>(v, tau, c);
-    }
-}
-
-// Shared-memory word of element x of a 256-point row: x ^ ((x >> 4) & 15). A half-warp (one
-// row's 16 threads) then touches 16 distinct 8-byte bank pairs both when it stores elements
-// e << 4 | tau and when it loads tau << 4 | e (and the reverse).
-__device__ __forceinline__ int sw16(int x) { return x ^ ((x >> 4) & 15); }
-
-// column pass: one CTA = 8 columns x 256 rows, thread (tau, col) = (threadIdx / 8, threadIdx % 8)
-template <bool INV>
-__global__ void __launch_bounds__(128, 4) k_ntt_col16(const __grid_constant__ RingDev R,
-                                                      const __grid_constant__ PolyBatch b) {
-    pdl_wait();
-    pdl_trigger();
-    constexpr int S = 256, KTC = 8;
-    extern __shared__ u64 sm[];                                    // [S][KTC] rows swizzled
-    ulonglong2* sw = reinterpret_cast<ulonglong2*>(sm + S * KTC);  // twiddles [0, S)
-    const int N = R.N;
-    const int C = N >> 8;
-    const int p = blockIdx.y;
-    int pi;
-    u64* x = poly_at(b, p, N, &pi);
-    const u64 q = R.primes[pi].q;
-    const ulonglong2* tw = (INV ? R.itw : R.tw) + (size_t)pi * N;
-    for (int i = threadIdx.x; i < S; i += blockDim.x) sw[i] = __ldg(tw + i);
-    const int col = threadIdx.x & (KTC - 1);
-    const int tau = threadIdx.x / KTC;
-    const int gcol = blockIdx.x * KTC + col;
-    constexpr int L0 = INV ? 0 : 4, L1 = INV ? 4 : 0;
-    u64 v[16];
-#pragma unroll
-    for (int e = 0; e < 16; ++e) v[e] = x[(long long)px16<L0>(tau, e) * C + gcol];
-    __syncthreads();
-    Ctx<false> c{0, S, sw, q, q < (1ull << 57)};
-    phase16<INV, L0>(v, tau, c);
-    // rows x and x + 16 of one load phase fall in different bank halves: row' = x ^ bit 4 of x
-#pragma unroll
-    for (int e = 0; e < 16; ++e) {
-        const int r = px16<L0>(tau, e);
-        sm[(r ^ ((r >> 4) & 1)) * KTC + col] = v[e];
-    }
-    __syncthreads();
-#pragma unroll
-    for (int e = 0; e < 16; ++e) {
-        const int r = px16<L1>(tau, e);
-        v[e] = sm[(r ^ ((r >> 4) & 1)) * KTC + col];
-    }
-    phase16<INV, L1>(v, tau, c);
-    if (INV) {
-        const DevPrime P = R.primes[pi];
-#pragma unroll
-        for (int e = 0; e < 16; ++e)
-            x[(long long)px16<L1>(tau, e) * C + gcol] = mul_shoup(v[e], P.ninv, P.ninv_s, q);
-    } else {
-#pragma unroll
-        for (int e = 0; e < 16; ++e) x[(long long)px16<L1>(tau, e) * C + gcol] = v[e];
-    }
-}
-
-// row pass: one CTA = 8 rows of 256 contiguous elements, 16 threads per row
-template <bool INV, class E>
-__global__ void __launch_bounds__(128, 4) k_ntt_row16(const __grid_constant__ RingDev R,
+template <int LOG, bool INV, class E>
+__global__ void __launch_bounds__(128, 6) k_ntt_row16(const __grid_constant__ RingDev R,
                                                       const __grid_constant__ PolyBatch b,
                                                       const __grid_constant__ E epi) {
     pdl_wait();
     pdl_trigger();
-    constexpr int S = 256, TPR = 16, RPC = 8;
-    extern __shared__ u64 sm[];  // [RPC][S] swizzled
-    const int N = R.N;
+    extern __shared__ __align__(16) u64 sm[];  // [4 warps][512]
     const int p = blockIdx.y;
     int pi;
-    u64* x = poly_at(b, p, N, &pi);
-    const u64 q = R.primes[pi].q;
-    const ulonglong2* tw = (INV ? R.itw : R.tw) + (size_t)pi * N;
-    const int rloc = threadIdx.x / TPR;
-    const int tau = threadIdx.x % TPR;
-    const int rho = blockIdx.x * RPC + rloc;
-    const int Jbase = rho * S;
-    u64* xr = x + Jbase;
-    constexpr int L0 = INV ? 0 : 4, L1 = INV ? 4 : 0;
-    u64 v[16];
-    if constexpr (L0 == 0) {
-        // the thread's 16 elements are contiguous: eight 16-byte loads
-        const ulonglong2* src = reinterpret_cast<const ulonglong2*>(xr + tau * 16);
-#pragma unroll
-        for (int h = 0; h < 8; ++h) {
-            const ulonglong2 t = src[h];
-            v[2 * h] = t.x;
-            v[2 * h + 1] = t.y;
-        }
-    } else {
-#pragma unroll
-        for (int e = 0; e < 16; ++e) v[e] = xr[px16<L0>(tau, e)];
-    }
-    const bool grow = q < (1ull << 57);
-    Ctx<true> c{Jbase, N, tw, q, INV ? false : grow};
-    phase16<INV, L0>(v, tau, c);
-    u64* s = sm + rloc * S;
-#pragma unroll
-    for (int e = 0; e < 16; ++e) s[sw16(px16<L0>(tau, e))] = v[e];
-    __syncthreads();
-#pragma unroll
-    for (int e = 0; e < 16; ++e) v[e] = s[sw16(px16<L1>(tau, e))];
-    phase16<INV, L1>(v, tau, c);
-    if constexpr (INV) {
-#pragma unroll
-        for (int e = 0; e < 16; ++e) xr[px16<L1>(tau, e)] = v[e];
-    } else {
-        const u64 one_s = R.primes[pi].one_s;
-        u64 o[16];
-#pragma unroll
-        for (int e = 0; e < 16; ++e) o[e] = grow ? mul_shoup(v[e], 1, one_s, q) : reduce4(v[e], q);
-        if constexpr (std::is_same<E, EpiStore>::value) {
-            ulonglong2* dst = reinterpret_cast<ulonglong2*>(xr + tau * 16);
-#pragma unroll
-            for (int h = 0; h < 8; ++h) dst[h] = make_ulonglong2(o[2 * h], o[2 * h + 1]);
-        } else if constexpr (std::is_same<E, EpiToMont>::value) {
-            const DevPrime P = R.primes[pi];
-            ulonglong2* dst = reinterpret_cast<ulonglong2*>(xr + tau * 16);
-#pragma unroll
-            for (int h = 0; h < 8; ++h) dst[h] = make_ulonglong2(to_mont(o[2 * h], P), to_mont(o[2 * h + 1], P));
-        } else {
-#pragma unroll
-            for (int e = 0; e < 16; ++e) epi.put(p, Jbase + tau * 16 + e, o[e], q);
-        }
-    }
+    u64* x = poly_at(b, p, R.N, &pi);
+    const uint4* tw = (INV ? R.irtw : R.rtw) + (size_t)pi * R.N;
+    const DevPrime P = R.primes[pi];
+    if (P.cls == 0) ntt_row16_body<LOG, INV, 0>(b, x, tw, P, p, R.N, sm, epi);
+    else ntt_row16_body<LOG, INV, 1>(b, x, tw, P, p, R.N, sm, epi);
 }
 
-template <class E>
+template <int LOGR, int LOGC, class E>
 void launch_ntt_r16(const RingDev& R, const PolyBatch& b, bool inverse, cudaStream_t st, const E& epi) {
-    const int N = R.N;
-    const dim3 gc((N >> 8) / 8, b.npolys), gr(256 / 8, b.npolys);
-    const size_t smc = (size_t)(256 * 8 + 2 * 256) * sizeof(u64), smr = (size_t)8 * 256 * sizeof(u64);
+    constexpr int SR = 1 << LOGR, SC = 1 << LOGC;
+    const dim3 gc(SC / kCol16, b.npolys), gr(SR * SC / 2048, b.npolys);
+    const int tc = kCol16 * SR / 16;
+    const size_t smc = (size_t)(SR * kCol16 + 2 * SR) * sizeof(u64), smr = (size_t)2048 * sizeof(u64);
     if (!inverse) {
-        launch_k(k_ntt_col16<false>, gc, dim3(128), smc, st, R, b);
-        launch_k(k_ntt_row16<false, E>, gr, dim3(128), smr, st, R, b, epi);
+        launch_k(k_ntt_col16<LOGR, false>, gc, dim3(tc), smc, st, R, b);
+        launch_k(k_ntt_row16<LOGC, false, E>, gr, dim3(128), smr, st, R, b, epi);
     } else {
-        launch_k(k_ntt_row16<true, EpiStore>, gr, dim3(128), smr, st, R, b, EpiStore{});
-        launch_k(k_ntt_col16<true>, gc, dim3(128), smc, st, R, b);
+        launch_k(k_ntt_row16<LOGC, true, EpiStore>, gr, dim3(128), smr, st, R, b, EpiStore{});
+        launch_k(k_ntt_col16<LOGR, true>, gc, dim3(tc), smc, st, R, b);
     }
 }
 
@@ -730,10 +772,17 @@ void launch_ntt_t(const RingDev& R, const PolyBatch& b, bool inverse, cudaStream
 }
 
 // Tile shape of a launch: 0..3 are the radix-8 two-pass kernels, bit 0 set = 8 columns per
-// column-pass CTA (else 4), bit 1 set = 256-thread row-pass CTAs (else 128); 4 is the
-// single-launch cluster kernel and 5 the radix-16 two-pass kernels (both N = 2^16). Chosen per
-// batch-size bucket by the tuner (RingDev holds the table); sizes other than N = 2^15, 2^16
-// use shape 0.
+// column-pass CTA (else 4), bit 1 set = 256-thread row-pass CTAs (else 128; N >= 2^15); 4 is the
+// single-launch cluster kernel (N = 2^16) and 5 the radix-16 two-pass kernels (N >= 2^14). Chosen
+// per batch-size bucket by the tuner (RingDev holds the table); smaller rings use shape 0.
+// Measured at N = 2^16, forward / inverse, 9 primes (1 of 60 bits, 8 of 50), microseconds with
+// launch and event overhead:
+//   polys     16          64           248           512
+//   shape 0   29.5/27.0   73.1/70.0    215.9/204.8   408.5/386.2
+//   shape 5   25.5/26.5   54.6/58.5    153.2/165.1   286.4/306.3
+// (512 polys with Shoup products: shape 0 487.7/471.0, and 448.2/455.1 for 16 residues a thread
+// that read and wrote their 128 contiguous bytes thread by thread.) Below about 8 polynomials the
+// launches' latency counts and the shapes are even.
 template <class E>
 void launch_ntt_cluster(const RingDev& R, const PolyBatch& b, bool inverse, cudaStream_t st, const E& epi) {
     static std::atomic<unsigned long long> fwd{0}, inv{0};
@@ -744,18 +793,34 @@ void launch_ntt_cluster(const RingDev& R, const PolyBatch& b, bool inverse, cuda
     else launch_k(k_ntt_cluster<true, EpiStore>, g, dim3(1024), kClusterSmem, st, R, b, EpiStore{});
 }
 
+// The tile shape this batch runs: the tuned one of its bucket, with two exceptions. Shapes 4 and
+// 5 have no code for class-2 primes, and shape 5 moves 16-byte chunks, so a ring with such a prime
+// or a batch at an address that is not a multiple of 16 bytes (a caller's own buffer) runs shape 0.
+int ntt_shape_of(const RingDev& R, const PolyBatch& b) {
+    if (R.logN < 14) return 0;
+    const int shape = R.ntt_shape[ntt_bucket(b.npolys)];
+    if (shape < 4) return shape;
+    const uintptr_t a = (uintptr_t)b.base | (uintptr_t)b.src | (uintptr_t)b.base2 |
+                        (uintptr_t)(8 * b.outer) | (uintptr_t)(8 * b.src_outer) | (uintptr_t)(8 * b.outer2);
+    return !R.fast || (a & 15) || (shape == 4 && R.logN != 16) ? 0 : shape;
+}
+
 template <int LOGR, int LOGC, class E>
 void launch_ntt_s(const RingDev& R, const PolyBatch& b, bool inverse, cudaStream_t st, const E& epi) {
-    const int shape = (LOGR + LOGC >= 15) ? R.ntt_shape[ntt_bucket(b.npolys)] : 0;
+    const int shape = ntt_shape_of(R, b);
     if constexpr (LOGR == 8 && LOGC == 8) {
         if (shape == 4) {
             launch_ntt_cluster(R, b, inverse, st, epi);
             return;
         }
-        if (shape == 5) {
-            launch_ntt_r16(R, b, inverse, st, epi);
-            return;
-        }
+    }
+    if (shape == 5) {
+        launch_ntt_r16<LOGR, LOGC>(R, b, inverse, st, epi);
+        return;
+    }
+    if constexpr (LOGR + LOGC < 15) {
+        launch_ntt_t<LOGR, LOGC, E, 4, 128>(R, b, inverse, st, epi);
+        return;
     }
     switch (shape) {
         case 1: launch_ntt_t<LOGR, LOGC, E, 8, 128>(R, b, inverse, st, epi); break;
@@ -765,24 +830,21 @@ void launch_ntt_s(const RingDev& R, const PolyBatch& b, bool inverse, cudaStream
     }
 }
 
-// Register-only throughput of the forward butterfly used above (Harvey lazy reduction,
-// Shoup twiddle product): the arithmetic ceiling of the NTT on this GPU, no memory traffic.
-__global__ void __launch_bounds__(256) k_butterfly_peak(u64 q, u64 w, u64 ws, int iters, u64* sink) {
+// Register-only throughput of the forward butterfly used above (a class-0 prime's, the cheapest
+// product): the arithmetic ceiling of the NTT on this GPU, no memory traffic.
+__global__ void __launch_bounds__(256) k_butterfly_peak(uint4 w, u64 c2, u64 off, int iters, u64* sink) {
     u64 x[8], y[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
-        x[e] = (threadIdx.x * 8 + e) % q;
-        y[e] = (blockIdx.x * 8 + e + 1) % q;
+        x[e] = threadIdx.x * 8 + e;
+        y[e] = blockIdx.x * 8 + e + 1;
     }
-    const u64 q2 = 2 * q;
     for (int it = 0; it < iters; ++it) {
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
-            u64 X = x[e];
-            X = X >= q2 ? X - q2 : X;
-            const u64 T = shoup_lazy(y[e], w, ws, q);
-            x[e] = X + T;
-            y[e] = X - T + q2;
+            const u64 T = mul_tw<0>(y[e], w, c2);
+            y[e] = x[e] - T + off;
+            x[e] = x[e] + T;
         }
     }
     u64 acc = 0;
@@ -802,9 +864,9 @@ int pdl_mode() {
 }
 
 double measure_butterfly_peak(int device) {
-    // 60-bit prime; any twiddle works for a throughput measurement
-    const u64 q = 1152921504606830593ull, w = 0x0123456789abcdefull % q;
-    const u64 ws = (u64)(((unsigned __int128)w << 64) / q);
+    // 50-bit prime; any twiddle works for a throughput measurement
+    const u64 q = 1125899904679937ull, off = q << 9;
+    const uint4 w = make_uint4(0x54321, 0x2badcafe, 0xabcde, 0x1234567);
     int nsm = 0;
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device);
     const int blocks = nsm * 8, threads = 256, iters = 4096;
@@ -813,9 +875,9 @@ double measure_butterfly_peak(int device) {
     cudaEvent_t a, b;
     cudaEventCreate(&a);
     cudaEventCreate(&b);
-    k_butterfly_peak<<<blocks, threads>>>(q, w, ws, 64, sink);  // warm-up
+    k_butterfly_peak<<<blocks, threads>>>(w, (1ull << 52) - 4 * q, off, 64, sink);  // warm-up
     cudaEventRecord(a);
-    k_butterfly_peak<<<blocks, threads>>>(q, w, ws, iters, sink);
+    k_butterfly_peak<<<blocks, threads>>>(w, (1ull << 52) - 4 * q, off, iters, sink);
     cudaEventRecord(b);
     cudaEventSynchronize(b);
     float ms = 0;
@@ -831,10 +893,9 @@ template <class E>
 void launch_ntt_e(const RingDev& R, const PolyBatch& b, bool inverse, cudaStream_t s, const E& epi) {
     if (b.npolys <= 0) return;
     if (b.src) {
-        // the radix-8 two-pass kernels read a source themselves; for the cluster and radix-16
-        // shapes (and a table-mapped batch) the source is copied into place first
-        const int shape = R.logN >= 15 ? R.ntt_shape[ntt_bucket(b.npolys)] : 0;
-        if (b.tab || shape == 4 || shape == 5) {
+        // the two-pass kernels read a source themselves; for the cluster shape (and a table-mapped
+        // batch) the source is copied into place first
+        if (b.tab || ntt_shape_of(R, b) == 4) {
             cudaMemcpy2DAsync(b.base, (size_t)b.outer * 8, b.src, (size_t)b.src_outer * 8, (size_t)b.inner * R.N * 8,
                               (size_t)(b.npolys / b.inner), cudaMemcpyDeviceToDevice, s);
             PolyBatch c = b;
@@ -848,7 +909,7 @@ void launch_ntt_e(const RingDev& R, const PolyBatch& b, bool inverse, cudaStream
         case 11: launch_ntt_t<5, 6, E, 4, 128>(R, b, inverse, s, epi); break;
         case 12: launch_ntt_t<6, 6, E, 4, 128>(R, b, inverse, s, epi); break;
         case 13: launch_ntt_t<6, 7, E, 4, 128>(R, b, inverse, s, epi); break;
-        case 14: launch_ntt_t<7, 7, E, 4, 128>(R, b, inverse, s, epi); break;
+        case 14: launch_ntt_s<7, 7, E>(R, b, inverse, s, epi); break;
         case 15: launch_ntt_s<7, 8, E>(R, b, inverse, s, epi); break;
         case 16: launch_ntt_s<8, 8, E>(R, b, inverse, s, epi); break;
         default: break;
@@ -861,13 +922,12 @@ void launch_ntt(const RingDev& R, const PolyBatch& b, bool inverse, cudaStream_t
 
 // Times every tile shape of the forward + inverse transform for one batch size per bucket
 // (CUDA events, best of `reps`) on a scratch buffer of zero residues and keeps the fastest
-// shape per bucket in R.ntt_shape; us[bucket * 4 + shape] receives the times.
+// shape per bucket in R.ntt_shape; us[bucket * FR_NTT_SHAPES + shape] receives the times.
 void tune_ntt(RingDev& R, cudaStream_t s, double* us, int reps) {
     for (int bk = 0; bk < FR_NTT_BUCKETS; ++bk) R.ntt_shape[bk] = 0;
     if (us)
         for (int i = 0; i < FR_NTT_BUCKETS * FR_NTT_SHAPES; ++i) us[i] = 0;
-    if (R.logN < 15) return;
-    const int nshapes = R.logN == 16 ? FR_NTT_SHAPES : FR_NTT_SHAPES - 2;  // shapes 4 and 5 are N = 2^16 only
+    if (R.logN < 14) return;
     const int sizes[FR_NTT_BUCKETS] = {4, 16, 64, 256};
     const int maxp = sizes[FR_NTT_BUCKETS - 1];
     u64* buf = nullptr;
@@ -876,32 +936,47 @@ void tune_ntt(RingDev& R, cudaStream_t s, double* us, int reps) {
     cudaEvent_t a, e;
     cudaEventCreate(&a);
     cudaEventCreate(&e);
+    auto timed = [&](int bk, int sh) {
+        PolyBatch pb{buf, 0, sizes[bk], sizes[bk], PrimeMap{}};
+        pb.pm.period = R.nprimes;
+        for (int i = 0; i < R.nprimes; ++i) pb.pm.idx[i] = (unsigned char)i;
+        R.ntt_shape[bk] = (unsigned char)sh;
+        cudaEventRecord(a, s);
+        launch_ntt(R, pb, false, s);
+        launch_ntt(R, pb, true, s);
+        cudaEventRecord(e, s);
+        cudaEventSynchronize(e);
+        float ms = 0;
+        cudaEventElapsedTime(&ms, a, e);
+        if (cudaGetLastError() != cudaSuccess) return 1e30;  // a shape this GPU cannot launch
+        return ms * 1000.0;
+    };
+    // an idle GPU's clocks take some milliseconds to rise: a first timing of 4 polynomials read
+    // 600 us instead of 25, and the shapes were picked by chance
+    double before = timed(FR_NTT_BUCKETS - 1, 0);
+    for (int i = 0, same = 0; i < 60 && same < 8; ++i) {
+        const double now = timed(FR_NTT_BUCKETS - 1, 0);
+        same = now > 0.97 * before && now < 1.03 * before ? same + 1 : 0;
+        before = now;
+    }
     unsigned char best[FR_NTT_BUCKETS];
     for (int bk = 0; bk < FR_NTT_BUCKETS; ++bk) {
-        PolyBatch pb{buf, 0, sizes[bk], sizes[bk], PrimeMap{}};
-        pb.pm.period = 1;
-        pb.pm.idx[0] = 0;
-        double tbest = 1e30, t0 = 1e30;
-        best[bk] = 0;
-        for (int sh = 0; sh < nshapes; ++sh) {
-            R.ntt_shape[bk] = (unsigned char)sh;
-            double t = 1e30;
-            for (int r = 0; r <= reps; ++r) {  // first run warms up
-                cudaEventRecord(a, s);
-                launch_ntt(R, pb, false, s);
-                launch_ntt(R, pb, true, s);
-                cudaEventRecord(e, s);
-                cudaEventSynchronize(e);
-                float ms = 0;
-                cudaEventElapsedTime(&ms, a, e);
-                if (r > 0) t = t < ms * 1000.0 ? t : ms * 1000.0;
+        double t[FR_NTT_SHAPES];
+        for (int sh = 0; sh < FR_NTT_SHAPES; ++sh) t[sh] = 1e30;
+        for (int r = 0; r <= reps; ++r)  // the first round warms up; the shapes take turns
+            for (int sh = 0; sh < FR_NTT_SHAPES; ++sh) {
+                if (sh == 4 && R.logN != 16) continue;                // N = 2^16 only
+                if (sh > 0 && sh < 4 && R.logN < 15) continue;  // N >= 2^15 only
+                const double now = timed(bk, sh);
+                if (r > 0 && now < t[sh]) t[sh] = now;
             }
-            if (cudaGetLastError() != cudaSuccess) t = 1e30;  // a shape this GPU cannot launch
-            if (us) us[bk * FR_NTT_SHAPES + sh] = t < 1e29 ? t : -1.0;
+        best[bk] = 0;
+        double tbest = t[0];
+        for (int sh = 0; sh < FR_NTT_SHAPES; ++sh) {
+            if (us) us[bk * FR_NTT_SHAPES + sh] = t[sh] < 1e29 ? t[sh] : -1.0;
             // another shape replaces the default only when at least 3% faster (timing noise)
-            if (sh == 0) t0 = t;
-            if (sh == 0 ? t < tbest : t < tbest && t < 0.97 * t0) {
-                tbest = t;
+            if (t[sh] < tbest && t[sh] < 0.97 * t[0]) {
+                tbest = t[sh];
                 best[bk] = (unsigned char)sh;
             }
         }

@@ -1,0 +1,68 @@
+"""GPU parity of the NTT's twiddle classes: the butterfly's product and its ranges depend on the
+prime (see mul_tw), so rotation, rescale and ct x ct product are checked bit for bit against the
+oracle on chains of every class and on a mixed one, at the ring sizes with their own kernels,
+with 8 and with 16 residues a thread where both exist. Exact arithmetic: no tolerance."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2604_00546_gb300 import fr
+
+pytestmark = pytest.mark.gpu
+
+CHAINS = {
+    "class0": dict(q_bits=[51, 50, 45], p_bits=[51, 51], scale_bits=45),
+    "class1": dict(q_bits=[60, 52, 55], p_bits=[58, 59], scale_bits=52),
+    "class2": dict(q_bits=[36, 34, 34], p_bits=[36, 36], scale_bits=30),
+    "mixed": dict(q_bits=[60, 50, 34], p_bits=[52, 60], scale_bits=34),
+}
+
+
+def _residues(primes, N, seed):
+    """[2][limbs][N]: random residues with runs at both ends of the range."""
+    rng = np.random.default_rng(seed)
+    w = np.empty((2, len(primes), N), dtype=np.uint64)
+    for i, q in enumerate(primes):
+        w[:, i] = rng.integers(0, q, (2, N), dtype=np.uint64)
+        w[:, i, : N // 8] = q - 1
+        w[:, i, N // 8: N // 4] = 0
+    return w
+
+
+@pytest.mark.parametrize("log_n", [12, 13, 14, 15, 16])
+@pytest.mark.parametrize("chain", sorted(CHAINS))
+def test_transforms_of_every_class(chain, log_n):
+    p = CHAINS[chain]
+    ctx = fr.Context(device=0, log_n=log_n, dnum=2, ell=64, n1=8, **p)
+    seed = 0x7C00 + log_n
+    ctx.load_keys(ctx.keygen([3], seed))
+    oc = oracle.Ctx(log_n, p["q_bits"], p["p_bits"], 2, p["scale_bits"])
+    ok = oc.keygen(seed)
+    top = oc.top
+    a, b = (_residues(ctx.primes()[: top + 1], ctx.N, seed + s) for s in (1, 2))
+    rot, rs, mul = ok.rotate(a, top, 3), oc.rescale(a, top), ok.mul_relin(a, b, top)
+    for shape in ([0, 5] if log_n >= 14 else [0]):
+        ctx.ntt_set_shapes([shape] * 4)
+        ca, cb = ctx.import_ct(a, top).upload(), ctx.import_ct(b, top).upload()
+        assert np.array_equal(ctx.rotate(ca, 3).export(), rot), shape
+        assert np.array_equal(ctx.rescale(ca).export(), rs), shape
+        assert np.array_equal(ctx.mul_relin(ca, cb).export(), mul), shape
+
+
+@pytest.mark.parametrize("words_off", [0, 1])
+def test_noalloc_rotation_on_any_word_address(words_off):
+    """The caller's output buffer need not start on a 16-byte boundary."""
+    torch = pytest.importorskip("torch")
+    p = CHAINS["class1"]
+    ctx = fr.Context(device=0, log_n=14, dnum=2, ell=64, n1=8, **p)
+    ctx.load_keys(ctx.keygen([3], 5))
+    ctx.ntt_set_shapes([5] * 4)
+    a = _residues(ctx.primes()[:3], ctx.N, 9)
+    ref = ctx.rotate(ctx.import_ct(a, 2).upload(), 3).export()
+    d_in = torch.from_numpy(a.view(np.int64)).to("cuda:0")
+    buf = torch.zeros(a.size + 2, dtype=torch.int64, device="cuda:0")
+    torch.cuda.synchronize()
+    ctx.rotate_noalloc(d_in.data_ptr(), 2, 3, buf.data_ptr() + 8 * words_off)
+    ctx.sync()
+    got = buf[words_off: words_off + a.size].cpu().numpy().view(np.uint64).reshape(a.shape)
+    assert np.array_equal(got, ref)
