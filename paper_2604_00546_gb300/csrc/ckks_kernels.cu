@@ -16,64 +16,152 @@ __device__ __forceinline__ void fold(Acc128& a, u64 q) {
 }
 
 // ---------------------------------------------------------------------------
-// ModUp: per digit, fast-convert the digit's limbs to every other position of
-// Q_l u P (coefficient form); the digit's own positions are copied from the
-// evaluation-form input so they need no forward NTT afterwards.
-// in: coefficient form, job j at in + j * in_job; in_eval: evaluation form, job j at in_eval + j * eval_job
-// ext: [J][beta][npos][N]
+// Fast base conversions (ModUp, ModDown). A thread converts W = 2 consecutive coefficients, 16-byte
+// accesses, to every target in turn; the block's targets are staged in shared memory.
 // ---------------------------------------------------------------------------
-// sum_i ys_i [B/b_i]_t mod t from split residues: 30-bit multiply-accumulate, the high word
-// reduced mod t, then one Montgomery reduction (hat_m carries the 2^64 factor)
+constexpr int kBcW = 2;
+
+// (sum_i y_i [B/b_i]_t + add) mod t, canonical; add < 2^61
 template <int NS>
-__device__ __forceinline__ u64 bconv_sum(const u64 (&ys)[NS], const u64 (&hat_m)[FR_MAX_DIGIT_LIMBS][FR_MAX_PRIMES],
-                                         int pos, u64 t, u64 tinv, u64 t_one_s) {
-    AccK a{0, 0, 0};
+__device__ __forceinline__ void bconv(const BconvTarget& T, const u64 (&y)[NS][kBcW], const u64 (&add)[kBcW],
+                                      u64 (&out)[kBcW]) {
+    if (T.mode == 0) {
+        u64 a0[kBcW], a1[kBcW];
 #pragma unroll
-    for (int i = 0; i < NS; ++i) mack(a, ys[i], sum30(ys[i]), hat_m[i][pos]);
-    Acc128 acc{0, 0};
-    flushk(acc, a);
-    return redc(mul_shoup(acc.hi, 1, t_one_s, t), acc.lo, t, tinv);
+        for (int w = 0; w < kBcW; ++w) {
+            a0[w] = add[w];
+            a1[w] = 0;
+        }
+#pragma unroll
+        for (int i = 0; i < NS; ++i) {
+            const uint4 h = T.hat[i];
+#pragma unroll
+            for (int w = 0; w < kBcW; ++w) {
+                const u32 xl = (u32)y[i][w], xh = (u32)(y[i][w] >> 32);
+                a1[w] = mad_wide(xh, h.w, mad_wide(xl, h.y, a1[w]));
+                a0[w] = mad_wide(xh, h.z, mad_wide(xl, h.x, a0[w]));
+            }
+        }
+#pragma unroll
+        for (int w = 0; w < kBcW; ++w) {
+            const u64 r = mad_wide((u32)a1[w], T.mul, mad_wide((u32)(a1[w] >> 32), T.c2, a0[w]));
+            const u64 f = fold_top(r, T.bsh, T.c);
+            out[w] = min(f, f - T.q);
+        }
+    } else if (T.mode == 1) {
+        u64 sum[kBcW];
+#pragma unroll
+        for (int w = 0; w < kBcW; ++w) sum[w] = add[w];
+#pragma unroll
+        for (int i = 0; i < NS; i += 2) {
+            const uint4 h = T.hat[i], g = i + 1 < NS ? T.hat[i + 1 < NS ? i + 1 : i] : make_uint4(0, 0, 0, 0);
+#pragma unroll
+            for (int w = 0; w < kBcW; ++w) {
+                const u32 xl = (u32)y[i][w], xh = (u32)(y[i][w] >> 32);
+                u64 a1 = mad_wide(xh, h.w, mul_wide(xl, h.y));
+                u64 a0 = mad_wide(xh, h.z, mul_wide(xl, h.x));
+                if (i + 1 < NS) {
+                    const u64 z = y[i + 1 < NS ? i + 1 : i][w];
+                    a1 = mad_wide((u32)(z >> 32), g.w, mad_wide((u32)z, g.y, a1));
+                    a0 = mad_wide((u32)(z >> 32), g.z, mad_wide((u32)z, g.x, a0));
+                }
+                sum[w] += fold_top(mad_wide((u32)a1, T.mul, mad_wide((u32)(a1 >> 32), T.c2, a0)), T.bsh, T.c);
+            }
+        }
+#pragma unroll
+        for (int w = 0; w < kBcW; ++w) {
+            const u64 f = fold_top(sum[w], T.bsh, T.c);
+            out[w] = min(f, f - T.q);
+        }
+    } else {
+        for (int w = 0; w < kBcW; ++w) {
+            AccK a{0, 0, 0};
+#pragma unroll
+            for (int i = 0; i < NS; ++i) {
+                const u64 x = split30(y[i][w]);
+                mack(a, x, sum30(x), (u64)T.hat[i].y << 32 | T.hat[i].x);
+            }
+            Acc128 acc{0, 0};
+            flushk(acc, a);
+            const u64 r = redc(mul_shoup(acc.hi, 1, T.one_s, T.q), acc.lo, T.q, T.qinv);
+            out[w] = add_mod(r, mul_shoup(add[w], 1, T.one_s, T.q), T.q);
+        }
+    }
 }
 
+// sources of a conversion: limb i of the thread's points at x + i N, times inv_hat unless scaled
 template <int NS>
-__device__ __forceinline__ void modup_body(const ModUpTab& T, const u64* __restrict__ x,
-                                           const u64* __restrict__ xe, u64* __restrict__ out, int npos, int N,
-                                           int k) {
-    u64 ys[NS];
+__device__ __forceinline__ void bconv_load(u64 (&y)[NS][kBcW], const u64* __restrict__ x, int N, bool scaled,
+                                           const u64* inv_hat, const u64* inv_hat_s, const u64* q) {
 #pragma unroll
-    for (int i = 0; i < NS; ++i)
-        ys[i] = split30(mul_shoup(x[(long long)(T.lo + i) * N + k], T.inv_hat[i], T.inv_hat_s[i], T.src_q[i]));
-    for (int pos = 0; pos < npos; ++pos) {
-        u64 v;
-        if (pos >= T.lo && pos < T.lo + NS) v = xe[(long long)pos * N + k];
-        else v = bconv_sum<NS>(ys, T.hat_m, pos, T.tq[pos], T.tinv[pos], T.t_one_s[pos]);
-        out[(long long)pos * N + k] = v;
+    for (int i = 0; i < NS; ++i) {
+        const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(x + (long long)i * N);
+        y[i][0] = t.x;
+        y[i][1] = t.y;
+        if (!scaled) {
+#pragma unroll
+            for (int w = 0; w < kBcW; ++w) y[i][w] = mul_shoup(y[i][w], inv_hat[i], inv_hat_s[i], q[i]);
+        }
+    }
+}
+
+// n targets from global into shared memory
+__device__ __forceinline__ void stage_targets(BconvTarget* s, const BconvTarget* __restrict__ g, int n) {
+    static_assert(sizeof(BconvTarget) % 16 == 0, "copied in 16-byte words");
+    const uint4* src = reinterpret_cast<const uint4*>(g);
+    uint4* dst = reinterpret_cast<uint4*>(s);
+    for (int e = threadIdx.x; e < n * (int)(sizeof(BconvTarget) / 16); e += blockDim.x) dst[e] = src[e];
+    __syncthreads();
+}
+
+// ---------------------------------------------------------------------------
+// ModUp: per digit, fast-convert the digit's limbs to every other position of Q_l u P
+// (coefficient form). The digit's own positions are not written: the inner product reads them
+// from the switched polynomial itself, in evaluation form.
+// in: coefficient form, job j at in + j * in_job; ext: [J][beta][npos][N]
+// Bound by integer multiplies before (75 of 99 us in arithmetic for 15 inputs at level 7, 4 limbs a
+// digit: 3 wide products a source, 80 cycles of reduction a target, and the products by inv_hat);
+// now 4 wide products a source, 2 for the reduction, none for inv_hat, and a third of the traffic
+// (the copies of the own positions) is gone. Block z = job, y = (digit, chunk of positions): one
+// chunk when the jobs fill the GPU, up to npos of them for a single input.
+// ---------------------------------------------------------------------------
+template <int NS>
+__device__ __forceinline__ void modup_body(const ModUpTab& T, const BconvTarget* st, const u64* __restrict__ x,
+                                           u64* __restrict__ out, int pos0, int pos1, int N, int k, bool scaled) {
+    u64 y[NS][kBcW];
+    bconv_load(y, x + (long long)T.lo * N + k, N, scaled, T.inv_hat, T.inv_hat_s, T.src_q);
+    const u64 zero[kBcW] = {};
+    for (int pos = pos0; pos < pos1; ++pos) {
+        if (pos >= T.lo && pos < T.lo + NS) continue;
+        u64 v[kBcW];
+        bconv<NS>(st[pos - pos0], y, zero, v);
+        *reinterpret_cast<ulonglong2*>(out + (long long)pos * N + k) = make_ulonglong2(v[0], v[1]);
     }
 }
 
 __global__ void __launch_bounds__(kThreads) k_modup(const u64* __restrict__ in, long long in_job,
-                                                    const u64* __restrict__ in_eval, long long eval_job,
                                                     u64* __restrict__ ext, const ModUpTab* __restrict__ tabs, int beta,
-                                                    int npos, int N) {
+                                                    int npos, int N, int per, bool scaled) {
     pdl_wait();
     pdl_trigger();
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    const int d = blockIdx.y;
+    __shared__ BconvTarget st[FR_MAX_PRIMES];
+    const int k = (blockIdx.x * blockDim.x + threadIdx.x) * kBcW;
+    const int d = blockIdx.y % beta, pos0 = (blockIdx.y / beta) * per, pos1 = min(npos, pos0 + per);
     const int j = blockIdx.z;
-    if (k >= N) return;
     const ModUpTab& T = tabs[d];
+    stage_targets(st, T.t + pos0, pos1 - pos0);
+    if (k >= N) return;
     const u64* x = in + (long long)j * in_job;
-    const u64* xe = in_eval + (long long)j * eval_job;
     u64* out = ext + (((long long)j * beta + d) * npos) * N;
     switch (T.ns) {
-        case 1: modup_body<1>(T, x, xe, out, npos, N, k); break;
-        case 2: modup_body<2>(T, x, xe, out, npos, N, k); break;
-        case 3: modup_body<3>(T, x, xe, out, npos, N, k); break;
-        case 4: modup_body<4>(T, x, xe, out, npos, N, k); break;
-        case 5: modup_body<5>(T, x, xe, out, npos, N, k); break;
-        case 6: modup_body<6>(T, x, xe, out, npos, N, k); break;
-        case 7: modup_body<7>(T, x, xe, out, npos, N, k); break;
-        default: modup_body<8>(T, x, xe, out, npos, N, k); break;  // ns <= 8, checked on the host
+        case 1: modup_body<1>(T, st, x, out, pos0, pos1, N, k, scaled); break;
+        case 2: modup_body<2>(T, st, x, out, pos0, pos1, N, k, scaled); break;
+        case 3: modup_body<3>(T, st, x, out, pos0, pos1, N, k, scaled); break;
+        case 4: modup_body<4>(T, st, x, out, pos0, pos1, N, k, scaled); break;
+        case 5: modup_body<5>(T, st, x, out, pos0, pos1, N, k, scaled); break;
+        case 6: modup_body<6>(T, st, x, out, pos0, pos1, N, k, scaled); break;
+        case 7: modup_body<7>(T, st, x, out, pos0, pos1, N, k, scaled); break;
+        default: modup_body<8>(T, st, x, out, pos0, pos1, N, k, scaled); break;  // ns <= 8, checked on the host
     }
 }
 
@@ -84,15 +172,20 @@ __global__ void __launch_bounds__(kThreads) k_modup(const u64* __restrict__ in, 
 // all jobs of a launch use the same key (batched relinearisation), a thread
 // reads its key words once and applies them to every job.
 // ---------------------------------------------------------------------------
+// digit d's extension at position pos: its own limb of the switched polynomial, or ext
+__device__ __forceinline__ const u64* ip_ext(const IPJob& J, int d, int npos, int pos, int owner, int N) {
+    return d == owner ? J.own + (long long)pos * N : J.ext + ((long long)d * npos + pos) * N;
+}
+
 template <int BETA>
-__device__ __forceinline__ void ip_job(const IPJob& J, const u64 (&k0)[BETA], const u64 (&k1)[BETA], int npos, int pos,
+__device__ __forceinline__ void ip_job(const IPJob& J, int owner, const u64 (&k0)[BETA], const u64 (&k1)[BETA], int npos, int pos,
                                        int k, u64 q, u64 qinv, int logN, int N, int level, const u64* pmod,
                                        const u64* pmod_s) {
     const u32 src = J.galois != 1u ? galois_src_index((u32)k, J.galois, logN) : (u32)k;
     Acc128 a0{0, 0}, a1{0, 0};
 #pragma unroll
     for (int d = 0; d < BETA; ++d) {
-        const u64 e = J.ext[((long long)d * npos + pos) * N + src];
+        const u64 e = ip_ext(J, d, npos, pos, owner, N)[src];
         mac128(a0, e, k0[d]);
         mac128(a1, e, k1[d]);
         if ((d & 7) == 7) { fold(a0, q); fold(a1, q); }
@@ -119,7 +212,7 @@ __device__ __forceinline__ void ip_body(const IPJobs& jobs, int npos, int pos, i
         k1[d] = key[(((long long)d * 2 + 1) * T + klimb) * N + k];
     }
     for (int j = jobs.gstart[g]; j < jobs.gstart[g + 1]; ++j)
-        ip_job<BETA>(jobs.j[j], k0, k1, npos, pos, k, q, qinv, logN, N, level, pmod, pmod_s);
+        ip_job<BETA>(jobs.j[j], jobs.owner[pos], k0, k1, npos, pos, k, q, qinv, logN, N, level, pmod, pmod_s);
 }
 
 // key layout [digit][2][T][N]: Q limbs at positions 0.., P limbs from position kp. One
@@ -167,6 +260,7 @@ __global__ void __launch_bounds__(kThreads) k_ip_sum(const __grid_constant__ IPS
     const int pi = pos <= level ? pos : pbase + (pos - (level + 1));
     const u64 q = primes[pi].q, qinv = primes[pi].qinv;
     const int klimb = pos <= level ? pos : kp + (pos - (level + 1));
+    const int owner = jobs.owner[pos];
     Acc128 a0{0, 0}, a1{0, 0};
     u64 badd = 0;
     for (int jj = jobs.gstart[g]; jj < jobs.gstart[g + 1]; ++jj) {
@@ -174,7 +268,7 @@ __global__ void __launch_bounds__(kThreads) k_ip_sum(const __grid_constant__ IPS
         const u32 src = J.galois != 1u ? galois_src_index((u32)k, J.galois, logN) : (u32)k;
 #pragma unroll
         for (int d = 0; d < BETA; ++d) {
-            const u64 e = J.ext[((long long)d * npos + pos) * N + src];
+            const u64 e = ip_ext(J, d, npos, pos, owner, N)[src];
             mac128(a0, e, J.key[(((long long)d * 2 + 0) * T + klimb) * N + k]);
             mac128(a1, e, J.key[(((long long)d * 2 + 1) * T + klimb) * N + k]);
         }
@@ -195,36 +289,95 @@ __global__ void __launch_bounds__(kThreads) k_ip_sum(const __grid_constant__ IPS
 // conv: [J][2][level+1][N]
 // ---------------------------------------------------------------------------
 template <int NP>
-__device__ __forceinline__ void p2q_body(const u64* __restrict__ x, u64* __restrict__ o, const P2QTab* __restrict__ tab,
-                                         int level, int N, int k) {
-    u64 ys[NP];
-#pragma unroll
-    for (int i = 0; i < NP; ++i)
-        ys[i] = split30(mul_shoup(x[(long long)(level + 1 + i) * N + k], tab->inv_hat[i], tab->inv_hat_s[i], tab->pq[i]));
-    for (int i = 0; i <= level; ++i)
-        o[(long long)i * N + k] = bconv_sum<NP>(ys, tab->hat_m, i, tab->qq[i], tab->qinv[i], tab->q_one_s[i]);
+__device__ __forceinline__ void p2q_body(const u64* __restrict__ x, u64* __restrict__ o, const P2QTab& T,
+                                         const BconvTarget* st, int level, int N, int k, bool scaled) {
+    u64 y[NP][kBcW];
+    bconv_load(y, x + (long long)(level + 1) * N + k, N, scaled, T.inv_hat, T.inv_hat_s, T.pq);
+    const u64 zero[kBcW] = {};
+    for (int i = 0; i <= level; ++i) {
+        u64 v[kBcW];
+        bconv<NP>(st[i], y, zero, v);
+        *reinterpret_cast<ulonglong2*>(o + (long long)i * N + k) = make_ulonglong2(v[0], v[1]);
+    }
 }
 
 __global__ void __launch_bounds__(kThreads) k_p2q(const u64* __restrict__ acc, long long acc_job, int npos,
                                                   int level, u64* __restrict__ conv, const P2QTab* __restrict__ tab,
-                                                  int N) {
+                                                  int N, bool scaled) {
     pdl_wait();
     pdl_trigger();
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    __shared__ BconvTarget st[FR_MAX_PRIMES];
+    const int k = (blockIdx.x * blockDim.x + threadIdx.x) * kBcW;
     const int t = blockIdx.y;
     const int j = blockIdx.z;
+    stage_targets(st, tab->t, level + 1);
     if (k >= N) return;
     const u64* x = acc + (long long)j * acc_job + (long long)t * npos * N;
     u64* o = conv + ((long long)j * 2 + t) * (level + 1) * N;
     switch (tab->np) {
-        case 1: p2q_body<1>(x, o, tab, level, N, k); break;
-        case 2: p2q_body<2>(x, o, tab, level, N, k); break;
-        case 3: p2q_body<3>(x, o, tab, level, N, k); break;
-        case 4: p2q_body<4>(x, o, tab, level, N, k); break;
-        case 5: p2q_body<5>(x, o, tab, level, N, k); break;
-        case 6: p2q_body<6>(x, o, tab, level, N, k); break;
-        case 7: p2q_body<7>(x, o, tab, level, N, k); break;
-        default: p2q_body<8>(x, o, tab, level, N, k); break;  // np <= 8, checked on the host
+        case 1: p2q_body<1>(x, o, *tab, st, level, N, k, scaled); break;
+        case 2: p2q_body<2>(x, o, *tab, st, level, N, k, scaled); break;
+        case 3: p2q_body<3>(x, o, *tab, st, level, N, k, scaled); break;
+        case 4: p2q_body<4>(x, o, *tab, st, level, N, k, scaled); break;
+        case 5: p2q_body<5>(x, o, *tab, st, level, N, k, scaled); break;
+        case 6: p2q_body<6>(x, o, *tab, st, level, N, k, scaled); break;
+        case 7: p2q_body<7>(x, o, *tab, st, level, N, k, scaled); break;
+        default: p2q_body<8>(x, o, *tab, st, level, N, k, scaled); break;  // np <= 8, checked on the host
+    }
+}
+
+// The same conversion followed by a rescale's lift (moddown_rescale): the table's targets carry
+// [B/b_i]_t P^-1, so bconv gives conv_i P^-1. With zc = the last limb before the conversion's part
+// is taken off (coefficient form), the last limb is m = zc - conv_l P^-1 (mod q_l), and
+// y_i = conv_i P^-1 + [centered m]_{q_i} for i < l: m - q_l for m > half is added as m + (-q_l mod
+// q_i), unreduced, before the conversion's own reduction. acc: job j's P limbs (inv_hat in them);
+// zc [J][2][N]; y [J][2][l][N]. The conversions themselves no longer pass through memory.
+template <int NP>
+__device__ __forceinline__ void p2q_lift_body(const u64* __restrict__ x, const u64* __restrict__ zc,
+                                              u64* __restrict__ o, const BconvTarget* st, const RescaleTab& R, u64 ql,
+                                              int l, int N, int k) {
+    u64 y[NP][kBcW];
+    bconv_load(y, x + (long long)(l + 1) * N + k, N, true, nullptr, nullptr, nullptr);
+    const ulonglong2 z = *reinterpret_cast<const ulonglong2*>(zc + k);
+    const u64 zero[kBcW] = {};
+    u64 m[kBcW];
+    bconv<NP>(st[l], y, zero, m);
+    m[0] = sub_mod(z.x, m[0], ql);
+    m[1] = sub_mod(z.y, m[1], ql);
+    const bool n0 = m[0] > R.half, n1 = m[1] > R.half;
+    for (int i = 0; i < l; ++i) {
+        const u64 nq = R.q[i] - R.ql_mod[i];
+        const u64 add[kBcW] = {m[0] + (n0 ? nq : 0), m[1] + (n1 ? nq : 0)};
+        u64 v[kBcW];
+        bconv<NP>(st[i], y, add, v);
+        *reinterpret_cast<ulonglong2*>(o + (long long)i * N + k) = make_ulonglong2(v[0], v[1]);
+    }
+}
+
+__global__ void __launch_bounds__(kThreads) k_p2q_lift(const u64* __restrict__ acc, long long acc_job, int npos,
+                                                       const u64* __restrict__ zc, u64* __restrict__ y,
+                                                       const P2QTab* __restrict__ tab,
+                                                       const RescaleTab* __restrict__ rtab, u64 ql, int l, int N) {
+    pdl_wait();
+    pdl_trigger();
+    __shared__ BconvTarget st[FR_MAX_PRIMES];
+    const int k = (blockIdx.x * blockDim.x + threadIdx.x) * kBcW;
+    const int t = blockIdx.y;
+    const int j = blockIdx.z;
+    stage_targets(st, tab->t, l + 1);
+    if (k >= N) return;
+    const u64* x = acc + (long long)j * acc_job + (long long)t * npos * N;
+    const u64* z = zc + ((long long)j * 2 + t) * N;
+    u64* o = y + ((long long)j * 2 + t) * l * N;
+    switch (tab->np) {
+        case 1: p2q_lift_body<1>(x, z, o, st, *rtab, ql, l, N, k); break;
+        case 2: p2q_lift_body<2>(x, z, o, st, *rtab, ql, l, N, k); break;
+        case 3: p2q_lift_body<3>(x, z, o, st, *rtab, ql, l, N, k); break;
+        case 4: p2q_lift_body<4>(x, z, o, st, *rtab, ql, l, N, k); break;
+        case 5: p2q_lift_body<5>(x, z, o, st, *rtab, ql, l, N, k); break;
+        case 6: p2q_lift_body<6>(x, z, o, st, *rtab, ql, l, N, k); break;
+        case 7: p2q_lift_body<7>(x, z, o, st, *rtab, ql, l, N, k); break;
+        default: p2q_lift_body<8>(x, z, o, st, *rtab, ql, l, N, k); break;
     }
 }
 
@@ -319,32 +472,6 @@ __global__ void __launch_bounds__(kThreads) k_rs_last(const u64* __restrict__ ac
     const u64 a = acc[((long long)jt * npos + l) * N + k];
     const u64 dd = d ? d[(((long long)j * 3 + t) * (l + 1) + l) * N + k] : 0;
     z[(long long)jt * N + k] = add_mod(mul_shoup(a, pinv[l], pinv_s[l], q), dd, q);
-}
-
-// Relinearisation + rescale, lift: with zc = z in coefficient form and conv the P -> Q
-// conversion (coefficient form, [J][2][l+1][N]), the relinearised product's last limb is
-// m = zc - conv_l P^-1 (mod q_l); y_i = conv_i P^-1 + [centered m]_{q_i} for i < l, [J][2][l][N].
-__global__ void __launch_bounds__(kThreads) k_rs_lift(const u64* __restrict__ zc, const u64* __restrict__ conv,
-                                                      u64* __restrict__ y, const u64* __restrict__ pinv,
-                                                      const u64* __restrict__ pinv_s,
-                                                      const RescaleTab* __restrict__ tab,
-                                                      const DevPrime* __restrict__ primes, int l, int N) {
-    pdl_wait();
-    pdl_trigger();
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    const int jt = blockIdx.y;
-    if (k >= N) return;
-    const u64 ql = primes[l].q;
-    const u64* cv = conv + (long long)jt * (l + 1) * N;
-    const u64 m = sub_mod(zc[(long long)jt * N + k], mul_shoup(cv[(long long)l * N + k], pinv[l], pinv_s[l], ql), ql);
-    const bool neg = m > tab->half;
-    u64* o = y + (long long)jt * l * N;
-    for (int i = 0; i < l; ++i) {
-        const u64 q = tab->q[i];
-        u64 r = mul_shoup(m, 1, tab->one_s[i], q);
-        if (neg) r = sub_mod(r, tab->ql_mod[i], q);
-        o[(long long)i * N + k] = add_mod(mul_shoup(cv[(long long)i * N + k], pinv[i], pinv_s[i], q), r, q);
-    }
 }
 
 // out[b][t][i] = (x[b][t][i] - lifted[b][t][i]) * q_l^-1
@@ -1178,10 +1305,19 @@ __global__ void k_coef_residues(const long long* __restrict__ m, int nd, u64* __
 // launchers
 // ===========================================================================
 
-void launch_modup(const u64* in, long long in_job, const u64* in_eval, long long eval_job, u64* ext,
-                  const ModUpTab* tabs, int beta, int npos, int N, int J, cudaStream_t s) {
-    dim3 g((N + kThreads - 1) / kThreads, beta, J);
-    launch_k(k_modup, dim3(g), dim3(kThreads), 0, s, in, in_job, in_eval, eval_job, ext, tabs, beta, npos, N);
+// blocks of the base conversions: 2 points a thread
+static unsigned bconv_blocks(int N) { return (unsigned)((N + kThreads * kBcW - 1) / (kThreads * kBcW)); }
+
+void launch_modup(const u64* in, long long in_job, u64* ext, const ModUpTab* tabs, int beta, int npos, int N, int J,
+                  bool scaled, cudaStream_t s) {
+    // positions a block: all of them once the (job, digit) blocks alone give every SM 8 blocks,
+    // fewer for small batches (each chunk re-reads the digit's limbs)
+    const long long blocks = (long long)bconv_blocks(N) * beta * J;
+    int chunks = 1;
+    while (chunks < npos && blocks * chunks < 152 * 8) ++chunks;
+    const int per = (npos + chunks - 1) / chunks;
+    dim3 g(bconv_blocks(N), beta * ((npos + per - 1) / per), J);
+    launch_k(k_modup, dim3(g), dim3(kThreads), 0, s, in, in_job, ext, tabs, beta, npos, N, per, scaled);
 }
 
 void launch_ip(const IPJobs& jobs, int beta, int npos, int level, int kp, int T, const DevPrime* primes,
@@ -1218,9 +1354,15 @@ void launch_ip_sum(const IPSumJobs& jobs, int beta, int npos, int level, int kp,
 }
 
 void launch_p2q(const u64* acc, long long acc_job, int npos, int level, u64* conv, const P2QTab* tab, int N, int J,
-                cudaStream_t s) {
-    dim3 g((N + kThreads - 1) / kThreads, 2, J);
-    launch_k(k_p2q, dim3(g), dim3(kThreads), 0, s, acc, acc_job, npos, level, conv, tab, N);
+                bool scaled, cudaStream_t s) {
+    dim3 g(bconv_blocks(N), 2, J);
+    launch_k(k_p2q, dim3(g), dim3(kThreads), 0, s, acc, acc_job, npos, level, conv, tab, N, scaled);
+}
+
+void launch_p2q_lift(const u64* acc, long long acc_job, int npos, const u64* zc, u64* y, const P2QTab* tab_rs,
+                     const RescaleTab* rtab, u64 ql, int l, int N, int J, cudaStream_t s) {
+    dim3 g(bconv_blocks(N), 2, J);
+    launch_k(k_p2q_lift, dim3(g), dim3(kThreads), 0, s, acc, acc_job, npos, zc, y, tab_rs, rtab, ql, l, N);
 }
 
 void launch_moddown_combine(const MDJobs& jobs, int J, int npos, int level, const u64* pinv, const u64* pinv_s,
@@ -1240,12 +1382,6 @@ void launch_rs_last(const u64* acc, const u64* d, u64* z, const u64* pinv, const
                     const DevPrime* primes, int N, int J, cudaStream_t s) {
     dim3 g((N + kThreads - 1) / kThreads, 2 * J);
     launch_k(k_rs_last, g, dim3(kThreads), 0, s, acc, d, z, pinv, pinv_s, npos, l, primes, N);
-}
-
-void launch_rs_lift(const u64* zc, const u64* conv, u64* y, const u64* pinv, const u64* pinv_s, const RescaleTab* tab,
-                    const DevPrime* primes, int l, int N, int J, cudaStream_t s) {
-    dim3 g((N + kThreads - 1) / kThreads, 2 * J);
-    launch_k(k_rs_lift, g, dim3(kThreads), 0, s, zc, conv, y, pinv, pinv_s, tab, primes, l, N);
 }
 
 void launch_rescale_lift(const u64* last, u64* lifted, const RescaleTab* tab, int l, int N, int BT, cudaStream_t s) {

@@ -4,28 +4,35 @@
 
 #define FR_MAX_DIGIT_LIMBS 16
 
+// Fast base conversion, one target: sum_i y_i [B/b_i]_t mod t over at most 8 sources y_i < 2^61,
+// without a quotient per product (the scheme of mul_tw, dev_arith.cuh). hat[i] = (w mod 2^S, w >> S,
+// v mod 2^S, v >> S) with w = [B/b_i]_t and v = w 2^32 mod t; the products of several sources share
+// the two 64-bit sums a0, a1 and one reduction a0 + (a1 mod 2^32) 2^S + (a1 >> 32) c2.
+//   mode 0  all sources in one pair of sums (S = bits(t) - 28, targets of at most about 55 bits);
+//   mode 1  two sources at a time (S = 30), the reduced pairs folded and added (60-bit targets);
+//   mode 2  any target: hat[i].xy = w 2^64 mod t in 30-bit halves (mack), one Montgomery
+//           reduction with qinv and one_s.
+// The host picks the first mode whose sums provably fit (bconv_target).
+struct BconvTarget {
+    u64 q, qinv, one_s;
+    u32 mode, mul, c2, bsh, c, pad;  // mul = 2^S; bsh, c as in DevPrime
+    uint4 hat[8];
+};
+
 // ModUp constants of one digit at one level: sources are the digit's Q limbs
-// [lo, lo + ns); targets are every position of Q_l u P.
-// FastBConv constants. hat_m holds [B/b_i]_t in Montgomery form (times 2^64 mod t), split into
-// 30-bit halves (low half in bits 0..29, high half in bits 32..61) for the multiply-accumulate;
-// tinv = t^-1 mod 2^64 and t_one_s = floor(2^64 / t) reduce the sum.
+// [lo, lo + ns); targets are the other positions of Q_l u P. The coefficients come multiplied
+// by inv_hat = [(B/b_i)^-1]_{b_i} already (PolyBatch::post), or are multiplied here.
 struct ModUpTab {
     int ns, lo;
-    u64 src_q[FR_MAX_DIGIT_LIMBS];
-    u64 inv_hat[FR_MAX_DIGIT_LIMBS], inv_hat_s[FR_MAX_DIGIT_LIMBS];
-    u64 tq[FR_MAX_PRIMES];
-    u64 tinv[FR_MAX_PRIMES], t_one_s[FR_MAX_PRIMES];
-    u64 hat_m[FR_MAX_DIGIT_LIMBS][FR_MAX_PRIMES];
+    u64 src_q[8], inv_hat[8], inv_hat_s[8];
+    BconvTarget t[FR_MAX_PRIMES];
 };
 
 // ModDown constants: sources are the P limbs, targets Q limbs 0..l
 struct P2QTab {
     int np;
-    u64 pq[FR_MAX_DIGIT_LIMBS];
-    u64 inv_hat[FR_MAX_DIGIT_LIMBS], inv_hat_s[FR_MAX_DIGIT_LIMBS];
-    u64 qq[FR_MAX_PRIMES];
-    u64 qinv[FR_MAX_PRIMES], q_one_s[FR_MAX_PRIMES];
-    u64 hat_m[FR_MAX_DIGIT_LIMBS][FR_MAX_PRIMES];
+    u64 pq[8], inv_hat[8], inv_hat_s[8];
+    BconvTarget t[FR_MAX_PRIMES];
 };
 
 // Rescale constants at level l (divide by q_l)
@@ -38,11 +45,11 @@ struct RescaleTab {
 };
 
 struct IPJob {
-    const u64* ext;  // [beta][npos][N]
+    const u64* ext;  // [beta][npos][N]; a digit's own positions are not in it
+    const u64* own;  // the switched polynomial, limbs 0..level, stride N: the digits' own positions
     const u64* key;  // [digits][2][T][N], Montgomery form: Q limbs 0..kp-1, then P limbs
     u64* out;        // [2][npos][N]
     u32 galois;      // 1: no automorphism
-    u32 pad;
     const u64* addb = nullptr;  // non-null: add P sigma_galois(addb) to component 0 on the Q positions
                                 // (addb: limbs 0..level, stride N, evaluation form)
 };
@@ -71,6 +78,7 @@ struct TensorJob {
 // jobs grouped by key: group g uses gkey[g] for jobs gstart[g] .. gstart[g+1]-1
 struct IPJobs {
     IPJob j[FR_MAX_JOBS];
+    signed char owner[FR_MAX_PRIMES];  // digit that holds position pos (-1: none, the P limbs)
     const u64* gkey[FR_MAX_JOBS];
     int gstart[FR_MAX_JOBS + 1];
     int ngroups;
@@ -81,6 +89,7 @@ struct MDJobs { MDJob j[FR_MAX_JOBS]; };
 // addb (its rotated ciphertext's c0) are used as in IPJobs.
 struct IPSumJobs {
     IPJob j[FR_MAX_JOBS];
+    signed char owner[FR_MAX_PRIMES];
     int gstart[FR_MAX_JOBS + 1];
     int ngroups;
 };
@@ -115,26 +124,27 @@ void launch_ntt_rescale(const RingDev& R, const PolyBatch& b, const u64* x, int 
 void launch_baby0_pq(u64* babies, long long baby_q, const u64* q, long long q_bs, int q_cap, int B, int npos,
                      int level, const DevPrime* primes, const u64* pmod, const u64* pmod_s, int N, cudaStream_t s);
 // Relinearisation fused with the rescale after it (J products at level l): launch_rs_last forms
-// z = acc_l P^-1 + d_l [J][2][N]; after its inverse NTT, launch_rs_lift forms y = conv P^-1 +
-// centered lift [J][2][l][N]; the forward NTT of y with launch_ntt_relin_rescale writes
+// z = acc_l P^-1 + d_l [J][2][N]; after its inverse NTT and that of the P limbs, launch_p2q_lift
+// forms y = conv P^-1 + centered lift [J][2][l][N]; the forward NTT of y with launch_ntt_relin_rescale writes
 // out_j = (acc P^-1 + d - NTT(y)) q_l^-1 (+ the EpiRescale modes) at level l - 1.
 void launch_rs_last(const u64* acc, const u64* d, u64* z, const u64* pinv, const u64* pinv_s, int npos, int l,
                     const DevPrime* primes, int N, int J, cudaStream_t s);
-void launch_rs_lift(const u64* zc, const u64* conv, u64* y, const u64* pinv, const u64* pinv_s, const RescaleTab* tab,
-                    const DevPrime* primes, int l, int N, int J, cudaStream_t s);
+void launch_p2q_lift(const u64* acc, long long acc_job, int npos, const u64* zc, u64* y, const P2QTab* tab_rs,
+                     const RescaleTab* rtab, u64 ql, int l, int N, int J, cudaStream_t s);
 void launch_ntt_relin_rescale(const RingDev& R, const PolyBatch& b, const u64* acc, const u64* d, int npos, int l,
                               const u64* pinv, const u64* pinv_s, const RescaleTab* tab, u64* out, int out_cap,
                               long long out_bs, int mode, const u64* add, int add_cap, long long add_bs,
                               const u64* cres, cudaStream_t s);
-// ModUp of J inputs: coefficient form of input j at in + j in_job, evaluation form (for the
-// digits' own positions) at in_eval + j eval_job
-void launch_modup(const u64* in, long long in_job, const u64* in_eval, long long eval_job, u64* ext,
-                  const ModUpTab* tabs, int beta, int npos, int N, int J, cudaStream_t s);
+// ModUp of J inputs: coefficient form of input j at in + j in_job (scaled: already multiplied by
+// the digits' inv_hat); writes the positions of ext that are not the digit's own
+void launch_modup(const u64* in, long long in_job, u64* ext, const ModUpTab* tabs, int beta, int npos, int N, int J,
+                  bool scaled, cudaStream_t s);
 void launch_ip(const IPJobs& jobs, int beta, int npos, int level, int kp, int T, const DevPrime* primes,
                const PrimeMap& pos_prime, int logN, cudaStream_t s, const u64* pmod = nullptr,
                const u64* pmod_s = nullptr);
+// P limbs in coefficient form, multiplied by the tables' inv_hat (PolyBatch::post) when scaled
 void launch_p2q(const u64* acc, long long acc_job, int npos, int level, u64* conv, const P2QTab* tab, int N, int J,
-                cudaStream_t s);
+                bool scaled, cudaStream_t s);
 void launch_moddown_combine(const MDJobs& jobs, int J, int npos, int level, const u64* pinv, const u64* pinv_s,
                             const DevPrime* primes, int logN, cudaStream_t s);
 void launch_rescale_lift(const u64* last, u64* lifted, const RescaleTab* tab, int l, int N, int BT, cudaStream_t s);

@@ -104,6 +104,9 @@ struct fr_ctx {
     std::vector<int*> d_modup_ntt;       // per level: (offset, prime) of the ext positions to transform
     std::vector<int> modup_ntt_n;
     P2QTab* d_p2q = nullptr;
+    P2QTab* d_p2q_rs = nullptr;          // the same with [P]^-1 in the targets (moddown_rescale)
+    std::vector<uint4*> d_modup_post;    // per level: last constants of the ModUp input's inverse NTT, [level+1][2]
+    uint4* d_p2q_post = nullptr;         // likewise of the P limbs, [np][2]
     std::vector<RescaleTab*> d_rescale;  // per level (index level), level >= 1
     u64 *d_pinv = nullptr, *d_pinv_s = nullptr;
     u64 *d_pmod = nullptr, *d_pmod_s = nullptr;  // [P]_{q_i} and Shoup quotients, Q primes
@@ -261,27 +264,31 @@ PrimeMap pm_ext(const fr_ctx* c, int level) {
     return m;
 }
 
-void ntt(fr_ctx* c, u64* base, long long outer, int inner, int npolys, const PrimeMap& pm, bool inv) {
+// post (inverse): the polynomials' last constants (PolyBatch::post)
+void ntt(fr_ctx* c, u64* base, long long outer, int inner, int npolys, const PrimeMap& pm, bool inv,
+         const uint4* post = nullptr) {
     Prof p(c, "ntt", 16.0 * npolys * c->R.N);
     PolyBatch b{base, outer, inner, npolys, pm};
+    b.post = post;
     launch_ntt(c->rd, b, inv, c->cur);
     c->launches += 2;
 }
 // the same transform out of place: poly p read from src + (p / inner) src_outer + (p % inner) N
 // (npolys a multiple of inner), written to its place in base
 void ntt_from(fr_ctx* c, const u64* src, long long src_outer, u64* base, long long outer, int inner, int npolys,
-              const PrimeMap& pm, bool inv) {
+              const PrimeMap& pm, bool inv, const uint4* post = nullptr) {
     Prof p(c, "ntt", 16.0 * npolys * c->R.N);
     PolyBatch b{base, outer, inner, npolys, pm};
+    b.post = post;
     b.src = src;
     b.src_outer = src_outer;
     launch_ntt(c->rd, b, inv, c->cur);
     c->launches += 2;
 }
 // two transforms of the same direction in one launch: n polys of (base, outer, inner, pm), then
-// n2 polys of (base2, outer2, inner2, pm2)
+// n2 polys of (base2, outer2, inner2, pm2); post: the first segment's last constants
 void ntt_pair(fr_ctx* c, u64* base, long long outer, int inner, int n, const PrimeMap& pm, u64* base2,
-              long long outer2, int inner2, int n2, const PrimeMap& pm2, bool inv) {
+              long long outer2, int inner2, int n2, const PrimeMap& pm2, bool inv, const uint4* post) {
     Prof p(c, "ntt", 16.0 * (n + n2) * c->R.N);
     PolyBatch b{base, outer, inner, n + n2, pm};
     b.split = n;
@@ -289,6 +296,7 @@ void ntt_pair(fr_ctx* c, u64* base, long long outer, int inner, int n, const Pri
     b.outer2 = outer2;
     b.inner2 = inner2;
     b.pm2 = pm2;
+    b.post = post;
     launch_ntt(c->rd, b, inv, c->cur);
     c->launches += 2;
 }
@@ -336,6 +344,16 @@ struct KSReq {
     int sum_dst = -1;           // keyswitch_sums: index of the sum the rotation belongs to
 };
 
+// owner[pos]: the digit whose own limb position pos of Q_l u P is (-1: the P limbs)
+void digit_owners(const fr_ctx* c, int level, signed char* owner) {
+    for (int pos = 0; pos < level + 1 + c->R.np; ++pos) owner[pos] = -1;
+    for (int d = 0; d < c->R.digits_at(level); ++d) {
+        int lo, hi;
+        c->R.digit_range(level, d, &lo, &hi);
+        for (int pos = lo; pos < hi; ++pos) owner[pos] = (signed char)d;
+    }
+}
+
 // inner product + ModDown of up to FR_MAX_JOBS jobs; job j reads its ModUp output ext[j].
 // Jobs arrive sorted by key: consecutive jobs with one key form one group whose key
 // words are read once.
@@ -347,13 +365,14 @@ void ks_finish(fr_ctx* c, int level, const std::vector<const KSReq*>& reqs, cons
     Tmp conv(c, (size_t)nj * 2 * (level + 1) * N);
     IPJobs ij;
     ij.ngroups = 0;
+    digit_owners(c, level, ij.owner);
     int distinct_ext = 0;
     for (int j = 0; j < nj; ++j) {
         ij.j[j].ext = ext[j];
         ij.j[j].key = reqs[j]->key;
         ij.j[j].out = acc.p + (size_t)j * 2 * npos * N;
         ij.j[j].galois = reqs[j]->galois;
-        ij.j[j].pad = 0;
+        ij.j[j].own = reqs[j]->c;
         if (j == 0 || reqs[j]->key != reqs[j - 1]->key) {
             ij.gkey[ij.ngroups] = reqs[j]->key;
             ij.gstart[ij.ngroups] = j;
@@ -374,10 +393,10 @@ void ks_finish(fr_ctx* c, int level, const std::vector<const KSReq*>& reqs, cons
     PrimeMap pmP{};
     pmP.period = np;
     for (int j = 0; j < np; ++j) pmP.idx[j] = (unsigned char)(nq + j);
-    ntt(c, acc.p + (size_t)(level + 1) * N, (long long)npos * N, np, nj * 2 * np, pmP, true);
+    ntt(c, acc.p + (size_t)(level + 1) * N, (long long)npos * N, np, nj * 2 * np, pmP, true, c->d_p2q_post);
     {
         Prof p(c, "moddown", 8.0 * N * nj * 2.0 * (np + level + 1));
-        launch_p2q(acc.p, 2ll * npos * N, npos, level, conv.p, c->d_p2q, N, nj, c->cur);
+        launch_p2q(acc.p, 2ll * npos * N, npos, level, conv.p, c->d_p2q, N, nj, true, c->cur);
         c->launches++;
     }
     MDJobs md;
@@ -427,9 +446,9 @@ void modup_chunks(fr_ctx* c, int level, const std::vector<KSReq>& reqs, F finish
     for (size_t u0 = 0; u0 < ins.size(); u0 += UCH) {
         const int nu = (int)std::min<size_t>(UCH, ins.size() - u0);
         // inputs at one stride (the d2 parts of a batch of products, the ciphertexts of a batch)
-        // are read in place: the inverse NTT writes their coefficient form straight into `in`,
-        // and the ModUp takes the digits' own positions from the inputs themselves. Others are
-        // first gathered into a second half of `in`.
+        // are read in place: the inverse NTT writes their coefficient form, times the digits'
+        // inv_hat, straight into `in`. Others are first gathered into a second half of `in`. The
+        // inner products take the digits' own positions from the inputs themselves.
         const long long st = nu > 1 ? (long long)(ins[u0 + 1] - ins[u0]) : (long long)L1N;
         bool strided = st > 0;
         for (int u = 1; u < nu && strided; ++u) strided = ins[u0 + u] == ins[u0] + (long long)u * st;
@@ -442,11 +461,12 @@ void modup_chunks(fr_ctx* c, int level, const std::vector<KSReq>& reqs, F finish
             in_e = g;
             e_job = (long long)L1N;
         }
-        ntt_from(c, in_e, e_job, in.p, (long long)L1N, level + 1, nu * (level + 1), pm_level(level), true);
+        ntt_from(c, in_e, e_job, in.p, (long long)L1N, level + 1, nu * (level + 1), pm_level(level), true,
+                 c->d_modup_post[level]);
         Tmp ext(c, (size_t)nu * beta * npos * N);
         {
-            Prof p(c, "modup", 8.0 * N * nu * (2.0 * (level + 1) + (double)beta * npos));
-            launch_modup(in.p, (long long)L1N, in_e, e_job, ext.p, c->d_modup[level], beta, npos, N, nu, c->cur);
+            Prof p(c, "modup", 8.0 * N * nu * ((double)beta * npos));
+            launch_modup(in.p, (long long)L1N, ext.p, c->d_modup[level], beta, npos, N, nu, true, c->cur);
             c->launches++;
         }
         ntt_modup(c, ext.p, nu, level);
@@ -492,8 +512,6 @@ void keyswitch_sums(fr_ctx* c, int level, const std::vector<KSReq>& reqs, const 
         Prof p(c, "copy", 8.0 * ndst * aw);
         CU(cudaMemsetAsync(accs.p, 0, (size_t)ndst * aw * 8, c->cur));
     }
-    const int pbase = nq;
-    (void)pbase;
     modup_chunks(c, level, reqs, [&](const std::vector<const KSReq*>& rq, const std::vector<const u64*>& ex) {
         // the jobs of one sum form one group of the summing inner product
         const int nj = (int)rq.size();
@@ -505,10 +523,11 @@ void keyswitch_sums(fr_ctx* c, int level, const std::vector<KSReq>& reqs, const 
         std::stable_sort(ord.begin(), ord.end(), [&](int a, int b) { return rq[a]->sum_dst < rq[b]->sum_dst; });
         IPSumJobs ij;
         ij.ngroups = 0;
+        digit_owners(c, level, ij.owner);
         std::vector<const u64*> keys, exts;
         for (int t = 0; t < nj; ++t) {
             const KSReq* r = rq[ord[t]];
-            ij.j[t] = IPJob{ex[ord[t]], r->key, accs.p + (size_t)r->sum_dst * aw, r->galois, 0, r->add};
+            ij.j[t] = IPJob{ex[ord[t]], r->c, r->key, accs.p + (size_t)r->sum_dst * aw, r->galois, r->add};
             if (t == 0 || r->sum_dst != rq[ord[t - 1]]->sum_dst) ij.gstart[ij.ngroups++] = t;
             if (std::find(keys.begin(), keys.end(), r->key) == keys.end()) keys.push_back(r->key);
             if (std::find(exts.begin(), exts.end(), ex[ord[t]]) == exts.end()) exts.push_back(ex[ord[t]]);
@@ -526,11 +545,11 @@ void keyswitch_sums(fr_ctx* c, int level, const std::vector<KSReq>& reqs, const 
     PrimeMap pmP{};
     pmP.period = np;
     for (int j = 0; j < np; ++j) pmP.idx[j] = (unsigned char)(nq + j);
-    ntt(c, accs.p + (size_t)(level + 1) * N, (long long)npos * N, np, ndst * 2 * np, pmP, true);
+    ntt(c, accs.p + (size_t)(level + 1) * N, (long long)npos * N, np, ndst * 2 * np, pmP, true, c->d_p2q_post);
     Tmp conv(c, (size_t)ndst * 2 * (level + 1) * N);
     {
         Prof p(c, "moddown", 8.0 * N * ndst * 2.0 * (np + level + 1));
-        launch_p2q(accs.p, (long long)aw, npos, level, conv.p, c->d_p2q, N, ndst, c->cur);
+        launch_p2q(accs.p, (long long)aw, npos, level, conv.p, c->d_p2q, N, ndst, true, c->cur);
         c->launches++;
     }
     for (int o0 = 0; o0 < ndst; o0 += FR_MAX_JOBS) {
@@ -695,19 +714,15 @@ void moddown_rescale(fr_ctx* c, int l, u64* acc, const u64* d, int nj, u64* out,
         launch_rs_last(acc, d, z.p, c->d_pinv, c->d_pinv_s, npos, l, c->d_primes, N, nj, c->cur);
         c->launches++;
     }
-    // the P limbs and that last limb to coefficients, in one launch; the P -> Q conversion
-    ntt_pair(c, acc + (size_t)(l + 1) * N, (long long)npos * N, np, nj * 2 * np, pmP, z.p, N, 1, 2 * nj, pmL, true);
-    Tmp conv(c, (size_t)nj * 2 * (l + 1) * N);
-    {
-        Prof p(c, "moddown", 8.0 * N * nj * 2.0 * (np + l + 1));
-        launch_p2q(acc, (long long)aw, npos, l, conv.p, c->d_p2q, N, nj, c->cur);
-        c->launches++;
-    }
-    // the lift; one forward NTT with the combine as its epilogue
+    // the P limbs and that last limb to coefficients, in one launch; the P -> Q conversion and the
+    // lift; one forward NTT with the combine as its epilogue
+    ntt_pair(c, acc + (size_t)(l + 1) * N, (long long)npos * N, np, nj * 2 * np, pmP, z.p, N, 1, 2 * nj, pmL, true,
+             c->d_p2q_post);
     Tmp y(c, (size_t)nj * 2 * l * N);
     {
-        Prof p(c, "rescale", 8.0 * N * nj * 2.0 * (2.0 + 2.0 * l));
-        launch_rs_lift(z.p, conv.p, y.p, c->d_pinv, c->d_pinv_s, c->d_rescale[l], c->d_primes, l, N, nj, c->cur);
+        Prof p(c, "moddown", 8.0 * N * nj * 2.0 * (np + 1 + l));
+        launch_p2q_lift(acc, (long long)aw, npos, z.p, y.p, c->d_p2q_rs, c->d_rescale[l], c->R.primes[l], l, N, nj,
+                        c->cur);
         c->launches++;
     }
     Prof p(c, "ntt", 16.0 * nj * 2 * l * N);
@@ -751,12 +766,13 @@ void mul_relin_rescale(fr_ctx* c, int l, const std::vector<const u64*>& A, int a
         modup_chunks(c, l, reqs, [&](const std::vector<const KSReq*>& rq, const std::vector<const u64*>& ex) {
             IPJobs ij;
             ij.ngroups = 1;
+            digit_owners(c, l, ij.owner);
             ij.gkey[0] = rq[0]->key;
             ij.gstart[0] = 0;
             ij.gstart[1] = (int)rq.size();
             for (size_t t = 0; t < rq.size(); ++t) {
                 const int j = (int)(rq[t]->c - (d.p + 2 * (size_t)(l + 1) * N)) / (int)dw;  // job of this request
-                ij.j[t] = IPJob{ex[t], rq[t]->key, acc.p + (size_t)j * aw, 1u, 0};
+                ij.j[t] = IPJob{ex[t], rq[t]->c, rq[t]->key, acc.p + (size_t)j * aw, 1u};
             }
             Prof p(c, "ip", 8.0 * N * npos * (2.0 * c->R.digits_at(l) + (double)rq.size() * (c->R.digits_at(l) + 2.0)));
             launch_ip(ij, c->R.digits_at(l), npos, l, c->key_level + 1, c->key_limbs, c->d_primes, pm_ext(c, l),
@@ -1257,6 +1273,54 @@ u64 inv_mod_2_64(u64 q) {
 // 30-bit halves of a residue below 2^60: low half in bits 0..29, high half in bits 32..61
 u64 split30_host(u64 x) { return (x & 0x3fffffffull) | ((x >> 30) << 32); }
 
+// Target t of a base conversion with constants hat (one per source, all sources below 2^61): the
+// first mode of BconvTarget whose sums fit in 64 bits, with an addend below 2^61 in the first.
+BconvTarget bconv_target(u64 t, const std::vector<u64>& hat) {
+    BconvTarget T;
+    std::memset(&T, 0, sizeof(T));
+    T.q = t;
+    T.qinv = inv_mod_2_64(t);
+    T.one_s = frh::shoup_quot(1, t);
+    int b = 64;
+    while (!(t >> (b - 1))) --b;
+    const int ns = (int)hat.size();
+    const u64 c = ((u64)1 << b) - t, r32 = ((u64)1 << 32) % t;
+    const u128 two64 = (u128)1 << 64;
+    auto fold_ok = [&](u128 v) {  // fold_top(v) is below 2t
+        return v < two64 && (v >> b) >> 32 == 0 && (((u128)1 << b) - 1) + (v >> b) * c < (u128)2 * t;
+    };
+    for (u32 mode = 0; mode < 2; ++mode) {
+        const int S = mode == 0 ? b - 28 : 30, group = mode == 0 ? ns : std::min(ns, 2);
+        if (b <= 33 || c >> 32 || S < 1 || S > 31) continue;
+        if ((t - 1) >> S >> 32) continue;
+        const u64 wl = ((u64)1 << S) - 1, wh = (t - 1) >> S, xl = 0xffffffffull, xh = 0x1fffffffull;
+        const u128 a1 = (u128)group * (u128)wh * (xl + xh), a0 = (u128)group * (u128)wl * (xl + xh);
+        const u64 c2 = (u64)(((u128)1 << (S + 32)) % t);
+        const u128 add = mode == 0 ? (u128)1 << 61 : 0;
+        if (a1 >= two64 || c2 >> 32) continue;
+        const u128 r = a0 + add + ((u128)0xffffffffu << S) + (a1 >> 32) * c2;
+        if (!fold_ok(r)) continue;
+        // mode 1: the folded pairs (below 2t) and an addend, folded once more
+        if (mode == 1 && !fold_ok((u128)((ns + 1) / 2) * 2 * t + ((u128)1 << 61))) continue;
+        T.mode = mode;
+        T.mul = (u32)1 << S;
+        T.c2 = (u32)c2;
+        T.bsh = (u32)(b - 32);
+        T.c = (u32)c;
+        for (int i = 0; i < ns; ++i) {
+            const u64 v = frh::mulm(hat[i], r32, t);
+            T.hat[i] = make_uint4((u32)(hat[i] & wl), (u32)(hat[i] >> S), (u32)(v & wl), (u32)(v >> S));
+        }
+        return T;
+    }
+    T.mode = 2;
+    for (int i = 0; i < ns; ++i) {
+        const u64 h = split30_host((u64)(((u128)hat[i] << 64) % t));
+        T.hat[i] = make_uint4((u32)h, (u32)(h >> 32), 0, 0);
+    }
+    return T;
+}
+
 // Twiddle class of prime q and its constants in d (see mul_tw): the first class whose sums
 // provably stay in 64 bits.
 void twiddle_class(u64 q, DevPrime& d) {
@@ -1363,18 +1427,29 @@ void build_tables(fr_ctx* c) {
     uint4 *tw, *itw, *rtw, *irtw;
     upload_tw(false, &tw, &rtw);
     upload_tw(true, &itw, &irtw);
-    c->rd = RingDev{R.logN, N, T, c->d_primes, tw, itw, rtw, irtw, fast};
+    c->rd = RingDev{R.logN, N, T, c->d_primes, tw, itw, rtw, irtw, fast, {0, 0, 0, 0}};
+    // untuned shapes: 16 residues a thread from 17 polynomials up (see launch_ntt)
+    if (rows) c->rd.ntt_shape[2] = c->rd.ntt_shape[3] = 5;
     c->d_rot = upload_persistent(c, R.rot_group.data(), R.rot_group.size());
     c->d_zr = upload_persistent(c, R.zr.data(), R.zr.size());
     c->d_zi = upload_persistent(c, R.zi.data(), R.zi.size());
     if (R.ndig > 8) raise(FR_ERR_UNSUPPORTED, "more than 8 key-switching digits");
+    // the last constants of prime pi's inverse transform, times k
+    auto post_of = [&](int pi, u64 k, std::vector<uint4>& out) {
+        const u64 q = R.primes[pi], n = frh::mulm(R.tabs[pi].ninv, k, q);
+        const Twiddler tw(dp[pi]);
+        out.push_back(tw(n));
+        out.push_back(tw(frh::mulm(n, R.tabs[pi].itw[1], q)));
+    };
     // ModUp tables per level
     c->d_modup.assign(R.nq, nullptr);
     c->d_modup_ntt.assign(R.nq, nullptr);
+    c->d_modup_post.assign(R.nq, nullptr);
     c->modup_ntt_n.assign(R.nq, 0);
     for (int l = 0; l < R.nq; ++l) {
         const int beta = R.digits_at(l), npos = l + 1 + R.np;
         std::vector<ModUpTab> tabs(beta);
+        std::vector<uint4> post;
         for (int d = 0; d < beta; ++d) {
             ModUpTab& t = tabs[d];
             std::memset(&t, 0, sizeof(t));
@@ -1385,23 +1460,21 @@ void build_tables(fr_ctx* c) {
             if (t.ns > 8) raise(FR_ERR_UNSUPPORTED, "key-switching digit wider than 8 limbs");
             std::vector<int> src;
             for (int i = lo; i < hi; ++i) src.push_back(i);
-            for (int i = 0; i < t.ns; ++i) t.src_q[i] = R.primes[lo + i];
+            std::vector<u64> ih, ht;
             for (int pos = 0; pos < npos; ++pos) {
                 const int pi = pos <= l ? pos : R.nq + pos - l - 1;
-                const u64 tp = R.primes[pi];
-                t.tq[pos] = tp;
-                t.tinv[pos] = inv_mod_2_64(tp);
-                t.t_one_s[pos] = (u64)(((unsigned __int128)1 << 64) / tp);
-                std::vector<u64> ih, ht;
                 frh::bconv_consts(R, src, pi, ih, ht);
-                for (int i = 0; i < t.ns; ++i) {
-                    t.inv_hat[i] = ih[i];
-                    t.inv_hat_s[i] = frh::shoup_quot(ih[i], R.primes[lo + i]);
-                    t.hat_m[i][pos] = split30_host((u64)(((unsigned __int128)ht[i] << 64) % tp));
-                }
+                if (pos < lo || pos >= hi) t.t[pos] = bconv_target(R.primes[pi], ht);
+            }
+            for (int i = 0; i < t.ns; ++i) {
+                t.src_q[i] = R.primes[lo + i];
+                t.inv_hat[i] = ih[i];
+                t.inv_hat_s[i] = frh::shoup_quot(ih[i], R.primes[lo + i]);
+                post_of(lo + i, ih[i], post);
             }
         }
         c->d_modup[l] = upload_persistent(c, tabs.data(), tabs.size());
+        c->d_modup_post[l] = upload_persistent(c, post.data(), post.size());
         std::vector<int> nt;
         for (int d = 0; d < beta; ++d)
             for (int pos = 0; pos < npos; ++pos) {
@@ -1414,33 +1487,37 @@ void build_tables(fr_ctx* c) {
     }
     // ModDown: P -> Q
     {
-        P2QTab t;
+        P2QTab t, trs;
         std::memset(&t, 0, sizeof(t));
         t.np = R.np;
         if (R.np > 8) raise(FR_ERR_UNSUPPORTED, "more than 8 special primes");
         std::vector<int> src;
         for (int j = 0; j < R.np; ++j) src.push_back(R.nq + j);
-        for (int j = 0; j < R.np; ++j) t.pq[j] = R.primes[R.nq + j];
-        std::vector<u64> pinv(R.nq), pinv_s(R.nq), pmod(R.nq), pmod_s(R.nq);
+        std::vector<u64> pinv(R.nq), pinv_s(R.nq), pmod(R.nq), pmod_s(R.nq), ih, ht;
+        trs = t;
         for (int i = 0; i < R.nq; ++i) {
-            t.qq[i] = R.primes[i];
-            std::vector<u64> ih, ht;
-            frh::bconv_consts(R, src, i, ih, ht);
-            t.qinv[i] = inv_mod_2_64(R.primes[i]);
-            t.q_one_s[i] = (u64)(((unsigned __int128)1 << 64) / R.primes[i]);
-            for (int j = 0; j < R.np; ++j) {
-                t.inv_hat[j] = ih[j];
-                t.inv_hat_s[j] = frh::shoup_quot(ih[j], t.pq[j]);
-                t.hat_m[j][i] = split30_host((u64)(((unsigned __int128)ht[j] << 64) % R.primes[i]));
-            }
+            const u64 q = R.primes[i];
             u64 P = 1;
-            for (int j = 0; j < R.np; ++j) P = frh::mulm(P, t.pq[j] % R.primes[i], R.primes[i]);
-            pinv[i] = frh::invm(P, R.primes[i]);
-            pinv_s[i] = frh::shoup_quot(pinv[i], R.primes[i]);
+            for (int j = 0; j < R.np; ++j) P = frh::mulm(P, R.primes[R.nq + j] % q, q);
+            pinv[i] = frh::invm(P, q);
+            pinv_s[i] = frh::shoup_quot(pinv[i], q);
             pmod[i] = P;
-            pmod_s[i] = frh::shoup_quot(P, R.primes[i]);
+            pmod_s[i] = frh::shoup_quot(P, q);
+            frh::bconv_consts(R, src, i, ih, ht);
+            t.t[i] = bconv_target(q, ht);
+            for (u64& h : ht) h = frh::mulm(h, pinv[i], q);
+            trs.t[i] = bconv_target(q, ht);
+        }
+        std::vector<uint4> post;
+        for (int j = 0; j < R.np; ++j) {
+            t.pq[j] = trs.pq[j] = R.primes[R.nq + j];
+            t.inv_hat[j] = trs.inv_hat[j] = ih[j];
+            t.inv_hat_s[j] = trs.inv_hat_s[j] = frh::shoup_quot(ih[j], t.pq[j]);
+            post_of(R.nq + j, ih[j], post);
         }
         c->d_p2q = upload_persistent(c, &t, 1);
+        c->d_p2q_rs = upload_persistent(c, &trs, 1);
+        c->d_p2q_post = upload_persistent(c, post.data(), post.size());
         c->d_pinv = upload_persistent(c, pinv.data(), pinv.size());
         c->d_pinv_s = upload_persistent(c, pinv_s.data(), pinv_s.size());
         c->d_pmod = upload_persistent(c, pmod.data(), pmod.size());
@@ -2305,9 +2382,10 @@ void ondemand_scores(fr_ctx* c, const BatchPlan& P, const u64* q, const std::vec
             modup_chunks(c, L, reqs, [&](const std::vector<const KSReq*>& rq, const std::vector<const u64*>& ex) {
                 IPJobs ij;
                 ij.ngroups = 0;
+                digit_owners(c, L, ij.owner);
                 const int nj = (int)rq.size();
                 for (int j = 0; j < nj; ++j) {
-                    ij.j[j] = IPJob{ex[j], rq[j]->key, rq[j]->out, rq[j]->galois, 0, rq[j]->add};  // + P sigma(b)
+                    ij.j[j] = IPJob{ex[j], rq[j]->c, rq[j]->key, rq[j]->out, rq[j]->galois, rq[j]->add};  // + P sigma(b)
                     if (j == 0 || rq[j]->key != rq[j - 1]->key) {
                         ij.gkey[ij.ngroups] = rq[j]->key;
                         ij.gstart[ij.ngroups] = j;
@@ -3508,12 +3586,13 @@ extern "C" fr_status fr_rotate_noalloc(fr_ctx* c, const uint64_t* d_in, uint32_t
         CU(cudaMemcpyAsync(a, d_in + L1N, L1N * 8, cudaMemcpyDeviceToDevice, st));
         const PrimeMap pl = pm_level(l);
         launch_ntt(c->rd, PolyBatch{e, (long long)N, 2 * (l + 1), 2 * (l + 1), pl}, false, st);
-        launch_modup(a, 0, e + L1N, 0, ext, c->d_modup[l], beta, npos, N, 1, st);
+        launch_modup(a, 0, ext, c->d_modup[l], beta, npos, N, 1, false, st);
         launch_ntt(c->rd, PolyBatch{ext, (long long)beta * npos * N, 1, c->modup_ntt_n[l], PrimeMap{},
                                     c->d_modup_ntt[l], c->modup_ntt_n[l]},
                    false, st);
         IPJobs ij;
-        ij.j[0] = IPJob{ext, key, acc, (u32)g, 0};
+        digit_owners(c, l, ij.owner);
+        ij.j[0] = IPJob{ext, e + L1N, key, acc, (u32)g};
         ij.gkey[0] = key;
         ij.gstart[0] = 0;
         ij.gstart[1] = 1;
@@ -3523,7 +3602,7 @@ extern "C" fr_status fr_rotate_noalloc(fr_ctx* c, const uint64_t* d_in, uint32_t
         pmP.period = np;
         for (int j = 0; j < np; ++j) pmP.idx[j] = (unsigned char)(nq + j);
         launch_ntt(c->rd, PolyBatch{acc + L1N, (long long)npos * N, np, 2 * np, pmP}, true, st);
-        launch_p2q(acc, 2ll * npos * N, npos, l, conv, c->d_p2q, N, 1, st);
+        launch_p2q(acc, 2ll * npos * N, npos, l, conv, c->d_p2q, N, 1, false, st);
         launch_ntt(c->rd, PolyBatch{conv, (long long)L1N, l + 1, 2 * (l + 1), pl}, false, st);
         MDJobs md;
         md.j[0] = MDJob{acc, conv, e, d_out, l + 1, l + 1, 1, (u32)g};

@@ -92,6 +92,10 @@ struct PolyBatch {
     long long outer2 = 0;
     int inner2 = 1;
     PrimeMap pm2{};
+    // optional (inverse, first segment): poly p ends with the constants post[2e], post[2e + 1], e =
+    // p % pm.period, instead of its prime's N^-1 and N^-1 itw[1] (tw_ninv, tw_wninv): a constant
+    // factor on the coefficients costs nothing
+    const uint4* post = nullptr;
 };
 
 // NTT batch-size buckets for the tuned tile shapes: <= 4, <= 16, <= 64, larger.
@@ -133,16 +137,3 @@ void tune_ntt(RingDev& R, cudaStream_t s, double* us, int reps);
 double measure_butterfly_peak(int device);
 // FP64 operations per second of fused multiply-adds with operands in registers.
 double measure_fp64_peak(int device);
-
-// Fast base conversion tables for one (source set, target list).
-struct BconvTab {
-    int ns;                          // source limbs
-    int nt;                          // target limbs
-    int src_prime[FR_MAX_DIGITS];    // prime indices of the sources
-    int src_pos[FR_MAX_DIGITS];      // positions of the sources in the input layout
-    u64 inv_hat[FR_MAX_DIGITS];      // [(B/b_i)^-1]_{b_i}
-    u64 inv_hat_s[FR_MAX_DIGITS];
-    int tgt_prime[FR_MAX_PRIMES];    // prime index of target t
-    int tgt_pos[FR_MAX_PRIMES];      // position of target t in the output layout
-};
-// hat[i][t] = [B/b_i]_{q_t}, with Shoup quotients; stored on the device as [ns][nt] pairs

@@ -53,6 +53,11 @@ __device__ __forceinline__ const u64* poly_in(const PolyBatch& b, int p, int N, 
     return b.src ? b.src + (long long)(p / b.inner) * b.src_outer + (long long)(p % b.inner) * N : x;
 }
 
+// poly p's own final constants of an inverse transform, if its batch has them
+__device__ __forceinline__ const uint4* poly_post(const PolyBatch& b, int p) {
+    return b.post && !(b.split && p >= b.split) ? b.post + 2 * (p % b.pm.period) : nullptr;
+}
+
 // element index of register e of thread tau in a phase whose RB bits start at LO
 template <int RB, int LO>
 __device__ __forceinline__ int phase_x(int tau, int e) {
@@ -345,9 +350,11 @@ __device__ __forceinline__ void stages(u64 (&v)[1 << RB], int tau, const C& c) {
 
 // The phases of a pass, PH .. P - 1, exchanging through ex between them. An inverse column pass
 // ends with its last stage (twiddle 1 of the table) and the product by N^-1 in one: the sums are
-// multiplied by N^-1, the differences by N^-1 times the twiddle (FIN).
+// multiplied by N^-1, the differences by N^-1 times the twiddle (FIN), or by the batch's own
+// constants in their place (post).
 template <int CLS, int RB, int LOG, bool INV, bool FIN, int PH, class Ex, class C>
-__device__ __forceinline__ void phases(u64 (&v)[1 << RB], int tau, const C& c, Ex& ex, const DevPrime& P) {
+__device__ __forceinline__ void phases(u64 (&v)[1 << RB], int tau, const C& c, Ex& ex, const DevPrime& P,
+                                       const uint4* post = nullptr) {
     using I = PhaseInfo<RB, LOG, INV, PH>;
     constexpr bool last = PH == I::P - 1;
     if constexpr (PH > 0) {
@@ -358,7 +365,7 @@ __device__ __forceinline__ void phases(u64 (&v)[1 << RB], int tau, const C& c, E
     stages<INV, CLS, RB, I::LO, I::BFROM, BTO, 0>(v, tau, c);
     if constexpr (FIN && last) {
         constexpr int lb = LOG - 1 - I::LO, T = BTO - I::BFROM;
-        const uint4 wn = P.tw_ninv, ww = P.tw_wninv;
+        const uint4 wn = post ? __ldg(post) : P.tw_ninv, ww = post ? __ldg(post + 1) : P.tw_wninv;
         const u64 lift = CLS == 0 ? c.off << T : CLS == 1 ? c.big : 2 * c.q;
 #pragma unroll
         for (int e = 0; e < (1 << RB); ++e) {
@@ -374,7 +381,7 @@ __device__ __forceinline__ void phases(u64 (&v)[1 << RB], int tau, const C& c, E
         for (int e = 0; e < (1 << RB); ++e)
             if (!(e & (1 << lb))) v[e] = fold_top(v[e], c.bsh, c.c);
     }
-    if constexpr (!last) phases<CLS, RB, LOG, INV, FIN, PH + 1>(v, tau, c, ex, P);
+    if constexpr (!last) phases<CLS, RB, LOG, INV, FIN, PH + 1>(v, tau, c, ex, P, post);
 }
 
 // exchange through shared memory, column layout s[x'][KTC]. With 4 columns x' = x ^ x3 ^
@@ -466,7 +473,7 @@ __device__ __forceinline__ void ntt_col_body(const PolyBatch& b, u64* x, const u
     __syncthreads();
     const Ctx<CLS, 0, LOG> c(0, S, sw, P);
     ColEx<KTC> ex{sm, col};
-    phases<CLS, RB, LOG, INV, INV, 0>(v, tau, c, ex, P);
+    phases<CLS, RB, LOG, INV, INV, 0>(v, tau, c, ex, P, poly_post(b, p));
 #pragma unroll
     for (int e = 0; e < (1 << RB); ++e) x[(long long)phase_x<RB, LL>(tau, e) * C + gcol] = INV ? c.canon(v[e]) : v[e];
 }
@@ -549,7 +556,7 @@ constexpr size_t kClusterSmem = (size_t)(2 * 8192 + 2 * 256) * sizeof(u64);
 
 template <bool INV, int CLS, class E>
 __device__ __forceinline__ void ntt_cluster_body(const RingDev& R, u64* x, const uint4* tw, const DevPrime& P, int p,
-                                                 u64* sm, const E& epi) {
+                                                 u64* sm, const E& epi, const uint4* post) {
     namespace cg = cooperative_groups;
     constexpr int LOG = 8, S = 256;
     u64* A = sm;              // 32 rows x 256 (row layout) / 256 rows x 32 columns (column layout)
@@ -610,7 +617,7 @@ __device__ __forceinline__ void ntt_cluster_body(const RingDev& R, u64* x, const
 #pragma unroll
         for (int e = 0; e < 8; ++e) v[e] = A[phase_x<3, L0>(tauc, e) * 32 + col];
         ColEx<32> exc{Bb, col};
-        phases<CLS, 3, LOG, true, true, 0>(v, tauc, c, exc, P);
+        phases<CLS, 3, LOG, true, true, 0>(v, tauc, c, exc, P, post);
 #pragma unroll
         for (int e = 0; e < 8; ++e) x[(long long)phase_x<3, LL>(tauc, e) * S + gcol] = c.canon(v[e]);
     }
@@ -628,8 +635,8 @@ __global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(1024, 1)
     u64* x = poly_at(b, p, R.N, &pi);
     const uint4* tw = (INV ? R.itw : R.tw) + (size_t)pi * R.N;
     const DevPrime P = R.primes[pi];  // class 0 or 1: the launcher checks
-    if (P.cls == 0) ntt_cluster_body<INV, 0>(R, x, tw, P, p, sm, epi);
-    else ntt_cluster_body<INV, 1>(R, x, tw, P, p, sm, epi);
+    if (P.cls == 0) ntt_cluster_body<INV, 0>(R, x, tw, P, p, sm, epi, poly_post(b, p));
+    else ntt_cluster_body<INV, 1>(R, x, tw, P, p, sm, epi, poly_post(b, p));
 }
 
 // ---------------------------------------------------------------------------
@@ -924,7 +931,6 @@ void launch_ntt(const RingDev& R, const PolyBatch& b, bool inverse, cudaStream_t
 // (CUDA events, best of `reps`) on a scratch buffer of zero residues and keeps the fastest
 // shape per bucket in R.ntt_shape; us[bucket * FR_NTT_SHAPES + shape] receives the times.
 void tune_ntt(RingDev& R, cudaStream_t s, double* us, int reps) {
-    for (int bk = 0; bk < FR_NTT_BUCKETS; ++bk) R.ntt_shape[bk] = 0;
     if (us)
         for (int i = 0; i < FR_NTT_BUCKETS * FR_NTT_SHAPES; ++i) us[i] = 0;
     if (R.logN < 14) return;
@@ -951,14 +957,6 @@ void tune_ntt(RingDev& R, cudaStream_t s, double* us, int reps) {
         if (cudaGetLastError() != cudaSuccess) return 1e30;  // a shape this GPU cannot launch
         return ms * 1000.0;
     };
-    // an idle GPU's clocks take some milliseconds to rise: a first timing of 4 polynomials read
-    // 600 us instead of 25, and the shapes were picked by chance
-    double before = timed(FR_NTT_BUCKETS - 1, 0);
-    for (int i = 0, same = 0; i < 60 && same < 8; ++i) {
-        const double now = timed(FR_NTT_BUCKETS - 1, 0);
-        same = now > 0.97 * before && now < 1.03 * before ? same + 1 : 0;
-        before = now;
-    }
     unsigned char best[FR_NTT_BUCKETS];
     for (int bk = 0; bk < FR_NTT_BUCKETS; ++bk) {
         double t[FR_NTT_SHAPES];

@@ -66,3 +66,26 @@ def test_noalloc_rotation_on_any_word_address(words_off):
     ctx.sync()
     got = buf[words_off: words_off + a.size].cpu().numpy().view(np.uint64).reshape(a.shape)
     assert np.array_equal(got, ref)
+
+
+@pytest.mark.parametrize("n_q,n_p", [(5, 5), (7, 6), (8, 8)])
+@pytest.mark.parametrize("log_n", [11, 14])
+def test_base_conversion_of_wide_digits(log_n, n_q, n_p):
+    """One digit of up to 8 limbs, up to 8 special primes, 50- and 60-bit targets: the sums of
+    every number of sources, without and with the rescale's lift (mul_relin, then rescale)."""
+    p = dict(q_bits=[60] + [50, 60, 45] * 3, p_bits=[60, 60, 59, 60] * 2, scale_bits=45)
+    p["q_bits"], p["p_bits"] = p["q_bits"][:n_q], p["p_bits"][:n_p]
+    ctx = fr.Context(device=0, log_n=log_n, dnum=1, ell=64, n1=8, **p)
+    ctx.load_keys(ctx.keygen([3], 77))
+    oc = oracle.Ctx(log_n, p["q_bits"], p["p_bits"], 1, p["scale_bits"])
+    ok = oc.keygen(77)
+    top = oc.top
+    a, b = (_residues(ctx.primes()[: top + 1], ctx.N, 177 + s) for s in (1, 2))
+    ca, cb = ctx.import_ct(a, top).upload(), ctx.import_ct(b, top).upload()
+    for l in (top, top - 1):
+        x = np.ascontiguousarray(a[:, : l + 1])
+        assert np.array_equal(ctx.rotate(ctx.import_ct(x, l).upload(), 3).export(), ok.rotate(x, l, 3)), l
+    mul = ok.mul_relin(a, b, top)
+    got = ctx.mul_relin(ca, cb)
+    assert np.array_equal(got.export(), mul)
+    assert np.array_equal(ctx.rescale(got).export(), oc.rescale(mul, top))
