@@ -20,8 +20,8 @@ struct BconvTarget {
 };
 
 // ModUp constants of one digit at one level: sources are the digit's Q limbs
-// [lo, lo + ns); targets are the other positions of Q_l u P. The coefficients come multiplied
-// by inv_hat = [(B/b_i)^-1]_{b_i} already (PolyBatch::post), or are multiplied here.
+// [lo, lo + ns); targets are the other positions of Q_l u P. inv_hat = [(B/b_i)^-1]_{b_i}; the
+// inverse transforms before a conversion multiply it in (PolyBatch::post).
 struct ModUpTab {
     int ns, lo;
     u64 src_q[8], inv_hat[8], inv_hat_s[8];
@@ -31,7 +31,6 @@ struct ModUpTab {
 // ModDown constants: sources are the P limbs, targets Q limbs 0..l
 struct P2QTab {
     int np;
-    u64 pq[8], inv_hat[8], inv_hat_s[8];
     BconvTarget t[FR_MAX_PRIMES];
 };
 
@@ -56,7 +55,6 @@ struct IPJob {
 
 struct MDJob {
     const u64* acc;   // [2][npos][N]
-    const u64* conv;  // [2][level+1][N]
     const u64* add;   // modes 1, 3: c0 limbs (stride N); mode 2: ct with add_cap
     u64* out;         // ct with out_cap
     int out_cap;
@@ -97,9 +95,9 @@ struct TensorJobs { TensorJob j[FR_MAX_JOBS]; };
 
 // Forward NTT that stores its values in Montgomery form (x 2^64 mod q), in place.
 void launch_ntt_tomont(const RingDev& R, const PolyBatch& b, cudaStream_t s);
-// Forward NTT of the P -> Q conversions of a ModDown fused with its combine: poly p of b is
-// (job p / (2(level+1)), component, limb); the transformed values never reach memory, the
-// jobs' outputs do (as launch_moddown_combine would write them).
+// Forward NTT of the P -> Q conversions of a ModDown (b.conv forms them) fused with its combine:
+// poly p of b is (job p / (2(level+1)), component, limb); the transformed values never reach
+// memory, the jobs' outputs do.
 void launch_ntt_moddown(const RingDev& R, const PolyBatch& b, const MDJobs& jobs, int npos, int level,
                         const u64* pinv, const u64* pinv_s, cudaStream_t s);
 // Forward NTT of a rescale's lifted last limb fused with its combine: poly p of b is
@@ -135,6 +133,10 @@ void launch_ntt_relin_rescale(const RingDev& R, const PolyBatch& b, const u64* a
                               const u64* pinv, const u64* pinv_s, const RescaleTab* tab, u64* out, int out_cap,
                               long long out_bs, int mode, const u64* add, int add_cap, long long add_bs,
                               const u64* cres, cudaStream_t s);
+// Target polynomials up to which a base conversion runs inside the column pass of the transform
+// after it (PolyBatch::conv) instead of in its own kernel: one launch less, at the price of reading
+// the sources once per target.
+constexpr int kConvFused = 16;
 // ModUp of J inputs: coefficient form of input j at in + j in_job (scaled: already multiplied by
 // the digits' inv_hat); writes the positions of ext that are not the digit's own
 void launch_modup(const u64* in, long long in_job, u64* ext, const ModUpTab* tabs, int beta, int npos, int N, int J,
@@ -142,11 +144,9 @@ void launch_modup(const u64* in, long long in_job, u64* ext, const ModUpTab* tab
 void launch_ip(const IPJobs& jobs, int beta, int npos, int level, int kp, int T, const DevPrime* primes,
                const PrimeMap& pos_prime, int logN, cudaStream_t s, const u64* pmod = nullptr,
                const u64* pmod_s = nullptr);
-// P limbs in coefficient form, multiplied by the tables' inv_hat (PolyBatch::post) when scaled
+// ModDown conversions of the P limbs (coefficient form, times inv_hat) of J accumulators
 void launch_p2q(const u64* acc, long long acc_job, int npos, int level, u64* conv, const P2QTab* tab, int N, int J,
-                bool scaled, cudaStream_t s);
-void launch_moddown_combine(const MDJobs& jobs, int J, int npos, int level, const u64* pinv, const u64* pinv_s,
-                            const DevPrime* primes, int logN, cudaStream_t s);
+                cudaStream_t s);
 void launch_rescale_lift(const u64* last, u64* lifted, const RescaleTab* tab, int l, int N, int BT, cudaStream_t s);
 void launch_rescale_combine(const u64* x, int x_cap, const u64* lifted, u64* out, int out_cap, const RescaleTab* tab,
                             int l, int N, int BT, cudaStream_t s);

@@ -109,6 +109,25 @@ __device__ __forceinline__ u64 redc(u64 hi, u64 lo, u64 q, u64 qinv) {
 struct Acc128 {
     u64 lo, hi;
 };
+// acc += x y
+__device__ __forceinline__ void mac_full(Acc128& a, u64 x, u64 y) {
+    const u32 xl = (u32)x, xh = (u32)(x >> 32), yl = (u32)y, yh = (u32)(y >> 32);
+    const u64 p0 = mul_wide(xl, yl), m0 = mad_wide(xh, yl, p0 >> 32), m1 = mad_wide(xl, yh, (u64)(u32)m0);
+    const u64 hi = mad_wide(xh, yh, (m0 >> 32) + (m1 >> 32)), lo = m1 << 32 | (u32)p0;
+    asm("add.cc.u64 %0, %0, %2;\n\taddc.u64 %1, %1, %3;" : "+l"(a.lo), "+l"(a.hi) : "l"(lo), "l"(hi));
+}
+// a sum of at most two products of residues to its canonical residue, for a prime of class 0 or 1:
+// everything from bit bits(q) up is worth c = 2^bits(q) - q per unit, three times over (no
+// quotient, no Montgomery factor: 40 issue cycles a warp against 45 for each of mul_mod's two
+// reductions)
+__device__ __forceinline__ u64 reduce_sum(const Acc128& a, const DevPrime& P) {
+    const u32 w1 = (u32)(a.lo >> 32), w2 = (u32)a.hi, w3 = (u32)(a.hi >> 32), mask = (1u << P.bsh) - 1;
+    const u64 p0 = mad_wide(__funnelshift_r(w1, w2, P.bsh), P.c, (u64)(w1 & mask) << 32 | (u32)a.lo);
+    const u64 p1 = mad_wide(__funnelshift_r(w2, w3, P.bsh), P.c, p0 >> 32);
+    const u64 r = mad_wide((u32)(p1 >> P.bsh), P.c, (u64)((u32)p1 & mask) << 32 | (u32)p0);
+    const u64 f = fold_top(r, P.bsh, P.c);
+    return min(f, f - P.q);
+}
 __device__ __forceinline__ void mac128(Acc128& a, u64 x, u64 y) {
     u64 l = x * y;
     u64 h = __umul64hi(x, y);

@@ -101,8 +101,7 @@ struct fr_ctx {
     int cmp_depth = 0;                   // levels the threshold consumes: d2 (+ 4 for the hybrid)
     int work_level = 0;                  // level of the query inside fr_match
     std::vector<ModUpTab*> d_modup;      // per level: digits_at(level) tables
-    std::vector<int*> d_modup_ntt;       // per level: (offset, prime) of the ext positions to transform
-    std::vector<int> modup_ntt_n;
+    std::vector<ExtMap> modup_ext;       // per level: the extension polynomials to transform
     P2QTab* d_p2q = nullptr;
     P2QTab* d_p2q_rs = nullptr;          // the same with [P]^-1 in the targets (moddown_rescale)
     std::vector<uint4*> d_modup_post;    // per level: last constants of the ModUp input's inverse NTT, [level+1][2]
@@ -300,14 +299,34 @@ void ntt_pair(fr_ctx* c, u64* base, long long outer, int inner, int n, const Pri
     launch_ntt(c->rd, b, inv, c->cur);
     c->launches += 2;
 }
-// forward NTT of the non-own positions of nj ModUp outputs [nj][beta][npos][N]
-void ntt_modup(fr_ctx* c, u64* ext, int nj, int level) {
-    const int beta = c->R.digits_at(level), npos = level + 1 + c->R.np;
-    const int cnt = c->modup_ntt_n[level];
-    Prof p(c, "ntt", 16.0 * nj * cnt * c->R.N);
-    PolyBatch b{ext, (long long)beta * npos * c->R.N, 1, nj * cnt, PrimeMap{}, c->d_modup_ntt[level], cnt};
+// ModUp of nj inputs and its forward NTT: in [nj][level+1][N] (coefficient form, times inv_hat) ->
+// the non-own positions of ext [nj][beta][npos][N]
+void ntt_modup(fr_ctx* c, const u64* in, u64* ext, int nj, int level) {
+    const int N = c->R.N, beta = c->R.digits_at(level), npos = level + 1 + c->R.np;
+    const int cnt = c->modup_ext[level].n;
+    PolyBatch b{ext, (long long)beta * npos * N, 1, nj * cnt, PrimeMap{}, c->modup_ext[level]};
+    if (b.npolys <= kConvFused) {
+        b.conv = ConvSrc{c->d_modup[level]->t, (long long)sizeof(ModUpTab), in, (long long)(level + 1) * N, 0};
+    } else {
+        Prof p(c, "modup", 8.0 * N * nj * ((double)beta * npos));
+        launch_modup(in, (long long)(level + 1) * N, ext, c->d_modup[level], beta, npos, N, nj, true, c->cur);
+        c->launches++;
+    }
+    Prof p(c, "ntt", 16.0 * nj * cnt * N);
     launch_ntt(c->rd, b, false, c->cur);
     c->launches += 2;
+}
+// the conversions P -> Q of nj accumulators acc [nj][2][npos][N] at `level` (P limbs in
+// coefficient form, times inv_hat), as the input of the forward NTT b [nj][2][level+1] of them
+void p2q_into(fr_ctx* c, const u64* acc, int nj, int level, PolyBatch& b) {
+    const long long N = c->R.N, npos = level + 1 + c->R.np;
+    if (b.npolys <= kConvFused) {
+        b.conv = ConvSrc{c->d_p2q->t, 0, acc + (level + 1) * N, npos * N, c->R.np};
+        return;
+    }
+    Prof p(c, "moddown", 8.0 * N * nj * 2.0 * (c->R.np + level + 1));
+    launch_p2q(acc, 2 * npos * N, (int)npos, level, b.base, c->d_p2q, (int)N, nj, c->cur);
+    c->launches++;
 }
 // all limbs 0..level of a ciphertext batch [B][2][cap][N]
 void ntt_cts(fr_ctx* c, u64* p, int B, int level, int cap, bool inv) {
@@ -394,16 +413,10 @@ void ks_finish(fr_ctx* c, int level, const std::vector<const KSReq*>& reqs, cons
     pmP.period = np;
     for (int j = 0; j < np; ++j) pmP.idx[j] = (unsigned char)(nq + j);
     ntt(c, acc.p + (size_t)(level + 1) * N, (long long)npos * N, np, nj * 2 * np, pmP, true, c->d_p2q_post);
-    {
-        Prof p(c, "moddown", 8.0 * N * nj * 2.0 * (np + level + 1));
-        launch_p2q(acc.p, 2ll * npos * N, npos, level, conv.p, c->d_p2q, N, nj, true, c->cur);
-        c->launches++;
-    }
     MDJobs md;
     for (int j = 0; j < nj; ++j) {
         MDJob& m = md.j[j];
         m.acc = acc.p + (size_t)j * 2 * npos * N;
-        m.conv = conv.p + (size_t)j * 2 * (level + 1) * N;
         m.add = reqs[j]->add;
         m.add_cap = reqs[j]->add_cap;
         m.out = reqs[j]->out;
@@ -412,11 +425,12 @@ void ks_finish(fr_ctx* c, int level, const std::vector<const KSReq*>& reqs, cons
         m.galois = reqs[j]->galois;
         m.add2 = reqs[j]->add2;
     }
-    // forward NTT of the conversions with the combine as its epilogue
-    // the region counts the transform's 16 B per coefficient (its butterflies); the fused
-    // epilogue's reads of acc and the addend are not added
-    Prof p(c, "ntt", 16.0 * nj * 2 * (level + 1) * N);
+    // the P -> Q conversions and their forward NTT with the combine as its epilogue. The ntt region
+    // counts the transform's 16 B per coefficient (its butterflies); the fused epilogue's reads of
+    // acc and the addend are not added
     PolyBatch pb{conv.p, (long long)(level + 1) * N, level + 1, nj * 2 * (level + 1), pm_level(level)};
+    p2q_into(c, acc.p, nj, level, pb);
+    Prof p(c, "ntt", 16.0 * nj * 2 * (level + 1) * N);
     launch_ntt_moddown(c->rd, pb, md, npos, level, c->d_pinv, c->d_pinv_s, c->cur);
     c->launches += 2;
 }
@@ -464,12 +478,7 @@ void modup_chunks(fr_ctx* c, int level, const std::vector<KSReq>& reqs, F finish
         ntt_from(c, in_e, e_job, in.p, (long long)L1N, level + 1, nu * (level + 1), pm_level(level), true,
                  c->d_modup_post[level]);
         Tmp ext(c, (size_t)nu * beta * npos * N);
-        {
-            Prof p(c, "modup", 8.0 * N * nu * ((double)beta * npos));
-            launch_modup(in.p, (long long)L1N, ext.p, c->d_modup[level], beta, npos, N, nu, true, c->cur);
-            c->launches++;
-        }
-        ntt_modup(c, ext.p, nu, level);
+        ntt_modup(c, in.p, ext.p, nu, level);
         std::vector<int> js;
         for (size_t j = 0; j < reqs.size(); ++j)
             if (in_of[j] >= (int)u0 && in_of[j] < (int)u0 + nu) js.push_back((int)j);
@@ -541,24 +550,18 @@ void keyswitch_sums(fr_ctx* c, int level, const std::vector<KSReq>& reqs, const 
                       c->d_pmod, c->d_pmod_s, c->cur);
         c->launches++;
     });
-    // one ModDown per sum: P limbs to coefficients, P -> Q conversion, forward NTT + combine
+    // one ModDown per sum: P limbs to coefficients, forward NTT of their P -> Q conversion + combine
     PrimeMap pmP{};
     pmP.period = np;
     for (int j = 0; j < np; ++j) pmP.idx[j] = (unsigned char)(nq + j);
     ntt(c, accs.p + (size_t)(level + 1) * N, (long long)npos * N, np, ndst * 2 * np, pmP, true, c->d_p2q_post);
     Tmp conv(c, (size_t)ndst * 2 * (level + 1) * N);
-    {
-        Prof p(c, "moddown", 8.0 * N * ndst * 2.0 * (np + level + 1));
-        launch_p2q(accs.p, (long long)aw, npos, level, conv.p, c->d_p2q, N, ndst, true, c->cur);
-        c->launches++;
-    }
     for (int o0 = 0; o0 < ndst; o0 += FR_MAX_JOBS) {
         const int no = std::min(FR_MAX_JOBS, ndst - o0);
         MDJobs md;
         for (int o = 0; o < no; ++o) {
             MDJob& m = md.j[o];
             m.acc = accs.p + (size_t)(o0 + o) * aw;
-            m.conv = conv.p + (size_t)(o0 + o) * 2 * (level + 1) * N;
             m.add = base[o0 + o];
             m.add_cap = base_cap;
             m.out = out[o0 + o];
@@ -567,9 +570,10 @@ void keyswitch_sums(fr_ctx* c, int level, const std::vector<KSReq>& reqs, const 
             m.galois = 1;
             m.add2 = nullptr;
         }
-        Prof p(c, "ntt", 16.0 * no * 2 * (level + 1) * N);
         PolyBatch pb{conv.p + (size_t)o0 * 2 * (level + 1) * N, (long long)(level + 1) * N, level + 1,
                      no * 2 * (level + 1), pm_level(level)};
+        p2q_into(c, accs.p + (size_t)o0 * aw, no, level, pb);
+        Prof p(c, "ntt", 16.0 * no * 2 * (level + 1) * N);
         launch_ntt_moddown(c->rd, pb, md, npos, level, c->d_pinv, c->d_pinv_s, c->cur);
         c->launches += 2;
     }
@@ -1391,6 +1395,7 @@ void build_tables(fr_ctx* c) {
     // primes
     std::vector<DevPrime> dp(T);
     bool fast = true;
+    unsigned long long cls1 = 0, cls2 = 0;
     for (int i = 0; i < T; ++i) {
         const u64 q = R.primes[i];
         DevPrime& d = dp[i];
@@ -1402,6 +1407,8 @@ void build_tables(fr_ctx* c) {
         d.one_s = frh::shoup_quot(1, q);
         twiddle_class(q, d);
         fast = fast && d.cls != 2;
+        cls1 |= (unsigned long long)(d.cls == 1) << i;
+        cls2 |= (unsigned long long)(d.cls == 2) << i;
         const u64 ninv = R.tabs[i].ninv;
         d.tw_ninv = Twiddler(d)(ninv);
         d.tw_wninv = Twiddler(d)(frh::mulm(ninv, R.tabs[i].itw[1], q));
@@ -1427,7 +1434,7 @@ void build_tables(fr_ctx* c) {
     uint4 *tw, *itw, *rtw, *irtw;
     upload_tw(false, &tw, &rtw);
     upload_tw(true, &itw, &irtw);
-    c->rd = RingDev{R.logN, N, T, c->d_primes, tw, itw, rtw, irtw, fast, {0, 0, 0, 0}};
+    c->rd = RingDev{R.logN, N, T, c->d_primes, tw, itw, rtw, irtw, fast, cls1, cls2, {0, 0, 0, 0}};
     // untuned shapes: 16 residues a thread from 17 polynomials up (see launch_ntt)
     if (rows) c->rd.ntt_shape[2] = c->rd.ntt_shape[3] = 5;
     c->d_rot = upload_persistent(c, R.rot_group.data(), R.rot_group.size());
@@ -1443,9 +1450,8 @@ void build_tables(fr_ctx* c) {
     };
     // ModUp tables per level
     c->d_modup.assign(R.nq, nullptr);
-    c->d_modup_ntt.assign(R.nq, nullptr);
+    c->modup_ext.assign(R.nq, ExtMap{});
     c->d_modup_post.assign(R.nq, nullptr);
-    c->modup_ntt_n.assign(R.nq, 0);
     for (int l = 0; l < R.nq; ++l) {
         const int beta = R.digits_at(l), npos = l + 1 + R.np;
         std::vector<ModUpTab> tabs(beta);
@@ -1475,15 +1481,16 @@ void build_tables(fr_ctx* c) {
         }
         c->d_modup[l] = upload_persistent(c, tabs.data(), tabs.size());
         c->d_modup_post[l] = upload_persistent(c, post.data(), post.size());
-        std::vector<int> nt;
-        for (int d = 0; d < beta; ++d)
-            for (int pos = 0; pos < npos; ++pos) {
-                if (pos >= tabs[d].lo && pos < tabs[d].lo + tabs[d].ns) continue;
-                nt.push_back(d * npos + pos);
-                nt.push_back(pos <= l ? pos : R.nq + pos - l - 1);
-            }
-        c->modup_ntt_n[l] = (int)nt.size() / 2;
-        c->d_modup_ntt[l] = upload_persistent(c, nt.data(), nt.size());
+        ExtMap& em = c->modup_ext[l];
+        em.ndig = beta;
+        em.npos = npos;
+        em.limbs = l + 1;
+        em.pbase = R.nq;
+        for (int d = 0; d < beta; ++d) {
+            em.lo[d] = (unsigned char)tabs[d].lo;
+            em.ns[d] = (unsigned char)tabs[d].ns;
+            em.n += npos - tabs[d].ns;
+        }
     }
     // ModDown: P -> Q
     {
@@ -1509,12 +1516,7 @@ void build_tables(fr_ctx* c) {
             trs.t[i] = bconv_target(q, ht);
         }
         std::vector<uint4> post;
-        for (int j = 0; j < R.np; ++j) {
-            t.pq[j] = trs.pq[j] = R.primes[R.nq + j];
-            t.inv_hat[j] = trs.inv_hat[j] = ih[j];
-            t.inv_hat_s[j] = trs.inv_hat_s[j] = frh::shoup_quot(ih[j], t.pq[j]);
-            post_of(R.nq + j, ih[j], post);
-        }
+        for (int j = 0; j < R.np; ++j) post_of(R.nq + j, ih[j], post);
         c->d_p2q = upload_persistent(c, &t, 1);
         c->d_p2q_rs = upload_persistent(c, &trs, 1);
         c->d_p2q_post = upload_persistent(c, post.data(), post.size());
@@ -3577,18 +3579,25 @@ extern "C" fr_status fr_rotate_noalloc(fr_ctx* c, const uint64_t* d_in, uint32_t
                                           std::to_string(FR_NOALLOC_SCRATCH_WORDS));
         u64* sc = noalloc_scratch(c->device);
         u64* e = sc;                     // [2][l+1][N] input, evaluation form
-        u64* a = e + 2 * L1N;            // [l+1][N] c1, coefficient form
+        u64* a = e + 2 * L1N;            // [l+1][N] c1, coefficient form (a misaligned input's copy)
         u64* ext = a + L1N;              // [beta][npos][N]
         u64* acc = ext + (size_t)beta * npos * N;  // [2][npos][N]
         u64* conv = acc + (size_t)2 * npos * N;    // [2][l+1][N]
+        u64* res = a;                    // [2][l+1][N] result, evaluation form (a and ext are done by then)
         cudaStream_t st = c->cur;
-        CU(cudaMemcpyAsync(e, d_in, 2 * L1N * 8, cudaMemcpyDeviceToDevice, st));
-        CU(cudaMemcpyAsync(a, d_in + L1N, L1N * 8, cudaMemcpyDeviceToDevice, st));
         const PrimeMap pl = pm_level(l);
-        launch_ntt(c->rd, PolyBatch{e, (long long)N, 2 * (l + 1), 2 * (l + 1), pl}, false, st);
-        launch_modup(a, 0, ext, c->d_modup[l], beta, npos, N, 1, false, st);
-        launch_ntt(c->rd, PolyBatch{ext, (long long)beta * npos * N, 1, c->modup_ntt_n[l], PrimeMap{},
-                                    c->d_modup_ntt[l], c->modup_ntt_n[l]},
+        PolyBatch in{e, 2 * (long long)L1N, 2 * (l + 1), 2 * (l + 1), pl};
+        in.src = d_in;  // out of place
+        in.src_outer = in.outer;
+        launch_ntt(c->rd, in, false, st);
+        // the conversion reads 16 bytes at a time
+        const u64* c1 = d_in + L1N;
+        if ((uintptr_t)c1 & 15) {
+            CU(cudaMemcpyAsync(a, c1, L1N * 8, cudaMemcpyDeviceToDevice, st));
+            c1 = a;
+        }
+        launch_modup(c1, 0, ext, c->d_modup[l], beta, npos, N, 1, false, st);
+        launch_ntt(c->rd, PolyBatch{ext, (long long)beta * npos * N, 1, c->modup_ext[l].n, PrimeMap{}, c->modup_ext[l]},
                    false, st);
         IPJobs ij;
         digit_owners(c, l, ij.owner);
@@ -3601,14 +3610,19 @@ extern "C" fr_status fr_rotate_noalloc(fr_ctx* c, const uint64_t* d_in, uint32_t
         PrimeMap pmP{};
         pmP.period = np;
         for (int j = 0; j < np; ++j) pmP.idx[j] = (unsigned char)(nq + j);
-        launch_ntt(c->rd, PolyBatch{acc + L1N, (long long)npos * N, np, 2 * np, pmP}, true, st);
-        launch_p2q(acc, 2ll * npos * N, npos, l, conv, c->d_p2q, N, 1, false, st);
-        launch_ntt(c->rd, PolyBatch{conv, (long long)L1N, l + 1, 2 * (l + 1), pl}, false, st);
+        PolyBatch pP{acc + L1N, (long long)npos * N, np, 2 * np, pmP};
+        pP.post = c->d_p2q_post;
+        launch_ntt(c->rd, pP, true, st);
         MDJobs md;
-        md.j[0] = MDJob{acc, conv, e, d_out, l + 1, l + 1, 1, (u32)g};
-        launch_moddown_combine(md, 1, npos, l, c->d_pinv, c->d_pinv_s, c->d_primes, c->R.logN, st);
-        launch_ntt(c->rd, PolyBatch{d_out, (long long)N, 2 * (l + 1), 2 * (l + 1), pl}, true, st);
-        c->launches += 13;
+        md.j[0] = MDJob{acc, e, res, l + 1, l + 1, 1, (u32)g};
+        PolyBatch pc{conv, (long long)L1N, l + 1, 2 * (l + 1), pl};
+        pc.conv = ConvSrc{c->d_p2q->t, 0, acc + L1N, (long long)npos * N, np};
+        launch_ntt_moddown(c->rd, pc, md, npos, l, c->d_pinv, c->d_pinv_s, st);
+        PolyBatch out{d_out, 2 * (long long)L1N, 2 * (l + 1), 2 * (l + 1), pl};
+        out.src = res;
+        out.src_outer = out.outer;
+        launch_ntt(c->rd, out, true, st);
+        c->launches += 12;
         CU(cudaGetLastError());
     });
 }

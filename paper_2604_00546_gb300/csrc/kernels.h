@@ -68,23 +68,45 @@ struct PrimeMap {
     unsigned char idx[FR_MAX_PRIMES];
 };
 
+// The polynomials of a ModUp extension [ndig][npos][N] that a digit does not own: of digit d's
+// npos positions all but [lo[d], lo[d] + ns[d]). n of them in all; position pos uses prime pos up to
+// limbs - 1, then pbase, pbase + 1, ...
+struct ExtMap {
+    int n = 0, ndig = 0, npos = 0, limbs = 0, pbase = 0;
+    unsigned char lo[8] = {}, ns[8] = {};
+};
+
+struct BconvTarget;
+
+// A batch whose forward transform starts from a fast base conversion: the column pass forms
+// poly p's coefficients itself, target `pos` of digit d's table from the digit's sources, instead
+// of reading them. With an extension map (ModUp) p names (job, d, pos) as above and the sources
+// are limbs lo[d] .. of src + job src_job; without one (ModDown) pos = p % inner, job = p / inner,
+// d = 0 and the sources are ns limbs from src + job src_job. Sources come multiplied by inv_hat.
+struct ConvSrc {
+    const BconvTarget* t = nullptr;  // digit 0's targets
+    long long t_bytes = 0;           // from one digit's targets to the next's
+    const u64* src = nullptr;
+    long long src_job = 0;
+    int ns = 0;                      // sources (no extension map)
+};
+
 // A batch of N-point polynomials: poly p lives at base + (p / inner) * outer + (p % inner) * N
-// and uses prime pm.idx[p % pm.period]. With an index table (tab != nullptr, tab_n entries
-// of (offset, prime) pairs) poly p instead lives at base + (p / tab_n) * outer + tab[2e] * N,
-// e = p % tab_n, and uses prime tab[2e + 1].
+// and uses prime pm.idx[p % pm.period]. With an extension map (ext.n > 0) poly p is polynomial
+// p % ext.n of the extension at base + (p / ext.n) * outer. Everything is in the launch's
+// parameters, so a pass starts its loads without waiting for another.
 struct PolyBatch {
     u64* base;
     long long outer;
     int inner;
     int npolys;
     PrimeMap pm;
-    const int* tab = nullptr;
-    int tab_n = 0;
+    ExtMap ext{};
     // optional source of the first pass (out of place): poly p read from
     // src + (p / inner) src_outer + (p % inner) N and written to its place in base
     const u64* src = nullptr;
     long long src_outer = 0;
-    // optional second segment (no source, no table): polys split .. npolys - 1 live at
+    // optional second segment (no source, no extension map): polys split .. npolys - 1 live at
     // base2 + (q / inner2) outer2 + (q % inner2) N, q = p - split, with primes pm2, so the
     // transforms of two buffers share one launch
     int split = 0;
@@ -96,6 +118,8 @@ struct PolyBatch {
     // p % pm.period, instead of its prime's N^-1 and N^-1 itw[1] (tw_ninv, tw_wninv): a constant
     // factor on the coefficients costs nothing
     const uint4* post = nullptr;
+    // optional (forward): the coefficients come from a base conversion
+    ConvSrc conv{};
 };
 
 // NTT batch-size buckets for the tuned tile shapes: <= 4, <= 16, <= 64, larger.
@@ -125,6 +149,7 @@ struct RingDev {
     const uint4* rtw;        // [nprimes][N] the same twiddles in the order of the radix-16 row pass
     const uint4* irtw;       // (row_tw_index; N >= 2^14, null otherwise)
     bool fast;               // no prime of twiddle class 2
+    unsigned long long cls1, cls2;  // bit i: prime i is of twiddle class 1, of class 2
     unsigned char ntt_shape[FR_NTT_BUCKETS];  // tile shape per batch-size bucket (see launch_ntt)
 };
 

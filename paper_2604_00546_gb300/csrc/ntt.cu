@@ -28,10 +28,19 @@
 #include <cstdlib>
 #include <type_traits>
 
+#include "bconv.cuh"
 #include "ckks_kernels.h"
 
 namespace {
 
+
+// polynomial e of an extension map: digit and position
+__device__ __forceinline__ void ext_at(const ExtMap& m, int e, int* digit, int* pos) {
+    int d = 0;
+    while (d + 1 < m.ndig && e >= m.npos - m.ns[d]) e -= m.npos - m.ns[d++];
+    *digit = d;
+    *pos = e < m.lo[d] ? e : e + m.ns[d];
+}
 
 __device__ __forceinline__ u64* poly_at(const PolyBatch& b, int p, int N, int* prime) {
     if (b.split && p >= b.split) {
@@ -39,13 +48,45 @@ __device__ __forceinline__ u64* poly_at(const PolyBatch& b, int p, int N, int* p
         *prime = b.pm2.idx[q % b.pm2.period];
         return b.base2 + (long long)(q / b.inner2) * b.outer2 + (long long)(q % b.inner2) * N;
     }
-    if (b.tab) {
-        const int e = p % b.tab_n;
-        *prime = __ldg(b.tab + 2 * e + 1);
-        return b.base + (long long)(p / b.tab_n) * b.outer + (long long)__ldg(b.tab + 2 * e) * N;
+    if (b.ext.n) {
+        int d, pos;
+        ext_at(b.ext, p % b.ext.n, &d, &pos);
+        *prime = pos < b.ext.limbs ? pos : b.ext.pbase + pos - b.ext.limbs;
+        return b.base + (long long)(p / b.ext.n) * b.outer + (long long)(d * b.ext.npos + pos) * N;
     }
     *prime = b.pm.idx[p % b.pm.period];
     return b.base + (long long)(p / b.inner) * b.outer + (long long)(p % b.inner) * N;
+}
+
+// The coefficients of poly p that a base conversion gives: v[e] = element at(e). Eight elements
+// share each pass over the sources, whose number stays a loop (unrolled for every count, the
+// conversion filled the instruction cache).
+template <int RB, class At>
+__device__ __forceinline__ void conv_load(u64 (&v)[1 << RB], const PolyBatch& b, int p, int N, At at) {
+    int d = 0, pos, job, lo = 0, ns = b.conv.ns;
+    if (b.ext.n) {
+        ext_at(b.ext, p % b.ext.n, &d, &pos);
+        job = p / b.ext.n;
+        lo = b.ext.lo[d];
+        ns = b.ext.ns[d];
+    } else {
+        pos = p % b.inner;
+        job = p / b.inner;
+    }
+    const BconvTarget& T =
+        reinterpret_cast<const BconvTarget*>(reinterpret_cast<const char*>(b.conv.t) + d * b.conv.t_bytes)[pos];
+    const u64* src = b.conv.src + job * b.conv.src_job + (long long)lo * N;
+    constexpr int W = 8;
+#pragma unroll
+    for (int e0 = 0; e0 < (1 << RB); e0 += W) {
+        int idx[W];
+        u64 o[W];
+#pragma unroll
+        for (int w = 0; w < W; ++w) idx[w] = at(e0 + w);
+        bconv_rt<W>(T, src, ns, N, idx, o);
+#pragma unroll
+        for (int w = 0; w < W; ++w) v[e0 + w] = o[w];
+    }
 }
 
 // where the first pass reads poly p: its source when the batch has one, else its place
@@ -87,7 +128,11 @@ struct LastLo {
 
 // Epilogues of the forward row pass (the last pass of a forward transform): instead of
 // storing the transformed values of poly p in place, the fused epilogue finishes the operation
-// the transform belonged to, on W = 1 or 2 consecutive indices from k (16-byte accesses for 2).
+// the transform belonged to, on W = 1 or 2 consecutive indices from k (16-byte accesses for 2). It
+// has two parts: load() fetches the operands, put() computes and stores. The outputs may alias the
+// operands, so the compiler cannot move a load above the store before it; a thread loads the
+// operands of four places and then stores four (one by one, their memory latencies added up: the
+// row pass of EpiRelinRescale took 141 us for 192 polynomials, 74 more than without an epilogue).
 // Values arrive below 2q; every epilogue ends them in a product by a constant, and Shoup's product
 // is exact for any 64-bit operand, so differences are lifted by 2q instead of reduced.
 struct EpiStore {};
@@ -97,6 +142,11 @@ struct EpiToMont {};
 
 template <class E>
 constexpr bool in_place = std::is_same<E, EpiStore>::value || std::is_same<E, EpiToMont>::value;
+
+template <int W>
+struct EpiOps {
+    u64 a[W], b[W], c[W];
+};
 
 template <int W>
 __device__ __forceinline__ void ld_vec(u64 (&r)[W], const u64* p) {
@@ -115,9 +165,7 @@ __device__ __forceinline__ void st_vec(u64* p, const u64 (&r)[W]) {
 }
 // r += a term below q, mod q
 template <int W>
-__device__ __forceinline__ void add_vec(u64 (&r)[W], const u64* p, u64 q) {
-    u64 a[W];
-    ld_vec(a, p);
+__device__ __forceinline__ void add_vec(u64 (&r)[W], const u64 (&a)[W], u64 q) {
 #pragma unroll
     for (int w = 0; w < W; ++w) r[w] = add_mod(r[w], a[w], q);
 }
@@ -131,24 +179,28 @@ struct EpiModDown {
     const u64* pinv;
     const u64* pinv_s;
     template <int W>
-    __device__ __forceinline__ void put(int p, int k, const u64 (&v)[W], u64 q) const {
+    __device__ __forceinline__ void load(EpiOps<W>& o, int p, int k) const {
         const int L1 = level + 1, N = 1 << logN;
-        const int j = p / (2 * L1), r = p % (2 * L1), t = r / L1, i = r % L1;
-        const MDJob& J = jobs.j[j];
-        u64 o[W];
-        ld_vec(o, J.acc + ((long long)t * npos + i) * N + k);
+        const int r = p % (2 * L1), t = r / L1, i = r % L1;
+        const MDJob& J = jobs.j[p / (2 * L1)];
+        ld_vec(o.a, J.acc + ((long long)t * npos + i) * N + k);
+        if ((J.mode & 1) && t == 0) {  // modes 1, 3
 #pragma unroll
-        for (int w = 0; w < W; ++w) o[w] = mul_shoup(o[w] + 2 * q - v[w], pinv[i], pinv_s[i], q);
-        if (J.mode == 1 || J.mode == 3) {
-            if (t == 0) {
-#pragma unroll
-                for (int w = 0; w < W; ++w)
-                    o[w] = add_mod(o[w], J.add[(long long)i * N + galois_src_index((u32)(k + w), J.galois, logN)], q);
-            }
-            if (J.mode == 3) add_vec(o, J.add2 + ((long long)t * J.add_cap + i) * N + k, q);
-        } else if (J.mode == 2) {
-            add_vec(o, J.add + ((long long)t * J.add_cap + i) * N + k, q);
+            for (int w = 0; w < W; ++w)
+                o.b[w] = J.add[(long long)i * N + galois_src_index((u32)(k + w), J.galois, logN)];
         }
+        if (J.mode & 2) ld_vec(o.c, (J.mode == 3 ? J.add2 : J.add) + ((long long)t * J.add_cap + i) * N + k);
+    }
+    template <int W>
+    __device__ __forceinline__ void put(const EpiOps<W>& x, int p, int k, const u64 (&v)[W], u64 q) const {
+        const int L1 = level + 1, N = 1 << logN;
+        const int r = p % (2 * L1), t = r / L1, i = r % L1;
+        const MDJob& J = jobs.j[p / (2 * L1)];
+        u64 o[W];
+#pragma unroll
+        for (int w = 0; w < W; ++w) o[w] = mul_shoup(x.a[w] + 2 * q - v[w], pinv[i], pinv_s[i], q);
+        if ((J.mode & 1) && t == 0) add_vec(o, x.b, q);
+        if (J.mode & 2) add_vec(o, x.c, q);
         st_vec(J.out + ((long long)t * J.out_cap + i) * N + k, o);
     }
 };
@@ -167,14 +219,19 @@ struct EpiRescale {
     long long add_bs;
     const u64* cres;    // mode 2: [l] constants
     template <int W>
-    __device__ __forceinline__ void put(int p, int k, const u64 (&v)[W], u64 q) const {
+    __device__ __forceinline__ void load(EpiOps<W>& o, int p, int k) const {
+        const int bt = p / l, i = p % l;
+        ld_vec(o.a, x + ((long long)bt * x_cap + i) * N + k);
+        if (mode == 1) ld_vec(o.b, add + (long long)(bt >> 1) * add_bs + ((long long)(bt & 1) * add_cap + i) * N + k);
+    }
+    template <int W>
+    __device__ __forceinline__ void put(const EpiOps<W>& o, int p, int k, const u64 (&v)[W], u64 q) const {
         const int bt = p / l, i = p % l;
         u64 r[W];
-        ld_vec(r, x + ((long long)bt * x_cap + i) * N + k);
 #pragma unroll
-        for (int w = 0; w < W; ++w) r[w] = mul_shoup(r[w] + 2 * q - v[w], tab->qlinv[i], tab->qlinv_s[i], q);
+        for (int w = 0; w < W; ++w) r[w] = mul_shoup(o.a[w] + 2 * q - v[w], tab->qlinv[i], tab->qlinv_s[i], q);
         if (mode == 1) {
-            add_vec(r, add + (long long)(bt >> 1) * add_bs + ((long long)(bt & 1) * add_cap + i) * N + k, q);
+            add_vec(r, o.b, q);
         } else if (mode == 2) {
 #pragma unroll
             for (int w = 0; w < W; ++w) {
@@ -204,14 +261,18 @@ struct EpiLeafRescale {
     const RescaleTab* tab;
     int l, N;
     template <int W>
-    __device__ __forceinline__ void put(int p, int k, const u64 (&v)[W], u64 q) const {
-        const int bjt = p / l, i = p % l, t = bjt & 1, bj = bjt >> 1, j = bj % nl, b = bj / nl;
+    __device__ __forceinline__ void load(EpiOps<W>& o, int p, int k) const {
+        const int bjt = p / l, i = p % l, t = bjt & 1, b = (bjt >> 1) / nl;
+        ld_vec(o.a, x + (long long)b * x_bs + ((long long)t * x_cap + i) * N + k);
+    }
+    template <int W>
+    __device__ __forceinline__ void put(const EpiOps<W>& o, int p, int k, const u64 (&v)[W], u64 q) const {
+        const int bjt = p / l, i = p % l, t = bjt & 1, j = (bjt >> 1) % nl;
         const u64 lift = 2 * q + (t == 0 ? ca[j * L1 + i] : 0);
         u64 r[W];
-        ld_vec(r, x + (long long)b * x_bs + ((long long)t * x_cap + i) * N + k);
 #pragma unroll
         for (int w = 0; w < W; ++w) {
-            const u64 a = mul_shoup_lazy(r[w], cb[j * L1 + i], cb_s[j * L1 + i], q);  // the sum is below 5q
+            const u64 a = mul_shoup_lazy(o.a[w], cb[j * L1 + i], cb_s[j * L1 + i], q);  // the sum is below 5q
             r[w] = mul_shoup(a + lift - v[w], tab->qlinv[i], tab->qlinv_s[i], q);
         }
         st_vec(out + ((long long)bjt * out_cap + i) * N + k, r);
@@ -240,19 +301,24 @@ struct EpiRelinRescale {
     long long add_bs;
     const u64* cres;   // mode 2: [l] constants
     template <int W>
-    __device__ __forceinline__ void put(int p, int k, const u64 (&v)[W], u64 q) const {
+    __device__ __forceinline__ void load(EpiOps<W>& o, int p, int k) const {
         const int jt = p / l, i = p % l, j = jt >> 1, t = jt & 1;
-        u64 r[W], dd[W];
-        ld_vec(r, acc + ((long long)jt * npos + i) * N + k);
-        if (d) ld_vec(dd, d + (((long long)j * 3 + t) * (l + 1) + i) * N + k);
+        ld_vec(o.a, acc + ((long long)jt * npos + i) * N + k);
+        if (d) ld_vec(o.b, d + (((long long)j * 3 + t) * (l + 1) + i) * N + k);
+        if (mode == 1) ld_vec(o.c, add + (long long)j * add_bs + ((long long)t * add_cap + i) * N + k);
+    }
+    template <int W>
+    __device__ __forceinline__ void put(const EpiOps<W>& o, int p, int k, const u64 (&v)[W], u64 q) const {
+        const int jt = p / l, i = p % l, j = jt >> 1, t = jt & 1;
+        u64 r[W];
 #pragma unroll
         for (int w = 0; w < W; ++w) {
-            u64 m = mul_shoup_lazy(r[w], pinv[i], pinv_s[i], q) + 2 * q - v[w];  // below 4q
-            if (d) m += dd[w];
+            u64 m = mul_shoup_lazy(o.a[w], pinv[i], pinv_s[i], q) + 2 * q - v[w];  // below 4q
+            if (d) m += o.b[w];
             r[w] = mul_shoup(m, tab->qlinv[i], tab->qlinv_s[i], q);
         }
         if (mode == 1) {
-            add_vec(r, add + (long long)j * add_bs + ((long long)t * add_cap + i) * N + k, q);
+            add_vec(r, o.c, q);
         } else if (mode == 2) {
 #pragma unroll
             for (int w = 0; w < W; ++w) {
@@ -285,23 +351,17 @@ struct Ctx {
             else w[u] = __ldg(tw + row_tw_index(LOG, LO != 0, lb, u, tau));
         }
     }
-    // a value of the transform to below 2q, and to its canonical residue
-    __device__ __forceinline__ u64 fold(u64 v) const {
-        if constexpr (CLS == 2) return min(v, v - 2 * q);
-        else return fold_top(v, bsh, c);
-    }
-    __device__ __forceinline__ u64 canon(u64 v) const {
-        v = fold(v);
-        return min(v, v - q);
-    }
-    // what a pass that ends in epilogue E keeps of v: the epilogues take values below 2q
-    template <class E>
-    __device__ __forceinline__ u64 finish(u64 v, const DevPrime& P) const {
-        if constexpr (std::is_same<E, EpiStore>::value) return canon(v);
-        else if constexpr (std::is_same<E, EpiToMont>::value) return to_mont(v, P);
-        else return fold(v);
-    }
+
 };
+
+// What a pass that ends in epilogue E keeps of v: canonical residues, or for the epilogues
+// values below 2q. C2: the prime is of class 2 (classes 0 and 1 end alike).
+template <class E, bool C2>
+__device__ __forceinline__ u64 finish(u64 v, const DevPrime& P) {
+    if constexpr (std::is_same<E, EpiToMont>::value) return to_mont(v, P);
+    const u64 f = C2 ? min(v, v - 2 * P.q) : fold_top(v, P.bsh, P.c);
+    return std::is_same<E, EpiStore>::value ? min(f, f - P.q) : f;
+}
 
 // One radix-2 stage on bit B of the registers of a phase with base bit LO. The butterfly of
 // registers e and e + 2^lb (lb = B - LO) takes twiddle (M + J + x) >> (B + 1), x its element
@@ -453,74 +513,101 @@ struct RowEx16 {
     }
 };
 
-// column pass: one CTA = KTC columns x S rows; thread (tau, col) with col = threadIdx % KTC
-template <int RB, int LOG, bool INV, int KTC, int CLS>
-__device__ __forceinline__ void ntt_col_body(const PolyBatch& b, u64* x, const uint4* tw, const DevPrime& P, int p,
-                                             int N, u64* sm) {
-    constexpr int S = 1 << LOG;
-    uint4* sw = reinterpret_cast<uint4*>(sm + S * KTC);  // twiddles [0, S)
-    const int C = N >> LOG;
-    for (int i = threadIdx.x; i < S; i += blockDim.x) sw[i] = __ldg(tw + i);
-    const int col = threadIdx.x & (KTC - 1);
-    const int tau = threadIdx.x / KTC;
-    const int gcol = blockIdx.x * KTC + col;
-    constexpr int L0 = PhaseInfo<RB, LOG, INV, 0>::LO;
-    constexpr int LL = LastLo<RB, LOG, INV>::v;
-    const u64* xin = INV ? x : poly_in(b, p, N, x);  // the column pass is the forward transform's first
-    u64 v[1 << RB];
-#pragma unroll
-    for (int e = 0; e < (1 << RB); ++e) v[e] = xin[(long long)phase_x<RB, L0>(tau, e) * C + gcol];
-    __syncthreads();
-    const Ctx<CLS, 0, LOG> c(0, S, sw, P);
-    ColEx<KTC> ex{sm, col};
-    phases<CLS, RB, LOG, INV, INV, 0>(v, tau, c, ex, P, poly_post(b, p));
-#pragma unroll
-    for (int e = 0; e < (1 << RB); ++e) x[(long long)phase_x<RB, LL>(tau, e) * C + gcol] = INV ? c.canon(v[e]) : v[e];
+// The twiddle class of prime pi, from the launch's parameters: the branch on it waits for no load.
+__device__ __forceinline__ int prime_class(const RingDev& R, int pi) {
+    return (int)(R.cls1 >> pi & 1) + 2 * (int)(R.cls2 >> pi & 1);
 }
 
-template <int LOG, bool INV, int KTC>
-__global__ void __launch_bounds__(KTC * (1 << LOG) / 8, 5) k_ntt_col(const __grid_constant__ RingDev R, const __grid_constant__ PolyBatch b) {
+// column pass: one CTA = KTC columns x S rows; thread (tau, col) with col = threadIdx % KTC. The
+// loads of the elements, the twiddles and the prime's constants are all issued before the first
+// use of any of them: a small batch runs one or two CTAs an SM and waits for every dependent load.
+template <int RB, int LOG, bool INV, int KTC, int CLS>
+__device__ __forceinline__ void ntt_col_body(u64 (&v)[1 << RB], const DevPrime& P, const uint4* post, u64* sm) {
+    constexpr int S = 1 << LOG;
+    const int col = threadIdx.x & (KTC - 1), tau = threadIdx.x / KTC;
+    const Ctx<CLS, 0, LOG> c(0, S, reinterpret_cast<const uint4*>(sm + S * KTC), P);
+    ColEx<KTC> ex{sm, col};
+    phases<CLS, RB, LOG, INV, INV, 0>(v, tau, c, ex, P, post);
+    if constexpr (INV && CLS == 2) {
+#pragma unroll
+        for (int e = 0; e < (1 << RB); ++e) v[e] = finish<EpiStore, true>(v[e], P);
+    }
+}
+
+template <int RB, int LOG, bool INV, int KTC, bool C2, bool CONV>
+__device__ __forceinline__ void ntt_col(const RingDev& R, const PolyBatch& b, u64* sm) {
+    constexpr int S = 1 << LOG, T = KTC * (S >> RB);
+    const int p = blockIdx.y, N = R.N, C = N >> LOG;
+    int pi;
+    u64* x = poly_at(b, p, N, &pi);
+    const uint4* tw = (INV ? R.itw : R.tw) + (size_t)pi * N;
+    const u64* xin = INV ? x : poly_in(b, p, N, x);  // the column pass is the forward transform's first
+    const int col = threadIdx.x & (KTC - 1), tau = threadIdx.x / KTC;
+    constexpr int L0 = PhaseInfo<RB, LOG, INV, 0>::LO;
+    u64 v[1 << RB];
+    auto at = [&](int e) { return phase_x<RB, L0>(tau, e) * C + (int)blockIdx.x * KTC + col; };
+    if constexpr (!CONV) {
+#pragma unroll
+        for (int e = 0; e < (1 << RB); ++e) v[e] = xin[at(e)];
+    }
+    uint4* sw = reinterpret_cast<uint4*>(sm + S * KTC);  // twiddles [0, S)
+#pragma unroll
+    for (int i = 0; i < (S + T - 1) / T; ++i)
+        if (i * T + (int)threadIdx.x < S) sw[i * T + threadIdx.x] = __ldg(tw + i * T + threadIdx.x);
+    if constexpr (CONV) conv_load<RB>(v, b, p, N, at);
+    const DevPrime P = R.primes[pi];
+    const uint4* post = poly_post(b, p);
+    __syncthreads();
+    const int cls = prime_class(R, pi);
+    if (cls == 0) ntt_col_body<RB, LOG, INV, KTC, 0>(v, P, post, sm);
+    else if (!C2 || cls == 1) ntt_col_body<RB, LOG, INV, KTC, 1>(v, P, post, sm);
+    else if constexpr (C2) ntt_col_body<RB, LOG, INV, KTC, 2>(v, P, post, sm);
+    constexpr int LL = LastLo<RB, LOG, INV>::v;
+#pragma unroll
+    for (int e = 0; e < (1 << RB); ++e)
+        x[phase_x<RB, LL>(tau, e) * C + (int)blockIdx.x * KTC + col] =
+            INV && !(C2 && cls == 2) ? finish<EpiStore, false>(v[e], P) : v[e];
+}
+
+template <int LOG, bool INV, int KTC, bool CONV>
+__global__ void __launch_bounds__(KTC * (1 << LOG) / 8, CONV ? 4 : 5) k_ntt_col(const __grid_constant__ RingDev R, const __grid_constant__ PolyBatch b) {
     pdl_wait();
     pdl_trigger();
     extern __shared__ __align__(16) u64 sm[];
-    const int p = blockIdx.y;
-    int pi;
-    u64* x = poly_at(b, p, R.N, &pi);
-    const uint4* tw = (INV ? R.itw : R.tw) + (size_t)pi * R.N;
-    const DevPrime P = R.primes[pi];
-    if (P.cls == 0) ntt_col_body<3, LOG, INV, KTC, 0>(b, x, tw, P, p, R.N, sm);
-    else if (P.cls == 1) ntt_col_body<3, LOG, INV, KTC, 1>(b, x, tw, P, p, R.N, sm);
-    else ntt_col_body<3, LOG, INV, KTC, 2>(b, x, tw, P, p, R.N, sm);
+    ntt_col<3, LOG, INV, KTC, true, CONV>(R, b, sm);
 }
 
 // row pass: one CTA = RPC rows of S contiguous elements (RT threads), S/8 threads per row
-template <int LOG, int RPC, bool INV, int CLS, class E>
-__device__ __forceinline__ void ntt_row_body(const PolyBatch& b, u64* x, const uint4* tw, const DevPrime& P, int p,
-                                             int N, u64* sm, const E& epi) {
-    constexpr int S = 1 << LOG;
-    constexpr int TPR = S / 8;  // threads per row
-    const int rloc = threadIdx.x / TPR;
-    const int tau = threadIdx.x % TPR;
-    const int Jbase = (blockIdx.x * RPC + rloc) * S;
-    u64* xr = x + Jbase;
-    const u64* xin = (INV ? poly_in(b, p, N, x) : x) + Jbase;  // the row pass is the inverse's first
-    constexpr int L0 = PhaseInfo<3, LOG, INV, 0>::LO;
-    constexpr int LL = LastLo<3, LOG, INV>::v;
-    u64 v[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) v[e] = xin[phase_x<3, L0>(tau, e)];
+template <int LOG, bool INV, int CLS, class E>
+__device__ __forceinline__ void ntt_row_body(u64 (&v)[8], const uint4* tw, const DevPrime& P, int Jbase, int N,
+                                             u64* s) {
     const Ctx<CLS, 1, LOG> c(Jbase, N, tw, P);
-    RowEx ex{sm + rloc * S};
-    phases<CLS, 3, LOG, INV, false, 0>(v, tau, c, ex, P);
+    RowEx ex{s};
+    phases<CLS, 3, LOG, INV, false, 0>(v, threadIdx.x % ((1 << LOG) / 8), c, ex, P);
+    if constexpr (!INV) {
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-        const int k = phase_x<3, LL>(tau, e);
-        if constexpr (INV) {
-            xr[k] = v[e];
-        } else {
-            const u64 o[1] = {c.template finish<E>(v[e], P)};
-            if constexpr (in_place<E>) xr[k] = o[0];
-            else epi.put(p, Jbase + k, o, P.q);
+        for (int e = 0; e < 8; ++e) v[e] = finish<E, CLS == 2>(v[e], P);
+    }
+}
+
+// a thread's finished values at consecutive places of its row (element e at k + e) to where the
+// epilogue puts them
+template <class E>
+__device__ __forceinline__ void row_put(const u64 (&v)[8], u64* x, int p, int k, const E& epi, u64 q) {
+    if constexpr (in_place<E>) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) x[k + e] = v[e];
+    } else {
+#pragma unroll
+        for (int g = 0; g < 8; g += 4) {
+            EpiOps<1> o[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) epi.load(o[e], p, k + g + e);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const u64 w[1] = {v[g + e]};
+                epi.put(o[e], p, k + g + e, w, q);
+            }
         }
     }
 }
@@ -530,17 +617,34 @@ __global__ void __launch_bounds__(RT, RT == 128 ? 9 : 4) k_ntt_row(const __grid_
                                                                    const __grid_constant__ E epi) {
     pdl_wait();
     pdl_trigger();
-    constexpr int TPR = (1 << LOG) / 8;
+    constexpr int S = 1 << LOG, TPR = S / 8;  // threads per row
     constexpr int RPC = (RT / TPR < (1 << LOGR)) ? RT / TPR : (1 << LOGR);  // rows per CTA
     extern __shared__ __align__(16) u64 sm[];
-    const int p = blockIdx.y;
+    const int p = blockIdx.y, N = R.N;
     int pi;
-    u64* x = poly_at(b, p, R.N, &pi);
-    const uint4* tw = (INV ? R.itw : R.tw) + (size_t)pi * R.N;
+    u64* x = poly_at(b, p, N, &pi);
+    const uint4* tw = (INV ? R.itw : R.tw) + (size_t)pi * N;
+    const int rloc = threadIdx.x / TPR, tau = threadIdx.x % TPR;
+    const int Jbase = (blockIdx.x * RPC + rloc) * S;
+    const u64* xin = (INV ? poly_in(b, p, N, x) : x) + Jbase;  // the row pass is the inverse's first
+    constexpr int L0 = PhaseInfo<3, LOG, INV, 0>::LO;
+    u64 v[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[e] = xin[phase_x<3, L0>(tau, e)];
     const DevPrime P = R.primes[pi];
-    if (P.cls == 0) ntt_row_body<LOG, RPC, INV, 0>(b, x, tw, P, p, R.N, sm, epi);
-    else if (P.cls == 1) ntt_row_body<LOG, RPC, INV, 1>(b, x, tw, P, p, R.N, sm, epi);
-    else ntt_row_body<LOG, RPC, INV, 2>(b, x, tw, P, p, R.N, sm, epi);
+    u64* s = sm + rloc * S;
+    const int cls = prime_class(R, pi);
+    if (cls == 0) ntt_row_body<LOG, INV, 0, E>(v, tw, P, Jbase, N, s);
+    else if (cls == 1) ntt_row_body<LOG, INV, 1, E>(v, tw, P, Jbase, N, s);
+    else ntt_row_body<LOG, INV, 2, E>(v, tw, P, Jbase, N, s);
+    constexpr int LL = LastLo<3, LOG, INV>::v;
+    if constexpr (INV) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) x[Jbase + phase_x<3, LL>(tau, e)] = v[e];
+    } else {
+        static_assert(LL == 0, "the last forward phase holds the low bits");
+        row_put(v, x, p, Jbase + tau * 8, epi, P.q);
+    }
 }
 
 // Single-launch NTT of N = 2^16 (256 x 256) for small batches. A cluster of 8 CTAs of 1024
@@ -596,12 +700,8 @@ __device__ __forceinline__ void ntt_cluster_body(const RingDev& R, u64* x, const
         RowEx exr{A + rloc * S};
         phases<CLS, 3, LOG, false, false, 0>(v, taur, cr, exr, P);
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const int k = phase_x<3, LL>(taur, e);
-            const u64 o[1] = {cr.template finish<E>(v[e], P)};
-            if constexpr (in_place<E>) xr[k] = o[0];
-            else epi.put(p, rho * S + k, o, P.q);
-        }
+        for (int e = 0; e < 8; ++e) v[e] = finish<E, false>(v[e], P);
+        row_put(v, x, p, rho * S + taur * 8, epi, P.q);
     } else {
 #pragma unroll
         for (int e = 0; e < 8; ++e) v[e] = xr[phase_x<3, L0>(taur, e)];
@@ -619,7 +719,7 @@ __device__ __forceinline__ void ntt_cluster_body(const RingDev& R, u64* x, const
         ColEx<32> exc{Bb, col};
         phases<CLS, 3, LOG, true, true, 0>(v, tauc, c, exc, P, post);
 #pragma unroll
-        for (int e = 0; e < 8; ++e) x[(long long)phase_x<3, LL>(tauc, e) * S + gcol] = c.canon(v[e]);
+        for (int e = 0; e < 8; ++e) x[(long long)phase_x<3, LL>(tauc, e) * S + gcol] = finish<EpiStore, false>(v[e], P);
     }
 }
 
@@ -635,7 +735,7 @@ __global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(1024, 1)
     u64* x = poly_at(b, p, R.N, &pi);
     const uint4* tw = (INV ? R.itw : R.tw) + (size_t)pi * R.N;
     const DevPrime P = R.primes[pi];  // class 0 or 1: the launcher checks
-    if (P.cls == 0) ntt_cluster_body<INV, 0>(R, x, tw, P, p, sm, epi, poly_post(b, p));
+    if (prime_class(R, pi) == 0) ntt_cluster_body<INV, 0>(R, x, tw, P, p, sm, epi, poly_post(b, p));
     else ntt_cluster_body<INV, 1>(R, x, tw, P, p, sm, epi, poly_post(b, p));
 }
 
@@ -647,19 +747,13 @@ __global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(1024, 1)
 // ---------------------------------------------------------------------------
 constexpr int kCol16 = 8;  // columns of a column-pass CTA: 64-byte row segments
 
-template <int LOG, bool INV>
-__global__ void __launch_bounds__(kCol16 * (1 << LOG) / 16, (INV ? 6 : 5) * (256 >> LOG))
+template <int LOG, bool INV, bool CONV>
+__global__ void __launch_bounds__(kCol16 * (1 << LOG) / 16, (INV ? 6 : CONV ? 4 : 5) * (256 >> LOG))
     k_ntt_col16(const __grid_constant__ RingDev R, const __grid_constant__ PolyBatch b) {
     pdl_wait();
     pdl_trigger();
     extern __shared__ __align__(16) u64 sm[];
-    const int p = blockIdx.y;
-    int pi;
-    u64* x = poly_at(b, p, R.N, &pi);
-    const uint4* tw = (INV ? R.itw : R.tw) + (size_t)pi * R.N;
-    const DevPrime P = R.primes[pi];
-    if (P.cls == 0) ntt_col_body<4, LOG, INV, kCol16, 0>(b, x, tw, P, p, R.N, sm);
-    else ntt_col_body<4, LOG, INV, kCol16, 1>(b, x, tw, P, p, R.N, sm);
+    ntt_col<4, LOG, INV, kCol16, false, CONV>(R, b, sm);
 }
 
 __device__ __forceinline__ void ld_async16(void* dst, const void* src) {
@@ -673,20 +767,36 @@ __device__ __forceinline__ void ld_async16(void* dst, const void* src) {
 // (thread & 7), so that the global side moves 512 contiguous bytes per instruction and epilogues
 // see consecutive elements in consecutive lanes. Reading and writing them thread by thread
 // touches 32 cache lines per instruction, which bounded the pass (the epilogues above all).
-template <int LOG, bool INV, int CLS, class E>
-__device__ __forceinline__ void ntt_row16_body(const PolyBatch& b, u64* x, const uint4* tw, const DevPrime& P, int p,
-                                               int N, u64* sm, const E& epi) {
+template <int LOG, bool INV, int CLS>
+__device__ __forceinline__ void ntt_row16_body(u64 (&v)[16], const uint4* tw, const DevPrime& P, int rho, int N,
+                                               u64* ws) {
     constexpr int S = 1 << LOG, TPR = S / 16;
+    const int lane = threadIdx.x & 31;
+    const Ctx<CLS, 2, LOG> c(rho * S, N, tw + (size_t)rho * S, P);
+    RowEx16<LOG> ex{ws + (lane / TPR) * S, rho & 1};
+    phases<CLS, 4, LOG, INV, false, 0>(v, lane % TPR, c, ex, P);
+}
+
+template <int LOG, bool INV, class E>
+__global__ void __launch_bounds__(128, 6) k_ntt_row16(const __grid_constant__ RingDev R,
+                                                      const __grid_constant__ PolyBatch b,
+                                                      const __grid_constant__ E epi) {
+    pdl_wait();
+    pdl_trigger();
+    extern __shared__ __align__(16) u64 sm[];  // [4 warps][512]
+    constexpr int S = 1 << LOG, TPR = S / 16;
+    const int p = blockIdx.y, N = R.N;
+    int pi;
+    u64* x = poly_at(b, p, N, &pi);
+    const uint4* tw = (INV ? R.irtw : R.rtw) + (size_t)pi * N;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int tau = lane % TPR;
     const int Wbase = (blockIdx.x * 4 + warp) * 512;  // the warp's first element
     const int rho = Wbase / S + lane / TPR;
     u64* ws = sm + warp * 512;
-    ulonglong2* wc = reinterpret_cast<ulonglong2*>(ws);
-    const Ctx<CLS, 2, LOG> c(rho * S, N, tw + (size_t)rho * S, P);
-    RowEx16<LOG> ex{ws + (lane / TPR) * S, rho & 1};
     u64 v[16];
+    const DevPrime P = R.primes[pi];
     if constexpr (INV) {
+        ulonglong2* wc = reinterpret_cast<ulonglong2*>(ws);
         const u64* xin = poly_in(b, p, N, x) + Wbase;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
@@ -703,45 +813,41 @@ __device__ __forceinline__ void ntt_row16_body(const PolyBatch& b, u64* x, const
             v[2 * h + 1] = t.y;
         }
         __syncwarp();
-        phases<CLS, 4, LOG, true, false, 0>(v, tau, c, ex, P);
-        u64* xr = x + (long long)rho * S;
-#pragma unroll
-        for (int e = 0; e < 16; ++e) xr[phase_x<4, LOG - 4>(tau, e)] = v[e];
     } else {
         const u64* xr = x + (long long)rho * S;
 #pragma unroll
-        for (int e = 0; e < 16; ++e) v[e] = xr[phase_x<4, LOG - 4>(tau, e)];
-        phases<CLS, 4, LOG, false, false, 0>(v, tau, c, ex, P);
+        for (int e = 0; e < 16; ++e) v[e] = xr[phase_x<4, LOG - 4>(lane % TPR, e)];
+    }
+    if (prime_class(R, pi) == 0) ntt_row16_body<LOG, INV, 0>(v, tw, P, rho, N, ws);
+    else ntt_row16_body<LOG, INV, 1>(v, tw, P, rho, N, ws);
+    if constexpr (INV) {
+        u64* xr = x + (long long)rho * S;
+#pragma unroll
+        for (int e = 0; e < 16; ++e) xr[phase_x<4, LOG - 4>(lane % TPR, e)] = v[e];
+    } else {
+        ulonglong2* wc = reinterpret_cast<ulonglong2*>(ws);
 #pragma unroll
         for (int h = 0; h < 8; ++h)
             wc[lane * 8 + (h ^ (lane & 7))] =
-                make_ulonglong2(c.template finish<E>(v[2 * h], P), c.template finish<E>(v[2 * h + 1], P));
+                make_ulonglong2(finish<E, false>(v[2 * h], P), finish<E, false>(v[2 * h + 1], P));
         __syncwarp();
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int ch = j * 32 + lane;
-            u64 o[2];
-            ld_vec(o, ws + 2 * (ch ^ ((ch >> 3) & 7)));
-            if constexpr (in_place<E>) st_vec(x + Wbase + 2 * ch, o);
-            else epi.put(p, Wbase + 2 * ch, o, P.q);
+        for (int g = 0; g < 8; g += 4) {
+            EpiOps<2> ops[4];
+            if constexpr (!in_place<E>) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) epi.load(ops[j], p, Wbase + 2 * ((g + j) * 32 + lane));
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int ch = (g + j) * 32 + lane;
+                u64 o[2];
+                ld_vec(o, ws + 2 * (ch ^ ((ch >> 3) & 7)));
+                if constexpr (in_place<E>) st_vec(x + Wbase + 2 * ch, o);
+                else epi.put(ops[j], p, Wbase + 2 * ch, o, P.q);
+            }
         }
     }
-}
-
-template <int LOG, bool INV, class E>
-__global__ void __launch_bounds__(128, 6) k_ntt_row16(const __grid_constant__ RingDev R,
-                                                      const __grid_constant__ PolyBatch b,
-                                                      const __grid_constant__ E epi) {
-    pdl_wait();
-    pdl_trigger();
-    extern __shared__ __align__(16) u64 sm[];  // [4 warps][512]
-    const int p = blockIdx.y;
-    int pi;
-    u64* x = poly_at(b, p, R.N, &pi);
-    const uint4* tw = (INV ? R.irtw : R.rtw) + (size_t)pi * R.N;
-    const DevPrime P = R.primes[pi];
-    if (P.cls == 0) ntt_row16_body<LOG, INV, 0>(b, x, tw, P, p, R.N, sm, epi);
-    else ntt_row16_body<LOG, INV, 1>(b, x, tw, P, p, R.N, sm, epi);
 }
 
 template <int LOGR, int LOGC, class E>
@@ -751,11 +857,12 @@ void launch_ntt_r16(const RingDev& R, const PolyBatch& b, bool inverse, cudaStre
     const int tc = kCol16 * SR / 16;
     const size_t smc = (size_t)(SR * kCol16 + 2 * SR) * sizeof(u64), smr = (size_t)2048 * sizeof(u64);
     if (!inverse) {
-        launch_k(k_ntt_col16<LOGR, false>, gc, dim3(tc), smc, st, R, b);
+        if (b.conv.t) launch_k(k_ntt_col16<LOGR, false, true>, gc, dim3(tc), smc, st, R, b);
+        else launch_k(k_ntt_col16<LOGR, false, false>, gc, dim3(tc), smc, st, R, b);
         launch_k(k_ntt_row16<LOGC, false, E>, gr, dim3(128), smr, st, R, b, epi);
     } else {
         launch_k(k_ntt_row16<LOGC, true, EpiStore>, gr, dim3(128), smr, st, R, b, EpiStore{});
-        launch_k(k_ntt_col16<LOGR, true>, gc, dim3(tc), smc, st, R, b);
+        launch_k(k_ntt_col16<LOGR, true, false>, gc, dim3(tc), smc, st, R, b);
     }
 }
 
@@ -770,11 +877,12 @@ void launch_ntt_t(const RingDev& R, const PolyBatch& b, bool inverse, cudaStream
     dim3 gr(SR / RPC, b.npolys);
     const size_t smr = (size_t)RPC * SC * sizeof(u64);
     if (!inverse) {
-        launch_k(k_ntt_col<LOGR, false, KTC>, dim3(gc), dim3(tc), smc, st, R, b);
+        if (b.conv.t) launch_k(k_ntt_col<LOGR, false, KTC, true>, dim3(gc), dim3(tc), smc, st, R, b);
+        else launch_k(k_ntt_col<LOGR, false, KTC, false>, dim3(gc), dim3(tc), smc, st, R, b);
         launch_k(k_ntt_row<LOGC, LOGR, false, E, RT>, dim3(gr), dim3(RPC * TPR), smr, st, R, b, epi);
     } else {
         launch_k(k_ntt_row<LOGC, LOGR, true, EpiStore, RT>, dim3(gr), dim3(RPC * TPR), smr, st, R, b, EpiStore{});
-        launch_k(k_ntt_col<LOGR, true, KTC>, dim3(gc), dim3(tc), smc, st, R, b);
+        launch_k(k_ntt_col<LOGR, true, KTC, false>, dim3(gc), dim3(tc), smc, st, R, b);
     }
 }
 
@@ -800,16 +908,17 @@ void launch_ntt_cluster(const RingDev& R, const PolyBatch& b, bool inverse, cuda
     else launch_k(k_ntt_cluster<true, EpiStore>, g, dim3(1024), kClusterSmem, st, R, b, EpiStore{});
 }
 
-// The tile shape this batch runs: the tuned one of its bucket, with two exceptions. Shapes 4 and
+// The tile shape this batch runs: the tuned one of its bucket, with exceptions. Shapes 4 and
 // 5 have no code for class-2 primes, and shape 5 moves 16-byte chunks, so a ring with such a prime
-// or a batch at an address that is not a multiple of 16 bytes (a caller's own buffer) runs shape 0.
+// or a batch at an address that is not a multiple of 16 bytes (a caller's own buffer) runs shape 0;
+// so does a base conversion's batch in place of shape 4.
 int ntt_shape_of(const RingDev& R, const PolyBatch& b) {
     if (R.logN < 14) return 0;
     const int shape = R.ntt_shape[ntt_bucket(b.npolys)];
     if (shape < 4) return shape;
     const uintptr_t a = (uintptr_t)b.base | (uintptr_t)b.src | (uintptr_t)b.base2 |
                         (uintptr_t)(8 * b.outer) | (uintptr_t)(8 * b.src_outer) | (uintptr_t)(8 * b.outer2);
-    return !R.fast || (a & 15) || (shape == 4 && R.logN != 16) ? 0 : shape;
+    return !R.fast || (a & 15) || (shape == 4 && (R.logN != 16 || b.conv.t)) ? 0 : shape;
 }
 
 template <int LOGR, int LOGC, class E>
@@ -900,9 +1009,9 @@ template <class E>
 void launch_ntt_e(const RingDev& R, const PolyBatch& b, bool inverse, cudaStream_t s, const E& epi) {
     if (b.npolys <= 0) return;
     if (b.src) {
-        // the two-pass kernels read a source themselves; for the cluster shape (and a table-mapped
-        // batch) the source is copied into place first
-        if (b.tab || ntt_shape_of(R, b) == 4) {
+        // the two-pass kernels read a source themselves; for the cluster shape (and a batch
+        // with an extension map) the source is copied into place first
+        if (b.ext.n || ntt_shape_of(R, b) == 4) {
             cudaMemcpy2DAsync(b.base, (size_t)b.outer * 8, b.src, (size_t)b.src_outer * 8, (size_t)b.inner * R.N * 8,
                               (size_t)(b.npolys / b.inner), cudaMemcpyDeviceToDevice, s);
             PolyBatch c = b;
