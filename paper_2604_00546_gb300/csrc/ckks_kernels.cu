@@ -458,94 +458,76 @@ __global__ void __launch_bounds__(kBcThreads) k_tensor(const TensorJobs jobs, in
 }
 
 // ---------------------------------------------------------------------------
-// Diagonal MAC (on-demand BSGS, Eq. eq:prerotation) for B queries at once:
-//   P_{b,j}[t][i][k] = sum_{i' < n1, j n1 + i' < ell} baby_{b,i'}[t][i][k] * D'_{j n1 + i'}[i][k]
-// A CTA owns TP evaluation points of one limb. The n1 baby words (both polys)
-// of its points are staged in shared memory for every query; JG thread groups
-// split the n2 giant steps. Every plaintext diagonal word is read once for all
-// B queries, eight at a time per thread; when every batch of eight is full (n1 a
-// multiple of 8 dividing ell), a word's register is refilled with the next batch's
-// word as soon as it has been multiplied, so the loads stay in flight.
+// Diagonal MAC (on-demand BSGS, Eq. eq:prerotation) of one query:
+//   P_j[t][i][k] = sum_{i' < n1, j n1 + i' < ell} baby_{i'}[t][i][k] * D'_{j n1 + i'}[i][k]
+// A CTA owns TP evaluation points of one limb. The n1 baby words (both polys) of its points are
+// staged in shared memory; JG thread groups split the n2 giant steps. The diagonals are streamed,
+// eight words a thread at a time; when every batch of eight is full (n1 a multiple of 8 dividing
+// ell), a word's register is refilled with the next batch's word as soon as it has been
+// multiplied, so the loads stay in flight.
+// Bound by HBM: the diagonals lie in tiles (diag_word), so a CTA reads one contiguous run of ell
+// kDiagTile words where rows 6.8 MB apart cost a fifth of the bandwidth, and already as 30-bit
+// halves. At the headline size (512 diagonals of 13 limbs, N = 2^16, 4.14 GB) 888 us, 4.67 TB/s ->
+// 637 us, 6.50 TB/s (tiles alone 668; 128 points x 4 rows 662; 64 x 8, two CTAs an SM, 666).
 // ---------------------------------------------------------------------------
-template <int B>
-__global__ void __launch_bounds__(512, (B == 1 ? 2 : 1)) k_mac(const u64* __restrict__ babies, long long baby_q, int cap_b,
-                                             const u64* __restrict__ diags, u64* __restrict__ out, long long out_q,
-                                             int cap_o, int nl, int n1, int n2, int ell, int TP, int JG,
-                                             const DevPrime* __restrict__ primes, int N) {
+template <int TP>
+__global__ void __launch_bounds__(256, 4) k_mac(const u64* __restrict__ babies, int cap_b,
+                                                const u64* __restrict__ diags, u64* __restrict__ out, int cap_o,
+                                                int nl, int n1, int n2, int ell, int JG,
+                                                const DevPrime* __restrict__ primes, int N) {
     pdl_wait();
     pdl_trigger();
-    extern __shared__ u64 sb[];  // [B][n1][2][TP]
+    extern __shared__ u64 sb[];  // [n1][2][TP]
     const int pl = threadIdx.x % TP;
     const int jg = threadIdx.x / TP;
     const int k = blockIdx.x * TP + pl;
     const int i = blockIdx.y;
     const u64 q = primes[i].q, qinv = primes[i].qinv, one_s = primes[i].one_s;
     const bool fold_each = n1 > 64;
-    const int per_q = n1 * 2 * TP;
-    // staging: thread (pl, jg) takes point pl of the rows r = 2 i' + t = jg, jg + JG, ... of
-    // every query (no index divisions)
+    // staging: thread (pl, jg) takes point pl of the rows r = 2 i' + t = jg, jg + JG, ... (no
+    // index divisions)
     {
         const long long rstep = (long long)cap_b * N;
-#pragma unroll
-        for (int b = 0; b < B; ++b) {
-            const u64* src = babies + (long long)b * baby_q + (long long)i * N + k;
-            u64* dst = sb + b * per_q + pl;
+        const u64* src = babies + (long long)i * N + k;
 #pragma unroll 8
-            for (int r = jg; r < 2 * n1; r += JG) dst[r * TP] = split30(src[r * rstep]);
-        }
+        for (int r = jg; r < 2 * n1; r += JG) sb[r * TP + pl] = split30(src[r * rstep]);
     }
     __syncthreads();
-    const long long dstride = (long long)nl * N;
     // the thread's work is a sequence of batches (giant step j, 8 diagonals from i0)
     int j = jg, i0 = 0;
     if (j >= n2) return;
     const u64* sbase = sb + pl;
-    const int TP2 = 2 * TP;
-    Acc128 acc[B][2];
-#pragma unroll
-    for (int b = 0; b < B; ++b) acc[b][0] = acc[b][1] = Acc128{0, 0};
-    // the products of one diagonal word d (both polys of every query's baby) into p
-    auto mul_word = [&](AccK (&p)[B][2], u64 d, const u64* sq) {
-        const u64 ds = split30(d);
-        const u32 dsum = sum30(ds);
-#pragma unroll
-        for (int b = 0; b < B; ++b) {
-            mack(p[b][0], ds, dsum, sq[b * per_q]);
-            mack(p[b][1], ds, dsum, sq[b * per_q + TP]);
-        }
+    Acc128 acc[2] = {};
+    // the products of one diagonal word d (both polys of the baby) into p
+    auto mul_word = [&](AccK (&p)[2], u64 d, const u64* sq) {
+        const u32 dsum = sum30(d);
+        mack(p[0], d, dsum, sq[0]);
+        mack(p[1], d, dsum, sq[TP]);
     };
     // after a batch of giant step j: add its sums (a flush adds less than 2^60 to the high word,
     // so up to 64 products per giant step, 8 flushes, need no fold and the high word is reduced
     // once before the REDC); when the giant step ends, store it
-    auto close_batch = [&](AccK (&p)[B][2], int jc, bool last) {
+    auto close_batch = [&](AccK (&p)[2], int jc, bool last) {
 #pragma unroll
-        for (int b = 0; b < B; ++b) {
-            flushk(acc[b][0], p[b][0]);
-            flushk(acc[b][1], p[b][1]);
-            if (fold_each) {
-                fold(acc[b][0], q);
-                fold(acc[b][1], q);
-            }
-        }
-        if (last) {
-#pragma unroll
-            for (int b = 0; b < B; ++b) {
-                u64* O = out + (long long)b * out_q + (long long)jc * 2 * cap_o * N;
-                O[(long long)i * N + k] = redc(mul_shoup(acc[b][0].hi, 1, one_s, q), acc[b][0].lo, q, qinv);
-                O[((long long)cap_o + i) * N + k] = redc(mul_shoup(acc[b][1].hi, 1, one_s, q), acc[b][1].lo, q, qinv);
-                acc[b][0] = acc[b][1] = Acc128{0, 0};
+        for (int t = 0; t < 2; ++t) {
+            flushk(acc[t], p[t]);
+            if (fold_each) fold(acc[t], q);
+            if (last) {
+                out[((long long)(2 * jc + t) * cap_o + i) * N + k] =
+                    redc(mul_shoup(acc[t].hi, 1, one_s, q), acc[t].lo, q, qinv);
+                acc[t] = Acc128{0, 0};
             }
         }
     };
-    const u64* dbase = diags + (long long)i * N + k;
+    const u64* dbase = diags + diag_word(i, k, 0, ell, N);
     if (ell % n1 == 0 && n1 % 8 == 0) {
         // every batch is full: while a batch is multiplied, each word's register is refilled with
         // the same word of the next batch, so eight loads per thread stay in flight throughout
         u64 d[8];
         {
-            const u64* D = dbase + (long long)j * n1 * dstride;
+            const u64* D = dbase + (long long)j * n1 * kDiagTile;
 #pragma unroll
-            for (int u = 0; u < 8; ++u) d[u] = __ldcs(D + u * dstride);
+            for (int u = 0; u < 8; ++u) d[u] = __ldcs(D + u * kDiagTile);
         }
         for (;;) {
             int jn = j, in = i0 + 8;
@@ -554,16 +536,14 @@ __global__ void __launch_bounds__(512, (B == 1 ? 2 : 1)) k_mac(const u64* __rest
                 in = 0;
             }
             const bool more = jn < n2;
-            const u64* Dn = dbase + ((long long)(more ? jn : j) * n1 + (more ? in : i0)) * dstride;
-            const u64* s0 = sbase + i0 * TP2;
-            AccK p[B][2];
-#pragma unroll
-            for (int b = 0; b < B; ++b) p[b][0] = p[b][1] = AccK{0, 0, 0};
+            const u64* Dn = dbase + (long long)((more ? jn : j) * n1 + (more ? in : i0)) * kDiagTile;
+            const u64* s0 = sbase + i0 * 2 * TP;
+            AccK p[2] = {};
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 const u64 w = d[u];
-                if (more) d[u] = __ldcs(Dn + u * dstride);
-                mul_word(p, w, s0 + u * TP2);
+                if (more) d[u] = __ldcs(Dn + u * kDiagTile);
+                mul_word(p, w, s0 + u * 2 * TP);
             }
             close_batch(p, j, jn != j);
             if (!more) break;
@@ -574,20 +554,18 @@ __global__ void __launch_bounds__(512, (B == 1 ? 2 : 1)) k_mac(const u64* __rest
     }
     for (;;) {
         const int cnt = min(n1, ell - j * n1);
-        const u64* D = dbase + ((long long)j * n1 + i0) * dstride;
-        const u64* s0 = sbase + i0 * TP2;
-        AccK p[B][2];
-#pragma unroll
-        for (int b = 0; b < B; ++b) p[b][0] = p[b][1] = AccK{0, 0, 0};
+        const u64* D = dbase + (long long)(j * n1 + i0) * kDiagTile;
+        const u64* s0 = sbase + i0 * 2 * TP;
+        AccK p[2] = {};
         if (i0 + 8 <= cnt) {
             // full batch: no bounds checks
             u64 d[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) d[u] = __ldcs(D + u * dstride);
+            for (int u = 0; u < 8; ++u) d[u] = __ldcs(D + u * kDiagTile);
 #pragma unroll
-            for (int u = 0; u < 8; ++u) mul_word(p, d[u], s0 + u * TP2);
+            for (int u = 0; u < 8; ++u) mul_word(p, d[u], s0 + u * 2 * TP);
         } else {
-            for (int u = 0; i0 + u < cnt; ++u) mul_word(p, __ldcs(D + (long long)u * dstride), s0 + u * TP2);
+            for (int u = 0; i0 + u < cnt; ++u) mul_word(p, __ldcs(D + u * kDiagTile), s0 + u * 2 * TP);
         }
         // next batch
         int jn = j, in = i0 + 8;
@@ -628,11 +606,12 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 template <int B, int TP, int JG>
 __global__ void __launch_bounds__(TP * JG) k_mac_pipe(const u64* __restrict__ babies, long long baby_q, int cap_b,
                                                       const u64* __restrict__ diags, u64* __restrict__ out,
-                                                      long long out_q, int cap_o, int nl, int n1, int n2,
+                                                      long long out_q, int cap_o, int n1, int n2,
                                                       const DevPrime* __restrict__ primes, int N) {
     pdl_wait();
     pdl_trigger();
     constexpr int SD = kMpSD;
+    const int ell = n1 * n2;
     constexpr int NT = TP * JG;                       // threads
     constexpr int ROWS = JG * SD;                     // diagonal rows per stage
     constexpr int CHUNKS = ROWS * TP / 2;             // 16-byte chunks per stage
@@ -657,7 +636,7 @@ __global__ void __launch_bounds__(TP * JG) k_mac_pipe(const u64* __restrict__ ba
                 const int row = ch / (TP / 2), w = (ch % (TP / 2)) * 2;
                 const int g = row / SD, u = row % SD;
                 const long long d = (long long)(jb * JG + g) * n1 + i0 + u;
-                cp_async16(dst + (size_t)row * TP + w, diags + (d * nl + i) * N + k0 + w);
+                cp_async16(dst + (size_t)row * TP + w, diags + diag_word(i, k0, d, ell, N) + w);
             }
         }
         cp_async_commit();  // an empty group past the last stage keeps the group count uniform
@@ -683,7 +662,7 @@ __global__ void __launch_bounds__(TP * JG) k_mac_pipe(const u64* __restrict__ ba
         for (int qb = 0; qb < B; ++qb) p[qb][0] = p[qb][1] = AccK{0, 0, 0};
 #pragma unroll
         for (int u = 0; u < SD; ++u) {
-            const u64 ds = split30(st[(size_t)u * TP]);
+            const u64 ds = st[(size_t)u * TP];
             const u32 dsum = sum30(ds);
 #pragma unroll
             for (int qb = 0; qb < B; ++qb) {
@@ -759,7 +738,7 @@ __global__ void __launch_bounds__(kMrTP * kMrJG) k_mac_ring(const u64* __restric
     const int mt = (int)blockIdx.x < ntile ? (ntile - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
     constexpr int spb = N1 / SD;           // stages per giant-step block
     const int nst = (n2 / JG) * spb;       // stages per tile
-    const long long dstep = (long long)nl * N;  // one diagonal
+    const int ell = n2 * N1;
     auto at_tile = [&](MrCursor& c) {
         c.tile = (int)blockIdx.x + c.m * (int)gridDim.x;
         c.i = c.tile / tpl;
@@ -777,13 +756,13 @@ __global__ void __launch_bounds__(kMrTP * kMrJG) k_mac_ring(const u64* __restric
         if (c.m < mt) {
             const int jb = c.sl / spb, i0 = (c.sl - jb * spb) * SD;
             u64* dst = sd + (size_t)c.slot * ROWS * TP;
-            const u64* src = diags + ((long long)jb * JG * N1 + i0) * dstep + (long long)c.i * N + c.k0;
+            const u64* src = diags + diag_word(c.i, c.k0, jb * JG * N1 + i0, ell, N);
 #pragma unroll
             for (int r = 0; r < CHUNKS / NT; ++r) {
                 const int ch = threadIdx.x + r * NT;
                 const int row = ch / (TP / 2), w = (ch % (TP / 2)) * 2;
                 const int gg = row / SD, u = row % SD;
-                cp_async16(dst + (size_t)row * TP + w, src + ((long long)gg * N1 + u) * dstep + w);
+                cp_async16(dst + (size_t)row * TP + w, src + (gg * N1 + u) * kDiagTile + w);
             }
             // the babies of tile 0 ride on its first stage, those of tile m + 1 on tile m's last
             const int mb = (c.m == 0 && c.sl == 0) ? 0 : (c.sl == nst - 1 ? c.m + 1 : -1);
@@ -832,7 +811,7 @@ __global__ void __launch_bounds__(kMrTP * kMrJG) k_mac_ring(const u64* __restric
         for (int qb = 0; qb < B; ++qb) p[qb][0] = p[qb][1] = AccK{0, 0, 0};
 #pragma unroll
         for (int u = 0; u < SD; ++u) {
-            const u64 ds = split30(st[u * TP]);
+            const u64 ds = st[u * TP];
             const u32 dsum = sum30(ds);
 #pragma unroll
             for (int qb = 0; qb < B; ++qb) {
@@ -870,8 +849,9 @@ __global__ void __launch_bounds__(kMrTP * kMrJG) k_mac_ring(const u64* __restric
 //   d0 += b0 e0,  d1 += b0 e1 + b1 e0,  d2 += b1 e1.
 // The middle term takes one product (Karatsuba): d1 = sum (b0 + b1)(e0 + e1) - d0 - d2, the
 // same residue mod q as the two products it replaces.
-// babies: [n1][2][cap_b][N] evaluation form; diags: [ell][2][nl][N] evaluation form in
-// Montgomery form (e0 R + e1 R = (e0 + e1) R), so one REDC of each sum gives it in plain form;
+// babies: [n1][2][cap_b][N] evaluation form; diags: component t of ciphertext d is row 2 d + t
+// of the tiles of diag_word, whole words in Montgomery form (e0 R + e1 R = (e0 + e1) R), so one
+// REDC of each sum gives it in plain form;
 // out: [n2][3][cap_o][N]. Tiling as k_mac: the babies of a point tile are staged in shared
 // memory as 30-bit halves of b0, b1 and b0 + b1, giant steps run over the thread rows.
 // Diagonals go in batches of 4 (one carry step per batch).
@@ -899,11 +879,10 @@ __global__ void __launch_bounds__(512, 2) k_mac_ct(const u64* __restrict__ babie
         dst[2 * TP] = split30(add_mod(b0, b1, q));
     }
     __syncthreads();
-    const long long dstride = 2LL * nl * N;  // one diagonal ciphertext
-    const long long cstride = (long long)nl * N;
+    constexpr int dstride = 2 * kDiagTile, cstride = kDiagTile;  // one diagonal ciphertext, one component
     for (int j = jg; j < n2; j += JG) {
         const int cnt = min(n1, ell - j * n1);
-        const u64* D = diags + (long long)j * n1 * dstride + (long long)i * N + k;
+        const u64* D = diags + diag_word(i, k, 2LL * j * n1, 2 * ell, N);
         Acc128 a0{0, 0}, am{0, 0}, a2{0, 0};
         for (int i0 = 0; i0 < cnt; i0 += 4) {
             AccK p0{0, 0, 0}, pm{0, 0, 0}, p2{0, 0, 0};
@@ -954,8 +933,8 @@ __global__ void __launch_bounds__(512, 2) k_mac_ct(const u64* __restrict__ babie
 // Table-schedule MAC (Algorithm 1, step 4): S_g = sum_{m < ell} rotQ[m] (.) D_{g,m}
 // for GG groups per CTA column. One thread per evaluation point of one limb; the two
 // table words of a point are read once for the GG groups, the diagonal words streamed.
-// table: [ell][2][cap_t][N]; diagonal m of group g, limb i at diags + g dgrp + (m nl + i) N
-// (Montgomery form); output of group g at out + g og, [2][cap_o][N]. Products use the 30-bit
+// table: [ell][2][cap_t][N]; diagonal m of group g at row m of the tiles at diags + g dgrp
+// (diag_word; Montgomery form, 30-bit halves); output of group g at out + g og, [2][cap_o][N]. Products use the 30-bit
 // split multiply-accumulate (four per carry step).
 // ---------------------------------------------------------------------------
 template <int GG>
@@ -970,10 +949,10 @@ __global__ void __launch_bounds__(256) k_mac_table(const u64* __restrict__ table
     const int g0 = blockIdx.z * GG;
     if (k >= N) return;
     const u64 q = primes[i].q, qinv = primes[i].qinv;
-    const long long ts = 2ll * cap_t * N, ds = (long long)nl * N;
+    const long long ts = 2ll * cap_t * N;
     const u64* t0 = table + (long long)i * N + k;
     const u64* t1 = t0 + (long long)cap_t * N;
-    const u64* d0 = diags + (long long)g0 * dgrp + (long long)i * N + k;
+    const u64* d0 = diags + (long long)g0 * dgrp + diag_word(i, k, 0, ell, N);
     Acc128 acc[GG][2];
 #pragma unroll
     for (int gg = 0; gg < GG; ++gg) acc[gg][0] = acc[gg][1] = Acc128{0, 0};
@@ -991,7 +970,7 @@ __global__ void __launch_bounds__(256) k_mac_table(const u64* __restrict__ table
                 AccK p0{0, 0, 0}, p1{0, 0, 0};
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
-                    const u64 d = split30(m0 + u < ell ? __ldcs(d0 + gg * dgrp + (long long)(m0 + u) * ds) : 0ull);
+                    const u64 d = m0 + u < ell ? __ldcs(d0 + gg * dgrp + (long long)(m0 + u) * kDiagTile) : 0ull;
                     const u32 dsum = sum30(d);
                     mack(p0, d, dsum, a[u]);
                     mack(p1, d, dsum, b[u]);
@@ -1082,6 +1061,19 @@ __global__ void k_to_mont(u64* x, long long n_per_poly, PrimeMap pm, const DevPr
         const DevPrime P = primes[pm.idx[p % pm.period]];
         x[e] = to_mont(x[e], P);
     }
+}
+
+// ciphertext polynomials src [rows][nl][N] in Montgomery form into rows row0, row0 + 1, ... of the
+// tiles of a database of `total` rows
+__global__ void __launch_bounds__(kThreads) k_tile_mont(const u64* __restrict__ src, u64* __restrict__ diags,
+                                                        long long row0, int total, int nl,
+                                                        const DevPrime* __restrict__ primes, int N) {
+    pdl_wait();
+    pdl_trigger();
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = blockIdx.y, r = blockIdx.z;
+    if (k >= N) return;
+    diags[diag_word(i, k, row0 + r, total, N)] = to_mont(src[((long long)r * nl + i) * N + k], primes[i]);
 }
 
 // ---------------------------------------------------------------------------
@@ -1197,11 +1189,18 @@ __device__ __forceinline__ long long fft_coef(const cplx* __restrict__ z, int lo
     return llround(__dmul_rn(__dmul_rn(v, inv_n), delta));
 }
 
-// m mod q for a signed coefficient: |m| reduced with the Shoup quotient of 1
+// m mod q for a signed coefficient: |m| < 2^63 reduced by its bits from bits(q) up where that is
+// enough for the prime (13 issue cycles a warp against 44), else with the Shoup quotient of 1
 __device__ __forceinline__ u64 coef_residue(long long m, const DevPrime& P) {
     const bool neg = m < 0;
     const u64 a = neg ? (u64)(-(m + 1)) : (u64)m;
-    const u64 ra = mul_shoup(a, 1, P.one_s, P.q);
+    u64 ra;
+    if (P.fold63) {
+        const u64 f = fold_top(a, P.bsh, P.c);
+        ra = min(f, f - P.q);
+    } else {
+        ra = mul_shoup(a, 1, P.one_s, P.q);
+    }
     return neg ? P.q - 1 - ra : ra;
 }
 
@@ -1339,20 +1338,15 @@ void launch_tensor(const TensorJobs& jobs, int J, int level, const DevPrime* pri
     launch_k(k_tensor, dim3(g), dim3(kBcThreads), 0, s, jobs, level, primes, N);
 }
 
-template <int B>
-static void launch_mac_t(const u64* babies, long long baby_q, int cap_b, const u64* diags, u64* out, long long out_q,
-                         int cap_o, int nl, int n1, int n2, int ell, const DevPrime* primes, int N, cudaStream_t s) {
-    // points per CTA: staged babies (B n1 2 TP words) within 128 KiB; giant-step groups up to 512 threads
-    int TP = 128;
-    while (TP > 16 && (size_t)B * n1 * 2 * TP * 8 > (128u << 10)) TP >>= 1;
-    int JG = 512 / TP;
-    if (JG > n2) JG = n2;
-    if (JG < 1) JG = 1;
-    const size_t sm = (size_t)B * n1 * 2 * TP * sizeof(u64);
+template <int TP>
+static void launch_mac_t(const u64* babies, int cap_b, const u64* diags, u64* out, int cap_o, int nl, int n1, int n2,
+                         int ell, const DevPrime* primes, int N, cudaStream_t s) {
+    const int JG = std::max(1, std::min(256 / TP, n2));
+    const size_t sm = (size_t)n1 * 2 * TP * sizeof(u64);
     static std::atomic<unsigned long long> attr{0};
-    smem_limit_once(k_mac<B>, 200 * 1024, attr);
-    dim3 g(N / TP, nl);
-    launch_k(k_mac<B>, dim3(g), dim3(TP * JG), sm, s, babies, baby_q, cap_b, diags, out, out_q, cap_o, nl, n1, n2, ell, TP, JG, primes, N);
+    smem_limit_once(k_mac<TP>, 200 * 1024, attr);
+    launch_k(k_mac<TP>, dim3(N / TP, nl), dim3(TP * JG), sm, s, babies, cap_b, diags, out, cap_o, nl, n1, n2, ell, JG,
+             primes, N);
 }
 
 static size_t mac_ring_smem(int B, int n1) {
@@ -1414,8 +1408,8 @@ static void launch_mac_pipe_s(const u64* babies, long long baby_q, int cap_b, co
     static std::atomic<unsigned long long> attr{0};
     smem_limit_once(k_mac_pipe<B, TP, JG>, 200 * 1024, attr);
     dim3 g(N / TP, nl);
-    launch_k(k_mac_pipe<B, TP, JG>, g, dim3(TP * JG), sm, s, babies, baby_q, cap_b, diags, out, out_q, cap_o, nl, n1,
-             n2, primes, N);
+    launch_k(k_mac_pipe<B, TP, JG>, g, dim3(TP * JG), sm, s, babies, baby_q, cap_b, diags, out, out_q, cap_o, n1, n2,
+             primes, N);
 }
 
 template <int B>
@@ -1444,15 +1438,13 @@ void launch_mac_pipe(const u64* babies, long long baby_q, int cap_b, const u64* 
     }
 }
 
-void launch_mac(const u64* babies, long long baby_q, int cap_b, const u64* diags, u64* out, long long out_q,
-                int cap_o, int nl, int n1, int n2, int ell, int B, const DevPrime* primes, int N, cudaStream_t s) {
-    switch (B) {
-        case 1: launch_mac_t<1>(babies, baby_q, cap_b, diags, out, out_q, cap_o, nl, n1, n2, ell, primes, N, s); break;
-        case 2: launch_mac_t<2>(babies, baby_q, cap_b, diags, out, out_q, cap_o, nl, n1, n2, ell, primes, N, s); break;
-        case 3: launch_mac_t<3>(babies, baby_q, cap_b, diags, out, out_q, cap_o, nl, n1, n2, ell, primes, N, s); break;
-        case 4: launch_mac_t<4>(babies, baby_q, cap_b, diags, out, out_q, cap_o, nl, n1, n2, ell, primes, N, s); break;
-        default: break;  // the engine splits larger batches
-    }
+void launch_mac(const u64* babies, int cap_b, const u64* diags, u64* out, int cap_o, int nl, int n1, int n2, int ell,
+                const DevPrime* primes, int N, cudaStream_t s) {
+    // points per CTA: a whole tile unless its staged babies (n1 2 TP words) exceed 128 KiB
+    const int TP = n1 <= 128 ? 64 : n1 <= 256 ? 32 : 16;
+    if (TP == 64) launch_mac_t<64>(babies, cap_b, diags, out, cap_o, nl, n1, n2, ell, primes, N, s);
+    else if (TP == 32) launch_mac_t<32>(babies, cap_b, diags, out, cap_o, nl, n1, n2, ell, primes, N, s);
+    else launch_mac_t<16>(babies, cap_b, diags, out, cap_o, nl, n1, n2, ell, primes, N, s);
 }
 
 void launch_mac_ct(const u64* babies, int cap_b, const u64* diags, u64* out, int cap_o, int nl, int n1, int n2, int ell,
@@ -1507,8 +1499,15 @@ void launch_to_mont(u64* x, long long n_per_poly, const PrimeMap& pm, const DevP
     launch_k(k_to_mont, dim3((unsigned)blocks), dim3(kThreads), 0, s, x, n_per_poly, pm, primes, total);
 }
 
-static void encode_fft(const float* T, long long K, int ell, int logn, long long grp, int d0, int nd, int n1,
-                       cplx* z, const unsigned* rot, const double* zr, const double* zi, cudaStream_t s) {
+void launch_tile_mont(const u64* src, int rows, u64* diags, long long row0, int total, int nl, const DevPrime* primes,
+                      int N, cudaStream_t s) {
+    dim3 g((N + kThreads - 1) / kThreads, nl, rows);
+    launch_k(k_tile_mont, g, dim3(kThreads), 0, s, src, diags, row0, total, nl, primes, N);
+}
+
+void launch_encode_fft(const float* T, long long K, int ell, int logn, long long grp, int d0, int nd, int n1, void* zbuf,
+                       const unsigned* rot, const double* zr, const double* zi, cudaStream_t s) {
+    cplx* z = (cplx*)zbuf;
     const int n = 1 << logn;
     {
         dim3 g((n + kThreads - 1) / kThreads, nd);
@@ -1531,24 +1530,17 @@ static void encode_fft(const float* T, long long K, int ell, int logn, long long
     }
 }
 
-void launch_encode_diags(const float* T, long long K, int ell, int logn, long long grp, int d0, int nd, int n1,
-                         void* zbuf, u64* out_coeff, int nl, const DevPrime* primes, int scale_bits,
-                         const unsigned* rot, const double* zr, const double* zi, cudaStream_t s) {
+void launch_fft_residues(const void* zbuf, int z0, int logn, int nd, u64* out_coeff, int nl, const DevPrime* primes,
+                         int scale_bits, cudaStream_t s) {
     const int n = 1 << logn;
-    cplx* z = (cplx*)zbuf;
-    encode_fft(T, K, ell, logn, grp, d0, nd, n1, z, rot, zr, zi, s);
     dim3 g((2 * n + kThreads - 1) / kThreads, nd);
-    launch_k(k_fft_finish, dim3(g), dim3(kThreads), 0, s, z, logn, nd, out_coeff, nl, primes, scale_bits);
+    launch_k(k_fft_finish, dim3(g), dim3(kThreads), 0, s, (const cplx*)zbuf + (size_t)z0 * n, logn, nd, out_coeff, nl,
+             primes, scale_bits);
 }
 
-void launch_encode_diags_int(const float* T, long long K, int ell, int logn, long long grp, int d0, int nd, int n1,
-                             void* zbuf, long long* out_int, int scale_bits, const unsigned* rot, const double* zr,
-                             const double* zi, cudaStream_t s) {
-    const int n = 1 << logn;
-    cplx* z = (cplx*)zbuf;
-    encode_fft(T, K, ell, logn, grp, d0, nd, n1, z, rot, zr, zi, s);
-    dim3 g((2 * n + kThreads - 1) / kThreads, nd);
-    launch_k(k_fft_round, dim3(g), dim3(kThreads), 0, s, z, logn, nd, out_int, scale_bits);
+void launch_fft_round(const void* zbuf, int logn, int nd, long long* out_int, int scale_bits, cudaStream_t s) {
+    dim3 g(((2 << logn) + kThreads - 1) / kThreads, nd);
+    launch_k(k_fft_round, dim3(g), dim3(kThreads), 0, s, (const cplx*)zbuf, logn, nd, out_int, scale_bits);
 }
 
 void launch_coef_residues(const long long* m, int nd, u64* out, int nl, const DevPrime* primes, int N,

@@ -93,8 +93,21 @@ struct IPSumJobs {
 };
 struct TensorJobs { TensorJob j[FR_MAX_JOBS]; };
 
-// Forward NTT that stores its values in Montgomery form (x 2^64 mod q), in place.
-void launch_ntt_tomont(const RingDev& R, const PolyBatch& b, cudaStream_t s);
+// Layout of a database's diagonals in evaluation form: tiles of kDiagTile points, [limb][N /
+// kDiagTile][row][kDiagTile], so that a CTA of the MAC, which takes all rows at a few points of one
+// limb, reads one contiguous run. Rows are the diagonals (or, encrypted, the two components of
+// each). Offset of point k of limb i of row r among `rows` rows of N points:
+constexpr int kDiagTile = 64;
+__host__ __device__ __forceinline__ long long diag_word(int i, int k, long long r, int rows, int N) {
+    return (((long long)i * (N / kDiagTile) + k / kDiagTile) * rows + r) * kDiagTile + k % kDiagTile;
+}
+// Forward NTT of encoded diagonals into a database: poly p of b is limb p % nl of diagonal d0 +
+// p / nl; the values go to diags (ell rows) in Montgomery form (x 2^64 mod q), as 30-bit halves
+// (split30).
+void launch_ntt_diags(const RingDev& R, const PolyBatch& b, u64* diags, int d0, int ell, int nl, cudaStream_t s);
+// src [rows][nl][N] (evaluation form) into rows row0.. of a database of total rows, Montgomery form
+void launch_tile_mont(const u64* src, int rows, u64* diags, long long row0, int total, int nl, const DevPrime* primes,
+                      int N, cudaStream_t s);
 // Forward NTT of the P -> Q conversions of a ModDown (b.conv forms them) fused with its combine:
 // poly p of b is (job p / (2(level+1)), component, limb); the transformed values never reach
 // memory, the jobs' outputs do.
@@ -151,7 +164,6 @@ void launch_rescale_lift(const u64* last, u64* lifted, const RescaleTab* tab, in
 void launch_rescale_combine(const u64* x, int x_cap, const u64* lifted, u64* out, int out_cap, const RescaleTab* tab,
                             int l, int N, int BT, cudaStream_t s);
 void launch_tensor(const TensorJobs& jobs, int J, int level, const DevPrime* primes, int N, cudaStream_t s);
-// B <= 4 queries: babies of query b at babies + b * baby_q, outputs at out + b * out_q
 // Sums of rotations with one ModDown (double hoisting), without the per-job inner products in
 // memory: for each group g and position,
 // out_g += sum_{jobs of g} (IP_j + P sigma_j(addb_j) on the Q positions of component 0), the
@@ -159,7 +171,7 @@ void launch_tensor(const TensorJobs& jobs, int J, int level, const DevPrime* pri
 void launch_ip_sum(const IPSumJobs& jobs, int beta, int npos, int level, int kp, int T, const DevPrime* primes,
                    const PrimeMap& pos_prime, int logN, const u64* pmod, const u64* pmod_s, cudaStream_t s);
 // Encrypted-database MAC: (d0, d1, d2)_j = sum_i B_i (x) E_{j n1 + i} for every giant step j.
-// babies [n1][2][cap_b][N]; diags [ell][2][nl][N] (evaluation form, Montgomery); out [n2][3][cap_o][N].
+// babies [n1][2][cap_b][N]; diags: 2 ell rows (evaluation form, Montgomery); out [n2][3][cap_o][N].
 void launch_mac_ct(const u64* babies, int cap_b, const u64* diags, u64* out, int cap_o, int nl, int n1, int n2, int ell,
                    const DevPrime* primes, int N, cudaStream_t s);
 // The diagonal MAC of B = 1..4 queries against one database with the diagonals streamed
@@ -175,8 +187,9 @@ void launch_mac_ring(const u64* babies, long long baby_q, int cap_b, const u64* 
                      int cap_o, int nl, int n1, int ell, int B, const DevPrime* primes, int N, cudaStream_t s);
 void launch_mac_pipe(const u64* babies, long long baby_q, int cap_b, const u64* diags, u64* out, long long out_q,
                      int cap_o, int nl, int n1, int ell, int B, const DevPrime* primes, int N, cudaStream_t s);
-void launch_mac(const u64* babies, long long baby_q, int cap_b, const u64* diags, u64* out, long long out_q,
-                int cap_o, int nl, int n1, int n2, int ell, int B, const DevPrime* primes, int N, cudaStream_t s);
+// The diagonal MAC of one query: babies [n1][2][cap_b][N], outputs [n2][2][cap_o][N].
+void launch_mac(const u64* babies, int cap_b, const u64* diags, u64* out, int cap_o, int nl, int n1, int n2, int ell,
+                const DevPrime* primes, int N, cudaStream_t s);
 // Table schedule (Algorithm 1): out_g = sum_{m < ell} table[m] (.) D_{g,m} for g < G (evaluation form,
 // not rescaled); table [ell][2][cap_t][N], group g's diagonals at diags + g * dgrp.
 void launch_mac_table(const u64* table, int cap_t, const u64* diags, long long dgrp, int G, u64* out, int cap_o,
@@ -187,13 +200,15 @@ void launch_sum(const u64* a, int cap, long long js, int J, u64* out, int o_cap,
                 int N, cudaStream_t s);
 void launch_to_mont(u64* x, long long n_per_poly, const PrimeMap& pm, const DevPrime* primes, long long total,
                     cudaStream_t s);
-void launch_encode_diags(const float* T, long long K, int ell, int logn, long long grp, int d0, int nd, int n1,
-                         void* zbuf, u64* out_coeff, int nl, const DevPrime* primes, int scale_bits,
-                         const unsigned* rot, const double* zr, const double* zi, cudaStream_t s);
-// Storage tier B: the same encoding up to the rounded integer coefficients, out_int [nd][N].
-void launch_encode_diags_int(const float* T, long long K, int ell, int logn, long long grp, int d0, int nd, int n1,
-                             void* zbuf, long long* out_int, int scale_bits, const unsigned* rot, const double* zr,
-                             const double* zi, cudaStream_t s);
+// Slot encoding of diagonals d0 .. d0 + nd - 1 of template group grp, up to the rounding: z [nd][n]
+// complex doubles
+void launch_encode_fft(const float* T, long long K, int ell, int logn, long long grp, int d0, int nd, int n1, void* zbuf,
+                       const unsigned* rot, const double* zr, const double* zi, cudaStream_t s);
+// The rounded coefficients of diagonals z0 .. z0 + nd - 1 of z as residues, out_coeff [nd][nl][N], or
+// (storage tier B) of all nd of z as integers, out_int [nd][N]
+void launch_fft_residues(const void* zbuf, int z0, int logn, int nd, u64* out_coeff, int nl, const DevPrime* primes,
+                         int scale_bits, cudaStream_t s);
+void launch_fft_round(const void* zbuf, int logn, int nd, long long* out_int, int scale_bits, cudaStream_t s);
 // Residues of stored integer coefficients: m [nd][N] -> out [nd][nl][N] (coefficient form).
 void launch_coef_residues(const long long* m, int nd, u64* out, int nl, const DevPrime* primes, int N,
                           cudaStream_t s);

@@ -25,7 +25,7 @@ struct DevPrime {
     u32 bsh;     // classes 0, 1: bits(q) - 32
     u32 c;       // classes 0, 1: 2^bits(q) - q
     u32 cls;     // twiddle class
-    u32 pad;
+    u32 fold63;  // fold_top brings every value below 2^63 to below 2q
     uint4 tw_ninv;   // N^-1 as a twiddle of the class
     uint4 tw_wninv;  // N^-1 times the inverse transform's last twiddle, likewise
 };

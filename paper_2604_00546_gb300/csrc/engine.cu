@@ -5,8 +5,8 @@
 //   ciphertext batch : [B][2][cap][N] u64, evaluation (NTT) form, limbs 0..level
 //                      valid (cap >= level+1, dropping a level keeps the buffer)
 //   key-switching key: [ndig][2][nq+np][N] u64, Montgomery form (x * 2^64 mod q)
-//   template database: [G][ell][nq][N] u64, pre-rotated diagonals (Eq.
-//                      eq:prerotation), evaluation + Montgomery form
+//   template database: [G] groups of ell pre-rotated diagonals (Eq. eq:prerotation), in tiles
+//                      (diag_word), evaluation + Montgomery form, 30-bit halves
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -174,7 +174,8 @@ struct fr_db {
                              // 4 (E): encrypted pre-rotated diagonals (ciphertexts, evaluation form)
     int schedule = 0;        // 0: on-demand BSGS (diagonals pre-rotated by j n1); 1: rotated-query table (plain diagonals)
     int nl = 0;              // limbs per plaintext diagonal: level + 1, or level + 1 + n_p over Q_l u P (hoist_babies)
-    u64* diags = nullptr;    // tier 1: [G][ell][level+1][N]; tier 4: [G][ell][2][level+1][N] (Montgomery form)
+    u64* diags = nullptr;    // tier 1: [G] groups of ell rows of nl limbs (diag_word), Montgomery form as 30-bit
+                             // halves; tier 4: [G] groups of 2 ell rows of level+1 limbs, whole words
     float* templates = nullptr;  // tier 2: [K][ell] FP32
     long long* coeffs = nullptr; // tier 3: [G][ell][N] integer coefficients of the diagonals
     size_t bytes = 0;
@@ -1062,32 +1063,46 @@ int diag_limbs(const fr_ctx* c, int schedule) {
     return c->work_level + 1 + (c->hoist_babies && schedule == 0 ? c->R.np : 0);
 }
 
-// Encode the diagonals of template group g at the working level into dst [ell][nl][N]
-// (evaluation + Montgomery form; nl = level + 1, or the positions of Q_l u P when
-// nl > level + 1), diagonal d pre-rotated by (d / n1_enc) n1_enc slots (n1_enc = ell: plain
-// diagonals).
+// Diagonals whose residues are transformed together: as many as keep the column-to-row
+// intermediate (nl limbs each) in 96 MB of the 126 MB L2, at least 4, at most 64.
+int encode_chunk(const fr_ctx* c, int nl) {
+    const size_t fit = ((size_t)96 << 20) / ((size_t)nl * c->R.N * 8);
+    return (int)std::min<size_t>(c->ell, std::max<size_t>(4, std::min<size_t>(64, fit)));
+}
+// residues o [nd][nl][N] of diagonals d0 .. of a database group -> dst: forward NTT, Montgomery
+// form and tiling in its epilogue
+void ntt_diags(fr_ctx* c, u64* o, int nd, int nl, const PrimeMap& pm, u64* dst, int d0) {
+    Prof p(c, "ntt", 16.0 * nd * nl * c->R.N);
+    PolyBatch pb{o, (long long)nl * c->R.N, nl, nd * nl, pm};
+    launch_ntt_diags(c->rd, pb, dst, d0, (int)c->ell, nl, c->cur);
+    c->launches += 2;
+}
+
+// Encode the diagonals of template group g at the working level into dst, ell rows of nl limbs in
+// the layout of diag_word (nl = level + 1, or the positions of Q_l u P when nl > level + 1),
+// diagonal d pre-rotated by (d / n1_enc) n1_enc slots (n1_enc = ell: plain diagonals).
 void encode_group(fr_ctx* c, const float* dT, long long K, long long g, u64* dst, int n1_enc, int nl) {
     const int N = c->R.N, n = N / 2, L = c->work_level, ell = (int)c->ell;
-    const int chunk = 64;
-    Tmp z(c, (size_t)chunk * n * 2);
+    const int fft = std::min(ell, 64), chunk = std::min(fft, encode_chunk(c, nl));
+    Tmp z(c, (size_t)fft * n * 2), o(c, (size_t)chunk * nl * N);
     const bool ext = nl > L + 1;
     const PrimeMap pm = ext ? pm_ext(c, L) : pm_level(L);
     const DevPrime* primes = ext ? primes_ext(c, L) : c->d_primes;
-    for (int d0 = 0; d0 < ell; d0 += chunk) {
-        const int nd = std::min(chunk, ell - d0);
-        u64* o = dst + (size_t)d0 * nl * N;
+    for (int f0 = 0; f0 < ell; f0 += fft) {
+        const int nf = std::min(fft, ell - f0);
         {
-            Prof p(c, "encode", 8.0 * N * nd * nl);
-            launch_encode_diags(dT, K, ell, c->R.logN - 1, g, d0, nd, n1_enc, z.p, o, nl, primes,
-                                c->R.scale_bits, c->d_rot, c->d_zr, c->d_zi, c->cur);
-            c->launches += 4;
+            Prof p(c, "encode", 16.0 * N * nf);
+            launch_encode_fft(dT, K, ell, c->R.logN - 1, g, f0, nf, n1_enc, z.p, c->d_rot, c->d_zr, c->d_zi, c->cur);
+            c->launches += 3;
         }
-        {
-            // forward NTT with the Montgomery conversion in its epilogue
-            Prof p(c, "ntt", 16.0 * nd * nl * N);
-            PolyBatch pb{o, (long long)nl * N, nl, nd * nl, pm};
-            launch_ntt_tomont(c->rd, pb, c->cur);
-            c->launches += 2;
+        for (int d0 = 0; d0 < nf; d0 += chunk) {
+            const int nd = std::min(chunk, nf - d0);
+            {
+                Prof p(c, "encode", 8.0 * N * nd * (1.0 + nl));
+                launch_fft_residues(z.p, d0, c->R.logN - 1, nd, o.p, nl, primes, c->R.scale_bits, c->cur);
+                c->launches++;
+            }
+            ntt_diags(c, o.p, nd, nl, pm, dst, f0 + d0);
         }
     }
 }
@@ -1195,32 +1210,29 @@ void encode_group_int(fr_ctx* c, const float* dT, long long K, long long g, long
     for (int d0 = 0; d0 < ell; d0 += chunk) {
         const int nd = std::min(chunk, ell - d0);
         Prof p(c, "encode", 8.0 * N * nd);
-        launch_encode_diags_int(dT, K, ell, c->R.logN - 1, g, d0, nd, n1_enc, z.p, dst + (size_t)d0 * N,
-                                c->R.scale_bits, c->d_rot, c->d_zr, c->d_zi, c->cur);
+        launch_encode_fft(dT, K, ell, c->R.logN - 1, g, d0, nd, n1_enc, z.p, c->d_rot, c->d_zr, c->d_zi, c->cur);
+        launch_fft_round(z.p, c->R.logN - 1, nd, dst + (size_t)d0 * N, c->R.scale_bits, c->cur);
         c->launches += 4;
     }
 }
 
 // Storage tier B, per query: residues of the stored coefficients at the working level, then
-// the forward NTT with the Montgomery conversion: dst [ell][nl][N] as encode_group writes.
+// the forward NTT into dst as encode_group writes it.
 void expand_group(fr_ctx* c, const long long* src, u64* dst, int nl) {
     const int N = c->R.N, L = c->work_level, ell = (int)c->ell;
-    const int chunk = 64;
+    const int chunk = encode_chunk(c, nl);
+    Tmp o(c, (size_t)chunk * nl * N);
     const bool ext = nl > L + 1;
     const PrimeMap pm = ext ? pm_ext(c, L) : pm_level(L);
     const DevPrime* primes = ext ? primes_ext(c, L) : c->d_primes;
     for (int d0 = 0; d0 < ell; d0 += chunk) {
         const int nd = std::min(chunk, ell - d0);
-        u64* o = dst + (size_t)d0 * nl * N;
         {
             Prof p(c, "encode", 8.0 * N * nd * (1.0 + nl));
-            launch_coef_residues(src + (size_t)d0 * N, nd, o, nl, primes, N, c->cur);
+            launch_coef_residues(src + (size_t)d0 * N, nd, o.p, nl, primes, N, c->cur);
             c->launches++;
         }
-        Prof p(c, "ntt", 16.0 * nd * nl * N);
-        PolyBatch pb{o, (long long)nl * N, nl, nd * nl, pm};
-        launch_ntt_tomont(c->rd, pb, c->cur);
-        c->launches += 2;
+        ntt_diags(c, o.p, nd, nl, pm, dst, d0);
     }
 }
 
@@ -1357,9 +1369,11 @@ void twiddle_class(u64 q, DevPrime& d) {
         d.c2 = e - m;
         d.bsh = (u32)(b - 32);
         d.c = (u32)c;
+        d.fold63 = folded((u128)1 << 63) < (u128)2 * q && b > 32;
         return;
     }
     d.cls = 2;
+    d.fold63 = 0;
     d.off = d.big = 0;
 }
 // Twiddles of one prime in the format of its class.
@@ -1930,46 +1944,40 @@ fr_status fr_load_db_encrypted(fr_ctx* c, const uint64_t* cts, size_t K, size_t 
                   std::string("cannot hold the encrypted diagonals: ") + cudaGetErrorString(e));
         }
         db->diags = (u64*)p;
-        // limbs 0..L of both components, 64 ciphertexts per copy, then the NTT (into Montgomery
-        // form when the enroller pre-rotated them)
-        for (size_t e0 = 0; e0 < ncts; e0 += 64) {
-            const size_t ne = std::min<size_t>(64, ncts - e0);
-            u64* dst = db->diags + e0 * 2 * L1 * N;
-            CU(cudaMemcpy2DAsync(dst, (size_t)L1 * N * 8, cts + e0 * 2 * lw * N, lw * N * 8, (size_t)L1 * N * 8, 2 * ne,
+        // limbs 0..L of both components, 16 ciphertexts at a time: copy, NTT, the server-side
+        // pre-rotation unless the enroller did it (Eq. eq:prerotation on ciphertexts: diagonal j n1 +
+        // i, j >= 1, rotated by -j n1 with the negative giant-step key), then tiled in Montgomery form
+        const int n1 = (int)c->n1;
+        const size_t cw1 = (size_t)2 * L1 * N;
+        constexpr size_t kChunk = 16;
+        Tmp nat(c, kChunk * cw1), rot(c, prerotated ? 1 : kChunk * cw1);
+        for (size_t e0 = 0; e0 < ncts; e0 += kChunk) {
+            const size_t ne = std::min(kChunk, ncts - e0);
+            CU(cudaMemcpy2DAsync(nat.p, (size_t)L1 * N * 8, cts + e0 * 2 * lw * N, lw * N * 8, (size_t)L1 * N * 8, 2 * ne,
                                  cudaMemcpyHostToDevice, c->cur));
-            if (prerotated) {
-                PolyBatch pb{dst, (long long)L1 * N, L1, (int)(2 * ne * L1), pm_level(L)};
-                launch_ntt_tomont(c->rd, pb, c->cur);
-                c->launches++;
-            } else {
-                ntt(c, dst, (long long)L1 * N, L1, (int)(2 * ne * L1), pm_level(L), false);
-            }
-        }
-        if (!prerotated) {
-            // server-side pre-rotation (Eq. eq:prerotation on ciphertexts): diagonal j n1 + i,
-            // j >= 1, is rotated by -j n1 with the negative giant-step key, 64 at a time into
-            // scratch and copied back; then the whole database into Montgomery form
-            const int n1 = (int)c->n1;
-            const size_t cw1 = (size_t)2 * L1 * N;
-            std::vector<size_t> todo;
-            for (size_t e = 0; e < ncts; ++e)
-                if ((int)(e % ell) >= n1) todo.push_back(e);
-            Tmp rot(c, 64 * cw1);
-            for (size_t t0 = 0; t0 < todo.size(); t0 += 64) {
-                const size_t nt = std::min<size_t>(64, todo.size() - t0);
+            ntt(c, nat.p, (long long)L1 * N, L1, (int)(2 * ne * L1), pm_level(L), false);
+            if (!prerotated) {
                 std::vector<KSReq> reqs;
-                for (size_t t = 0; t < nt; ++t) {
-                    const size_t e = todo[t0 + t];
-                    const long j = (long)(e % ell) / n1;
+                for (size_t t = 0; t < ne; ++t) {
+                    const u64* src = nat.p + t * cw1;
+                    const long j = (long)((e0 + t) % ell) / n1;
+                    if (j == 0) {
+                        copy_d2d(c, rot.p + t * cw1, src, cw1);
+                        continue;
+                    }
                     const u64 gk = frh::galois_of_rotation(c->R, -j * n1);
-                    const u64* src = db->diags + e * cw1;
                     reqs.push_back(KSReq{src + (size_t)L1 * N, rot_key(c, gk), (u32)gk, 1, src, L1, rot.p + t * cw1, L1});
                 }
                 keyswitch(c, L, reqs);
-                for (size_t t = 0; t < nt; ++t) copy_d2d(c, db->diags + todo[t0 + t] * cw1, rot.p + t * cw1, cw1);
             }
-            launch_to_mont(db->diags, N, pm_level(L), c->d_primes, (long long)(ncts * cw1), c->cur);
-            c->launches++;
+            // a chunk may span groups, whose tiles are their own
+            for (size_t t = 0; t < ne;) {
+                const size_t g = (e0 + t) / ell, d = (e0 + t) % ell, n = std::min(ne - t, ell - d);
+                launch_tile_mont((prerotated ? nat.p : rot.p) + t * cw1, (int)(2 * n), db->diags + g * ell * cw1, 2 * d,
+                                 (int)(2 * ell), L1, c->d_primes, N, c->cur);
+                c->launches++;
+                t += n;
+            }
         }
         CU(cudaStreamSynchronize(c->cur));
         c->resident += db->bytes;
@@ -2462,7 +2470,7 @@ void ondemand_scores(fr_ctx* c, const BatchPlan& P, const u64* q, const std::vec
                 // up to 4 queries against the same diagonals (consecutive babies) share one launch
                 // that reads each diagonal word once for all of them: the persistent pipeline
                 // k_mac_ring where its tiling fits, else k_mac_pipe. A single query runs k_mac
-                // below (measured faster for one query: 0.98 ms against 1.13 ms at the headline)
+                // below
                 int cnt = 1;
                 if (d->tier != 4 && (mac_ring_fits(n1, ell, N, 2) || mac_pipe_fits(n1, ell, N)))
                     while (cnt < 4 && t + cnt < nb && sel[s0 + t + cnt] == b + cnt &&
@@ -2501,8 +2509,8 @@ void ondemand_scores(fr_ctx* c, const BatchPlan& P, const u64* q, const std::vec
                     continue;
                 }
                 Prof p(c, "mac", 8.0 * N * nlx * ((double)ell + 2.0 * n1 + 2.0 * n2));
-                launch_mac(babies.p + (size_t)b * n1 * bw, (long long)n1 * bw, nlx, diag_of(d),
-                           Pj.p + (size_t)t * n2 * bw, (long long)n2 * bw, nlx, nlx, n1, n2, ell, 1, mprimes, N, c->cur);
+                launch_mac(babies.p + (size_t)b * n1 * bw, nlx, diag_of(d), Pj.p + (size_t)t * n2 * bw, nlx, nlx, n1, n2,
+                           ell, mprimes, N, c->cur);
                 c->launches++;
             }
             if (!relin.empty()) {

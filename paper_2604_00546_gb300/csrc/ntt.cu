@@ -137,11 +137,8 @@ struct LastLo {
 // is exact for any 64-bit operand, so differences are lifted by 2q instead of reduced.
 struct EpiStore {};
 
-// Montgomery form of the transformed value, stored in place (template diagonals).
-struct EpiToMont {};
-
 template <class E>
-constexpr bool in_place = std::is_same<E, EpiStore>::value || std::is_same<E, EpiToMont>::value;
+constexpr bool in_place = std::is_same<E, EpiStore>::value;
 
 template <int W>
 struct EpiOps {
@@ -170,6 +167,21 @@ __device__ __forceinline__ void add_vec(u64 (&r)[W], const u64 (&a)[W], u64 q) {
     for (int w = 0; w < W; ++w) r[w] = add_mod(r[w], a[w], q);
 }
 
+// Template diagonals: Montgomery form as 30-bit halves into the database's tiles.
+struct EpiDiag {
+    u64* diags;
+    int d0, ell, nl, N;
+    template <int W>
+    __device__ __forceinline__ void load(EpiOps<W>&, int, int) const {}
+    template <int W>
+    __device__ __forceinline__ void put(const EpiOps<W>&, int p, int k, const u64 (&v)[W], const DevPrime& P) const {
+        u64 o[W];
+#pragma unroll
+        for (int w = 0; w < W; ++w) o[w] = split30(to_mont(v[w], P));
+        st_vec(diags + diag_word(p % nl, k, d0 + p / nl, ell, N), o);
+    }
+};
+
 // ModDown combine: poly p = (job, component t, limb i) of the P -> Q conversions; out =
 // (acc_Q - v) P^-1 (+ sigma_g(c0) for rotations, + the ct addend for relinearisation; a
 // rotation may add a ciphertext as well, as in x + Rot(x)).
@@ -192,7 +204,8 @@ struct EpiModDown {
         if (J.mode & 2) ld_vec(o.c, (J.mode == 3 ? J.add2 : J.add) + ((long long)t * J.add_cap + i) * N + k);
     }
     template <int W>
-    __device__ __forceinline__ void put(const EpiOps<W>& x, int p, int k, const u64 (&v)[W], u64 q) const {
+    __device__ __forceinline__ void put(const EpiOps<W>& x, int p, int k, const u64 (&v)[W], const DevPrime& P) const {
+        const u64 q = P.q;
         const int L1 = level + 1, N = 1 << logN;
         const int r = p % (2 * L1), t = r / L1, i = r % L1;
         const MDJob& J = jobs.j[p / (2 * L1)];
@@ -225,7 +238,8 @@ struct EpiRescale {
         if (mode == 1) ld_vec(o.b, add + (long long)(bt >> 1) * add_bs + ((long long)(bt & 1) * add_cap + i) * N + k);
     }
     template <int W>
-    __device__ __forceinline__ void put(const EpiOps<W>& o, int p, int k, const u64 (&v)[W], u64 q) const {
+    __device__ __forceinline__ void put(const EpiOps<W>& o, int p, int k, const u64 (&v)[W], const DevPrime& P) const {
+        const u64 q = P.q;
         const int bt = p / l, i = p % l;
         u64 r[W];
 #pragma unroll
@@ -266,7 +280,8 @@ struct EpiLeafRescale {
         ld_vec(o.a, x + (long long)b * x_bs + ((long long)t * x_cap + i) * N + k);
     }
     template <int W>
-    __device__ __forceinline__ void put(const EpiOps<W>& o, int p, int k, const u64 (&v)[W], u64 q) const {
+    __device__ __forceinline__ void put(const EpiOps<W>& o, int p, int k, const u64 (&v)[W], const DevPrime& P) const {
+        const u64 q = P.q;
         const int bjt = p / l, i = p % l, t = bjt & 1, j = (bjt >> 1) % nl;
         const u64 lift = 2 * q + (t == 0 ? ca[j * L1 + i] : 0);
         u64 r[W];
@@ -308,7 +323,8 @@ struct EpiRelinRescale {
         if (mode == 1) ld_vec(o.c, add + (long long)j * add_bs + ((long long)t * add_cap + i) * N + k);
     }
     template <int W>
-    __device__ __forceinline__ void put(const EpiOps<W>& o, int p, int k, const u64 (&v)[W], u64 q) const {
+    __device__ __forceinline__ void put(const EpiOps<W>& o, int p, int k, const u64 (&v)[W], const DevPrime& P) const {
+        const u64 q = P.q;
         const int jt = p / l, i = p % l, j = jt >> 1, t = jt & 1;
         u64 r[W];
 #pragma unroll
@@ -358,7 +374,7 @@ struct Ctx {
 // values below 2q. C2: the prime is of class 2 (classes 0 and 1 end alike).
 template <class E, bool C2>
 __device__ __forceinline__ u64 finish(u64 v, const DevPrime& P) {
-    if constexpr (std::is_same<E, EpiToMont>::value) return to_mont(v, P);
+    if constexpr (std::is_same<E, EpiDiag>::value) return v;  // to_mont takes any value
     const u64 f = C2 ? min(v, v - 2 * P.q) : fold_top(v, P.bsh, P.c);
     return std::is_same<E, EpiStore>::value ? min(f, f - P.q) : f;
 }
@@ -593,7 +609,7 @@ __device__ __forceinline__ void ntt_row_body(u64 (&v)[8], const uint4* tw, const
 // a thread's finished values at consecutive places of its row (element e at k + e) to where the
 // epilogue puts them
 template <class E>
-__device__ __forceinline__ void row_put(const u64 (&v)[8], u64* x, int p, int k, const E& epi, u64 q) {
+__device__ __forceinline__ void row_put(const u64 (&v)[8], u64* x, int p, int k, const E& epi, const DevPrime& P) {
     if constexpr (in_place<E>) {
 #pragma unroll
         for (int e = 0; e < 8; ++e) x[k + e] = v[e];
@@ -606,7 +622,7 @@ __device__ __forceinline__ void row_put(const u64 (&v)[8], u64* x, int p, int k,
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const u64 w[1] = {v[g + e]};
-                epi.put(o[e], p, k + g + e, w, q);
+                epi.put(o[e], p, k + g + e, w, P);
             }
         }
     }
@@ -643,7 +659,7 @@ __global__ void __launch_bounds__(RT, RT == 128 ? 9 : 4) k_ntt_row(const __grid_
         for (int e = 0; e < 8; ++e) x[Jbase + phase_x<3, LL>(tau, e)] = v[e];
     } else {
         static_assert(LL == 0, "the last forward phase holds the low bits");
-        row_put(v, x, p, Jbase + tau * 8, epi, P.q);
+        row_put(v, x, p, Jbase + tau * 8, epi, P);
     }
 }
 
@@ -701,7 +717,7 @@ __device__ __forceinline__ void ntt_cluster_body(const RingDev& R, u64* x, const
         phases<CLS, 3, LOG, false, false, 0>(v, taur, cr, exr, P);
 #pragma unroll
         for (int e = 0; e < 8; ++e) v[e] = finish<E, false>(v[e], P);
-        row_put(v, x, p, rho * S + taur * 8, epi, P.q);
+        row_put(v, x, p, rho * S + taur * 8, epi, P);
     } else {
 #pragma unroll
         for (int e = 0; e < 8; ++e) v[e] = xr[phase_x<3, L0>(taur, e)];
@@ -844,7 +860,7 @@ __global__ void __launch_bounds__(128, 6) k_ntt_row16(const __grid_constant__ Ri
                 u64 o[2];
                 ld_vec(o, ws + 2 * (ch ^ ((ch >> 3) & 7)));
                 if constexpr (in_place<E>) st_vec(x + Wbase + 2 * ch, o);
-                else epi.put(ops[j], p, Wbase + 2 * ch, o, P.q);
+                else epi.put(ops[j], p, Wbase + 2 * ch, o, P);
             }
         }
     }
@@ -1095,8 +1111,8 @@ void tune_ntt(RingDev& R, cudaStream_t s, double* us, int reps) {
     cudaStreamSynchronize(s);
 }
 
-void launch_ntt_tomont(const RingDev& R, const PolyBatch& b, cudaStream_t s) {
-    launch_ntt_e(R, b, false, s, EpiToMont{});
+void launch_ntt_diags(const RingDev& R, const PolyBatch& b, u64* diags, int d0, int ell, int nl, cudaStream_t s) {
+    launch_ntt_e(R, b, false, s, EpiDiag{diags, d0, ell, nl, R.N});
 }
 
 void launch_ntt_moddown(const RingDev& R, const PolyBatch& b, const MDJobs& jobs, int npos, int level,
