@@ -118,89 +118,110 @@ __global__ void __launch_bounds__(kBcThreads) k_modup(const u64* __restrict__ in
 // the canonical residue. The automorphism is a gather on the ext index. When
 // all jobs of a launch use the same key (batched relinearisation), a thread
 // reads its key words once and applies them to every job.
+// A thread takes two consecutive points (16-byte loads, twice the bytes in flight of one: the
+// kernel is bound by HBM latency). The automorphism keeps aligned pairs together: position k's
+// source is src(k), and src(k + 1) = src(k) ^ 1 for even k, because the low bits of a position are
+// the high bits of the exponent 2 brev(k) + 1, which an odd factor permutes among themselves. So a
+// gathered pair is one aligned load, its halves swapped when src(k) is odd.
+// Measured at the headline size: baby steps (31 keys, 3 digits, 13 positions, 1.73 GB) 343 us with
+// one point a thread.
 // ---------------------------------------------------------------------------
+constexpr int kIpThreads = 128;
+
+struct U64x2 {
+    u64 v[2];
+};
+__device__ __forceinline__ U64x2 ld2(const u64* p) {
+    const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(p);
+    return U64x2{{t.x, t.y}};
+}
+// the pair gathered for the even position whose source is src
+__device__ __forceinline__ U64x2 ld2_from(const u64* p, u32 src) {
+    const U64x2 t = ld2(p + (src & ~1u));
+    return (src & 1) ? U64x2{{t.v[1], t.v[0]}} : t;
+}
+__device__ __forceinline__ void st2(u64* p, u64 a, u64 b) { *reinterpret_cast<ulonglong2*>(p) = make_ulonglong2(a, b); }
+
 // digit d's extension at position pos: its own limb of the switched polynomial, or ext
 __device__ __forceinline__ const u64* ip_ext(const IPJob& J, int d, int npos, int pos, int owner, int N) {
     return d == owner ? J.own + (long long)pos * N : J.ext + ((long long)d * npos + pos) * N;
 }
 
-template <int BETA>
-__device__ __forceinline__ void ip_job(const IPJob& J, int owner, const u64 (&k0)[BETA], const u64 (&k1)[BETA], int npos, int pos,
-                                       int k, u64 q, u64 qinv, int logN, int N, int level, const u64* pmod,
-                                       const u64* pmod_s) {
-    const u32 src = J.galois != 1u ? galois_src_index((u32)k, J.galois, logN) : (u32)k;
-    Acc128 a0{0, 0}, a1{0, 0};
-#pragma unroll
-    for (int d = 0; d < BETA; ++d) {
-        const u64 e = ip_ext(J, d, npos, pos, owner, N)[src];
-        mac128(a0, e, k0[d]);
-        mac128(a1, e, k1[d]);
-        if ((d & 7) == 7) { fold(a0, q); fold(a1, q); }
-    }
-    fold(a0, q);
-    fold(a1, q);
-    u64 r0 = redc(a0.hi, a0.lo, q, qinv);
-    if (J.addb && pos <= level)  // a rotation kept in Q_l u P: + P sigma(b) on the Q positions
-        r0 = add_mod(r0, mul_shoup(J.addb[(long long)pos * N + src], pmod[pos], pmod_s[pos], q), q);
-    J.out[(long long)pos * N + k] = r0;
-    J.out[((long long)npos + pos) * N + k] = redc(a1.hi, a1.lo, q, qinv);
-}
-
-template <int BETA>
-__device__ __forceinline__ void ip_body(const IPJobs& jobs, int npos, int pos, int klimb, int T, int k, u64 q,
-                                        u64 qinv, int logN, int N, int level, const u64* pmod, const u64* pmod_s) {
-    // one key group per blockIdx.y: its key words are read once and applied to every job of the group
-    const int g = blockIdx.y;
-    const u64* key = jobs.gkey[g];
-    u64 k0[BETA], k1[BETA];
-#pragma unroll
-    for (int d = 0; d < BETA; ++d) {
-        k0[d] = key[(((long long)d * 2 + 0) * T + klimb) * N + k];
-        k1[d] = key[(((long long)d * 2 + 1) * T + klimb) * N + k];
-    }
-    for (int j = jobs.gstart[g]; j < jobs.gstart[g + 1]; ++j)
-        ip_job<BETA>(jobs.j[j], jobs.owner[pos], k0, k1, npos, pos, k, q, qinv, logN, N, level, pmod, pmod_s);
-}
-
 // key layout [digit][2][T][N]: Q limbs at positions 0.., P limbs from position kp. One
-// instantiation per digit count, so the registers a launch needs follow its beta.
+// instantiation per digit count, so the registers a launch needs follow its beta. One key group
+// per blockIdx.y: its key words are read once and applied to every job of the group.
 template <int BETA>
-__global__ void __launch_bounds__(kThreads) k_ip(const __grid_constant__ IPJobs jobs, int npos, int level, int kp,
-                                                 int T, const DevPrime* __restrict__ primes, int pbase, int logN,
-                                                 const u64* __restrict__ pmod, const u64* __restrict__ pmod_s) {
+__global__ void __launch_bounds__(kIpThreads) k_ip(const __grid_constant__ IPJobs jobs, int npos, int level, int kp,
+                                                   int T, const DevPrime* __restrict__ primes, int pbase, int logN,
+                                                   const u64* __restrict__ pmod, const u64* __restrict__ pmod_s) {
     pdl_wait();
     pdl_trigger();
     const int N = 1 << logN;
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    const int k = (blockIdx.x * kIpThreads + threadIdx.x) * 2;
     // position-major grid: the key groups of one position run back to back, so a ModUp
     // extension that several groups gather from (hoisted rotations) is read from L2
-    const int pos = blockIdx.z;
+    const int pos = blockIdx.z, g = blockIdx.y;
     if (k >= N) return;
     // positions 0..level are Q limbs 0..level; the P limbs follow (prime indices from pbase)
     const int pi = pos <= level ? pos : pbase + (pos - (level + 1));
     const u64 q = primes[pi].q, qinv = primes[pi].qinv;
     const int klimb = pos <= level ? pos : kp + (pos - (level + 1));
-    ip_body<BETA>(jobs, npos, pos, klimb, T, k, q, qinv, logN, N, level, pmod, pmod_s);
+    const int owner = jobs.owner[pos];
+    const u64* key = jobs.gkey[g] + (long long)klimb * N + k;
+    U64x2 k0[BETA], k1[BETA];
+#pragma unroll
+    for (int d = 0; d < BETA; ++d) {
+        k0[d] = ld2(key + (long long)(2 * d) * T * N);
+        k1[d] = ld2(key + (long long)(2 * d + 1) * T * N);
+    }
+    for (int jj = jobs.gstart[g]; jj < jobs.gstart[g + 1]; ++jj) {
+        const IPJob& J = jobs.j[jj];
+        const u32 src = J.galois != 1u ? galois_src_index((u32)k, J.galois, logN) : (u32)k;
+        U64x2 e[BETA], badd{{0, 0}};
+#pragma unroll
+        for (int d = 0; d < BETA; ++d) e[d] = ld2_from(ip_ext(J, d, npos, pos, owner, N), src);
+        const bool addb = J.addb && pos <= level;  // a rotation kept in Q_l u P: + P sigma(b) on the Q positions
+        if (addb) badd = ld2_from(J.addb + (long long)pos * N, src);
+        u64 r0[2], r1[2];
+#pragma unroll
+        for (int w = 0; w < 2; ++w) {
+            Acc128 a0{0, 0}, a1{0, 0};
+#pragma unroll
+            for (int d = 0; d < BETA; ++d) {
+                mac_full(a0, e[d].v[w], k0[d].v[w]);
+                mac_full(a1, e[d].v[w], k1[d].v[w]);
+            }
+            fold(a0, q);
+            fold(a1, q);
+            r0[w] = redc(a0.hi, a0.lo, q, qinv);
+            if (addb) r0[w] = add_mod(r0[w], mul_shoup(badd.v[w], pmod[pos], pmod_s[pos], q), q);
+            r1[w] = redc(a1.hi, a1.lo, q, qinv);
+        }
+        st2(J.out + (long long)pos * N + k, r0[0], r0[1]);
+        st2(J.out + ((long long)npos + pos) * N + k, r1[0], r1[1]);
+    }
 }
 
 // Inner products summed into their accumulator (double-hoisted sums of rotations): thread
-// (point k, group g, position pos) runs the jobs of group g, each a key-switch inner product
-// of its ext under its automorphism (the same products as ip_job), in one 128-bit sum per
+// (points k, k + 1, group g, position pos) runs the jobs of group g, each a key-switch inner product
+// of its ext under its automorphism (the same products as k_ip), in one 128-bit sum per
 // component, folded after every job: a product of two residues below q < 2^61 adds less than
 // q/8 to the high word, so a job's beta <= 8 products leave it below 2q before the fold. Then
 // it adds P sigma_j(addb_j) on the Q positions of component 0 and the value already in the
-// accumulator. The grid is (points, groups, positions), groups fastest after the points:
+// accumulator. The words of U jobs are loaded together: the jobs' keys come from HBM one after the
+// other otherwise. The grid is (points, groups, positions), groups fastest after the points:
 // the key words of one position, which every group's job with that key reads, are L2 hits
 // after the first group.
 template <int BETA>
-__global__ void __launch_bounds__(kThreads) k_ip_sum(const __grid_constant__ IPSumJobs jobs, int npos, int level,
-                                                     int kp, int T, const DevPrime* __restrict__ primes, int pbase,
-                                                     int logN, const u64* __restrict__ pmod,
-                                                     const u64* __restrict__ pmod_s) {
+__global__ void __launch_bounds__(kIpThreads) k_ip_sum(const __grid_constant__ IPSumJobs jobs, int npos, int level,
+                                                       int kp, int T, const DevPrime* __restrict__ primes, int pbase,
+                                                       int logN, const u64* __restrict__ pmod,
+                                                       const u64* __restrict__ pmod_s) {
     pdl_wait();
     pdl_trigger();
+    constexpr int U = BETA == 1 ? 4 : BETA == 2 ? 2 : 1;
     const int N = 1 << logN;
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    const int k = (blockIdx.x * kIpThreads + threadIdx.x) * 2;
     const int g = blockIdx.y;
     const int pos = blockIdx.z;
     if (k >= N) return;
@@ -208,26 +229,52 @@ __global__ void __launch_bounds__(kThreads) k_ip_sum(const __grid_constant__ IPS
     const u64 q = primes[pi].q, qinv = primes[pi].qinv;
     const int klimb = pos <= level ? pos : kp + (pos - (level + 1));
     const int owner = jobs.owner[pos];
-    Acc128 a0{0, 0}, a1{0, 0};
-    u64 badd = 0;
-    for (int jj = jobs.gstart[g]; jj < jobs.gstart[g + 1]; ++jj) {
-        const IPJob& J = jobs.j[jj];
-        const u32 src = J.galois != 1u ? galois_src_index((u32)k, J.galois, logN) : (u32)k;
+    Acc128 a0[2] = {}, a1[2] = {};
+    u64 badd[2] = {0, 0};
+    const int end = jobs.gstart[g + 1];
+    for (int j0 = jobs.gstart[g]; j0 < end; j0 += U) {
+        U64x2 e[U][BETA], k0[U][BETA], k1[U][BETA], bb[U];
 #pragma unroll
-        for (int d = 0; d < BETA; ++d) {
-            const u64 e = ip_ext(J, d, npos, pos, owner, N)[src];
-            mac128(a0, e, J.key[(((long long)d * 2 + 0) * T + klimb) * N + k]);
-            mac128(a1, e, J.key[(((long long)d * 2 + 1) * T + klimb) * N + k]);
+        for (int u = 0; u < U; ++u) {
+            const IPJob& J = jobs.j[min(j0 + u, end - 1)];
+            const u32 src = J.galois != 1u ? galois_src_index((u32)k, J.galois, logN) : (u32)k;
+            const u64* key = J.key + (long long)klimb * N + k;
+#pragma unroll
+            for (int d = 0; d < BETA; ++d) {
+                e[u][d] = ld2_from(ip_ext(J, d, npos, pos, owner, N), src);
+                k0[u][d] = ld2(key + (long long)(2 * d) * T * N);
+                k1[u][d] = ld2(key + (long long)(2 * d + 1) * T * N);
+            }
+            if (J.addb && pos <= level) bb[u] = ld2_from(J.addb + (long long)pos * N, src);
         }
-        fold(a0, q);
-        fold(a1, q);
-        if (J.addb && pos <= level)
-            badd = add_mod(badd, mul_shoup(J.addb[(long long)pos * N + src], pmod[pos], pmod_s[pos], q), q);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (j0 + u >= end) break;
+            const bool addb = jobs.j[j0 + u].addb && pos <= level;
+#pragma unroll
+            for (int w = 0; w < 2; ++w) {
+#pragma unroll
+                for (int d = 0; d < BETA; ++d) {
+                    mac_full(a0[w], e[u][d].v[w], k0[u][d].v[w]);
+                    mac_full(a1[w], e[u][d].v[w], k1[u][d].v[w]);
+                }
+                fold(a0[w], q);
+                fold(a1[w], q);
+                if (addb) badd[w] = add_mod(badd[w], mul_shoup(bb[u].v[w], pmod[pos], pmod_s[pos], q), q);
+            }
+        }
     }
-    u64* O = jobs.j[jobs.gstart[g]].out;
-    const long long o0 = (long long)pos * N + k, o1 = ((long long)npos + pos) * N + k;
-    O[o0] = add_mod(O[o0], add_mod(redc(a0.hi, a0.lo, q, qinv), badd, q), q);
-    O[o1] = add_mod(O[o1], redc(a1.hi, a1.lo, q, qinv), q);
+    u64* O0 = jobs.j[jobs.gstart[g]].out + (long long)pos * N + k;
+    u64* O1 = O0 + (long long)npos * N;
+    const U64x2 o0 = ld2(O0), o1 = ld2(O1);
+    u64 r0[2], r1[2];
+#pragma unroll
+    for (int w = 0; w < 2; ++w) {
+        r0[w] = add_mod(o0.v[w], add_mod(redc(a0[w].hi, a0[w].lo, q, qinv), badd[w], q), q);
+        r1[w] = add_mod(o1.v[w], redc(a1[w].hi, a1[w].lo, q, qinv), q);
+    }
+    st2(O0, r0[0], r0[1]);
+    st2(O1, r1[0], r1[1]);
 }
 
 // ---------------------------------------------------------------------------
@@ -336,22 +383,27 @@ __global__ void __launch_bounds__(kBcThreads) k_p2q_lift(const u64* __restrict__
 // Rescale. lift: centered last limb (coefficient form) to each q_i, i < l.
 // last: [B][2][N] ; lifted: [B][2][l][N]
 // ---------------------------------------------------------------------------
+// the centered lift of x < q_l (x, or x - q_l above half) mod q_i: x plus -q_l mod q_i, reduced once
+__device__ __forceinline__ u64 centered_residue(u64 x, const RescaleTab& tab, const DevPrime& P, int i) {
+    const u64 v = x + (x > tab.half ? P.q - tab.ql_mod[i] : 0);  // below 2^62
+    if (P.fold63) {
+        const u64 f = fold_top(v, P.bsh, P.c);
+        return min(f, f - P.q);
+    }
+    return mul_shoup(v, 1, P.one_s, P.q);
+}
+
 __global__ void __launch_bounds__(kThreads) k_rescale_lift(const u64* __restrict__ last, u64* __restrict__ lifted,
-                                                           const RescaleTab* __restrict__ tab, int l, int N) {
+                                                           const RescaleTab* __restrict__ tab,
+                                                           const DevPrime* __restrict__ primes, int l, int N) {
     pdl_wait();
     pdl_trigger();
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     const int bt = blockIdx.y;
     if (k >= N) return;
     const u64 x = last[(long long)bt * N + k];
-    const bool neg = x > tab->half;
-    u64* o = lifted + (long long)bt * l * N;
-    for (int i = 0; i < l; ++i) {
-        const u64 q = tab->q[i];
-        u64 r = mul_shoup(x, 1, tab->one_s[i], q);  // x mod q
-        if (neg) r = sub_mod(r, tab->ql_mod[i], q);
-        o[(long long)i * N + k] = r;
-    }
+    u64* o = lifted + (long long)bt * l * N + k;
+    for (int i = 0; i < l; ++i) o[(long long)i * N] = centered_residue(x, *tab, primes[i], i);
 }
 
 // Baby steps kept in Q_l u P (double hoisting of the baby steps): baby 0 of query b is P q_b on
@@ -394,23 +446,6 @@ __global__ void __launch_bounds__(kThreads) k_rs_last(const u64* __restrict__ ac
     const u64 a = acc[((long long)jt * npos + l) * N + k];
     const u64 dd = d ? d[(((long long)j * 3 + t) * (l + 1) + l) * N + k] : 0;
     z[(long long)jt * N + k] = add_mod(mul_shoup(a, pinv[l], pinv_s[l], q), dd, q);
-}
-
-// out[b][t][i] = (x[b][t][i] - lifted[b][t][i]) * q_l^-1
-__global__ void __launch_bounds__(kThreads) k_rescale_combine(const u64* __restrict__ x, int x_cap,
-                                                              const u64* __restrict__ lifted, u64* __restrict__ out,
-                                                              int out_cap, const RescaleTab* __restrict__ tab, int l,
-                                                              int N) {
-    pdl_wait();
-    pdl_trigger();
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    const int i = blockIdx.y % l;
-    const int bt = blockIdx.y / l;
-    if (k >= N) return;
-    const u64 q = tab->q[i];
-    const u64 a = x[((long long)bt * x_cap + i) * N + k];
-    const u64 c = lifted[((long long)bt * l + i) * N + k];
-    out[((long long)bt * out_cap + i) * N + k] = mul_shoup(sub_mod(a, c, q), tab->qlinv[i], tab->qlinv_s[i], q);
 }
 
 // ---------------------------------------------------------------------------
@@ -1033,25 +1068,20 @@ __global__ void k_sum(const u64* a, int cap, long long js, int J, u64* out, int 
 // lifted [B nl][2][l][N]; grid (N / 256, 2 nl, B).
 __global__ void k_leaf_lift(const u64* __restrict__ u, const u64* __restrict__ cb, const u64* __restrict__ cb_s,
                             const u64* __restrict__ ca, int nl, int L1, u64* __restrict__ lifted,
-                            const RescaleTab* __restrict__ tab, u64 ql, int l, int N) {
+                            const RescaleTab* __restrict__ tab, const DevPrime* __restrict__ primes, int l, int N) {
     pdl_wait();
     pdl_trigger();
+    const u64 ql = primes[l].q;
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y >> 1, t = blockIdx.y & 1, b = blockIdx.z;
     if (k >= N) return;
     u64 r = mul_shoup(u[((long long)b * 2 + t) * N + k], cb[j * L1 + l], cb_s[j * L1 + l], ql);
     if (t == 0 && k == 0) r = add_mod(r, ca[j * L1 + l], ql);
-    const bool neg = r > tab->half;
     u64* o = lifted + ((((long long)b * nl + j) * 2 + t) * l) * N + k;
-    for (int i = 0; i < l; ++i) {
-        const u64 q = tab->q[i];
-        u64 w = mul_shoup(r, 1, tab->one_s[i], q);
-        if (neg) w = sub_mod(w, tab->ql_mod[i], q);
-        o[(long long)i * N] = w;
-    }
+    for (int i = 0; i < l; ++i) o[(long long)i * N] = centered_residue(r, *tab, primes[i], i);
 }
 
-// x <- 2 x - c (c added to the constant term: every evaluation point of c0)
+// x to Montgomery form (evaluation keys)
 __global__ void k_to_mont(u64* x, long long n_per_poly, PrimeMap pm, const DevPrime* primes, long long total) {
     pdl_wait();
     pdl_trigger();
@@ -1176,6 +1206,20 @@ __global__ void __launch_bounds__(256) k_fft_row(cplx* z, int logn, int logR, in
     for (int e = threadIdx.x; e < tile; e += blockDim.x) x[e] = sc[e];
 }
 
+// v 2^shift rounded half away from zero. Both factors of the encoder (1/n and Delta) are powers
+// of two, so the product is exact and the rounding is a shift of the mantissa: GB300 has two FP64
+// lanes an SM partition, and two multiplications and llround per coefficient cost more than the
+// rest of the kernel. Values that do not fit go through the FP64 form.
+__device__ __forceinline__ long long scale_round(double v, int shift) {
+    const u64 b = (u64)__double_as_longlong(v);
+    const int ex = (int)(b >> 52) & 0x7ff, s = ex - 1075 + shift;  // |v| = m 2^(ex - 1075)
+    if (ex == 0x7ff || s > 9) return llround(ldexp(v, shift));
+    if (ex == 0 || s < -63) return 0;
+    const u64 m = (b & 0xfffffffffffffull) | (1ull << 52);
+    const u64 r = s >= 0 ? m << s : (m + (1ull << (-s - 1))) >> -s;
+    return (b >> 63) ? -(long long)r : (long long)r;
+}
+
 // coefficient c of the encoded diagonal di: bit reversal, times 1/n and Delta, rounded half
 // away from zero
 __device__ __forceinline__ long long fft_coef(const cplx* __restrict__ z, int logn, int di, int c, int scale_bits) {
@@ -1183,10 +1227,7 @@ __device__ __forceinline__ long long fft_coef(const cplx* __restrict__ z, int lo
     const int cc = c < n ? c : c - n;
     const int src = __brev(cc) >> (32 - logn);
     const cplx w = z[(long long)di * n + src];
-    const double v = c < n ? w.r : w.i;
-    const double inv_n = 1.0 / (double)n;
-    const double delta = ldexp(1.0, scale_bits);
-    return llround(__dmul_rn(__dmul_rn(v, inv_n), delta));
+    return scale_round(c < n ? w.r : w.i, scale_bits - logn);
 }
 
 // m mod q for a signed coefficient: |m| < 2^63 reduced by its bits from bits(q) up where that is
@@ -1268,14 +1309,14 @@ void launch_modup(const u64* in, long long in_job, u64* ext, const ModUpTab* tab
 void launch_ip(const IPJobs& jobs, int beta, int npos, int level, int kp, int T, const DevPrime* primes,
                const PrimeMap& pos_prime, int logN, cudaStream_t s, const u64* pmod, const u64* pmod_s) {
     const int N = 1 << logN;
-    dim3 g((N + kThreads - 1) / kThreads, jobs.ngroups, npos);
+    dim3 g((N / 2 + kIpThreads - 1) / kIpThreads, jobs.ngroups, npos);
     const int pbase = npos > level + 1 ? pos_prime.idx[level + 1] : 0;
     switch (beta) {
 #define FR_IP_CASE(B) \
-    case B: launch_k(k_ip<B>, g, dim3(kThreads), 0, s, jobs, npos, level, kp, T, primes, pbase, logN, pmod, pmod_s); \
+    case B: launch_k(k_ip<B>, g, dim3(kIpThreads), 0, s, jobs, npos, level, kp, T, primes, pbase, logN, pmod, pmod_s); \
         break;
         FR_IP_CASE(1) FR_IP_CASE(2) FR_IP_CASE(3) FR_IP_CASE(4) FR_IP_CASE(5) FR_IP_CASE(6) FR_IP_CASE(7)
-        default: launch_k(k_ip<8>, g, dim3(kThreads), 0, s, jobs, npos, level, kp, T, primes, pbase, logN, pmod, pmod_s);
+        default: launch_k(k_ip<8>, g, dim3(kIpThreads), 0, s, jobs, npos, level, kp, T, primes, pbase, logN, pmod, pmod_s);
             break;
 #undef FR_IP_CASE
     }
@@ -1284,14 +1325,14 @@ void launch_ip(const IPJobs& jobs, int beta, int npos, int level, int kp, int T,
 void launch_ip_sum(const IPSumJobs& jobs, int beta, int npos, int level, int kp, int T, const DevPrime* primes,
                    const PrimeMap& pos_prime, int logN, const u64* pmod, const u64* pmod_s, cudaStream_t s) {
     const int N = 1 << logN;
-    dim3 g((N + kThreads - 1) / kThreads, jobs.ngroups, npos);
+    dim3 g((N / 2 + kIpThreads - 1) / kIpThreads, jobs.ngroups, npos);
     const int pbase = npos > level + 1 ? pos_prime.idx[level + 1] : 0;
     switch (beta) {
 #define FR_IPS_CASE(B) \
-    case B: launch_k(k_ip_sum<B>, g, dim3(kThreads), 0, s, jobs, npos, level, kp, T, primes, pbase, logN, pmod, pmod_s); \
+    case B: launch_k(k_ip_sum<B>, g, dim3(kIpThreads), 0, s, jobs, npos, level, kp, T, primes, pbase, logN, pmod, pmod_s); \
         break;
         FR_IPS_CASE(1) FR_IPS_CASE(2) FR_IPS_CASE(3) FR_IPS_CASE(4) FR_IPS_CASE(5) FR_IPS_CASE(6) FR_IPS_CASE(7)
-        default: launch_k(k_ip_sum<8>, g, dim3(kThreads), 0, s, jobs, npos, level, kp, T, primes, pbase, logN, pmod,
+        default: launch_k(k_ip_sum<8>, g, dim3(kIpThreads), 0, s, jobs, npos, level, kp, T, primes, pbase, logN, pmod,
                           pmod_s);
             break;
 #undef FR_IPS_CASE
@@ -1322,15 +1363,10 @@ void launch_rs_last(const u64* acc, const u64* d, u64* z, const u64* pinv, const
     launch_k(k_rs_last, g, dim3(kThreads), 0, s, acc, d, z, pinv, pinv_s, npos, l, primes, N);
 }
 
-void launch_rescale_lift(const u64* last, u64* lifted, const RescaleTab* tab, int l, int N, int BT, cudaStream_t s) {
+void launch_rescale_lift(const u64* last, u64* lifted, const RescaleTab* tab, const DevPrime* primes, int l, int N,
+                         int BT, cudaStream_t s) {
     dim3 g((N + kThreads - 1) / kThreads, BT);
-    launch_k(k_rescale_lift, dim3(g), dim3(kThreads), 0, s, last, lifted, tab, l, N);
-}
-
-void launch_rescale_combine(const u64* x, int x_cap, const u64* lifted, u64* out, int out_cap, const RescaleTab* tab,
-                            int l, int N, int BT, cudaStream_t s) {
-    dim3 g((N + kThreads - 1) / kThreads, BT * l);
-    launch_k(k_rescale_combine, dim3(g), dim3(kThreads), 0, s, x, x_cap, lifted, out, out_cap, tab, l, N);
+    launch_k(k_rescale_lift, dim3(g), dim3(kThreads), 0, s, last, lifted, tab, primes, l, N);
 }
 
 void launch_tensor(const TensorJobs& jobs, int J, int level, const DevPrime* primes, int N, cudaStream_t s) {
@@ -1487,9 +1523,9 @@ void launch_sum(const u64* a, int cap, long long js, int J, u64* out, int o_cap,
 }
 
 void launch_leaf_lift(const u64* u, const u64* cb, const u64* cb_s, const u64* ca, int nl, int L1, u64* lifted,
-                      const RescaleTab* tab, u64 ql, int l, int N, int B, cudaStream_t s) {
+                      const RescaleTab* tab, const DevPrime* primes, int l, int N, int B, cudaStream_t s) {
     dim3 g((N + kThreads - 1) / kThreads, 2 * nl, B);
-    launch_k(k_leaf_lift, dim3(g), dim3(kThreads), 0, s, u, cb, cb_s, ca, nl, L1, lifted, tab, ql, l, N);
+    launch_k(k_leaf_lift, dim3(g), dim3(kThreads), 0, s, u, cb, cb_s, ca, nl, L1, lifted, tab, primes, l, N);
 }
 
 void launch_to_mont(u64* x, long long n_per_poly, const PrimeMap& pm, const DevPrime* primes, long long total,

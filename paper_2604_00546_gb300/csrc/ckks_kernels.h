@@ -123,7 +123,7 @@ void launch_ntt_moddown(const RingDev& R, const PolyBatch& b, const MDJobs& jobs
 // (b: poly ((b nl + j) 2 + t) l + i) and writes leaf (b, j) at out + (b nl + j) 2 out_cap N.
 // T1 of query b at x + b x_bs (cap x_cap); constants [nl][L1] each.
 void launch_leaf_lift(const u64* u, const u64* cb, const u64* cb_s, const u64* ca, int nl, int L1, u64* lifted,
-                      const RescaleTab* tab, u64 ql, int l, int N, int B, cudaStream_t s);
+                      const RescaleTab* tab, const DevPrime* primes, int l, int N, int B, cudaStream_t s);
 void launch_ntt_leaf_rescale(const RingDev& R, const PolyBatch& b, const u64* x, long long x_bs, int x_cap,
                              const u64* cb, const u64* cb_s, const u64* ca, int nl, int L1, u64* out, int out_cap,
                              const RescaleTab* tab, int l, cudaStream_t s);
@@ -160,9 +160,8 @@ void launch_ip(const IPJobs& jobs, int beta, int npos, int level, int kp, int T,
 // ModDown conversions of the P limbs (coefficient form, times inv_hat) of J accumulators
 void launch_p2q(const u64* acc, long long acc_job, int npos, int level, u64* conv, const P2QTab* tab, int N, int J,
                 cudaStream_t s);
-void launch_rescale_lift(const u64* last, u64* lifted, const RescaleTab* tab, int l, int N, int BT, cudaStream_t s);
-void launch_rescale_combine(const u64* x, int x_cap, const u64* lifted, u64* out, int out_cap, const RescaleTab* tab,
-                            int l, int N, int BT, cudaStream_t s);
+void launch_rescale_lift(const u64* last, u64* lifted, const RescaleTab* tab, const DevPrime* primes, int l, int N,
+                         int BT, cudaStream_t s);
 void launch_tensor(const TensorJobs& jobs, int J, int level, const DevPrime* primes, int N, cudaStream_t s);
 // Sums of rotations with one ModDown (double hoisting), without the per-job inner products in
 // memory: for each group g and position,

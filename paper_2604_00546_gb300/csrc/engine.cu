@@ -629,7 +629,7 @@ void rescale(fr_ctx* c, const u64* in, int B, int level, int in_cap, u64* out, i
     Tmp lifted(c, (size_t)2 * B * l * N);
     {
         Prof p(c, "rescale", 8.0 * N * 2 * B * (1.0 + l));
-        launch_rescale_lift(last.p, lifted.p, c->d_rescale[l], l, N, 2 * B, c->cur);
+        launch_rescale_lift(last.p, lifted.p, c->d_rescale[l], c->d_primes, l, N, 2 * B, c->cur);
         c->launches++;
     }
     // forward NTT of the lifted limb with the combine as its epilogue
@@ -658,7 +658,7 @@ void leaves_rescaled(fr_ctx* c, const u64* x, int B, int x_cap, int l, int nl, c
     Tmp lifted(c, (size_t)B * nl * 2 * l * N);
     {
         Prof p(c, "rescale", 8.0 * N * B * 2.0 * (1.0 + (double)nl * l));
-        launch_leaf_lift(u.p, cb, cb_s, ca, nl, L1, lifted.p, c->d_rescale[l], c->R.primes[l], l, N, B, c->cur);
+        launch_leaf_lift(u.p, cb, cb_s, ca, nl, L1, lifted.p, c->d_rescale[l], c->d_primes, l, N, B, c->cur);
         c->launches++;
     }
     Prof p(c, "ntt", 16.0 * B * nl * 2 * l * N);
