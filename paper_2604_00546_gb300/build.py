@@ -16,7 +16,7 @@ CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "libfr.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-CU_SOURCES = ["ntt.cu", "ckks_kernels.cu", "engine.cu"]
+CU_SOURCES = ["ntt.cu", "ntt_small.cu", "ckks_kernels.cu", "engine.cu"]
 CXX_SOURCES = ["host_ring.cpp"]
 
 

@@ -3624,7 +3624,7 @@ extern "C" fr_status fr_rotate_noalloc(fr_ctx* c, const uint64_t* d_in, uint32_t
         MDJobs md;
         md.j[0] = MDJob{acc, e, res, l + 1, l + 1, 1, (u32)g};
         PolyBatch pc{conv, (long long)L1N, l + 1, 2 * (l + 1), pl};
-        pc.conv = ConvSrc{c->d_p2q->t, 0, acc + L1N, (long long)npos * N, np};
+        p2q_into(c, acc, 1, l, pc);
         launch_ntt_moddown(c->rd, pc, md, npos, l, c->d_pinv, c->d_pinv_s, st);
         PolyBatch out{d_out, 2 * (long long)L1N, 2 * (l + 1), 2 * (l + 1), pl};
         out.src = res;
