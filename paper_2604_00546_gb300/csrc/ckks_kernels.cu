@@ -207,8 +207,8 @@ __global__ void __launch_bounds__(kIpThreads) k_ip(const __grid_constant__ IPJob
 // of its ext under its automorphism (the same products as k_ip), in one 128-bit sum per
 // component, folded after every job: a product of two residues below q < 2^61 adds less than
 // q/8 to the high word, so a job's beta <= 8 products leave it below 2q before the fold. Then
-// it adds P sigma_j(addb_j) on the Q positions of component 0 and the value already in the
-// accumulator. The words of U jobs are loaded together: the jobs' keys come from HBM one after the
+// it adds P sum_j sigma_j(addb_j) on the Q positions of component 0 (one product by P for all
+// jobs) and, where an earlier launch started the sum (add), the value already in the accumulator. The words of U jobs are loaded together: the jobs' keys come from HBM one after the
 // other otherwise. The grid is (points, groups, positions), groups fastest after the points:
 // the key words of one position, which every group's job with that key reads, are L2 hits
 // after the first group.
@@ -260,17 +260,22 @@ __global__ void __launch_bounds__(kIpThreads) k_ip_sum(const __grid_constant__ I
                 }
                 fold(a0[w], q);
                 fold(a1[w], q);
-                if (addb) badd[w] = add_mod(badd[w], mul_shoup(bb[u].v[w], pmod[pos], pmod_s[pos], q), q);
+                if (addb) badd[w] = add_mod(badd[w], bb[u].v[w], q);
             }
         }
     }
     u64* O0 = jobs.j[jobs.gstart[g]].out + (long long)pos * N + k;
     u64* O1 = O0 + (long long)npos * N;
-    const U64x2 o0 = ld2(O0), o1 = ld2(O1);
+    U64x2 o0{{0, 0}}, o1{{0, 0}};
+    if (jobs.add[g]) {
+        o0 = ld2(O0);
+        o1 = ld2(O1);
+    }
     u64 r0[2], r1[2];
 #pragma unroll
     for (int w = 0; w < 2; ++w) {
-        r0[w] = add_mod(o0.v[w], add_mod(redc(a0[w].hi, a0[w].lo, q, qinv), badd[w], q), q);
+        const u64 pb = pos <= level ? mul_shoup(badd[w], pmod[pos], pmod_s[pos], q) : 0;
+        r0[w] = add_mod(o0.v[w], add_mod(redc(a0[w].hi, a0[w].lo, q, qinv), pb, q), q);
         r1[w] = add_mod(o1.v[w], redc(a1[w].hi, a1[w].lo, q, qinv), q);
     }
     st2(O0, r0[0], r0[1]);
@@ -428,24 +433,6 @@ __global__ void __launch_bounds__(kThreads) k_baby0_pq(u64* __restrict__ babies,
     }
     const u64 qp = primes[pos].q;
     *o = mul_shoup(q[(long long)b * q_bs + ((long long)t * q_cap + pos) * N + k], pmod[pos], pmod_s[pos], qp);
-}
-
-// Relinearisation + rescale, last limb: z = acc_l P^-1 + d_l (evaluation form), the last limb
-// of the relinearised product before the rescale. acc [J][2][npos][N], d [J][3][l+1][N] or
-// null (a ModDown with no addend), z [J][2][N].
-__global__ void __launch_bounds__(kThreads) k_rs_last(const u64* __restrict__ acc, const u64* __restrict__ d,
-                                                      u64* __restrict__ z, const u64* __restrict__ pinv,
-                                                      const u64* __restrict__ pinv_s, int npos, int l,
-                                                      const DevPrime* __restrict__ primes, int N) {
-    pdl_wait();
-    pdl_trigger();
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    const int jt = blockIdx.y, j = jt >> 1, t = jt & 1;
-    if (k >= N) return;
-    const u64 q = primes[l].q;
-    const u64 a = acc[((long long)jt * npos + l) * N + k];
-    const u64 dd = d ? d[(((long long)j * 3 + t) * (l + 1) + l) * N + k] : 0;
-    z[(long long)jt * N + k] = add_mod(mul_shoup(a, pinv[l], pinv_s[l], q), dd, q);
 }
 
 // ---------------------------------------------------------------------------
@@ -1355,12 +1342,6 @@ void launch_baby0_pq(u64* babies, long long baby_q, const u64* q, long long q_bs
                      int level, const DevPrime* primes, const u64* pmod, const u64* pmod_s, int N, cudaStream_t s) {
     dim3 g((N + kThreads - 1) / kThreads, npos, 2 * B);
     launch_k(k_baby0_pq, g, dim3(kThreads), 0, s, babies, baby_q, q, q_bs, q_cap, npos, level, primes, pmod, pmod_s, N);
-}
-
-void launch_rs_last(const u64* acc, const u64* d, u64* z, const u64* pinv, const u64* pinv_s, int npos, int l,
-                    const DevPrime* primes, int N, int J, cudaStream_t s) {
-    dim3 g((N + kThreads - 1) / kThreads, 2 * J);
-    launch_k(k_rs_last, g, dim3(kThreads), 0, s, acc, d, z, pinv, pinv_s, npos, l, primes, N);
 }
 
 void launch_rescale_lift(const u64* last, u64* lifted, const RescaleTab* tab, const DevPrime* primes, int l, int N,

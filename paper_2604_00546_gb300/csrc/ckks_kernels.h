@@ -83,11 +83,12 @@ struct IPJobs {
 };
 struct MDJobs { MDJob j[FR_MAX_JOBS]; };
 // Inner products summed straight into the accumulators of their sums of rotations: group g
-// (jobs gstart[g] .. gstart[g+1]-1) adds into j[gstart[g]].out. Each job's ext, key, galois and
+// (jobs gstart[g] .. gstart[g+1]-1) writes, or with add[g] adds into, j[gstart[g]].out. Each job's ext, key, galois and
 // addb (its rotated ciphertext's c0) are used as in IPJobs.
 struct IPSumJobs {
     IPJob j[FR_MAX_JOBS];
     signed char owner[FR_MAX_PRIMES];
+    bool add[FR_MAX_JOBS];  // group g continues a sum (else it starts one)
     int gstart[FR_MAX_JOBS + 1];
     int ngroups;
 };
@@ -134,12 +135,10 @@ void launch_ntt_rescale(const RingDev& R, const PolyBatch& b, const u64* x, int 
 // babies [B][n1][2][npos][N]; babies 1..n1-1 are inner products with IPJob::addb set.
 void launch_baby0_pq(u64* babies, long long baby_q, const u64* q, long long q_bs, int q_cap, int B, int npos,
                      int level, const DevPrime* primes, const u64* pmod, const u64* pmod_s, int N, cudaStream_t s);
-// Relinearisation fused with the rescale after it (J products at level l): launch_rs_last forms
-// z = acc_l P^-1 + d_l [J][2][N]; after its inverse NTT and that of the P limbs, launch_p2q_lift
+// Relinearisation fused with the rescale after it (J products at level l): z = acc_l P^-1 + d_l
+// [J][2][N] is formed by its inverse NTT (PolyBatch::rs); after that and the P limbs', launch_p2q_lift
 // forms y = conv P^-1 + centered lift [J][2][l][N]; the forward NTT of y with launch_ntt_relin_rescale writes
 // out_j = (acc P^-1 + d - NTT(y)) q_l^-1 (+ the EpiRescale modes) at level l - 1.
-void launch_rs_last(const u64* acc, const u64* d, u64* z, const u64* pinv, const u64* pinv_s, int npos, int l,
-                    const DevPrime* primes, int N, int J, cudaStream_t s);
 void launch_p2q_lift(const u64* acc, long long acc_job, int npos, const u64* zc, u64* y, const P2QTab* tab_rs,
                      const RescaleTab* rtab, u64 ql, int l, int N, int J, cudaStream_t s);
 void launch_ntt_relin_rescale(const RingDev& R, const PolyBatch& b, const u64* acc, const u64* d, int npos, int l,
@@ -165,8 +164,8 @@ void launch_rescale_lift(const u64* last, u64* lifted, const RescaleTab* tab, co
 void launch_tensor(const TensorJobs& jobs, int J, int level, const DevPrime* primes, int N, cudaStream_t s);
 // Sums of rotations with one ModDown (double hoisting), without the per-job inner products in
 // memory: for each group g and position,
-// out_g += sum_{jobs of g} (IP_j + P sigma_j(addb_j) on the Q positions of component 0), the
-// inner products as launch_ip computes them. out_g: [2][npos][N], read and written.
+// out_g (+)= sum_{jobs of g} (IP_j + P sigma_j(addb_j) on the Q positions of component 0), the
+// inner products as launch_ip computes them. out_g: [2][npos][N].
 void launch_ip_sum(const IPSumJobs& jobs, int beta, int npos, int level, int kp, int T, const DevPrime* primes,
                    const PrimeMap& pos_prime, int logN, const u64* pmod, const u64* pmod_s, cudaStream_t s);
 // Encrypted-database MAC: (d0, d1, d2)_j = sum_i B_i (x) E_{j n1 + i} for every giant step j.

@@ -287,8 +287,10 @@ void ntt_from(fr_ctx* c, const u64* src, long long src_outer, u64* base, long lo
 }
 // two transforms of the same direction in one launch: n polys of (base, outer, inner, pm), then
 // n2 polys of (base2, outer2, inner2, pm2); post: the first segment's last constants
+// and the second's source (PolyBatch::rs)
 void ntt_pair(fr_ctx* c, u64* base, long long outer, int inner, int n, const PrimeMap& pm, u64* base2,
-              long long outer2, int inner2, int n2, const PrimeMap& pm2, bool inv, const uint4* post) {
+              long long outer2, int inner2, int n2, const PrimeMap& pm2, bool inv, const uint4* post,
+              const decltype(PolyBatch::rs)& rs) {
     Prof p(c, "ntt", 16.0 * (n + n2) * c->R.N);
     PolyBatch b{base, outer, inner, n + n2, pm};
     b.split = n;
@@ -297,6 +299,7 @@ void ntt_pair(fr_ctx* c, u64* base, long long outer, int inner, int n, const Pri
     b.inner2 = inner2;
     b.pm2 = pm2;
     b.post = post;
+    b.rs = rs;
     launch_ntt(c->rd, b, inv, c->cur);
     c->launches += 2;
 }
@@ -518,9 +521,13 @@ void keyswitch_sums(fr_ctx* c, int level, const std::vector<KSReq>& reqs, const 
     const int ndst = (int)out.size();
     const size_t aw = (size_t)2 * npos * N;
     Tmp accs(c, (size_t)ndst * aw);
-    {
-        Prof p(c, "copy", 8.0 * ndst * aw);
-        CU(cudaMemsetAsync(accs.p, 0, (size_t)ndst * aw * 8, c->cur));
+    // the first inner product of a sum starts its accumulator; a sum without any starts at zero
+    std::vector<bool> begun(ndst, false);
+    for (const KSReq& r : reqs)
+        if (r.sum_dst >= 0 && r.sum_dst < ndst) begun[r.sum_dst] = true;
+    for (int o = 0; o < ndst; ++o) {
+        if (!begun[o]) CU(cudaMemsetAsync(accs.p + (size_t)o * aw, 0, aw * 8, c->cur));
+        begun[o] = !begun[o];
     }
     modup_chunks(c, level, reqs, [&](const std::vector<const KSReq*>& rq, const std::vector<const u64*>& ex) {
         // the jobs of one sum form one group of the summing inner product
@@ -538,7 +545,11 @@ void keyswitch_sums(fr_ctx* c, int level, const std::vector<KSReq>& reqs, const 
         for (int t = 0; t < nj; ++t) {
             const KSReq* r = rq[ord[t]];
             ij.j[t] = IPJob{ex[ord[t]], r->c, r->key, accs.p + (size_t)r->sum_dst * aw, r->galois, r->add};
-            if (t == 0 || r->sum_dst != rq[ord[t - 1]]->sum_dst) ij.gstart[ij.ngroups++] = t;
+            if (t == 0 || r->sum_dst != rq[ord[t - 1]]->sum_dst) {
+                ij.add[ij.ngroups] = begun[r->sum_dst];
+                begun[r->sum_dst] = true;
+                ij.gstart[ij.ngroups++] = t;
+            }
             if (std::find(keys.begin(), keys.end(), r->key) == keys.end()) keys.push_back(r->key);
             if (std::find(exts.begin(), exts.end(), ex[ord[t]]) == exts.end()) exts.push_back(ex[ord[t]]);
         }
@@ -711,18 +722,13 @@ void moddown_rescale(fr_ctx* c, int l, u64* acc, const u64* d, int nj, u64* out,
     PrimeMap pmL{};
     pmL.period = 1;
     pmL.idx[0] = (unsigned char)l;
-    // the last limb of the result before the rescale, in evaluation form (it reads only limb l of
-    // acc and d, not the P limbs)
+    // the P limbs, and the last limb of the result before the rescale (limb l of acc P^-1 + d, formed
+    // as it is read), to coefficients in one launch; the P -> Q conversion and the lift; one forward
+    // NTT with the combine as its epilogue
     Tmp z(c, (size_t)nj * 2 * N);
-    {
-        Prof p(c, "rescale", 8.0 * N * nj * 2.0 * (d ? 3.0 : 2.0));
-        launch_rs_last(acc, d, z.p, c->d_pinv, c->d_pinv_s, npos, l, c->d_primes, N, nj, c->cur);
-        c->launches++;
-    }
-    // the P limbs and that last limb to coefficients, in one launch; the P -> Q conversion and the
-    // lift; one forward NTT with the combine as its epilogue
+    decltype(PolyBatch::rs) rs{acc, d, c->d_pinv, c->d_pinv_s, npos, l};
     ntt_pair(c, acc + (size_t)(l + 1) * N, (long long)npos * N, np, nj * 2 * np, pmP, z.p, N, 1, 2 * nj, pmL, true,
-             c->d_p2q_post);
+             c->d_p2q_post, rs);
     Tmp y(c, (size_t)nj * 2 * l * N);
     {
         Prof p(c, "moddown", 8.0 * N * nj * 2.0 * (np + 1 + l));
@@ -921,17 +927,21 @@ void chebyshev(fr_ctx* c, const u64* x, int B, int ls, int x_cap, u64* out, int 
                 A.push_back(v->p + ((size_t)b * 2 * P + 2 * i) * ctw(c, vcap));
                 Bv.push_back(pw[s]->p + (size_t)b * ctw(c, pw_cap[s]));
             }
-        std::unique_ptr<Tmp> w(new Tmp(c, (size_t)B * P * ctw(c, lc)));
+        // the last level's products are the result
+        const bool last = s == d2 - 1;
+        std::unique_ptr<Tmp> w(last ? nullptr : new Tmp(c, (size_t)B * P * ctw(c, lc)));
         RescaleEpi addc;  // + child(2i+1), the odd children, in the rescale's epilogue
         addc.mode = 1;
         addc.add = v->p + ctw(c, vcap);
         addc.add_cap = vcap;
         addc.add_bs = 2 * ctw(c, vcap);
-        mul_relin_rescale(c, lc, A, vcap, Bv, pw_cap[s], w->p, lc, ctw(c, lc), addc);
+        mul_relin_rescale(c, lc, A, vcap, Bv, pw_cap[s], last ? out : w->p, last ? out_cap : lc,
+                          ctw(c, last ? out_cap : lc), addc);
+        if (last) break;
         v = std::move(w);
         vcap = lc;
     }
-    copy_cts(c, out, out_cap, v->p, vcap, B, ls - d2);
+    if (d2 == 1) copy_cts(c, out, out_cap, v->p, vcap, B, ls - d2);  // one leaf
     // join the side branch back into the main stream
     CU(cudaEventRecord(c->evs[d2], side));
     c->cur = main;
@@ -1063,12 +1073,12 @@ int diag_limbs(const fr_ctx* c, int schedule) {
     return c->work_level + 1 + (c->hoist_babies && schedule == 0 ? c->R.np : 0);
 }
 
-// Diagonals whose residues are transformed together: as many as keep the column-to-row
-// intermediate (nl limbs each) in 96 MB of the 126 MB L2, at least 4, at most 64.
-int encode_chunk(const fr_ctx* c, int nl) {
-    const size_t fit = ((size_t)96 << 20) / ((size_t)nl * c->R.N * 8);
-    return (int)std::min<size_t>(c->ell, std::max<size_t>(4, std::min<size_t>(64, fit)));
-}
+// Diagonals whose residues are transformed together: 32 (218 MB of scratch at the headline size).
+// Chunks that keep the column-to-row intermediate in L2 (14 diagonals, 96 MB) measured slower: the
+// transforms are bound by arithmetic, and shorter launches leave their last wave emptier (per-query
+// encoding of 4 groups 47.7 ms against 46.0 with 64 diagonals; the same chunking of the threshold's
+// batches cost 1 to 5% at 128 and 64 MB).
+constexpr int kEncodeChunk = 32;
 // residues o [nd][nl][N] of diagonals d0 .. of a database group -> dst: forward NTT, Montgomery
 // form and tiling in its epilogue
 void ntt_diags(fr_ctx* c, u64* o, int nd, int nl, const PrimeMap& pm, u64* dst, int d0) {
@@ -1083,7 +1093,7 @@ void ntt_diags(fr_ctx* c, u64* o, int nd, int nl, const PrimeMap& pm, u64* dst, 
 // diagonal d pre-rotated by (d / n1_enc) n1_enc slots (n1_enc = ell: plain diagonals).
 void encode_group(fr_ctx* c, const float* dT, long long K, long long g, u64* dst, int n1_enc, int nl) {
     const int N = c->R.N, n = N / 2, L = c->work_level, ell = (int)c->ell;
-    const int fft = std::min(ell, 64), chunk = std::min(fft, encode_chunk(c, nl));
+    const int fft = std::min(ell, 64), chunk = std::min(fft, kEncodeChunk);
     Tmp z(c, (size_t)fft * n * 2), o(c, (size_t)chunk * nl * N);
     const bool ext = nl > L + 1;
     const PrimeMap pm = ext ? pm_ext(c, L) : pm_level(L);
@@ -1220,7 +1230,7 @@ void encode_group_int(fr_ctx* c, const float* dT, long long K, long long g, long
 // the forward NTT into dst as encode_group writes it.
 void expand_group(fr_ctx* c, const long long* src, u64* dst, int nl) {
     const int N = c->R.N, L = c->work_level, ell = (int)c->ell;
-    const int chunk = encode_chunk(c, nl);
+    const int chunk = std::min(ell, kEncodeChunk);
     Tmp o(c, (size_t)chunk * nl * N);
     const bool ext = nl > L + 1;
     const PrimeMap pm = ext ? pm_ext(c, L) : pm_level(L);
@@ -1262,8 +1272,7 @@ void export_words(fr_ctx* c, const fr_ct* ct, u64* buf) {
     }
     std::lock_guard<std::recursive_mutex> ctx_lock(c->mu);
     Tmp t(c, 2 * L1 * N);
-    copy_cts(c, t.p, (int)L1, ct->dev, ct->cap, 1, ct->level);
-    ntt_cts(c, t.p, 1, ct->level, (int)L1, true);
+    ntt_from(c, ct->dev, (long long)ct->cap * N, t.p, (long long)L1 * N, (int)L1, (int)(2 * L1), pm_level(ct->level), true);
     CU(cudaMemcpyAsync(buf, t.p, 2 * L1 * N * 8, cudaMemcpyDeviceToHost, c->cur));
     CU(cudaStreamSynchronize(c->cur));
 }
@@ -2548,26 +2557,29 @@ void ondemand_scores(fr_ctx* c, const BatchPlan& P, const u64* q, const std::vec
                 continue;
             }
             if (n2 > 1) {
+                // rotated giant steps beside the first, unrotated one, for the sum
                 Tmp Pr(c, (size_t)nb * n2 * cw);
-                copy_d2d(c, Pr.p, Gs.p, (size_t)nb * n2 * cw);
+                for (int t = 0; t < nb; ++t) copy_d2d(c, Pr.p + (size_t)t * n2 * cw, Gs.p + (size_t)t * n2 * cw, cw);
                 std::vector<KSReq> reqs;
                 for (int j = 1; j < n2; ++j) {
                     const u64 gk = frh::galois_of_rotation(c->R, (long)j * n1);
                     const u64* key = rot_key(c, gk);
                     for (int t = 0; t < nb; ++t) {
-                        const u64* src = Pr.p + ((size_t)t * n2 + j) * cw;
+                        const u64* src = Gs.p + ((size_t)t * n2 + j) * cw;
                         reqs.push_back(KSReq{src + (size_t)L * N, key, (u32)gk, 1, src, L,
-                                             Gs.p + ((size_t)t * n2 + j) * cw, L});
+                                             Pr.p + ((size_t)t * n2 + j) * cw, L});
                     }
                 }
                 keyswitch(c, L - 1, reqs);
-            }
-            for (int t = 0; t < nb; ++t) {
-                const int b = sel[s0 + t];
-                Prof p(c, "misc", 8.0 * N * 2.0 * L * (n2 + 1));
-                launch_sum(Gs.p + (size_t)t * n2 * cw, L, cw, n2, S + ((size_t)P.soff[qs[b]] + g) * cw, L, L - 1,
-                           c->d_primes, N, c->cur);
-                c->launches++;
+                for (int t = 0; t < nb; ++t) {
+                    Prof p(c, "misc", 8.0 * N * 2.0 * L * (n2 + 1));
+                    launch_sum(Pr.p + (size_t)t * n2 * cw, L, cw, n2, S + ((size_t)P.soff[qs[sel[s0 + t]]] + g) * cw, L,
+                               L - 1, c->d_primes, N, c->cur);
+                    c->launches++;
+                }
+            } else {
+                for (int t = 0; t < nb; ++t)  // a single giant step is the score
+                    copy_d2d(c, S + ((size_t)P.soff[qs[sel[s0 + t]]] + g) * cw, Gs.p + (size_t)t * n2 * cw, cw);
             }
             stage.reset();
             s0 = s1;
@@ -2670,12 +2682,14 @@ void match_pipeline(fr_ctx* c, const std::vector<const fr_db*>& dbs, const u64* 
         CU(cudaGetLastError());  // a launch the device refused (configuration, resources) fails the match
         return;
     }
-    Tmp cbuf(c, (size_t)total * cwo);
+    // one group each: the thresholds are the sums over groups
+    const bool single = total == B;
+    Tmp cbuf(c, single ? 1 : (size_t)total * cwo);
     stage.reset(new Prof(c, "stage:cheb"));
-    threshold(c, S, (int)total, L - 1, L, cbuf.p, lo + 1);
+    threshold(c, S, (int)total, L - 1, L, single ? out : cbuf.p, lo + 1);
     // S7: per query, sum over its groups, then RotateAndSum over all slots
     stage.reset(new Prof(c, "stage:sum"));
-    for (int b = 0; b < B; ++b) {
+    for (int b = 0; b < B && !single; ++b) {
         Prof p(c, "misc");
         launch_sum(cbuf.p + (size_t)P.soff[b] * cwo, lo + 1, cwo, (int)dbs[b]->G, out + (size_t)b * cwo, lo + 1, lo,
                    c->d_primes, N, c->cur);

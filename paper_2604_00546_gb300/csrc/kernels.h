@@ -118,6 +118,15 @@ struct PolyBatch {
     // p % pm.period, instead of its prime's N^-1 and N^-1 itw[1] (tw_ninv, tw_wninv): a constant
     // factor on the coefficients costs nothing
     const uint4* post = nullptr;
+    // optional (inverse, second segment): its poly (job j, component t) = 2 j + t starts from acc_l P^-1
+    // + d_l, limb l of acc [J][2][npos][N] and of d [J][3][l+1][N] (null: no addend), instead of its
+    // memory
+    struct {
+        const u64* acc = nullptr;
+        const u64* d = nullptr;
+        const u64 *pinv = nullptr, *pinv_s = nullptr;
+        int npos = 0, l = 0;
+    } rs{};
     // optional (forward): the coefficients come from a base conversion
     ConvSrc conv{};
 };

@@ -94,6 +94,34 @@ __device__ __forceinline__ void conv_load(u64 (&v)[1 << RB], const PolyBatch& b,
     }
 }
 
+template <int W>
+__device__ __forceinline__ void ld_vec(u64 (&r)[W], const u64* p) {
+    if constexpr (W == 2) {
+        const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(p);
+        r[0] = t.x;
+        r[1] = t.y;
+    } else {
+        r[0] = *p;
+    }
+}
+template <int W>
+__device__ __forceinline__ void st_vec(u64* p, const u64 (&r)[W]) {
+    if constexpr (W == 2) *reinterpret_cast<ulonglong2*>(p) = make_ulonglong2(r[0], r[1]);
+    else *p = r[0];
+}
+// W consecutive values from index k of second-segment poly p (PolyBatch::rs)
+template <int W>
+__device__ __forceinline__ void rs_load(u64 (&v)[W], const PolyBatch& b, int p, int k, int N, u64 q) {
+    const int jt = p - b.split, l = b.rs.l;
+    const u64 w = __ldg(b.rs.pinv + l), ws = __ldg(b.rs.pinv_s + l);
+    u64 dd[W] = {};
+    ld_vec(v, b.rs.acc + ((long long)jt * b.rs.npos + l) * N + k);
+    if (b.rs.d) ld_vec(dd, b.rs.d + (((long long)(jt >> 1) * 3 + (jt & 1)) * (l + 1) + l) * N + k);
+#pragma unroll
+    for (int i = 0; i < W; ++i) v[i] = add_mod(mul_shoup(v[i], w, ws, q), dd[i], q);
+}
+__device__ __forceinline__ bool rs_poly(const PolyBatch& b, int p) { return b.rs.acc && p >= b.split; }
+
 // where the first pass reads poly p: its source when the batch has one, else its place
 __device__ __forceinline__ const u64* poly_in(const PolyBatch& b, int p, int N, const u64* x) {
     return b.src ? b.src + (long long)(p / b.inner) * b.src_outer + (long long)(p % b.inner) * N : x;
@@ -157,21 +185,6 @@ template <class E>
 constexpr bool in_place = std::is_same<E, EpiStore>::value;
 
 
-template <int W>
-__device__ __forceinline__ void ld_vec(u64 (&r)[W], const u64* p) {
-    if constexpr (W == 2) {
-        const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(p);
-        r[0] = t.x;
-        r[1] = t.y;
-    } else {
-        r[0] = *p;
-    }
-}
-template <int W>
-__device__ __forceinline__ void st_vec(u64* p, const u64 (&r)[W]) {
-    if constexpr (W == 2) *reinterpret_cast<ulonglong2*>(p) = make_ulonglong2(r[0], r[1]);
-    else *p = r[0];
-}
 // r += a term below q, mod q
 template <int W>
 __device__ __forceinline__ void add_vec(u64 (&r)[W], const u64 (&a)[W], u64 q) {
@@ -679,10 +692,19 @@ __global__ void __launch_bounds__(kRowThreads, 9) k_ntt_row(const __grid_constan
     const int Jbase = (blockIdx.x * RPC + rloc) * S;
     const u64* xin = (INV ? poly_in(b, p, N, x) : x) + Jbase;  // the row pass is the inverse's first
     constexpr int L0 = PhaseInfo<3, LOG, INV, 0>::LO;
-    u64 v[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) v[e] = xin[phase_x<3, L0>(tau, e)];
     const DevPrime P = R.primes[pi];
+    u64 v[8];
+    if (INV && rs_poly(b, p)) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            u64 t[1];
+            rs_load(t, b, p, Jbase + phase_x<3, L0>(tau, e), N, P.q);
+            v[e] = t[0];
+        }
+    } else {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[e] = xin[phase_x<3, L0>(tau, e)];
+    }
     const EpiK K = epi.consts(p);
     u64* s = sm + rloc * S;
     const int cls = prime_class(R, pi);
@@ -813,11 +835,14 @@ __global__ void __launch_bounds__(ClusterShape<LOGR, LOGC, CL>::T)
     }
     u64 v[8];
     if constexpr (INV) {
-        const u64* xin = poly_in(b, p, N, x) + (rank * RPC + threadIdx.x / (C / 8)) * C + (threadIdx.x % (C / 8)) * 8;
+        const int k = (rank * RPC + threadIdx.x / (C / 8)) * C + (threadIdx.x % (C / 8)) * 8;
+        const u64* xin = poly_in(b, p, N, x) + k;
+        const bool rs = rs_poly(b, p);
 #pragma unroll
         for (int h = 0; h < 4; ++h) {
             u64 t[2];
-            ld_vec(t, xin + 2 * h);
+            if (rs) rs_load(t, b, p, k + 2 * h, N, R.primes[pi].q);
+            else ld_vec(t, xin + 2 * h);
             v[2 * h] = t[0];
             v[2 * h + 1] = t[1];
         }
@@ -925,13 +950,23 @@ __global__ void __launch_bounds__(128, 6) k_ntt_row16(const __grid_constant__ Ri
     const EpiK K = epi.consts(p);
     if constexpr (INV) {
         ulonglong2* wc = reinterpret_cast<ulonglong2*>(ws);
-        const u64* xin = poly_in(b, p, N, x) + Wbase;
+        if (rs_poly(b, p)) {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int ch = j * 32 + lane;
-            ld_async16(wc + (ch ^ ((ch >> 3) & 7)), xin + 2 * ch);
+            for (int j = 0; j < 8; ++j) {
+                const int ch = j * 32 + lane;
+                u64 t[2];
+                rs_load(t, b, p, Wbase + 2 * ch, N, P.q);
+                wc[ch ^ ((ch >> 3) & 7)] = make_ulonglong2(t[0], t[1]);
+            }
+        } else {
+            const u64* xin = poly_in(b, p, N, x) + Wbase;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const int ch = j * 32 + lane;
+                ld_async16(wc + (ch ^ ((ch >> 3) & 7)), xin + 2 * ch);
+            }
+            ld_async_wait();
         }
-        ld_async_wait();
         __syncwarp();
 #pragma unroll
         for (int h = 0; h < 8; ++h) {
