@@ -38,7 +38,6 @@ struct P2QTab {
 struct RescaleTab {
     u64 half;  // (q_l - 1) / 2
     u64 q[FR_MAX_PRIMES];
-    u64 one_s[FR_MAX_PRIMES];  // floor(2^64 / q_i): Shoup quotient of 1, for x mod q_i
     u64 ql_mod[FR_MAX_PRIMES];
     u64 qlinv[FR_MAX_PRIMES], qlinv_s[FR_MAX_PRIMES];
 };

@@ -128,12 +128,6 @@ __device__ __forceinline__ u64 reduce_sum(const Acc128& a, const DevPrime& P) {
     const u64 f = fold_top(r, P.bsh, P.c);
     return min(f, f - P.q);
 }
-__device__ __forceinline__ void mac128(Acc128& a, u64 x, u64 y) {
-    u64 l = x * y;
-    u64 h = __umul64hi(x, y);
-    a.lo += l;
-    a.hi += h + (a.lo < l ? 1ull : 0ull);
-}
 
 // Products of residues below 2^60 from 30-bit halves: x = xh 2^30 + xl, y = yh 2^30 + yl,
 // x y = xl yl + (xl yh + xh yl) 2^30 + xh yh 2^60. Each partial product is below 2^60, so up

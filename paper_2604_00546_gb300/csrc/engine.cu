@@ -1558,7 +1558,6 @@ void build_tables(fr_ctx* c) {
         for (int i = 0; i < l; ++i) {
             const u64 q = R.primes[i];
             t.q[i] = q;
-            t.one_s[i] = frh::shoup_quot(1, q);
             t.ql_mod[i] = ql % q;
             t.qlinv[i] = frh::invm(ql % q, q);
             t.qlinv_s[i] = frh::shoup_quot(t.qlinv[i], q);

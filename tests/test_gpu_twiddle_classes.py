@@ -89,3 +89,22 @@ def test_base_conversion_of_wide_digits(log_n, n_q, n_p):
     got = ctx.mul_relin(ca, cb)
     assert np.array_equal(got.export(), mul)
     assert np.array_equal(ctx.rescale(got).export(), oc.rescale(mul, top))
+
+
+@pytest.mark.parametrize("log_n", [11, 13, 15])
+@pytest.mark.parametrize("bits", [34, 45, 52], ids=["class2", "class0", "class1"])
+def test_threshold_of_every_class(bits, log_n):
+    """The whole threshold (products relinearised and rescaled through one transform, leaves, tree) on a
+    chain of each class, at rings that run the cluster kernel, the two-pass kernels and, for class 2,
+    the 8-residue fallback."""
+    q_bits, p_bits = [bits + 2] + [bits] * 7, [bits + 2] * 3
+    ctx = fr.Context(device=0, log_n=log_n, q_bits=q_bits, p_bits=p_bits, dnum=3, scale_bits=bits - 4, ell=64, n1=8,
+                     cheb_degree=27, threshold=0.5)
+    ctx.load_keys(ctx.keygen([], 91))
+    oc = oracle.Ctx(log_n, q_bits, p_bits, 3, bits - 4)
+    ok = oc.keygen(91)
+    a = _residues(ctx.primes()[: oc.top + 1], ctx.N, 191)
+    for shape in ([0, 5] if log_n >= 14 else [0]):
+        ctx.ntt_set_shapes([shape] * 4)
+        got = ctx.chebyshev(ctx.import_ct(a, oc.top).upload())
+        assert np.array_equal(got.export(), ok.cheb_eval(a, oc.top, 27, 0.5)), shape
