@@ -731,8 +731,8 @@ __global__ void __launch_bounds__(kRowThreads, 9) k_ntt_row(const __grid_constan
 // pass), not by its arithmetic. Everything the kernel reads is asked for at its start: elements,
 // both passes' twiddles and, before the cluster barrier, the epilogue's operands. For N <= 2^13 it
 // is the faster form at every batch size (microseconds, forward / inverse, launches in a graph):
-//   N = 2^13   8 polys 4.6/4.7 (two passes 5.8/5.8), 128: 13.4/14.4 (14.8/15.7), 1024: 76.8/82.5 (90.9/87.6)
-//   N = 2^12   8 polys 4.6/4.3 (5.3/5.5), 128: 7.4/7.8 (9.7/9.9), 1024: 37.1/39.2 (45.6/44.0)
+//   N = 2^13   8 polys 4.6/4.8 (two passes 5.8/5.8), 128: 13.4/14.5 (14.8/15.7), 1024: 76.8/83.6 (90.9/87.6)
+//   N = 2^12   8 polys 4.7/4.5 (5.3/5.5), 128: 7.4/7.8 (9.7/9.9), 1024: 36.9/39.9 (45.6/44.0)
 // At N = 2^16, 16 CTAs of 4096 elements, it took 15.7 us for 8 polynomials where two passes take
 // 10.0: a cluster that large leaves most of the SMs' slots empty.
 template <int LOGR, int LOGC, int CL>
@@ -749,6 +749,13 @@ __device__ __forceinline__ void ld_async_wait() {
     asm volatile("cp.async.commit_group;" ::: "memory");
     asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
+
+// The shared memory of another CTA of the cluster may be written only once that CTA has started:
+// every thread arrives as its kernel begins and waits before its first remote store, so the loads
+// and the first pass lie between the two. Relaxed: nothing but the start is ordered by it. It costs
+// 0 to 0.2 us a launch (times below; 8 polynomials without it: 4.6/4.7 at N = 2^13, 4.6/4.3 at 2^12).
+__device__ __forceinline__ void cluster_arrive_started() { asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait_started() { asm volatile("barrier.cluster.wait;" ::: "memory"); }
 
 template <int LOGR, int LOGC, int CL, bool INV, int CLS, class E>
 __device__ __forceinline__ void ntt_cluster_body(u64 (&v)[8], const PolyBatch& b, u64* x, const DevPrime& P, int p, int rank, u64* sm, const E& epi) {
@@ -769,6 +776,7 @@ __device__ __forceinline__ void ntt_cluster_body(u64 (&v)[8], const PolyBatch& b
     if constexpr (!INV) {
         ColEx<KTC> exc{A, col};
         phases<CLS, 3, LOGR, false, false, 0>(v, tauc, cc, exc, P);
+        cluster_wait_started();
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
             const int row = phase_x<3, CLL>(tauc, e);
@@ -796,6 +804,7 @@ __device__ __forceinline__ void ntt_cluster_body(u64 (&v)[8], const PolyBatch& b
     } else {
         RowEx exr{B + rloc * C};
         phases<CLS, 3, LOGC, true, false, 0>(v, taur, cr, exr, P);
+        cluster_wait_started();
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
             const int k = phase_x<3, RLL>(taur, e);
@@ -816,6 +825,7 @@ template <int LOGR, int LOGC, int CL, bool INV, class E, bool CONV>
 __global__ void __launch_bounds__(ClusterShape<LOGR, LOGC, CL>::T)
     k_ntt_cluster(const __grid_constant__ RingDev R, const __grid_constant__ PolyBatch b,
                   const __grid_constant__ E epi) {
+    cluster_arrive_started();
     pdl_wait();
     pdl_trigger();
     using Sh = ClusterShape<LOGR, LOGC, CL>;
