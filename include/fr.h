@@ -416,7 +416,8 @@ fr_status fr_butterfly_peak(int device, double* butterflies_per_s);
  * thread with register operands, 8 CTAs of 256 threads per SM (an FMA counts as two). The
  * ceiling of the encoder's FP64 special FFT. FR_ERR_CUDA without such a device. */
 fr_status fr_fp64_peak(int device, double* flops_per_s);
-/* Number of kernel launches issued by the library so far. */
+/* Number of kernels launched by this context's calls so far (replays of a match's graph count the
+ * graph's kernels; fr_setup's tuning launches are not counted). */
 uint64_t fr_launch_count(const fr_ctx* ctx);
 
 /* Context facts: primes (Q then P), digit boundaries, resident HBM bytes. */

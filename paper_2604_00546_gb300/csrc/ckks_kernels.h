@@ -104,14 +104,14 @@ __host__ __device__ __forceinline__ long long diag_word(int i, int k, long long 
 // Forward NTT of encoded diagonals into a database: poly p of b is limb p % nl of diagonal d0 +
 // p / nl; the values go to diags (ell rows) in Montgomery form (x 2^64 mod q), as 30-bit halves
 // (split30).
-void launch_ntt_diags(const RingDev& R, const PolyBatch& b, u64* diags, int d0, int ell, int nl, cudaStream_t s);
+int launch_ntt_diags(const RingDev& R, const PolyBatch& b, u64* diags, int d0, int ell, int nl, cudaStream_t s);
 // src [rows][nl][N] (evaluation form) into rows row0.. of a database of total rows, Montgomery form
 void launch_tile_mont(const u64* src, int rows, u64* diags, long long row0, int total, int nl, const DevPrime* primes,
                       int N, cudaStream_t s);
 // Forward NTT of the P -> Q conversions of a ModDown (b.conv forms them) fused with its combine:
 // poly p of b is (job p / (2(level+1)), component, limb); the transformed values never reach
 // memory, the jobs' outputs do.
-void launch_ntt_moddown(const RingDev& R, const PolyBatch& b, const MDJobs& jobs, int npos, int level,
+int launch_ntt_moddown(const RingDev& R, const PolyBatch& b, const MDJobs& jobs, int npos, int level,
                         const u64* pinv, const u64* pinv_s, cudaStream_t s);
 // Forward NTT of a rescale's lifted last limb fused with its combine: poly p of b is
 // (ct component p / l, limb p % l); writes out = (x - NTT(lifted)) q_l^-1, then mode 1 adds
@@ -124,10 +124,10 @@ void launch_ntt_moddown(const RingDev& R, const PolyBatch& b, const MDJobs& jobs
 // T1 of query b at x + b x_bs (cap x_cap); constants [nl][L1] each.
 void launch_leaf_lift(const u64* u, const u64* cb, const u64* cb_s, const u64* ca, int nl, int L1, u64* lifted,
                       const RescaleTab* tab, const DevPrime* primes, int l, int N, int B, cudaStream_t s);
-void launch_ntt_leaf_rescale(const RingDev& R, const PolyBatch& b, const u64* x, long long x_bs, int x_cap,
+int launch_ntt_leaf_rescale(const RingDev& R, const PolyBatch& b, const u64* x, long long x_bs, int x_cap,
                              const u64* cb, const u64* cb_s, const u64* ca, int nl, int L1, u64* out, int out_cap,
                              const RescaleTab* tab, int l, cudaStream_t s);
-void launch_ntt_rescale(const RingDev& R, const PolyBatch& b, const u64* x, int x_cap, u64* out, int out_cap,
+int launch_ntt_rescale(const RingDev& R, const PolyBatch& b, const u64* x, int x_cap, u64* out, int out_cap,
                         const RescaleTab* tab, int l, int mode, const u64* add, int add_cap, long long add_bs,
                         const u64* cres, cudaStream_t s);
 // Baby steps kept in Q_l u P: baby 0 = P q (zero on the P positions) of each of B queries,
@@ -140,7 +140,7 @@ void launch_baby0_pq(u64* babies, long long baby_q, const u64* q, long long q_bs
 // out_j = (acc P^-1 + d - NTT(y)) q_l^-1 (+ the EpiRescale modes) at level l - 1.
 void launch_p2q_lift(const u64* acc, long long acc_job, int npos, const u64* zc, u64* y, const P2QTab* tab_rs,
                      const RescaleTab* rtab, u64 ql, int l, int N, int J, cudaStream_t s);
-void launch_ntt_relin_rescale(const RingDev& R, const PolyBatch& b, const u64* acc, const u64* d, int npos, int l,
+int launch_ntt_relin_rescale(const RingDev& R, const PolyBatch& b, const u64* acc, const u64* d, int npos, int l,
                               const u64* pinv, const u64* pinv_s, const RescaleTab* tab, u64* out, int out_cap,
                               long long out_bs, int mode, const u64* add, int add_cap, long long add_bs,
                               const u64* cres, cudaStream_t s);

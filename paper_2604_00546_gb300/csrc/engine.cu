@@ -270,8 +270,7 @@ void ntt(fr_ctx* c, u64* base, long long outer, int inner, int npolys, const Pri
     Prof p(c, "ntt", 16.0 * npolys * c->R.N);
     PolyBatch b{base, outer, inner, npolys, pm};
     b.post = post;
-    launch_ntt(c->rd, b, inv, c->cur);
-    c->launches += 2;
+    c->launches += launch_ntt(c->rd, b, inv, c->cur);
 }
 // the same transform out of place: poly p read from src + (p / inner) src_outer + (p % inner) N
 // (npolys a multiple of inner), written to its place in base
@@ -282,8 +281,7 @@ void ntt_from(fr_ctx* c, const u64* src, long long src_outer, u64* base, long lo
     b.post = post;
     b.src = src;
     b.src_outer = src_outer;
-    launch_ntt(c->rd, b, inv, c->cur);
-    c->launches += 2;
+    c->launches += launch_ntt(c->rd, b, inv, c->cur);
 }
 // two transforms of the same direction in one launch: n polys of (base, outer, inner, pm), then
 // n2 polys of (base2, outer2, inner2, pm2); post: the first segment's last constants
@@ -300,8 +298,7 @@ void ntt_pair(fr_ctx* c, u64* base, long long outer, int inner, int n, const Pri
     b.pm2 = pm2;
     b.post = post;
     b.rs = rs;
-    launch_ntt(c->rd, b, inv, c->cur);
-    c->launches += 2;
+    c->launches += launch_ntt(c->rd, b, inv, c->cur);
 }
 // ModUp of nj inputs and its forward NTT: in [nj][level+1][N] (coefficient form, times inv_hat) ->
 // the non-own positions of ext [nj][beta][npos][N]
@@ -317,8 +314,7 @@ void ntt_modup(fr_ctx* c, const u64* in, u64* ext, int nj, int level) {
         c->launches++;
     }
     Prof p(c, "ntt", 16.0 * nj * cnt * N);
-    launch_ntt(c->rd, b, false, c->cur);
-    c->launches += 2;
+    c->launches += launch_ntt(c->rd, b, false, c->cur);
 }
 // the conversions P -> Q of nj accumulators acc [nj][2][npos][N] at `level` (P limbs in
 // coefficient form, times inv_hat), as the input of the forward NTT b [nj][2][level+1] of them
@@ -435,8 +431,7 @@ void ks_finish(fr_ctx* c, int level, const std::vector<const KSReq*>& reqs, cons
     PolyBatch pb{conv.p, (long long)(level + 1) * N, level + 1, nj * 2 * (level + 1), pm_level(level)};
     p2q_into(c, acc.p, nj, level, pb);
     Prof p(c, "ntt", 16.0 * nj * 2 * (level + 1) * N);
-    launch_ntt_moddown(c->rd, pb, md, npos, level, c->d_pinv, c->d_pinv_s, c->cur);
-    c->launches += 2;
+    c->launches += launch_ntt_moddown(c->rd, pb, md, npos, level, c->d_pinv, c->d_pinv_s, c->cur);
 }
 
 // Hybrid key switching of a list of requests. Requests that switch the same
@@ -586,8 +581,7 @@ void keyswitch_sums(fr_ctx* c, int level, const std::vector<KSReq>& reqs, const 
                      no * 2 * (level + 1), pm_level(level)};
         p2q_into(c, accs.p + (size_t)o0 * aw, no, level, pb);
         Prof p(c, "ntt", 16.0 * no * 2 * (level + 1) * N);
-        launch_ntt_moddown(c->rd, pb, md, npos, level, c->d_pinv, c->d_pinv_s, c->cur);
-        c->launches += 2;
+        c->launches += launch_ntt_moddown(c->rd, pb, md, npos, level, c->d_pinv, c->d_pinv_s, c->cur);
     }
 }
 
@@ -646,9 +640,8 @@ void rescale(fr_ctx* c, const u64* in, int B, int level, int in_cap, u64* out, i
     // forward NTT of the lifted limb with the combine as its epilogue
     Prof p(c, "ntt", 16.0 * 2 * B * l * N);
     PolyBatch pb{lifted.p, (long long)l * N, l, 2 * B * l, pm_level(l - 1)};
-    launch_ntt_rescale(c->rd, pb, in, in_cap, out, out_cap, c->d_rescale[l], l, ep.mode, ep.add, ep.add_cap, ep.add_bs,
-                       ep.cres, c->cur);
-    c->launches += 2;
+    c->launches += launch_ntt_rescale(c->rd, pb, in, in_cap, out, out_cap, c->d_rescale[l], l, ep.mode, ep.add,
+                                      ep.add_cap, ep.add_bs, ep.cres, c->cur);
 }
 
 // Rescale(T1 round(c1 Delta) + round(c0 Delta) Delta) for nl leaves of each of B cts T1 at level
@@ -674,9 +667,8 @@ void leaves_rescaled(fr_ctx* c, const u64* x, int B, int x_cap, int l, int nl, c
     }
     Prof p(c, "ntt", 16.0 * B * nl * 2 * l * N);
     PolyBatch pb{lifted.p, (long long)l * N, l, B * nl * 2 * l, pm_level(l - 1)};
-    launch_ntt_leaf_rescale(c->rd, pb, x, ctw(c, x_cap), x_cap, cb, cb_s, ca, nl, L1, out, out_cap, c->d_rescale[l], l,
-                            c->cur);
-    c->launches += 2;
+    c->launches += launch_ntt_leaf_rescale(c->rd, pb, x, ctw(c, x_cap), x_cap, cb, cb_s, ca, nl, L1, out, out_cap,
+                                           c->d_rescale[l], l, c->cur);
 }
 
 // ---------------------------------------------------------------------------
@@ -738,9 +730,8 @@ void moddown_rescale(fr_ctx* c, int l, u64* acc, const u64* d, int nj, u64* out,
     }
     Prof p(c, "ntt", 16.0 * nj * 2 * l * N);
     PolyBatch pb{y.p, (long long)l * N, l, nj * 2 * l, pm_level(l - 1)};
-    launch_ntt_relin_rescale(c->rd, pb, acc, d, npos, l, c->d_pinv, c->d_pinv_s, c->d_rescale[l], out, out_cap, out_bs,
-                             ep.mode, ep.add, ep.add_cap, ep.add_bs, ep.cres, c->cur);
-    c->launches += 2;
+    c->launches += launch_ntt_relin_rescale(c->rd, pb, acc, d, npos, l, c->d_pinv, c->d_pinv_s, c->d_rescale[l], out,
+                                            out_cap, out_bs, ep.mode, ep.add, ep.add_cap, ep.add_bs, ep.cres, c->cur);
 }
 
 // Products of ciphertext pairs at level l, relinearised and rescaled, with the relinearisation's
@@ -1084,8 +1075,7 @@ constexpr int kEncodeChunk = 32;
 void ntt_diags(fr_ctx* c, u64* o, int nd, int nl, const PrimeMap& pm, u64* dst, int d0) {
     Prof p(c, "ntt", 16.0 * nd * nl * c->R.N);
     PolyBatch pb{o, (long long)nl * c->R.N, nl, nd * nl, pm};
-    launch_ntt_diags(c->rd, pb, dst, d0, (int)c->ell, nl, c->cur);
-    c->launches += 2;
+    c->launches += launch_ntt_diags(c->rd, pb, dst, d0, (int)c->ell, nl, c->cur);
 }
 
 // Encode the diagonals of template group g at the working level into dst, ell rows of nl limbs in
@@ -1815,6 +1805,7 @@ fr_status fr_load_keys(fr_ctx* c, const fr_keys* k) {
             CU(cudaMalloc(&dptr, words * 8));
             CU(cudaMemcpy(dptr, stage.data(), words * 8, cudaMemcpyHostToDevice));
             launch_to_mont(dptr, N, pm, c->d_primes, (long long)words, c->cur);
+            c->launches++;
             CU(cudaStreamSynchronize(c->cur));
             return dptr;
         };
@@ -2842,6 +2833,7 @@ void match_queries(fr_ctx* c, const std::vector<const fr_db*>& dbs, const fr_ct*
             try {
                 match_pipeline(c, dbs, mg.in, mode, mg.out);
             } catch (...) {
+                c->launches = k0;
                 graph = nullptr;
                 if (cudaStreamEndCapture(c->cur, &graph) == cudaSuccess && graph) cudaGraphDestroy(graph);
                 cudaGetLastError();
@@ -3486,7 +3478,7 @@ fr_status fr_ntt_time(fr_ctx* c, uint32_t npolys, uint32_t level, uint32_t reps,
         for (uint32_t r = 0; r <= reps; ++r) {  // the first round warms up
             for (int inv = 0; inv < 2; ++inv) {
                 cudaEventRecord(a, c->cur);
-                launch_ntt(c->rd, pb, inv != 0, c->cur);
+                c->launches += launch_ntt(c->rd, pb, inv != 0, c->cur);
                 cudaEventRecord(b, c->cur);
                 cudaEventSynchronize(b);
                 float ms = 0;
@@ -3610,16 +3602,17 @@ extern "C" fr_status fr_rotate_noalloc(fr_ctx* c, const uint64_t* d_in, uint32_t
         PolyBatch in{e, 2 * (long long)L1N, 2 * (l + 1), 2 * (l + 1), pl};
         in.src = d_in;  // out of place
         in.src_outer = in.outer;
-        launch_ntt(c->rd, in, false, st);
+        c->launches += launch_ntt(c->rd, in, false, st);
         // the conversion reads 16 bytes at a time
         const u64* c1 = d_in + L1N;
         if ((uintptr_t)c1 & 15) {
             CU(cudaMemcpyAsync(a, c1, L1N * 8, cudaMemcpyDeviceToDevice, st));
             c1 = a;
         }
+        c->launches += 2;  // the conversion, the inner product
         launch_modup(c1, 0, ext, c->d_modup[l], beta, npos, N, 1, false, st);
-        launch_ntt(c->rd, PolyBatch{ext, (long long)beta * npos * N, 1, c->modup_ext[l].n, PrimeMap{}, c->modup_ext[l]},
-                   false, st);
+        PolyBatch pe{ext, (long long)beta * npos * N, 1, c->modup_ext[l].n, PrimeMap{}, c->modup_ext[l]};
+        c->launches += launch_ntt(c->rd, pe, false, st);
         IPJobs ij;
         digit_owners(c, l, ij.owner);
         ij.j[0] = IPJob{ext, e + L1N, key, acc, (u32)g};
@@ -3633,17 +3626,16 @@ extern "C" fr_status fr_rotate_noalloc(fr_ctx* c, const uint64_t* d_in, uint32_t
         for (int j = 0; j < np; ++j) pmP.idx[j] = (unsigned char)(nq + j);
         PolyBatch pP{acc + L1N, (long long)npos * N, np, 2 * np, pmP};
         pP.post = c->d_p2q_post;
-        launch_ntt(c->rd, pP, true, st);
+        c->launches += launch_ntt(c->rd, pP, true, st);
         MDJobs md;
         md.j[0] = MDJob{acc, e, res, l + 1, l + 1, 1, (u32)g};
         PolyBatch pc{conv, (long long)L1N, l + 1, 2 * (l + 1), pl};
         p2q_into(c, acc, 1, l, pc);
-        launch_ntt_moddown(c->rd, pc, md, npos, l, c->d_pinv, c->d_pinv_s, st);
+        c->launches += launch_ntt_moddown(c->rd, pc, md, npos, l, c->d_pinv, c->d_pinv_s, st);
         PolyBatch out{d_out, 2 * (long long)L1N, 2 * (l + 1), 2 * (l + 1), pl};
         out.src = res;
         out.src_outer = out.outer;
-        launch_ntt(c->rd, out, true, st);
-        c->launches += 12;
+        c->launches += launch_ntt(c->rd, out, true, st);
         CU(cudaGetLastError());
     });
 }

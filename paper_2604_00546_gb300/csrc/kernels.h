@@ -162,8 +162,9 @@ struct RingDev {
     unsigned char ntt_shape[FR_NTT_BUCKETS];  // tile shape per batch-size bucket (see launch_ntt)
 };
 
-// Batched negacyclic NTT (evaluation order: position k = value at psi^(2 brev(k)+1)).
-void launch_ntt(const RingDev& R, const PolyBatch& b, bool inverse, cudaStream_t s);
+// Batched negacyclic NTT (evaluation order: position k = value at psi^(2 brev(k)+1)). This and every
+// launch_ntt_* return the number of kernels launched: 1 for the cluster transform, 2 for two passes.
+int launch_ntt(const RingDev& R, const PolyBatch& b, bool inverse, cudaStream_t s);
 // Autotuner of the NTT tile shapes (see ntt.cu); us: FR_NTT_BUCKETS x FR_NTT_SHAPES times in
 // microseconds (-1: shape not available), or null.
 void tune_ntt(RingDev& R, cudaStream_t s, double* us, int reps);

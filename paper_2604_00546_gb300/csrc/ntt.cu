@@ -68,17 +68,17 @@ double measure_butterfly_peak(int device) {
 }
 
 template <class E>
-void launch_ntt_e(const RingDev& R, const PolyBatch& b, bool inverse, cudaStream_t s, const E& epi) {
-    if (b.npolys <= 0) return;
+int launch_ntt_e(const RingDev& R, const PolyBatch& b, bool inverse, cudaStream_t s, const E& epi) {
+    if (b.npolys <= 0) return 0;
     switch (R.logN) {
-        case 15: launch_ntt_s<7, 8>(R, b, inverse, s, epi); break;
-        case 16: launch_ntt_s<8, 8>(R, b, inverse, s, epi); break;
-        default: launch_ntt_small(R, b, inverse, s, epi); break;
+        case 15: return launch_ntt_s<7, 8>(R, b, inverse, s, epi);
+        case 16: return launch_ntt_s<8, 8>(R, b, inverse, s, epi);
+        default: return launch_ntt_small(R, b, inverse, s, epi);
     }
 }
 
-void launch_ntt(const RingDev& R, const PolyBatch& b, bool inverse, cudaStream_t s) {
-    launch_ntt_e(R, b, inverse, s, EpiStore{});
+int launch_ntt(const RingDev& R, const PolyBatch& b, bool inverse, cudaStream_t s) {
+    return launch_ntt_e(R, b, inverse, s, EpiStore{});
 }
 
 // Times every tile shape of the forward + inverse transform for one batch size per bucket
@@ -140,34 +140,34 @@ void tune_ntt(RingDev& R, cudaStream_t s, double* us, int reps) {
     cudaStreamSynchronize(s);
 }
 
-void launch_ntt_diags(const RingDev& R, const PolyBatch& b, u64* diags, int d0, int ell, int nl, cudaStream_t s) {
-    launch_ntt_e(R, b, false, s, EpiDiag{diags, d0, ell, nl, R.N});
+int launch_ntt_diags(const RingDev& R, const PolyBatch& b, u64* diags, int d0, int ell, int nl, cudaStream_t s) {
+    return launch_ntt_e(R, b, false, s, EpiDiag{diags, d0, ell, nl, R.N});
 }
 
-void launch_ntt_moddown(const RingDev& R, const PolyBatch& b, const MDJobs& jobs, int npos, int level,
+int launch_ntt_moddown(const RingDev& R, const PolyBatch& b, const MDJobs& jobs, int npos, int level,
                         const u64* pinv, const u64* pinv_s, cudaStream_t s) {
     EpiModDown e{jobs, npos, level, R.logN, pinv, pinv_s};
-    launch_ntt_e(R, b, false, s, e);
+    return launch_ntt_e(R, b, false, s, e);
 }
 
-void launch_ntt_relin_rescale(const RingDev& R, const PolyBatch& b, const u64* acc, const u64* d, int npos, int l,
+int launch_ntt_relin_rescale(const RingDev& R, const PolyBatch& b, const u64* acc, const u64* d, int npos, int l,
                               const u64* pinv, const u64* pinv_s, const RescaleTab* tab, u64* out, int out_cap,
                               long long out_bs, int mode, const u64* add, int add_cap, long long add_bs,
                               const u64* cres, cudaStream_t s) {
     EpiRelinRescale e{acc, d, out, tab, pinv, pinv_s, npos, l, R.N, out_cap, mode, out_bs, add, add_cap, add_bs, cres};
-    launch_ntt_e(R, b, false, s, e);
+    return launch_ntt_e(R, b, false, s, e);
 }
 
-void launch_ntt_leaf_rescale(const RingDev& R, const PolyBatch& b, const u64* x, long long x_bs, int x_cap,
+int launch_ntt_leaf_rescale(const RingDev& R, const PolyBatch& b, const u64* x, long long x_bs, int x_cap,
                              const u64* cb, const u64* cb_s, const u64* ca, int nl, int L1, u64* out, int out_cap,
                              const RescaleTab* tab, int l, cudaStream_t s) {
     EpiLeafRescale e{x, x_bs, x_cap, cb, cb_s, ca, nl, L1, out, out_cap, tab, l, R.N};
-    launch_ntt_e(R, b, false, s, e);
+    return launch_ntt_e(R, b, false, s, e);
 }
 
-void launch_ntt_rescale(const RingDev& R, const PolyBatch& b, const u64* x, int x_cap, u64* out, int out_cap,
+int launch_ntt_rescale(const RingDev& R, const PolyBatch& b, const u64* x, int x_cap, u64* out, int out_cap,
                         const RescaleTab* tab, int l, int mode, const u64* add, int add_cap, long long add_bs,
                         const u64* cres, cudaStream_t s) {
     EpiRescale e{x, out, tab, x_cap, out_cap, l, R.N, mode, add, add_cap, add_bs, cres};
-    launch_ntt_e(R, b, false, s, e);
+    return launch_ntt_e(R, b, false, s, e);
 }

@@ -753,7 +753,7 @@ __device__ __forceinline__ void ld_async_wait() {
 // The shared memory of another CTA of the cluster may be written only once that CTA has started:
 // every thread arrives as its kernel begins and waits before its first remote store, so the loads
 // and the first pass lie between the two. Relaxed: nothing but the start is ordered by it. It costs
-// 0 to 0.2 us a launch (times below; 8 polynomials without it: 4.6/4.7 at N = 2^13, 4.6/4.3 at 2^12).
+// 0 to 0.2 us a launch (times above; 8 polynomials without it: 4.6/4.7 at N = 2^13, 4.6/4.3 at 2^12).
 __device__ __forceinline__ void cluster_arrive_started() { asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait_started() { asm volatile("barrier.cluster.wait;" ::: "memory"); }
 
@@ -1079,32 +1079,34 @@ inline int ntt_shape_of(const RingDev& R, const PolyBatch& b) {
     return !R.fast || (a & 15) || (shape == 4 && R.logN > 14) ? 0 : shape;
 }
 
+// Returns the number of kernels launched.
 template <int LOGR, int LOGC, class E>
-void launch_ntt_s(const RingDev& R, const PolyBatch& b, bool inverse, cudaStream_t st, const E& epi) {
+int launch_ntt_s(const RingDev& R, const PolyBatch& b, bool inverse, cudaStream_t st, const E& epi) {
     const int shape = ntt_shape_of(R, b);
     if constexpr (LOGR + LOGC <= 14) {
         if (shape == 4) {
             launch_ntt_cluster<LOGR, LOGC>(R, b, inverse, st, epi);
-            return;
+            return 1;
         }
     }
     if constexpr (LOGR + LOGC >= 14) {
         if (shape == 5) {
             launch_ntt_r16<LOGR, LOGC>(R, b, inverse, st, epi);
-            return;
+            return 2;
         }
     }
     if constexpr (LOGR + LOGC >= 15) {
         if (shape & 1) {
             launch_ntt_t<LOGR, LOGC, E, 8>(R, b, inverse, st, epi);
-            return;
+            return 2;
         }
     }
     launch_ntt_t<LOGR, LOGC, E, 4>(R, b, inverse, st, epi);
+    return 2;
 }
 
 // The transform of a ring of N <= 2^14 (ntt_small.cu).
 template <class E>
-void launch_ntt_small(const RingDev& R, const PolyBatch& b, bool inverse, cudaStream_t s, const E& epi);
+int launch_ntt_small(const RingDev& R, const PolyBatch& b, bool inverse, cudaStream_t s, const E& epi);
 
 }  // namespace ntt_kernels
