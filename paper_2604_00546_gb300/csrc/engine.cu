@@ -234,7 +234,7 @@ struct Prof {
     Region* r = nullptr;
     cudaEvent_t a = nullptr, b = nullptr;
     Prof(fr_ctx* cc, const char* name, double bytes = 0) : c(cc) {
-        if (!c->prof) return;
+        if (!c->prof || !name) return;
         if (!c->prof_only.empty() && std::strncmp(name, c->prof_only.c_str(), c->prof_only.size()) != 0) return;
         r = &c->regions[name];
         r->bytes += (uint64_t)bytes;
@@ -317,14 +317,15 @@ void ntt_modup(fr_ctx* c, const u64* in, u64* ext, int nj, int level) {
     c->launches += launch_ntt(c->rd, b, false, c->cur);
 }
 // the conversions P -> Q of nj accumulators acc [nj][2][npos][N] at `level` (P limbs in
-// coefficient form, times inv_hat), as the input of the forward NTT b [nj][2][level+1] of them
-void p2q_into(fr_ctx* c, const u64* acc, int nj, int level, PolyBatch& b) {
+// coefficient form, times inv_hat), as the input of the forward NTT b [nj][2][level+1] of them;
+// region: where a conversion launched of its own is timed (null: nowhere)
+void p2q_into(fr_ctx* c, const u64* acc, int nj, int level, PolyBatch& b, const char* region = "moddown") {
     const long long N = c->R.N, npos = level + 1 + c->R.np;
     if (b.npolys <= kConvFused) {
         b.conv = ConvSrc{c->d_p2q->t, 0, acc + (level + 1) * N, npos * N, c->R.np};
         return;
     }
-    Prof p(c, "moddown", 8.0 * N * nj * 2.0 * (c->R.np + level + 1));
+    Prof p(c, region, 8.0 * N * nj * 2.0 * (c->R.np + level + 1));
     launch_p2q(acc, 2 * npos * N, (int)npos, level, b.base, c->d_p2q, (int)N, nj, c->cur);
     c->launches++;
 }
@@ -3630,7 +3631,7 @@ extern "C" fr_status fr_rotate_noalloc(fr_ctx* c, const uint64_t* d_in, uint32_t
         MDJobs md;
         md.j[0] = MDJob{acc, e, res, l + 1, l + 1, 1, (u32)g};
         PolyBatch pc{conv, (long long)L1N, l + 1, 2 * (l + 1), pl};
-        p2q_into(c, acc, 1, l, pc);
+        p2q_into(c, acc, 1, l, pc, nullptr);  // no events: the caller may be capturing this stream
         c->launches += launch_ntt_moddown(c->rd, pc, md, npos, l, c->d_pinv, c->d_pinv_s, st);
         PolyBatch out{d_out, 2 * (long long)L1N, 2 * (l + 1), 2 * (l + 1), pl};
         out.src = res;
