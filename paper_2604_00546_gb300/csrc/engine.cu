@@ -210,6 +210,25 @@ struct Tmp {
     Tmp(const Tmp&) = delete;
     Tmp& operator=(const Tmp&) = delete;
 };
+// cudaMalloc'ed memory of a handle being built: freed, once the work queued on it is done, unless
+// keep() hands it over
+struct DevHold {
+    fr_ctx* c;
+    void* p = nullptr;
+    explicit DevHold(fr_ctx* cc) : c(cc) {}
+    ~DevHold() {
+        if (!p) return;
+        cudaStreamSynchronize(c->cur);
+        cudaFree(p);
+    }
+    DevHold(const DevHold&) = delete;
+    DevHold& operator=(const DevHold&) = delete;
+    void* keep() {
+        void* r = p;
+        p = nullptr;
+        return r;
+    }
+};
 template <class T>
 T* upload_persistent(fr_ctx* c, const T* h, size_t count) {
     void* p = nullptr;
@@ -1856,33 +1875,32 @@ fr_status fr_load_db(fr_ctx* c, const float* templates, size_t K, size_t ell, fr
         db->bytes = tier == 1 ? dbytes : tier == 3 ? ibytes : tbytes;
         if (c->budget && c->resident + db->bytes > c->budget)
             raise(FR_ERR_HBM_BUDGET, "database exceeds the HBM budget");
-        float* dT = nullptr;
-        CU(cudaMalloc(&dT, tbytes));
+        DevHold hT(c), hold(c);
+        CU(cudaMalloc(&hT.p, tbytes));
+        float* dT = (float*)hT.p;
         CU(cudaMemcpyAsync(dT, templates, tbytes, cudaMemcpyHostToDevice, c->cur));
         if (tier == 1 || tier == 3) {
-            void* p = nullptr;
-            cudaError_t e = cudaMalloc(&p, tier == 1 ? dbytes : ibytes);
+            cudaError_t e = cudaMalloc(&hold.p, tier == 1 ? dbytes : ibytes);
             if (e != cudaSuccess) {
                 cudaGetLastError();
-                cudaFree(dT);
                 raise(e == cudaErrorMemoryAllocation ? FR_ERR_HBM_BUDGET : FR_ERR_CUDA,
                       std::string("cannot hold the database diagonals: ") + cudaGetErrorString(e));
             }
             for (long long g = 0; g < db->G; ++g) {
                 if (tier == 1) {
-                    db->diags = (u64*)p;
+                    db->diags = (u64*)hold.p;
                     encode_group(c, dT, (long long)K, g, db->diags + (size_t)g * ell * nl * N, db_n1_enc(c, db.get()),
                                  nl);
                 } else {
-                    db->coeffs = (long long*)p;
+                    db->coeffs = (long long*)hold.p;
                     encode_group_int(c, dT, (long long)K, g, db->coeffs + (size_t)g * ell * N, db_n1_enc(c, db.get()));
                 }
             }
             CU(cudaStreamSynchronize(c->cur));
-            CU(cudaFree(dT));
+            hold.keep();
         } else {
-            db->templates = dT;
             CU(cudaStreamSynchronize(c->cur));
+            db->templates = (float*)hT.keep();
         }
         c->resident += db->bytes;
         c->dbs.insert(db.get());
@@ -1936,14 +1954,14 @@ fr_status fr_load_db_encrypted(fr_ctx* c, const uint64_t* cts, size_t K, size_t 
             raise(FR_ERR_HBM_BUDGET, "database exceeds the HBM budget");
         if (!prerotated)  // the negative giant-step keys of the server-side pre-rotation
             for (long j = 1; j * (long)c->n1 < (long)ell; ++j) rot_key(c, frh::galois_of_rotation(c->R, -j * (long)c->n1));
-        void* p = nullptr;
-        cudaError_t e = cudaMalloc(&p, db->bytes);
+        DevHold hold(c);
+        cudaError_t e = cudaMalloc(&hold.p, db->bytes);
         if (e != cudaSuccess) {
             cudaGetLastError();
             raise(e == cudaErrorMemoryAllocation ? FR_ERR_HBM_BUDGET : FR_ERR_CUDA,
                   std::string("cannot hold the encrypted diagonals: ") + cudaGetErrorString(e));
         }
-        db->diags = (u64*)p;
+        db->diags = (u64*)hold.p;
         // limbs 0..L of both components, 16 ciphertexts at a time: copy, NTT, the server-side
         // pre-rotation unless the enroller did it (Eq. eq:prerotation on ciphertexts: diagonal j n1 +
         // i, j >= 1, rotated by -j n1 with the negative giant-step key), then tiled in Montgomery form
@@ -1980,6 +1998,7 @@ fr_status fr_load_db_encrypted(fr_ctx* c, const uint64_t* cts, size_t K, size_t 
             }
         }
         CU(cudaStreamSynchronize(c->cur));
+        hold.keep();
         c->resident += db->bytes;
         c->dbs.insert(db.get());
         *out = db.release();
