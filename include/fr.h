@@ -377,14 +377,14 @@ fr_status fr_profile_only(fr_ctx* ctx, const char* prefix);
  * FR_NTT_TUNE=0): for N >= 2^14 it times each shape of a forward + inverse transform on this
  * GPU for one batch size per bucket (<= 4, <= 16, <= 64, > 64 limb-polynomials; best of 3
  * runs after a warm-up) and keeps the fastest. Shapes 0..3: radix-8 two-pass kernels (8
- * residues per thread), bit 0 = 8 columns per column-pass CTA (else 4), bit 1 without effect;
- * shape 4: one launch per transform, a cluster of CTAs per polynomial exchanging through
- * distributed shared memory (N <= 2^14; below 2^14 every bucket runs it unless the ring's
- * primes need the general reduction); shape 5 (N >= 2^14): radix-16 two-pass
- * kernels (16 residues per thread, one exchange per pass). A shape that N or the primes rule
- * out runs shape 0. shapes[4]
- * receives the chosen shape per bucket, us[24] (may be NULL) the measured microseconds,
- * bucket-major, 6 per bucket (-1: shape not available). */
+ * residues per thread), bit 0 = 8 columns per column-pass CTA (else 4), bit 1 without effect (2
+ * and 3 are not timed: they report 0's and 1's times and are never chosen); shape 4: one launch
+ * per transform, a cluster of CTAs per polynomial exchanging through distributed shared memory
+ * (N <= 2^14; below 2^14 every bucket runs it unless the ring's primes need the general
+ * reduction); shape 5 (N >= 2^14): radix-16 two-pass kernels (16 residues per thread, one
+ * exchange per pass). A shape that N or the primes rule out runs shape 0. shapes[4] receives the
+ * chosen shape per bucket, us[24] (may be NULL) the measured microseconds, bucket-major, 6 per
+ * bucket (-1: shape not available). */
 fr_status fr_ntt_tuning(const fr_ctx* ctx, uint32_t* shapes, double* us);
 /* Override the shape per bucket (shapes[4], each 0..5); drops the captured match graphs.
  * Every shape computes the same transform, bit for bit. */

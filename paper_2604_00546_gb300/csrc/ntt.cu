@@ -117,11 +117,16 @@ void tune_ntt(RingDev& R, cudaStream_t s, double* us, int reps) {
         for (int sh = 0; sh < FR_NTT_SHAPES; ++sh) t[sh] = 1e30;
         for (int r = 0; r <= reps; ++r)  // the first round warms up; the shapes take turns
             for (int sh = 0; sh < FR_NTT_SHAPES; ++sh) {
-                // shapes that would run another's kernels
-                if ((sh > 0 && sh < 4 && R.logN < 15) || (sh >= 4 && !R.fast) || (sh == 4 && R.logN > 14)) continue;
+                // shapes that would run another's kernels (2 and 3 are 0 and 1, and take their times)
+                if (sh == 2 || sh == 3 || (sh == 1 && R.logN < 15) || (sh >= 4 && !R.fast) || (sh == 4 && R.logN > 14))
+                    continue;
                 const double now = timed(bk, sh);
                 if (r > 0 && now < t[sh]) t[sh] = now;
             }
+        if (R.logN >= 15) {
+            t[2] = t[0];
+            t[3] = t[1];
+        }
         best[bk] = 0;
         double tbest = t[0];
         for (int sh = 0; sh < FR_NTT_SHAPES; ++sh) {
