@@ -1049,7 +1049,13 @@ void launch_ntt_t(const RingDev& R, const PolyBatch& b, bool inverse, cudaStream
     dim3 gr(SR / RPC, b.npolys);
     const size_t smr = (size_t)RPC * SC * sizeof(u64);
     if (!inverse) {
-        if (b.conv.t) launch_k(k_ntt_col<LOGR, false, KTC, true>, dim3(gc), dim3(tc), smc, st, R, b);
+        // A pass that converts keeps eight points' sums beside its elements: with 8 columns, 64
+        // registers a thread, it spilled 1.2 KB a thread (membership with shape 1 for the batches of
+        // up to 16: 4.55 ms, with 4 columns 4.47, as with shape 0), so it has 4 under shape 1 as well.
+        constexpr int KC = 4;
+        if (b.conv.t)
+            launch_k(k_ntt_col<LOGR, false, KC, true>, dim3((N >> LOGR) / KC, b.npolys), dim3(KC * SR / 8),
+                     (size_t)(SR * KC + 2 * SR) * sizeof(u64), st, R, b);
         else launch_k(k_ntt_col<LOGR, false, KTC, false>, dim3(gc), dim3(tc), smc, st, R, b);
         launch_k(k_ntt_row<LOGC, LOGR, false, E>, dim3(gr), dim3(RPC * TPR), smr, st, R, b, epi);
     } else {
