@@ -57,12 +57,13 @@ __device__ __forceinline__ void bconv(const BconvTarget& T, const u64 (&y)[NS][W
     } else {
         for (int w = 0; w < W; ++w) {
             AccK a{0, 0, 0};
+            Acc128 acc{0, 0};
 #pragma unroll
             for (int i = 0; i < NS; ++i) {
                 const u64 x = split30(y[i][w]);
                 mack(a, x, sum30(x), (u64)T.hat[i].y << 32 | T.hat[i].x);
+                if (i % 4 == 3) flushk(acc, a);  // operands below 2^61
             }
-            Acc128 acc{0, 0};
             flushk(acc, a);
             const u64 r = redc(mul_shoup(acc.hi, 1, T.one_s, T.q), acc.lo, T.q, T.qinv);
             out[w] = add_mod(r, mul_shoup(add[w], 1, T.one_s, T.q), T.q);
@@ -117,11 +118,12 @@ __device__ __forceinline__ void bconv_rt(const BconvTarget& T, const u64* __rest
 #pragma unroll
         for (int w = 0; w < W; ++w) {
             AccK a{0, 0, 0};
+            Acc128 acc{0, 0};
             for (int i = 0; i < ns; ++i) {
                 const u64 x = split30(src[(long long)i * N + idx[w]]);
                 mack(a, x, sum30(x), (u64)T.hat[i].y << 32 | T.hat[i].x);
+                if (i % 4 == 3) flushk(acc, a);
             }
-            Acc128 acc{0, 0};
             flushk(acc, a);
             out[w] = redc(mul_shoup(acc.hi, 1, T.one_s, T.q), acc.lo, T.q, T.qinv);
         }

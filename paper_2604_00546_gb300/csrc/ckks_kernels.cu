@@ -485,15 +485,15 @@ __global__ void __launch_bounds__(kBcThreads) k_tensor(const TensorJobs jobs, in
 //   P_j[t][i][k] = sum_{i' < n1, j n1 + i' < ell} baby_{i'}[t][i][k] * D'_{j n1 + i'}[i][k]
 // A CTA owns TP evaluation points of one limb. The n1 baby words (both polys) of its points are
 // staged in shared memory; JG thread groups split the n2 giant steps. The diagonals are streamed,
-// eight words a thread at a time; when every batch of eight is full (n1 a multiple of 8 dividing
-// ell), a word's register is refilled with the next batch's word as soon as it has been
-// multiplied, so the loads stay in flight.
+// U = 8 words a thread at a time (4 on chains with 61-bit primes, where only 4 products sum without
+// a carry); when every batch is full (n1 a multiple of U dividing ell), a word's register is refilled
+// with the next batch's word as soon as it has been multiplied, so the loads stay in flight.
 // Bound by HBM: the diagonals lie in tiles (diag_word), so a CTA reads one contiguous run of ell
 // kDiagTile words where rows 6.8 MB apart cost a fifth of the bandwidth, and already as 30-bit
 // halves. At the headline size (512 diagonals of 13 limbs, N = 2^16, 4.14 GB) 888 us, 4.67 TB/s ->
 // 637 us, 6.50 TB/s (tiles alone 668; 128 points x 4 rows 662; 64 x 8, two CTAs an SM, 666).
 // ---------------------------------------------------------------------------
-template <int TP>
+template <int TP, int U>
 __global__ void __launch_bounds__(256, 4) k_mac(const u64* __restrict__ babies, int cap_b,
                                                 const u64* __restrict__ diags, u64* __restrict__ out, int cap_o,
                                                 int nl, int n1, int n2, int ell, int JG,
@@ -516,7 +516,7 @@ __global__ void __launch_bounds__(256, 4) k_mac(const u64* __restrict__ babies, 
         for (int r = jg; r < 2 * n1; r += JG) sb[r * TP + pl] = split30(src[r * rstep]);
     }
     __syncthreads();
-    // the thread's work is a sequence of batches (giant step j, 8 diagonals from i0)
+    // the thread's work is a sequence of batches (giant step j, U diagonals from i0)
     int j = jg, i0 = 0;
     if (j >= n2) return;
     const u64* sbase = sb + pl;
@@ -527,9 +527,9 @@ __global__ void __launch_bounds__(256, 4) k_mac(const u64* __restrict__ babies, 
         mack(p[0], d, dsum, sq[0]);
         mack(p[1], d, dsum, sq[TP]);
     };
-    // after a batch of giant step j: add its sums (a flush adds less than 2^60 to the high word,
-    // so up to 64 products per giant step, 8 flushes, need no fold and the high word is reduced
-    // once before the REDC); when the giant step ends, store it
+    // after a batch of giant step j: add its sums (a product adds less than 2^58 to the high word, so
+    // up to 64 per giant step need no fold and the high word is reduced once before the REDC); when
+    // the giant step ends, store it
     auto close_batch = [&](AccK (&p)[2], int jc, bool last) {
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
@@ -543,17 +543,17 @@ __global__ void __launch_bounds__(256, 4) k_mac(const u64* __restrict__ babies, 
         }
     };
     const u64* dbase = diags + diag_word(i, k, 0, ell, N);
-    if (ell % n1 == 0 && n1 % 8 == 0) {
+    if (ell % n1 == 0 && n1 % U == 0) {
         // every batch is full: while a batch is multiplied, each word's register is refilled with
-        // the same word of the next batch, so eight loads per thread stay in flight throughout
-        u64 d[8];
+        // the same word of the next batch, so U loads per thread stay in flight throughout
+        u64 d[U];
         {
             const u64* D = dbase + (long long)j * n1 * kDiagTile;
 #pragma unroll
-            for (int u = 0; u < 8; ++u) d[u] = __ldcs(D + u * kDiagTile);
+            for (int u = 0; u < U; ++u) d[u] = __ldcs(D + u * kDiagTile);
         }
         for (;;) {
-            int jn = j, in = i0 + 8;
+            int jn = j, in = i0 + U;
             if (in == n1) {
                 jn = j + JG;
                 in = 0;
@@ -563,7 +563,7 @@ __global__ void __launch_bounds__(256, 4) k_mac(const u64* __restrict__ babies, 
             const u64* s0 = sbase + i0 * 2 * TP;
             AccK p[2] = {};
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
+            for (int u = 0; u < U; ++u) {
                 const u64 w = d[u];
                 if (more) d[u] = __ldcs(Dn + u * kDiagTile);
                 mul_word(p, w, s0 + u * 2 * TP);
@@ -580,18 +580,18 @@ __global__ void __launch_bounds__(256, 4) k_mac(const u64* __restrict__ babies, 
         const u64* D = dbase + (long long)(j * n1 + i0) * kDiagTile;
         const u64* s0 = sbase + i0 * 2 * TP;
         AccK p[2] = {};
-        if (i0 + 8 <= cnt) {
+        if (i0 + U <= cnt) {
             // full batch: no bounds checks
-            u64 d[8];
+            u64 d[U];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) d[u] = __ldcs(D + u * kDiagTile);
+            for (int u = 0; u < U; ++u) d[u] = __ldcs(D + u * kDiagTile);
 #pragma unroll
-            for (int u = 0; u < 8; ++u) mul_word(p, d[u], s0 + u * 2 * TP);
+            for (int u = 0; u < U; ++u) mul_word(p, d[u], s0 + u * 2 * TP);
         } else {
             for (int u = 0; i0 + u < cnt; ++u) mul_word(p, __ldcs(D + u * kDiagTile), s0 + u * 2 * TP);
         }
         // next batch
-        int jn = j, in = i0 + 8;
+        int jn = j, in = i0 + U;
         if (in >= cnt) {
             jn = j + JG;
             in = 0;
@@ -1356,14 +1356,14 @@ void launch_tensor(const TensorJobs& jobs, int J, int level, const DevPrime* pri
     launch_k(k_tensor, dim3(g), dim3(kBcThreads), 0, s, jobs, level, primes, N);
 }
 
-template <int TP>
+template <int TP, int U>
 static void launch_mac_t(const u64* babies, int cap_b, const u64* diags, u64* out, int cap_o, int nl, int n1, int n2,
                          int ell, const DevPrime* primes, int N, cudaStream_t s) {
     const int JG = std::max(1, std::min(256 / TP, n2));
     const size_t sm = (size_t)n1 * 2 * TP * sizeof(u64);
     static std::atomic<unsigned long long> attr{0};
-    smem_limit_once(k_mac<TP>, 200 * 1024, attr);
-    launch_k(k_mac<TP>, dim3(N / TP, nl), dim3(TP * JG), sm, s, babies, cap_b, diags, out, cap_o, nl, n1, n2, ell, JG,
+    smem_limit_once(k_mac<TP, U>, 200 * 1024, attr);
+    launch_k(k_mac<TP, U>, dim3(N / TP, nl), dim3(TP * JG), sm, s, babies, cap_b, diags, out, cap_o, nl, n1, n2, ell, JG,
              primes, N);
 }
 
@@ -1371,7 +1371,8 @@ static size_t mac_ring_smem(int B, int n1) {
     return ((size_t)2 * B * n1 * 2 * kMrTP + (size_t)kMrNS * kMrJG * kMpSD * kMrTP) * sizeof(u64);
 }
 
-bool mac_ring_fits(int n1, int ell, int N, int B) {
+bool mac_ring_fits(int n1, int ell, int N, int B, bool wide) {
+    if (wide) return false;  // it sums eight products between carries
     // instantiated for n1 = 32 (the headline BSGS split); other splits take k_mac_pipe or k_mac
     if (n1 != 32 || ell % n1 != 0 || N % kMrTP != 0 || B < 1 || B > 4) return false;
     const int n2 = ell / n1;
@@ -1409,7 +1410,8 @@ void launch_mac_ring(const u64* babies, long long baby_q, int cap_b, const u64* 
     }
 }
 
-bool mac_pipe_fits(int n1, int ell, int N) {
+bool mac_pipe_fits(int n1, int ell, int N, bool wide) {
+    if (wide) return false;  // as the ring
     const int n2 = n1 > 0 ? ell / n1 : 0;
     return n1 % kMpSD == 0 && n1 <= 64 && ell % n1 == 0 && n2 % 4 == 0 && N % 64 == 0;
 }
@@ -1456,13 +1458,20 @@ void launch_mac_pipe(const u64* babies, long long baby_q, int cap_b, const u64* 
     }
 }
 
-void launch_mac(const u64* babies, int cap_b, const u64* diags, u64* out, int cap_o, int nl, int n1, int n2, int ell,
-                const DevPrime* primes, int N, cudaStream_t s) {
+template <int U>
+static void launch_mac_u(const u64* babies, int cap_b, const u64* diags, u64* out, int cap_o, int nl, int n1, int n2,
+                         int ell, const DevPrime* primes, int N, cudaStream_t s) {
     // points per CTA: a whole tile unless its staged babies (n1 2 TP words) exceed 128 KiB
     const int TP = n1 <= 128 ? 64 : n1 <= 256 ? 32 : 16;
-    if (TP == 64) launch_mac_t<64>(babies, cap_b, diags, out, cap_o, nl, n1, n2, ell, primes, N, s);
-    else if (TP == 32) launch_mac_t<32>(babies, cap_b, diags, out, cap_o, nl, n1, n2, ell, primes, N, s);
-    else launch_mac_t<16>(babies, cap_b, diags, out, cap_o, nl, n1, n2, ell, primes, N, s);
+    if (TP == 64) launch_mac_t<64, U>(babies, cap_b, diags, out, cap_o, nl, n1, n2, ell, primes, N, s);
+    else if (TP == 32) launch_mac_t<32, U>(babies, cap_b, diags, out, cap_o, nl, n1, n2, ell, primes, N, s);
+    else launch_mac_t<16, U>(babies, cap_b, diags, out, cap_o, nl, n1, n2, ell, primes, N, s);
+}
+
+void launch_mac(const u64* babies, int cap_b, const u64* diags, u64* out, int cap_o, int nl, int n1, int n2, int ell,
+                bool wide, const DevPrime* primes, int N, cudaStream_t s) {
+    if (wide) launch_mac_u<4>(babies, cap_b, diags, out, cap_o, nl, n1, n2, ell, primes, N, s);
+    else launch_mac_u<8>(babies, cap_b, diags, out, cap_o, nl, n1, n2, ell, primes, N, s);
 }
 
 void launch_mac_ct(const u64* babies, int cap_b, const u64* diags, u64* out, int cap_o, int nl, int n1, int n2, int ell,

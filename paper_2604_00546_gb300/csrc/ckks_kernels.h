@@ -175,18 +175,19 @@ void launch_mac_ct(const u64* babies, int cap_b, const u64* diags, u64* out, int
 // through a shared-memory ring of asynchronous copies, every diagonal word read once for all B
 // queries (the sums of launch_mac: babies of query b at babies + b baby_q, [n1][2][cap_b][N];
 // outputs at out + b out_q, [n2][2][cap_o][N]); usable when mac_pipe_fits.
-bool mac_pipe_fits(int n1, int ell, int N);
+bool mac_pipe_fits(int n1, int ell, int N, bool wide);
 // The same sums as a persistent pipeline (k_mac_ring): one CTA per GPU slot runs point tiles in
 // turn, the next tile's diagonals and babies in flight while this one is multiplied; B = 1..4
 // queries, each diagonal word read once for all of them. Usable when mac_ring_fits.
-bool mac_ring_fits(int n1, int ell, int N, int B);
+bool mac_ring_fits(int n1, int ell, int N, int B, bool wide);
 void launch_mac_ring(const u64* babies, long long baby_q, int cap_b, const u64* diags, u64* out, long long out_q,
                      int cap_o, int nl, int n1, int ell, int B, const DevPrime* primes, int N, cudaStream_t s);
 void launch_mac_pipe(const u64* babies, long long baby_q, int cap_b, const u64* diags, u64* out, long long out_q,
                      int cap_o, int nl, int n1, int ell, int B, const DevPrime* primes, int N, cudaStream_t s);
-// The diagonal MAC of one query: babies [n1][2][cap_b][N], outputs [n2][2][cap_o][N].
+// The diagonal MAC of one query: babies [n1][2][cap_b][N], outputs [n2][2][cap_o][N]. wide: some
+// prime has 61 bits (the batched forms above then do not fit).
 void launch_mac(const u64* babies, int cap_b, const u64* diags, u64* out, int cap_o, int nl, int n1, int n2, int ell,
-                const DevPrime* primes, int N, cudaStream_t s);
+                bool wide, const DevPrime* primes, int N, cudaStream_t s);
 // Table schedule (Algorithm 1): out_g = sum_{m < ell} table[m] (.) D_{g,m} for g < G (evaluation form,
 // not rescaled); table [ell][2][cap_t][N], group g's diagonals at diags + g * dgrp.
 void launch_mac_table(const u64* table, int cap_t, const u64* diags, long long dgrp, int G, u64* out, int cap_o,

@@ -132,7 +132,8 @@ __device__ __forceinline__ u64 reduce_sum(const Acc128& a, const DevPrime& P) {
 // Products of residues below 2^60 from 30-bit halves: x = xh 2^30 + xl, y = yh 2^30 + yl,
 // x y = xl yl + (xl yh + xh yl) 2^30 + xh yh 2^60. Each partial product is below 2^60, so up
 // to 8 products sum in three 64-bit words, a1 holding the middle terms (below 2^64), with no
-// carries. split30 packs (xl, xh) into the low and high 32-bit words.
+// carries. split30 packs (xl, xh) into the low and high 32-bit words. Residues below 2^61 have
+// xh, yh below 2^31, partial products below 2^62 and middle terms below 2^62: up to 4 products.
 struct Acc3 {
     u64 a0, a1, a2;
 };
@@ -152,7 +153,8 @@ __device__ __forceinline__ void flush30(Acc128& acc, Acc3& a) {
 // Karatsuba form of the same sums, three multiply-adds per product:
 //   x y = xl yl + ((xl + xh)(yl + yh) - xl yl - xh yh) 2^30 + xh yh 2^60.
 // am = sum (xl + xh)(yl + yh) may wrap modulo 2^64, but the middle term sum (xl yh + xh yl) is
-// below 8 * 2 * 2^60 = 2^64 for up to 8 products, so am - a0 - a2 modulo 2^64 is exact.
+// below 8 * 2 * 2^60 = 2^64 for up to 8 products (residues below 2^61: 4 * 2 * 2^61, up to 4), so
+// am - a0 - a2 modulo 2^64 is exact.
 // xsum = xl + xh is passed in (it is shared by every product with the same x).
 struct AccK {
     u64 a0, am, a2;

@@ -100,6 +100,7 @@ struct fr_ctx {
     int comparator = 0;                  // 0: step interpolant; 1: hybrid (sign interpolant, then (1 + f_4) / 2)
     int cmp_depth = 0;                   // levels the threshold consumes: d2 (+ 4 for the hybrid)
     int work_level = 0;                  // level of the query inside fr_match
+    bool wide = false;                   // some prime has 61 bits: four 30-bit-half products a carry, not eight
     std::vector<ModUpTab*> d_modup;      // per level: digits_at(level) tables
     std::vector<ExtMap> modup_ext;       // per level: the extension polynomials to transform
     P2QTab* d_p2q = nullptr;
@@ -1439,6 +1440,7 @@ void build_tables(fr_ctx* c) {
         d.r2 = frh::mulm(r1, r1, q);
         d.one_s = frh::shoup_quot(1, q);
         twiddle_class(q, d);
+        c->wide = c->wide || q >> 60;
         fast = fast && d.cls != 2;
         cls1 |= (unsigned long long)(d.cls == 1) << i;
         cls2 |= (unsigned long long)(d.cls == 2) << i;
@@ -2491,11 +2493,11 @@ void ondemand_scores(fr_ctx* c, const BatchPlan& P, const u64* q, const std::vec
                 // k_mac_ring where its tiling fits, else k_mac_pipe. A single query runs k_mac
                 // below
                 int cnt = 1;
-                if (d->tier != 4 && (mac_ring_fits(n1, ell, N, 2) || mac_pipe_fits(n1, ell, N)))
+                if (d->tier != 4 && (mac_ring_fits(n1, ell, N, 2, c->wide) || mac_pipe_fits(n1, ell, N, c->wide)))
                     while (cnt < 4 && t + cnt < nb && sel[s0 + t + cnt] == b + cnt &&
                            diag_of(P.dbs[qs[b + cnt]]) == diag_of(d))
                         ++cnt;
-                if (d->tier != 4 && cnt > 1 && mac_ring_fits(n1, ell, N, cnt)) {
+                if (d->tier != 4 && cnt > 1 && mac_ring_fits(n1, ell, N, cnt, c->wide)) {
                     Prof p(c, "mac", 8.0 * N * nlx * ((double)ell + cnt * (2.0 * n1 + 2.0 * n2)));
                     launch_mac_ring(babies.p + (size_t)b * n1 * bw, (long long)n1 * bw, nlx, diag_of(d),
                                     Pj.p + (size_t)t * n2 * bw, (long long)n2 * bw, nlx, nlx, n1, ell, cnt, mprimes, N,
@@ -2504,7 +2506,7 @@ void ondemand_scores(fr_ctx* c, const BatchPlan& P, const u64* q, const std::vec
                     t += cnt - 1;
                     continue;
                 }
-                if (cnt > 1 && mac_pipe_fits(n1, ell, N)) {
+                if (cnt > 1 && mac_pipe_fits(n1, ell, N, c->wide)) {
                     Prof p(c, "mac", 8.0 * N * nlx * ((double)ell + cnt * (2.0 * n1 + 2.0 * n2)));
                     launch_mac_pipe(babies.p + (size_t)b * n1 * bw, (long long)n1 * bw, nlx, diag_of(d),
                                     Pj.p + (size_t)t * n2 * bw, (long long)n2 * bw, nlx, nlx, n1, ell, cnt, mprimes, N,
@@ -2529,7 +2531,7 @@ void ondemand_scores(fr_ctx* c, const BatchPlan& P, const u64* q, const std::vec
                 }
                 Prof p(c, "mac", 8.0 * N * nlx * ((double)ell + 2.0 * n1 + 2.0 * n2));
                 launch_mac(babies.p + (size_t)b * n1 * bw, nlx, diag_of(d), Pj.p + (size_t)t * n2 * bw, nlx, nlx, n1, n2,
-                           ell, mprimes, N, c->cur);
+                           ell, c->wide, mprimes, N, c->cur);
                 c->launches++;
             }
             if (!relin.empty()) {
