@@ -2,7 +2,7 @@
 #pragma once
 #include "ckks_kernels.h"
 
-// (sum_i y_i [B/b_i]_t + add) mod t, canonical; add < 2^61
+// (sum_i y_i [B/b_i]_t + add) mod t, canonical; add up to the add_max the target was made for
 template <int NS, int W>
 __device__ __forceinline__ void bconv(const BconvTarget& T, const u64 (&y)[NS][W], const u64 (&add)[W],
                                       u64 (&out)[W]) {

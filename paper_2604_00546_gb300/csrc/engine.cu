@@ -1310,8 +1310,8 @@ u64 inv_mod_2_64(u64 q) {
 u64 split30_host(u64 x) { return (x & 0x3fffffffull) | ((x >> 30) << 32); }
 
 // Target t of a base conversion with constants hat (one per source, all sources below 2^61): the
-// first mode of BconvTarget whose sums fit in 64 bits, with an addend below 2^61 in the first.
-BconvTarget bconv_target(u64 t, const std::vector<u64>& hat) {
+// first mode of BconvTarget whose sums fit in 64 bits with an addend of up to add_max.
+BconvTarget bconv_target(u64 t, const std::vector<u64>& hat, u128 add_max = (u128)1 << 61) {
     BconvTarget T;
     std::memset(&T, 0, sizeof(T));
     T.q = t;
@@ -1332,12 +1332,12 @@ BconvTarget bconv_target(u64 t, const std::vector<u64>& hat) {
         const u64 wl = ((u64)1 << S) - 1, wh = (t - 1) >> S, xl = 0xffffffffull, xh = 0x1fffffffull;
         const u128 a1 = (u128)group * (u128)wh * (xl + xh), a0 = (u128)group * (u128)wl * (xl + xh);
         const u64 c2 = (u64)(((u128)1 << (S + 32)) % t);
-        const u128 add = mode == 0 ? (u128)1 << 61 : 0;
+        const u128 add = mode == 0 ? add_max : 0;
         if (a1 >= two64 || c2 >> 32) continue;
         const u128 r = a0 + add + ((u128)0xffffffffu << S) + (a1 >> 32) * c2;
         if (!fold_ok(r)) continue;
         // mode 1: the folded pairs (below 2t) and an addend, folded once more
-        if (mode == 1 && !fold_ok((u128)((ns + 1) / 2) * 2 * t + ((u128)1 << 61))) continue;
+        if (mode == 1 && !fold_ok((u128)((ns + 1) / 2) * 2 * t + add_max)) continue;
         T.mode = mode;
         T.mul = (u32)1 << S;
         T.c2 = (u32)c2;
@@ -1537,6 +1537,7 @@ void build_tables(fr_ctx* c) {
         for (int j = 0; j < R.np; ++j) src.push_back(R.nq + j);
         std::vector<u64> pinv(R.nq), pinv_s(R.nq), pmod(R.nq), pmod_s(R.nq), ih, ht;
         trs = t;
+        const u64 qmax = *std::max_element(R.primes.begin(), R.primes.begin() + R.nq);
         for (int i = 0; i < R.nq; ++i) {
             const u64 q = R.primes[i];
             u64 P = 1;
@@ -1548,7 +1549,8 @@ void build_tables(fr_ctx* c) {
             frh::bconv_consts(R, src, i, ih, ht);
             t.t[i] = bconv_target(q, ht);
             for (u64& h : ht) h = frh::mulm(h, pinv[i], q);
-            trs.t[i] = bconv_target(q, ht);
+            // k_p2q_lift adds a residue of the dropped limb and -q_l mod q
+            trs.t[i] = bconv_target(q, ht, std::max((u128)1 << 61, (u128)qmax + q));
         }
         std::vector<uint4> post;
         for (int j = 0; j < R.np; ++j) post_of(R.nq + j, ih[j], post);
