@@ -605,7 +605,7 @@ __global__ void __launch_bounds__(256, 4) k_mac(const u64* __restrict__ babies, 
 
 // ---------------------------------------------------------------------------
 // Diagonal MAC with the diagonals streamed through shared memory (the on-demand schedule's S4
-// for B = 1..4 queries against one database, when n1 is a multiple of SD = 8 and n2 of JG): the
+// for B = 2..4 queries against one database, when n1 is a multiple of SD = 8 and n2 of JG): the
 // sums of k_mac, P_{b,j}[t][i][k] = sum_{i'} B_{b,i'}[t][i][k] * D'_{j n1 + i'}[i][k], every
 // diagonal word read once for all B queries. A CTA owns TP points of one limb and JG giant-step
 // rows: thread (jg, point) accumulates giant steps jb JG + jg for its point. The babies of the
@@ -717,7 +717,7 @@ __global__ void __launch_bounds__(TP * JG) k_mac_pipe(const u64* __restrict__ ba
 }
 
 // ---------------------------------------------------------------------------
-// Diagonal MAC as a persistent pipeline (the on-demand schedule's S4 for B = 1..4 queries against
+// Diagonal MAC as a persistent pipeline (the on-demand schedule's S4 for B = 2..4 queries against
 // one database): the sums of k_mac, P_{b,j}[t][i][k] = sum_{i'} B_{b,i'}[t][i][k] D'_{j n1 + i'}[i][k].
 // A tile is TP = 16 points of one limb; each CTA runs the tiles blockIdx.x, blockIdx.x + gridDim.x,
 // ... with 256 threads, thread (giant-step row jg, point) accumulating giant steps jb 16 + jg. One
@@ -1196,7 +1196,7 @@ __global__ void __launch_bounds__(256) k_fft_row(cplx* z, int logn, int logR, in
 
 // v 2^shift rounded half away from zero. Both factors of the encoder (1/n and Delta) are powers
 // of two, so the product is exact and the rounding is a shift of the mantissa: GB300 has two FP64
-// lanes an SM partition, and two multiplications and llround per coefficient cost more than the
+// lanes an SM, and two multiplications and llround per coefficient cost more than the
 // rest of the kernel. Values that do not fit go through the FP64 form.
 __device__ __forceinline__ long long scale_round(double v, int shift) {
     const u64 b = (u64)__double_as_longlong(v);
@@ -1374,7 +1374,7 @@ static size_t mac_ring_smem(int B, int n1) {
 bool mac_ring_fits(int n1, int ell, int N, int B, bool wide) {
     if (wide) return false;  // it sums eight products between carries
     // instantiated for n1 = 32 (the headline BSGS split); other splits take k_mac_pipe or k_mac
-    if (n1 != 32 || ell % n1 != 0 || N % kMrTP != 0 || B < 1 || B > 4) return false;
+    if (n1 != 32 || ell % n1 != 0 || N % kMrTP != 0 || B < 2 || B > 4) return false;
     const int n2 = ell / n1;
     if (n1 > 64 || n2 % kMrJG != 0 || (n2 / kMrJG) * (n1 / kMpSD) < kMrNS) return false;
     return mac_ring_smem(B, n1) <= 200u * 1024;
@@ -1402,7 +1402,6 @@ void launch_mac_ring(const u64* babies, long long baby_q, int cap_b, const u64* 
                      int cap_o, int nl, int n1, int ell, int B, const DevPrime* primes, int N, cudaStream_t s) {
     const int n2 = ell / n1;
     switch (B) {
-        case 1: launch_mac_ring_t<1>(babies, baby_q, cap_b, diags, out, out_q, cap_o, nl, n1, n2, primes, N, s); break;
         case 2: launch_mac_ring_t<2>(babies, baby_q, cap_b, diags, out, out_q, cap_o, nl, n1, n2, primes, N, s); break;
         case 3: launch_mac_ring_t<3>(babies, baby_q, cap_b, diags, out, out_q, cap_o, nl, n1, n2, primes, N, s); break;
         case 4: launch_mac_ring_t<4>(babies, baby_q, cap_b, diags, out, out_q, cap_o, nl, n1, n2, primes, N, s); break;
@@ -1416,7 +1415,7 @@ bool mac_pipe_fits(int n1, int ell, int N, bool wide) {
     return n1 % kMpSD == 0 && n1 <= 64 && ell % n1 == 0 && n2 % 4 == 0 && N % 64 == 0;
 }
 
-// TP points x JG giant-step rows per CTA. One query: 64 points x 4 rows. Two to four queries:
+// TP points x JG giant-step rows per CTA:
 // 16 points x 16 rows when the giant steps come in blocks of 16 (256 threads; 8 B KiB of staged
 // babies and a 64 KiB ring, so two CTAs, 16 warps, share an SM), else 32 points x 4 rows.
 template <int B, int TP, int JG>
@@ -1436,21 +1435,16 @@ template <int B>
 static void launch_mac_pipe_t(const u64* babies, long long baby_q, int cap_b, const u64* diags, u64* out,
                               long long out_q, int cap_o, int nl, int n1, int n2, const DevPrime* primes, int N,
                               cudaStream_t s) {
-    if constexpr (B == 1) {
-        launch_mac_pipe_s<1, 64, 4>(babies, baby_q, cap_b, diags, out, out_q, cap_o, nl, n1, n2, primes, N, s);
-    } else {
-        if (n2 % 16 == 0 && N % 16 == 0)
-            launch_mac_pipe_s<B, 16, 16>(babies, baby_q, cap_b, diags, out, out_q, cap_o, nl, n1, n2, primes, N, s);
-        else
-            launch_mac_pipe_s<B, 32, 4>(babies, baby_q, cap_b, diags, out, out_q, cap_o, nl, n1, n2, primes, N, s);
-    }
+    if (n2 % 16 == 0 && N % 16 == 0)
+        launch_mac_pipe_s<B, 16, 16>(babies, baby_q, cap_b, diags, out, out_q, cap_o, nl, n1, n2, primes, N, s);
+    else
+        launch_mac_pipe_s<B, 32, 4>(babies, baby_q, cap_b, diags, out, out_q, cap_o, nl, n1, n2, primes, N, s);
 }
 
 void launch_mac_pipe(const u64* babies, long long baby_q, int cap_b, const u64* diags, u64* out, long long out_q,
                      int cap_o, int nl, int n1, int ell, int B, const DevPrime* primes, int N, cudaStream_t s) {
     const int n2 = ell / n1;
     switch (B) {
-        case 1: launch_mac_pipe_t<1>(babies, baby_q, cap_b, diags, out, out_q, cap_o, nl, n1, n2, primes, N, s); break;
         case 2: launch_mac_pipe_t<2>(babies, baby_q, cap_b, diags, out, out_q, cap_o, nl, n1, n2, primes, N, s); break;
         case 3: launch_mac_pipe_t<3>(babies, baby_q, cap_b, diags, out, out_q, cap_o, nl, n1, n2, primes, N, s); break;
         case 4: launch_mac_pipe_t<4>(babies, baby_q, cap_b, diags, out, out_q, cap_o, nl, n1, n2, primes, N, s); break;

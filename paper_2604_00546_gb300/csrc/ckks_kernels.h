@@ -2,8 +2,6 @@
 #pragma once
 #include "kernels.h"
 
-#define FR_MAX_DIGIT_LIMBS 16
-
 // Fast base conversion, one target: sum_i y_i [B/b_i]_t mod t over at most 8 sources y_i < 2^61,
 // without a quotient per product (the scheme of mul_tw, dev_arith.cuh). hat[i] = (w mod 2^S, w >> S,
 // v mod 2^S, v >> S) with w = [B/b_i]_t and v = w 2^32 mod t; the products of several sources share
@@ -171,13 +169,13 @@ void launch_ip_sum(const IPSumJobs& jobs, int beta, int npos, int level, int kp,
 // babies [n1][2][cap_b][N]; diags: 2 ell rows (evaluation form, Montgomery); out [n2][3][cap_o][N].
 void launch_mac_ct(const u64* babies, int cap_b, const u64* diags, u64* out, int cap_o, int nl, int n1, int n2, int ell,
                    const DevPrime* primes, int N, cudaStream_t s);
-// The diagonal MAC of B = 1..4 queries against one database with the diagonals streamed
+// The diagonal MAC of B = 2..4 queries against one database with the diagonals streamed
 // through a shared-memory ring of asynchronous copies, every diagonal word read once for all B
 // queries (the sums of launch_mac: babies of query b at babies + b baby_q, [n1][2][cap_b][N];
 // outputs at out + b out_q, [n2][2][cap_o][N]); usable when mac_pipe_fits.
 bool mac_pipe_fits(int n1, int ell, int N, bool wide);
 // The same sums as a persistent pipeline (k_mac_ring): one CTA per GPU slot runs point tiles in
-// turn, the next tile's diagonals and babies in flight while this one is multiplied; B = 1..4
+// turn, the next tile's diagonals and babies in flight while this one is multiplied; B = 2..4
 // queries, each diagonal word read once for all of them. Usable when mac_ring_fits.
 bool mac_ring_fits(int n1, int ell, int N, int B, bool wide);
 void launch_mac_ring(const u64* babies, long long baby_q, int cap_b, const u64* diags, u64* out, long long out_q,

@@ -60,7 +60,6 @@ inline void smem_limit_once(K* k, int bytes, std::atomic<unsigned long long>& do
 }
 
 #define FR_MAX_PRIMES 64
-#define FR_MAX_DIGITS 16
 
 // Periodic prime assignment of a batch of polynomials: poly p uses prime idx[p % period].
 struct PrimeMap {
