@@ -70,62 +70,3 @@ __device__ __forceinline__ void bconv(const BconvTarget& T, const u64 (&y)[NS][W
         }
     }
 }
-
-// The same sum for a number of sources known at run time only, source i's elements at src + i N:
-// element idx[w] of the target's polynomial into out[w]. The elements of four sources are asked for
-// before the first is used (a small batch waits for each dependent load).
-template <int W>
-__device__ __forceinline__ void bconv_rt(const BconvTarget& T, const u64* __restrict__ src, int ns, int N,
-                                         const int (&idx)[W], u64 (&out)[W]) {
-    u64 sum[W], a0[W], a1[W];
-#pragma unroll
-    for (int w = 0; w < W; ++w) sum[w] = a0[w] = a1[w] = 0;
-    if (T.mode < 2) {
-        for (int i0 = 0; i0 < ns; i0 += 4) {
-            u64 y[4][W];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int w = 0; w < W; ++w) y[i][w] = i0 + i < ns ? src[(long long)(i0 + i) * N + idx[w]] : 0;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                if (i0 + i < ns) {
-                    const uint4 h = T.hat[i0 + i];
-#pragma unroll
-                    for (int w = 0; w < W; ++w) {
-                        const u32 xl = (u32)y[i][w], xh = (u32)(y[i][w] >> 32);
-                        a1[w] = mad_wide(xh, h.w, mad_wide(xl, h.y, a1[w]));
-                        a0[w] = mad_wide(xh, h.z, mad_wide(xl, h.x, a0[w]));
-                    }
-                    // a full pair (mode 1), or everything: into the sum
-                    if (i0 + i == ns - 1 || (T.mode == 1 && (i & 1))) {
-#pragma unroll
-                        for (int w = 0; w < W; ++w) {
-                            sum[w] += fold_top(mad_wide((u32)a1[w], T.mul, mad_wide((u32)(a1[w] >> 32), T.c2, a0[w])),
-                                               T.bsh, T.c);
-                            a0[w] = a1[w] = 0;
-                        }
-                    }
-                }
-            }
-        }
-#pragma unroll
-        for (int w = 0; w < W; ++w) {
-            const u64 f = fold_top(sum[w], T.bsh, T.c);
-            out[w] = min(f, f - T.q);
-        }
-    } else {
-#pragma unroll
-        for (int w = 0; w < W; ++w) {
-            AccK a{0, 0, 0};
-            Acc128 acc{0, 0};
-            for (int i = 0; i < ns; ++i) {
-                const u64 x = split30(src[(long long)i * N + idx[w]]);
-                mack(a, x, sum30(x), (u64)T.hat[i].y << 32 | T.hat[i].x);
-                if (i % 4 == 3) flushk(acc, a);
-            }
-            flushk(acc, a);
-            out[w] = redc(mul_shoup(acc.hi, 1, T.one_s, T.q), acc.lo, T.q, T.qinv);
-        }
-    }
-}

@@ -55,8 +55,7 @@ __device__ __forceinline__ void stage_targets(BconvTarget* s, const BconvTarget*
 // ---------------------------------------------------------------------------
 // ModUp: per digit, fast-convert the digit's limbs to every other position of Q_l u P
 // (coefficient form). The digit's own positions are not written: the inner product reads them
-// from the switched polynomial itself, in evaluation form. For up to kConvFused target polynomials
-// the conversion runs inside the column pass of the transform after it instead (PolyBatch::conv).
+// from the switched polynomial itself, in evaluation form.
 // in: coefficient form, job j at in + j * in_job, already times inv_hat if SCALED;
 // ext: [J][beta][npos][N]
 // Bound by integer multiplies before (75 of 99 us in arithmetic for 15 inputs at level 7, 4 limbs a
@@ -284,8 +283,8 @@ __global__ void __launch_bounds__(kIpThreads) k_ip_sum(const __grid_constant__ I
 }
 
 // ---------------------------------------------------------------------------
-// ModDown base conversion P -> Q_l (batches beyond kConvFused): acc: job j's P limbs in
-// coefficient form, times inv_hat; conv [J][2][level+1][N]
+// ModDown base conversion P -> Q_l: acc: job j's P limbs in coefficient form, times inv_hat; conv
+// [J][2][level+1][N]
 template <int NP>
 __device__ __forceinline__ void p2q_body(const u64* __restrict__ x, u64* __restrict__ o, const BconvTarget* st,
                                          int level, int N, int k) {

@@ -106,7 +106,7 @@ int launch_ntt_diags(const RingDev& R, const PolyBatch& b, u64* diags, int d0, i
 // src [rows][nl][N] (evaluation form) into rows row0.. of a database of total rows, Montgomery form
 void launch_tile_mont(const u64* src, int rows, u64* diags, long long row0, int total, int nl, const DevPrime* primes,
                       int N, cudaStream_t s);
-// Forward NTT of the P -> Q conversions of a ModDown (b.conv forms them) fused with its combine:
+// Forward NTT of the P -> Q conversions of a ModDown fused with its combine:
 // poly p of b is (job p / (2(level+1)), component, limb); the transformed values never reach
 // memory, the jobs' outputs do.
 int launch_ntt_moddown(const RingDev& R, const PolyBatch& b, const MDJobs& jobs, int npos, int level,
@@ -142,10 +142,6 @@ int launch_ntt_relin_rescale(const RingDev& R, const PolyBatch& b, const u64* ac
                               const u64* pinv, const u64* pinv_s, const RescaleTab* tab, u64* out, int out_cap,
                               long long out_bs, int mode, const u64* add, int add_cap, long long add_bs,
                               const u64* cres, cudaStream_t s);
-// Target polynomials up to which a base conversion runs inside the column pass of the transform
-// after it (PolyBatch::conv) instead of in its own kernel: one launch less, at the price of reading
-// the sources once per target.
-constexpr int kConvFused = 16;
 // ModUp of J inputs: coefficient form of input j at in + j in_job (scaled: already multiplied by
 // the digits' inv_hat); writes the positions of ext that are not the digit's own
 void launch_modup(const u64* in, long long in_job, u64* ext, const ModUpTab* tabs, int beta, int npos, int N, int J,

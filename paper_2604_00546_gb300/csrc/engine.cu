@@ -321,14 +321,16 @@ void ntt_pair(fr_ctx* c, u64* base, long long outer, int inner, int n, const Pri
     c->launches += launch_ntt(c->rd, b, inv, c->cur);
 }
 // ModUp of nj inputs and its forward NTT: in [nj][level+1][N] (coefficient form, times inv_hat) ->
-// the non-own positions of ext [nj][beta][npos][N]
+// the non-own positions of ext [nj][beta][npos][N]. The conversion is a launch of its own at every
+// size: formed inside the column pass of the transform instead (batches of at most 16 polynomials,
+// one launch less), it read its sources once per target and cost registers, and the matches were
+// slower or the same: N = 2^13 membership 1357 us apart, 1422 fused; 2^14 scores 981, 994; 2^16
+// membership 4442, 4492; 2^12 scores 131 either way.
 void ntt_modup(fr_ctx* c, const u64* in, u64* ext, int nj, int level) {
     const int N = c->R.N, beta = c->R.digits_at(level), npos = level + 1 + c->R.np;
     const int cnt = c->modup_ext[level].n;
     PolyBatch b{ext, (long long)beta * npos * N, 1, nj * cnt, PrimeMap{}, c->modup_ext[level]};
-    if (b.npolys <= kConvFused) {
-        b.conv = ConvSrc{c->d_modup[level]->t, (long long)sizeof(ModUpTab), in, (long long)(level + 1) * N, 0};
-    } else {
+    {
         Prof p(c, "modup", 8.0 * N * nj * ((double)beta * npos));
         launch_modup(in, (long long)(level + 1) * N, ext, c->d_modup[level], beta, npos, N, nj, true, c->cur);
         c->launches++;
@@ -337,16 +339,12 @@ void ntt_modup(fr_ctx* c, const u64* in, u64* ext, int nj, int level) {
     c->launches += launch_ntt(c->rd, b, false, c->cur);
 }
 // the conversions P -> Q of nj accumulators acc [nj][2][npos][N] at `level` (P limbs in
-// coefficient form, times inv_hat), as the input of the forward NTT b [nj][2][level+1] of them;
-// region: where a conversion launched of its own is timed (null: nowhere)
-void p2q_into(fr_ctx* c, const u64* acc, int nj, int level, PolyBatch& b, const char* region = "moddown") {
+// coefficient form, times inv_hat) into conv [nj][2][level+1][N]; region: where they are timed
+// (null: nowhere)
+void p2q(fr_ctx* c, const u64* acc, int nj, int level, u64* conv, const char* region = "moddown") {
     const long long N = c->R.N, npos = level + 1 + c->R.np;
-    if (b.npolys <= kConvFused) {
-        b.conv = ConvSrc{c->d_p2q->t, 0, acc + (level + 1) * N, npos * N, c->R.np};
-        return;
-    }
     Prof p(c, region, 8.0 * N * nj * 2.0 * (c->R.np + level + 1));
-    launch_p2q(acc, 2 * npos * N, (int)npos, level, b.base, c->d_p2q, (int)N, nj, c->cur);
+    launch_p2q(acc, 2 * npos * N, (int)npos, level, conv, c->d_p2q, (int)N, nj, c->cur);
     c->launches++;
 }
 // all limbs 0..level of a ciphertext batch [B][2][cap][N]
@@ -450,7 +448,7 @@ void ks_finish(fr_ctx* c, int level, const std::vector<const KSReq*>& reqs, cons
     // counts the transform's 16 B per coefficient (its butterflies); the fused epilogue's reads of
     // acc and the addend are not added
     PolyBatch pb{conv.p, (long long)(level + 1) * N, level + 1, nj * 2 * (level + 1), pm_level(level)};
-    p2q_into(c, acc.p, nj, level, pb);
+    p2q(c, acc.p, nj, level, conv.p);
     Prof p(c, "ntt", 16.0 * nj * 2 * (level + 1) * N);
     c->launches += launch_ntt_moddown(c->rd, pb, md, npos, level, c->d_pinv, c->d_pinv_s, c->cur);
 }
@@ -600,7 +598,7 @@ void keyswitch_sums(fr_ctx* c, int level, const std::vector<KSReq>& reqs, const 
         }
         PolyBatch pb{conv.p + (size_t)o0 * 2 * (level + 1) * N, (long long)(level + 1) * N, level + 1,
                      no * 2 * (level + 1), pm_level(level)};
-        p2q_into(c, accs.p + (size_t)o0 * aw, no, level, pb);
+        p2q(c, accs.p + (size_t)o0 * aw, no, level, pb.base);
         Prof p(c, "ntt", 16.0 * no * 2 * (level + 1) * N);
         c->launches += launch_ntt_moddown(c->rd, pb, md, npos, level, c->d_pinv, c->d_pinv_s, c->cur);
     }
@@ -3654,7 +3652,7 @@ extern "C" fr_status fr_rotate_noalloc(fr_ctx* c, const uint64_t* d_in, uint32_t
         MDJobs md;
         md.j[0] = MDJob{acc, e, res, l + 1, l + 1, 1, (u32)g};
         PolyBatch pc{conv, (long long)L1N, l + 1, 2 * (l + 1), pl};
-        p2q_into(c, acc, 1, l, pc, nullptr);  // no events: the caller may be capturing this stream
+        p2q(c, acc, 1, l, conv, nullptr);  // no events: the caller may be capturing this stream
         c->launches += launch_ntt_moddown(c->rd, pc, md, npos, l, c->d_pinv, c->d_pinv_s, st);
         PolyBatch out{d_out, 2 * (long long)L1N, 2 * (l + 1), 2 * (l + 1), pl};
         out.src = res;

@@ -75,21 +75,6 @@ struct ExtMap {
     unsigned char lo[8] = {}, ns[8] = {};
 };
 
-struct BconvTarget;
-
-// A batch whose forward transform starts from a fast base conversion: the column pass forms
-// poly p's coefficients itself, target `pos` of digit d's table from the digit's sources, instead
-// of reading them. With an extension map (ModUp) p names (job, d, pos) as above and the sources
-// are limbs lo[d] .. of src + job src_job; without one (ModDown) pos = p % inner, job = p / inner,
-// d = 0 and the sources are ns limbs from src + job src_job. Sources come multiplied by inv_hat.
-struct ConvSrc {
-    const BconvTarget* t = nullptr;  // digit 0's targets
-    long long t_bytes = 0;           // from one digit's targets to the next's
-    const u64* src = nullptr;
-    long long src_job = 0;
-    int ns = 0;                      // sources (no extension map)
-};
-
 // A batch of N-point polynomials: poly p lives at base + (p / inner) * outer + (p % inner) * N
 // and uses prime pm.idx[p % pm.period]. With an extension map (ext.n > 0) poly p is polynomial
 // p % ext.n of the extension at base + (p / ext.n) * outer. Everything is in the launch's
@@ -126,8 +111,6 @@ struct PolyBatch {
         const u64 *pinv = nullptr, *pinv_s = nullptr;
         int npos = 0, l = 0;
     } rs{};
-    // optional (forward): the coefficients come from a base conversion
-    ConvSrc conv{};
 };
 
 // NTT batch-size buckets for the tuned tile shapes: <= 4, <= 16, <= 64, larger.

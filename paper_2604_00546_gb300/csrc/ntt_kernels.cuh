@@ -28,7 +28,6 @@
 #include <cooperative_groups.h>
 #include <type_traits>
 
-#include "bconv.cuh"
 #include "ckks_kernels.h"
 
 namespace ntt_kernels {
@@ -56,42 +55,6 @@ __device__ __forceinline__ u64* poly_at(const PolyBatch& b, int p, int N, int* p
     }
     *prime = b.pm.idx[p % b.pm.period];
     return b.base + (long long)(p / b.inner) * b.outer + (long long)(p % b.inner) * N;
-}
-
-// The coefficients of poly p that a base conversion gives: v[e] = element at(e). Eight elements
-// share each pass over the sources, whose number stays a loop (unrolled for every count, the
-// conversion filled the instruction cache).
-template <int RB, class At>
-__device__ __forceinline__ void conv_load(u64 (&v)[1 << RB], const PolyBatch& b, int p, int N, At at) {
-    int d = 0, pos, job, lo = 0, ns = b.conv.ns;
-    if (b.ext.n) {
-        ext_at(b.ext, p % b.ext.n, &d, &pos);
-        job = p / b.ext.n;
-        lo = b.ext.lo[d];
-        ns = b.ext.ns[d];
-    } else {
-        pos = p % b.inner;
-        job = p / b.inner;
-    }
-    const BconvTarget* Tg =
-        reinterpret_cast<const BconvTarget*>(reinterpret_cast<const char*>(b.conv.t) + d * b.conv.t_bytes) + pos;
-    const u64* src = b.conv.src + job * b.conv.src_job + (long long)lo * N;
-    __shared__ BconvTarget T;
-    constexpr int kWords = sizeof(BconvTarget) / 16;
-    if (threadIdx.x < kWords)
-        reinterpret_cast<uint4*>(&T)[threadIdx.x] = __ldg(reinterpret_cast<const uint4*>(Tg) + threadIdx.x);
-    __syncthreads();
-    constexpr int W = 8;
-#pragma unroll
-    for (int e0 = 0; e0 < (1 << RB); e0 += W) {
-        int idx[W];
-        u64 o[W];
-#pragma unroll
-        for (int w = 0; w < W; ++w) idx[w] = at(e0 + w);
-        bconv_rt<W>(T, src, ns, N, idx, o);
-#pragma unroll
-        for (int w = 0; w < W; ++w) v[e0 + w] = o[w];
-    }
 }
 
 template <int W>
@@ -595,7 +558,7 @@ __device__ __forceinline__ void ntt_col_body(u64 (&v)[1 << RB], const DevPrime& 
     }
 }
 
-template <int RB, int LOG, bool INV, int KTC, bool C2, bool CONV>
+template <int RB, int LOG, bool INV, int KTC, bool C2>
 __device__ __forceinline__ void ntt_col(const RingDev& R, const PolyBatch& b, u64* sm) {
     constexpr int S = 1 << LOG, T = KTC * (S >> RB);
     const int p = blockIdx.y, N = R.N, C = N >> LOG;
@@ -606,16 +569,12 @@ __device__ __forceinline__ void ntt_col(const RingDev& R, const PolyBatch& b, u6
     const int col = threadIdx.x & (KTC - 1), tau = threadIdx.x / KTC;
     constexpr int L0 = PhaseInfo<RB, LOG, INV, 0>::LO;
     u64 v[1 << RB];
-    auto at = [&](int e) { return phase_x<RB, L0>(tau, e) * C + (int)blockIdx.x * KTC + col; };
-    if constexpr (!CONV) {
 #pragma unroll
-        for (int e = 0; e < (1 << RB); ++e) v[e] = xin[at(e)];
-    }
+    for (int e = 0; e < (1 << RB); ++e) v[e] = xin[phase_x<RB, L0>(tau, e) * C + (int)blockIdx.x * KTC + col];
     uint4* sw = reinterpret_cast<uint4*>(sm + S * KTC);  // twiddles [0, S)
 #pragma unroll
     for (int i = 0; i < (S + T - 1) / T; ++i)
         if (i * T + (int)threadIdx.x < S) sw[i * T + threadIdx.x] = __ldg(tw + i * T + threadIdx.x);
-    if constexpr (CONV) conv_load<RB>(v, b, p, N, at);
     const DevPrime P = R.primes[pi];
     const uint4* post = poly_post(b, p);
     __syncthreads();
@@ -630,12 +589,12 @@ __device__ __forceinline__ void ntt_col(const RingDev& R, const PolyBatch& b, u6
             INV && !(C2 && cls == 2) ? finish<EpiStore, false>(v[e], P) : v[e];
 }
 
-template <int LOG, bool INV, int KTC, bool CONV>
-__global__ void __launch_bounds__(KTC * (1 << LOG) / 8, CONV ? 4 : 5) k_ntt_col(const __grid_constant__ RingDev R, const __grid_constant__ PolyBatch b) {
+template <int LOG, bool INV, int KTC>
+__global__ void __launch_bounds__(KTC * (1 << LOG) / 8, 5) k_ntt_col(const __grid_constant__ RingDev R, const __grid_constant__ PolyBatch b) {
     pdl_wait();
     pdl_trigger();
     extern __shared__ __align__(16) u64 sm[];
-    ntt_col<3, LOG, INV, KTC, true, CONV>(R, b, sm);
+    ntt_col<3, LOG, INV, KTC, true>(R, b, sm);
 }
 
 // row pass: one CTA = RPC rows of S contiguous elements (128 threads), S/8 threads per row
@@ -821,7 +780,7 @@ __device__ __forceinline__ void ntt_cluster_body(u64 (&v)[8], const PolyBatch& b
     }
 }
 
-template <int LOGR, int LOGC, int CL, bool INV, class E, bool CONV>
+template <int LOGR, int LOGC, int CL, bool INV, class E>
 __global__ void __launch_bounds__(ClusterShape<LOGR, LOGC, CL>::T)
     k_ntt_cluster(const __grid_constant__ RingDev R, const __grid_constant__ PolyBatch b,
                   const __grid_constant__ E epi) {
@@ -858,14 +817,10 @@ __global__ void __launch_bounds__(ClusterShape<LOGR, LOGC, CL>::T)
         }
     } else {
         const int col = threadIdx.x % KTC, tauc = threadIdx.x / KTC;
-        auto at = [&](int e) { return phase_x<3, PhaseInfo<3, LOGR, false, 0>::LO>(tauc, e) * C + rank * KTC + col; };
-        if constexpr (CONV) {
-            conv_load<3>(v, b, p, N, at);
-        } else {
-            const u64* xin = poly_in(b, p, N, x);
+        const u64* xin = poly_in(b, p, N, x);
 #pragma unroll
-            for (int e = 0; e < 8; ++e) v[e] = xin[at(e)];
-        }
+        for (int e = 0; e < 8; ++e)
+            v[e] = xin[phase_x<3, PhaseInfo<3, LOGR, false, 0>::LO>(tauc, e) * C + rank * KTC + col];
     }
     const DevPrime P = R.primes[pi];  // class 0 or 1: the launcher checks
     ld_async_wait();
@@ -874,10 +829,10 @@ __global__ void __launch_bounds__(ClusterShape<LOGR, LOGC, CL>::T)
     else ntt_cluster_body<LOGR, LOGC, CL, INV, 1>(v, b, x, P, p, rank, sm, epi);
 }
 
-template <int LOGR, int LOGC, int CL, bool INV, class E, bool CONV>
+template <int LOGR, int LOGC, int CL, bool INV, class E>
 void launch_cluster_k(const RingDev& R, const PolyBatch& b, cudaStream_t st, const E& epi) {
     using Sh = ClusterShape<LOGR, LOGC, CL>;
-    auto* k = k_ntt_cluster<LOGR, LOGC, CL, INV, E, CONV>;
+    auto* k = k_ntt_cluster<LOGR, LOGC, CL, INV, E>;
     static std::atomic<unsigned long long> lim{0};
     if (Sh::smem > 48 * 1024) smem_limit_once(k, (int)Sh::smem, lim);
     cudaLaunchConfig_t cfg{};
@@ -901,9 +856,8 @@ template <int LOGR, int LOGC, class E>
 void launch_ntt_cluster(const RingDev& R, const PolyBatch& b, bool inverse, cudaStream_t st, const E& epi) {
     // 1024 elements a CTA, 2048 at N = 2^14
     constexpr int CL = LOGR + LOGC >= 13 ? 8 : LOGR + LOGC == 12 ? 4 : LOGR + LOGC == 11 ? 2 : 1;
-    if (inverse) launch_cluster_k<LOGR, LOGC, CL, true, EpiStore, false>(R, b, st, EpiStore{});
-    else if (b.conv.t) launch_cluster_k<LOGR, LOGC, CL, false, E, true>(R, b, st, epi);
-    else launch_cluster_k<LOGR, LOGC, CL, false, E, false>(R, b, st, epi);
+    if (inverse) launch_cluster_k<LOGR, LOGC, CL, true, EpiStore>(R, b, st, EpiStore{});
+    else launch_cluster_k<LOGR, LOGC, CL, false, E>(R, b, st, epi);
 }
 
 // ---------------------------------------------------------------------------
@@ -914,13 +868,13 @@ void launch_ntt_cluster(const RingDev& R, const PolyBatch& b, bool inverse, cuda
 // ---------------------------------------------------------------------------
 constexpr int kCol16 = 8;  // columns of a column-pass CTA: 64-byte row segments
 
-template <int LOG, bool INV, bool CONV>
-__global__ void __launch_bounds__(kCol16 * (1 << LOG) / 16, (INV ? 6 : CONV ? 4 : 5) * (256 >> LOG))
+template <int LOG, bool INV>
+__global__ void __launch_bounds__(kCol16 * (1 << LOG) / 16, (INV ? 6 : 5) * (256 >> LOG))
     k_ntt_col16(const __grid_constant__ RingDev R, const __grid_constant__ PolyBatch b) {
     pdl_wait();
     pdl_trigger();
     extern __shared__ __align__(16) u64 sm[];
-    ntt_col<4, LOG, INV, kCol16, false, CONV>(R, b, sm);
+    ntt_col<4, LOG, INV, kCol16, false>(R, b, sm);
 }
 
 // Row pass: 128 threads, each warp on its own 512 contiguous elements (2 rows of 256 points or 4
@@ -1029,12 +983,11 @@ void launch_ntt_r16(const RingDev& R, const PolyBatch& b, bool inverse, cudaStre
     const int tc = kCol16 * SR / 16;
     const size_t smc = (size_t)(SR * kCol16 + 2 * SR) * sizeof(u64), smr = (size_t)2048 * sizeof(u64);
     if (!inverse) {
-        if (b.conv.t) launch_k(k_ntt_col16<LOGR, false, true>, gc, dim3(tc), smc, st, R, b);
-        else launch_k(k_ntt_col16<LOGR, false, false>, gc, dim3(tc), smc, st, R, b);
+        launch_k(k_ntt_col16<LOGR, false>, gc, dim3(tc), smc, st, R, b);
         launch_k(k_ntt_row16<LOGC, false, E>, gr, dim3(128), smr, st, R, b, epi);
     } else {
         launch_k(k_ntt_row16<LOGC, true, EpiStore>, gr, dim3(128), smr, st, R, b, EpiStore{});
-        launch_k(k_ntt_col16<LOGR, true, false>, gc, dim3(tc), smc, st, R, b);
+        launch_k(k_ntt_col16<LOGR, true>, gc, dim3(tc), smc, st, R, b);
     }
 }
 
@@ -1049,18 +1002,11 @@ void launch_ntt_t(const RingDev& R, const PolyBatch& b, bool inverse, cudaStream
     dim3 gr(SR / RPC, b.npolys);
     const size_t smr = (size_t)RPC * SC * sizeof(u64);
     if (!inverse) {
-        // A pass that converts keeps eight points' sums beside its elements: with 8 columns, 64
-        // registers a thread, it spilled 1.2 KB a thread (membership with shape 1 for the batches of
-        // up to 16: 4.55 ms, with 4 columns 4.47, as with shape 0), so it has 4 under shape 1 as well.
-        constexpr int KC = 4;
-        if (b.conv.t)
-            launch_k(k_ntt_col<LOGR, false, KC, true>, dim3((N >> LOGR) / KC, b.npolys), dim3(KC * SR / 8),
-                     (size_t)(SR * KC + 2 * SR) * sizeof(u64), st, R, b);
-        else launch_k(k_ntt_col<LOGR, false, KTC, false>, dim3(gc), dim3(tc), smc, st, R, b);
+        launch_k(k_ntt_col<LOGR, false, KTC>, dim3(gc), dim3(tc), smc, st, R, b);
         launch_k(k_ntt_row<LOGC, LOGR, false, E>, dim3(gr), dim3(RPC * TPR), smr, st, R, b, epi);
     } else {
         launch_k(k_ntt_row<LOGC, LOGR, true, EpiStore>, dim3(gr), dim3(RPC * TPR), smr, st, R, b, EpiStore{});
-        launch_k(k_ntt_col<LOGR, true, KTC, false>, dim3(gc), dim3(tc), smc, st, R, b);
+        launch_k(k_ntt_col<LOGR, true, KTC>, dim3(gc), dim3(tc), smc, st, R, b);
     }
 }
 

@@ -1,8 +1,8 @@
 """fr_launch_count counts kernels: a transform is one by the cluster kernel (rings up to 2^13 without
 primes of class 2, and shape 4 at 2^14) and two by the two-pass kernels. Expected figures are the
-calls' kernels, t a transform: upload and export t; rescale 2 t and the lift; rotation 4 t and the
-inner product (both conversions run inside transforms at these sizes); product the same and the
-tensor product; rotation on caller's buffers 5 t, the conversion and the inner product."""
+calls' kernels, t a transform: upload and export t; rescale 2 t and the lift; rotation 4 t, two
+conversions and the inner product; product the same and the tensor product; rotation on caller's
+buffers 5 t, two conversions and the inner product."""
 import numpy as np
 import pytest
 
@@ -34,9 +34,9 @@ def test_counts_of_the_calls(log_n, chain, shape, t):
     assert n == t
     assert count(ct.export)[0] == t
     assert count(lambda: ctx.rescale(ct))[0] == 2 * t + 1
-    assert count(lambda: ctx.rotate(ct, 3))[0] == 4 * t + 1
-    assert count(lambda: ctx.mul_relin(ct, ct))[0] == 4 * t + 2
+    assert count(lambda: ctx.rotate(ct, 3))[0] == 4 * t + 3
+    assert count(lambda: ctx.mul_relin(ct, ct))[0] == 4 * t + 4
     d = torch.from_numpy(a.view(np.int64)).to("cuda:0")
     torch.cuda.synchronize()
-    assert count(lambda: ctx.rotate_noalloc(d.data_ptr(), 2, 3, d.data_ptr()))[0] == 5 * t + 2
+    assert count(lambda: ctx.rotate_noalloc(d.data_ptr(), 2, 3, d.data_ptr()))[0] == 5 * t + 3
     ctx.sync()
