@@ -772,11 +772,11 @@ def run_reference(args):
 # line are these shares of the timed step; otherwise they come from the profiled replays and the
 # NTT traffic is null.
 LAUNCH_LIST = {
-    "sha256": ["969f0e566dcc25179c4566297aa52dbbca0d29ea2d21c99a4028238a1b6cc198"],
-    "share": {"ntt": 0.5839, "mac": 0.1457, "ip": 0.1370, "modup": 0.0399, "moddown": 0.0500, "rescale": 0.0110,
-              "tensor": 0.0324, "misc": 0.0, "copy": 0.0},
-    "ntt_dram_per_alg_byte": 1.755,
-    "keyswitch_dram_gbs": 3724.4,
+    "sha256": ["e3655d394a2a4d38574ec61af7d31fb6ca7047b7d7949df66cf54370656fcf44"],
+    "share": {"ntt": 0.5589, "mac": 0.1447, "ip": 0.1357, "modup": 0.0601, "moddown": 0.0574, "rescale": 0.0111,
+              "tensor": 0.0321, "misc": 0.0, "copy": 0.0},
+    "ntt_dram_per_alg_byte": 1.752,
+    "keyswitch_dram_gbs": 3318.7,
 }
 
 # kernel name prefix -> region class, for reading a launch list
