@@ -39,7 +39,7 @@ def test_capture_under_profiling_records_no_region():
 
 
 @pytest.mark.parametrize("in_off,out_off", [(0, 0), (0, 1), (1, 0), (1, 1), (None, 0), (None, 1)])
-@pytest.mark.parametrize("log_n", [12, 13, 14, 16])
+@pytest.mark.parametrize("log_n", [10, 11, 12, 13, 14, 16])
 def test_any_word_address(log_n, in_off, out_off):
     """Input and output at any word, or in place (in_off None): buffers off a 16-byte boundary leave
     the kernels that move 16 bytes, and c1 is copied before the conversion reads it. The words around
